@@ -180,10 +180,9 @@ void layout(ipm_ctx *c, char *base) {
   d.relpos = upload(cv, pl.relpos, st);
   d.sri = upload(cv, c->S.sri, st);
   d.build = upload(cv, pl.build_tasks, st);
-  d.gemm = upload(cv, pl.gemm_tasks, st);
   d.potrf = upload(cv, pl.potrf_tasks, st);
-  d.trsm = upload(cv, pl.trsm_tasks, st);
-  d.syrk = upload(cv, pl.syrk_tasks, st);
+  d.trsm = upload(cv, pl.trsm_ents, st);
+  d.upd = upload(cv, pl.upd_ents, st);
   d.gath = upload(cv, pl.gath_tasks, st);
   d.sdiag = upload(cv, pl.sdiag_tasks, st);
   d.sgemv = upload(cv, pl.sgemv_tasks, st);

@@ -13,7 +13,7 @@ namespace gipm {
 struct DevPlan {
   const FrontInfo *fronts;
   const int32_t *children, *inv, *relpos, *sri;
-  const Task *build, *gemm, *potrf, *trsm, *syrk, *gath, *sdiag, *sgemv, *rgemv;
+  const Task *build, *potrf, *trsm, *upd, *gath, *sdiag, *sgemv, *rgemv;
   const int64_t *toff;
   const Task *fs_inv, *ps_tasks;  // persistent FP32 solve
   const int64_t *ps_pbase;        // per front: first partial-sum row of its backward tasks
@@ -62,8 +62,6 @@ struct Carve {
   }
 };
 
-constexpr int kGemmTile = 64;
-constexpr int kTrsmRows = 128;
 constexpr int kGathPos = 256;
 constexpr int kSolveRows = 128;
 constexpr int kSolveCols = 256;

@@ -1,6 +1,7 @@
 // Internal data structures of the solver library (host + device).
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 #include <string>
 #include <vector>
@@ -83,14 +84,79 @@ enum SolveTaskKind : int32_t {
 };
 
 // Work of one level of the supernodal tree, as ranges into the task arrays.
-struct StepRange {
-  int32_t gemm_b, gemm_e, potrf_b, potrf_e, trsm_b, trsm_e;
+//
+// Panel solves and trailing updates of the FMA-pipe factor are numbered by
+// block: a launch's entries [b, e) hold one Task {front, a = number of the
+// front's first block of the launch, b = first column of the step} per front,
+// and a block finds its front by bisection, so a front's O((nf / tile)^2)
+// update tiles need no list.
+constexpr int kTrsmRows = 16;  // rows per batch of a panel solve's blocks
+// Batches per block, for `rows` rows in the launch: one while every block has an
+// SM of its own (a launch then lasts one batch), up to four beyond that, which
+// read the diagonal block once per 64 rows.
+inline int trsm_batches(int64_t rows) {
+  constexpr int64_t kSms = 152;
+  const int64_t b = (rows + kTrsmRows * kSms - 1) / (kTrsmRows * kSms);
+  return (int)(b < 1 ? 1 : b > 4 ? 4 : b);
+}
+constexpr int kUpdTile64 = 32;  // update tile, FP64
+constexpr int kUpdTile32 = 64;  // update tile, FP32
+// One trailing-update launch: columns from min(k1, ncol) to min(clim, ncol) of
+// the panels, and with_u the update matrices, by the columns [k0, min(k1, ncol)).
+struct UpdRange {
+  int32_t b = 0, e = 0, n = 0;  // entries, blocks
+  int32_t k0 = 0, k1 = 0, clim = 0, with_u = 0;
 };
+struct StepRange {
+  int32_t potrf_b = 0, potrf_e = 0, trsm_b = 0, trsm_e = 0, trsm_n = 0, trsm_bat = 1;
+  UpdRange upd64;         // FP64: everything right of the step's columns
+  UpdRange upd32, sup32;  // FP32: the rest of the super-step; at its end everything past it
+};
+
+// Tiles of a front's trailing update (TS x TS; see UpdRange): panel column tiles
+// from c0 = min(k1, ncol), each with the row tiles from its own first column
+// down, then the lower triangle of the update matrix's tiles.
+struct UpdTile {
+  int32_t r, c, cend;  // first row and column (front-local), end of its columns
+};
+#ifdef __CUDACC__
+#define GIPM_HD __host__ __device__
+#else
+#define GIPM_HD
+#endif
+GIPM_HD inline int64_t upd_tiles(int ncol, int nrow, int k1, int clim, int with_u, int TS) {
+  const int c0 = k1 < ncol ? k1 : ncol, lim = clim < ncol ? clim : ncol;
+  const int64_t A = (ncol + nrow - c0 + TS - 1) / TS, J = lim > c0 ? (lim - c0 + TS - 1) / TS : 0;
+  const int64_t B = with_u ? (nrow + TS - 1) / TS : 0;
+  return J * A - J * (J - 1) / 2 + B * (B + 1) / 2;
+}
+GIPM_HD inline UpdTile upd_decode(int ncol, int nrow, int k1, int clim, int with_u, int TS, int t) {
+  const int c0 = k1 < ncol ? k1 : ncol, lim = clim < ncol ? clim : ncol;
+  const int A = (ncol + nrow - c0 + TS - 1) / TS, J = lim > c0 ? (lim - c0 + TS - 1) / TS : 0;
+  const int64_t np = (int64_t)J * A - (int64_t)J * (J - 1) / 2;
+  if (t < np) {  // column tile j holds A - j row tiles: first of j is j A - j (j - 1) / 2
+    const double h = A + 0.5;
+    double disc = h * h - 2.0 * t;
+    int j = (int)(h - sqrt(disc > 0.0 ? disc : 0.0));
+    if (j > J - 1) j = J - 1;
+    if (j < 0) j = 0;
+    while (j > 0 && (int64_t)j * A - (int64_t)j * (j - 1) / 2 > t) j--;
+    while (j + 1 < J && (int64_t)(j + 1) * A - (int64_t)(j + 1) * j / 2 <= t) j++;
+    const int i = j + (int)(t - ((int64_t)j * A - (int64_t)j * (j - 1) / 2));
+    return UpdTile{c0 + TS * i, c0 + TS * j, lim};
+  }
+  const int u = (int)(t - np);  // row tile i of the lower triangle holds i + 1 tiles
+  int i = (int)((sqrt(8.0 * u + 1.0) - 1.0) * 0.5);
+  while (i > 0 && (int64_t)i * (i + 1) / 2 > u) i--;
+  while ((int64_t)(i + 1) * (i + 2) / 2 <= u) i++;
+  const int j = u - (int)((int64_t)i * (i + 1) / 2);
+  (void)with_u;
+  return UpdTile{ncol + TS * i, ncol + TS * j, ncol + nrow};
+}
 struct LevelPlan {
   int32_t front_b = 0, front_e = 0;  // into the level-ordered front list
   int32_t build_b = 0, build_e = 0;  // front-assembly tiles
   int64_t k_b = 0, k_e = 0;          // K entries of this level's fronts
-  int32_t syrk_b = 0, syrk_e = 0;    // update-matrix tiles
   int32_t gath_b = 0, gath_e = 0;    // solve gather tasks
   int32_t rg_b = 0, rg_e = 0;        // backward-solve tasks on the rows below the block
   int32_t sdiag_b = 0, sdiag_e = 0;  // solve diagonal-block tasks, by step: see solve_steps
@@ -102,6 +168,7 @@ struct LevelPlan {
 
 // Numeric plan: everything the kernels need, built on the host by analysis.
 struct Plan {
+  static constexpr int kSuper32 = 256;  // columns per super-step of the FP32 FMA-pipe factor
   int nb = 64;                       // factor block width
   int nbs = 64;                      // solve block width
   std::vector<FrontInfo> fronts;     // by supernode index
@@ -111,7 +178,7 @@ struct Plan {
   std::vector<int32_t> inv;          // child -> parent-front inverse maps
   std::vector<int32_t> relpos;       // child row -> position in parent's front (by sri offset)
   std::vector<LevelPlan> levels;
-  std::vector<Task> build_tasks, gemm_tasks, potrf_tasks, trsm_tasks, syrk_tasks;
+  std::vector<Task> build_tasks, potrf_tasks, trsm_ents, upd_ents;
   std::vector<Task> gath_tasks, sdiag_tasks, sgemv_tasks, rgemv_tasks;
   std::vector<int64_t> toff;         // per front: offset of its solve update vector (length nrow)
   int64_t t_entries = 0;

@@ -4,10 +4,10 @@
 //
 // Per level of the supernodal tree: build every frontal matrix of the level
 // (gather of the children's update matrices, each entry written once), add the
-// K entries owned by the level, then factor the fronts' panels block column by
-// block column (left-looking GEMM update, Cholesky of the diagonal block,
-// triangular solve of the rows below) and form their update matrices
-// U = F22 - L21 L21^T (SYRK). No atomics on values: results are bit-reproducible.
+// K entries owned by the level, then factor the fronts block column by block
+// column: Cholesky of the diagonal block, triangular solve of the rows below,
+// right-looking update of the rest of the panel and of the update matrix
+// U = F22 - L21 L21^T. No atomics on values: results are bit-reproducible.
 #include <cfloat>
 #include <climits>
 
@@ -149,266 +149,384 @@ __global__ void kadd_kernel(DevPlan dp, int64_t q0, int64_t q1, const double *__
   }
 }
 
-// C[M x N] -= A[M x K] * S * B[N x K]^T for one 64x64 tile (rows of A and B
-// are contiguous along K), 256 threads, 4x4 outputs per thread; S = diag(sk)
-// holds the pivot signs of the K columns of a signed factorisation (sk ==
-// nullptr: S = I).
-template <typename T>
-__device__ __forceinline__ void gemm_nt_tile(T *C, int64_t ldc, const T *A, int64_t lda,
-                                             const T *B, int64_t ldb, int M, int N, int K,
-                                             const int8_t *sk) {
-  constexpr int BK = 16;
-  __shared__ T As[BK][kGemmTile + 4], Bs[BK][kGemmTile + 4];
-  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-  T acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; i++)
-#pragma unroll
-    for (int j = 0; j < 4; j++) acc[i][j] = T(0);
-  for (int k0 = 0; k0 < K; k0 += BK) {
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-      const int e = tid + 256 * q, r = e / BK, kk = e % BK;
-      As[kk][r] = (r < M && k0 + kk < K) ? A[(int64_t)r * lda + k0 + kk] : T(0);
-      T bv = (r < N && k0 + kk < K) ? B[(int64_t)r * ldb + k0 + kk] : T(0);
-      if (sk && k0 + kk < K && sk[k0 + kk] < 0) bv = -bv;
-      Bs[kk][r] = bv;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < BK; kk++) {
-      T a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; i++) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 4; j++) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; i++)
-#pragma unroll
-        for (int j = 0; j < 4; j++) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
+// Trailing update of a level's fronts by the finished columns [k0, k1) (C -= A S
+// B^T, A and B rows of a front's panel, S = diag(pivot signs), nullptr: I): one
+// TS x TS tile of the columns [min(k1, ncol), min(clim, ncol)) of a panel, or,
+// with_u, also of the update matrix, per block (tile numbering: upd_decode).
+//
+// FP64 (32 x 32 tiles, 64 columns per launch, right-looking): GB300's FP64 pipe
+// starts two multiply-adds a cycle per SM, so a 32 x 32 x 64 tile is 16 us of pipe
+// time for 48 KB of L2 traffic, and nothing but spreading the tiles over all SMs
+// matters. A left-looking form (one block column at a time, K = all columns before
+// it) has 47 blocks of 64 x 64 for 152 SMs on a 3008-column front: 118 ms of updates
+// on the 32^3 grid LP against 37 ms (32 ms at the nominal FP64 rate). FP32 (64 x 64 tiles): the pipe
+// is 64 times faster, so the tile's reads and writes are spread over a longer K
+// (columns of a super-step: see Plan::kSuper32).
+template <typename T, int TS, int NT, int BK>
+__global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 3 : 2) upd_kernel(DevPlan dp, const Task *__restrict__ ents, int nent,
+                                                 int k0, int k1, int clim, int with_u,
+                                                 T *__restrict__ L, T *__restrict__ U) {
+  constexpr int TY = NT / 16, MI = TS / TY, NJ = TS / 16;
+  constexpr int VW = 16 / (int)sizeof(T), LD = BK + VW, NV = BK / VW;  // rows of BK values, 16-byte padded
+  constexpr int PER = 2 * TS * NV / NT;                                // 16-byte loads per thread and chunk
+  static_assert(sizeof(T) == 4 || BK >= 64, "an FP64 launch has at most 64 columns");
+  static_assert(2 * TS * NV % NT == 0 && TS * NV % NT == 0, "loader shape");
+  __shared__ __align__(16) T sA[TS * LD], sB[TS * LD];
+  int lo = 0, hi = nent - 1;  // the front this block's tile belongs to
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) / 2;
+    if (ents[mid].a <= (int)blockIdx.x) lo = mid;
+    else hi = mid - 1;
   }
-#pragma unroll
-  for (int i = 0; i < 4; i++) {
-    const int r = ty + 16 * i;
-    if (r >= M) continue;
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-      const int c = tx + 16 * j;
-      if (c < N) C[(int64_t)r * ldc + c] -= acc[i][j];
-    }
-  }
-}
-
-// Left-looking update of block column k of a panel: rows i0..i0+63 of
-// F[:, k:k+kb] -= L[:, 0:k] * L[k:k+kb, 0:k]^T.
-template <typename T>
-__global__ void __launch_bounds__(256) gemm_ll_kernel(DevPlan dp, int32_t task0, int nb,
-                                                      T *__restrict__ L) {
-  const Task tk = dp.gemm[task0 + blockIdx.x];
+  const Task tk = ents[lo];
   const FrontInfo F = dp.fronts[tk.front];
-  const int nf = F.ncol + F.nrow, i0 = tk.a, k = tk.b;
-  const int kb = min(nb, F.ncol - k), M = min(kGemmTile, nf - i0);
+  const int nf = F.ncol + F.nrow, K = min(k1, F.ncol) - k0;
+  const UpdTile tl = upd_decode(F.ncol, F.nrow, k1, clim, with_u, TS, (int)blockIdx.x - tk.a);
+  const int M = min(TS, nf - tl.r), N = min(TS, tl.cend - tl.c);
   T *P = L + F.loff;
-  gemm_nt_tile<T>(P + (int64_t)i0 * F.ld + k, F.ld, P + (int64_t)i0 * F.ld, F.ld,
-                  P + (int64_t)k * F.ld, F.ld, M, kb, k, dp.sgn ? dp.sgn + F.first : nullptr);
-}
-
-// Update matrix U = F22 - L21 L21^T, one 64x64 lower tile per block.
-template <typename T>
-__global__ void __launch_bounds__(256) syrk_kernel(DevPlan dp, int32_t task0,
-                                                   const T *__restrict__ L, T *__restrict__ U) {
-  const Task tk = dp.syrk[task0 + blockIdx.x];
-  const FrontInfo F = dp.fronts[tk.front];
-  const int i0 = tk.a, j0 = tk.b;
-  const int M = min(kGemmTile, F.nrow - i0), N = min(kGemmTile, F.nrow - j0);
-  const T *P = L + F.loff + (int64_t)F.ncol * F.ld;
-  gemm_nt_tile<T>(U + F.uoff + (int64_t)i0 * F.uld + j0, F.uld, P + (int64_t)i0 * F.ld, F.ld,
-                  P + (int64_t)j0 * F.ld, F.ld, M, N, F.ncol, dp.sgn ? dp.sgn + F.first : nullptr);
+  const T *A = P + (int64_t)tl.r * F.ld + k0, *B = P + (int64_t)tl.c * F.ld + k0;
+  T *C;
+  int64_t ldc;
+  if (tl.c < F.ncol) {
+    ldc = F.ld;
+    C = P + (int64_t)tl.r * ldc + tl.c;
+  } else {
+    ldc = F.uld;
+    C = U + F.uoff + (int64_t)(tl.r - F.ncol) * ldc + (tl.c - F.ncol);
+  }
+  const int8_t *sk = dp.sgn ? dp.sgn + F.first + k0 : nullptr;
+  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
+  struct __align__(16) V { T v[VW]; };
+  V reg[PER];
+  auto load = [&](int kc) {  // chunk [kc, kc + BK) of both operands (zero past K, M, N)
+#pragma unroll
+    for (int q = 0; q < PER; q++) {
+      const bool isb = q >= PER / 2;
+      const int e = tid + NT * (isb ? q - PER / 2 : q), r = e / NV, kk = kc + VW * (e % NV);
+      V x;
+#pragma unroll
+      for (int h = 0; h < VW; h++) x.v[h] = T(0);
+      if (r < (isb ? N : M) && kk < K) {
+        x = *reinterpret_cast<const V *>((isb ? B : A) + (int64_t)r * F.ld + kk);
+#pragma unroll
+        for (int h = 0; h < VW; h++) {
+          if (kk + h >= K) x.v[h] = T(0);
+          else if (isb && sk && sk[kk + h] < 0) x.v[h] = -x.v[h];
+        }
+      }
+      reg[q] = x;
+    }
+  };
+  load(0);
+  T acc[MI][NJ], cv[MI][NJ];  // the products' sum, the target's values
+#pragma unroll
+  for (int i = 0; i < MI; i++)
+#pragma unroll
+    for (int j = 0; j < NJ; j++) {
+      const int r = ty + TY * i, c = tx + 16 * j;
+      acc[i][j] = T(0);
+      cv[i][j] = (r < M && c < N) ? C[(int64_t)r * ldc + c] : T(0);
+    }
+  for (int kc = 0; kc < K; kc += BK) {
+    if (kc > 0) __syncthreads();
+#pragma unroll
+    for (int q = 0; q < PER; q++) {
+      const bool isb = q >= PER / 2;
+      const int e = tid + NT * (isb ? q - PER / 2 : q);
+      *reinterpret_cast<V *>((isb ? sB : sA) + (e / NV) * LD + VW * (e % NV)) = reg[q];
+    }
+    __syncthreads();
+    if (sizeof(T) == 4 && kc + BK < K) load(kc + BK);  // (FP64: one chunk)
+    const int kn = min(BK, K - kc);
+#pragma unroll (sizeof(T) == 8 ? 4 : 1)
+    for (int kk = 0; kk < kn; kk += VW) {
+      V a[MI], b[NJ];
+#pragma unroll
+      for (int i = 0; i < MI; i++) a[i] = *reinterpret_cast<const V *>(sA + (ty + TY * i) * LD + kk);
+#pragma unroll
+      for (int j = 0; j < NJ; j++) b[j] = *reinterpret_cast<const V *>(sB + (tx + 16 * j) * LD + kk);
+#pragma unroll
+      for (int h = 0; h < VW; h++)
+#pragma unroll
+        for (int i = 0; i < MI; i++)
+#pragma unroll
+          for (int j = 0; j < NJ; j++) acc[i][j] = fma(a[i].v[h], b[j].v[h], acc[i][j]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < MI; i++)
+#pragma unroll
+    for (int j = 0; j < NJ; j++) {
+      const int r = ty + TY * i, c = tx + 16 * j;
+      if (r < M && c < N) C[(int64_t)r * ldc + c] = cv[i][j] - acc[i][j];
+    }
 }
 
 template <typename T> __device__ __forceinline__ T big_pivot();
 template <> __device__ __forceinline__ float big_pivot<float>() { return 1e30f; }
 template <> __device__ __forceinline__ double big_pivot<double>() { return 1e64; }
 
-// Cholesky of one diagonal block (kb <= nb <= 128) in shared memory. A pivot
-// that is not positive is either reported (smallest failing column kept) or
-// replaced by a large value (static pivoting) and counted. With pivot signs
-// (dp.sgn, a quasi-definite matrix) the block is factored as L S L^T: the
-// pivot d_j must have the sign s_j, L_jj = sqrt(s_j d_j), the column below is
-// divided by s_j L_jj and the trailing update is -= L_ij s_j L_cj.
+// 1 / sqrt(d) for d > 0: the FP32 estimate and one third-order step,
+// r (1 + e/2 + 3 e^2 / 8) with e = 1 - d r^2 (|e| < 2^-21: the step's own error
+// is below 2^-62). Values outside FP32's normal range take the library functions.
+__device__ __forceinline__ double inv_sqrt(double d) {
+  if (!(d > 1e-36 && d < 1e36)) return 1.0 / sqrt(d);
+  const double r = (double)rsqrtf((float)d);
+  const double e = fma(-(d * r), r, 1.0);
+  return fma(r * e, fma(0.375, e, 0.5), r);
+}
+__device__ __forceinline__ float inv_sqrt(float d) {
+  if (!(d > 1e-30f && d < 1e30f)) return 1.f / sqrtf(d);
+  const float r = rsqrtf(d);
+  return fmaf(0.5f * r, fmaf(-d * r, r, 1.f), r);
+}
+// 1 / d for d > 0 is r0 (1 + e + e^2), r0 an FP32 reciprocal and e = 1 - d r0 (|e| <
+// 2^-21); a / d is a r0 plus (e + e^2) of it, a chain of three FP64 operations. r0 = 0
+// tells that d is outside FP32's normal range (the callers then divide).
+__device__ __forceinline__ double recip_start(double d) {
+  const unsigned ex = ((unsigned)__double2hiint(d) >> 20) & 0x7FFu;  // 2^-119 .. 2^119
+  return ex - 904u < 239u ? (double)__fdividef(1.f, (float)d) : 0.0;
+}
+__device__ __forceinline__ float recip_start(float d) { return 1.f / d; }
+__device__ __forceinline__ double recip_err(double d, double r0) {
+  const double e = fma(-d, r0, 1.0);
+  return fma(e, e, e);
+}
+__device__ __forceinline__ float recip_err(float, float) { return 0.f; }
+template <typename T> __device__ __forceinline__ T recip(T d) {
+  const T r0 = recip_start(d);
+  return r0 != T(0) ? fma(r0, recip_err(d, r0), r0) : T(1) / d;
+}
+// s v for s = +-1 and 0 < d < big_pivot^2 (false for NaN) on the integer pipe:
+// an FP64 multiplication or comparison costs as much as a multiply-add.
+__device__ __forceinline__ double flip(double v, bool neg) {
+  return __hiloint2double(__double2hiint(v) ^ (neg ? 0x80000000 : 0), __double2loint(v));
+}
+__device__ __forceinline__ float flip(float v, bool neg) { return neg ? -v : v; }
+__device__ __forceinline__ bool pivot_ok(double d) {
+  const long long b = __double_as_longlong(d);
+  return b > 0 && b < __double_as_longlong(1e128);
+}
+__device__ __forceinline__ bool pivot_ok(float d) { return d > 0.f && d < INFINITY; }
+
+// Cholesky of one diagonal block (kb <= 64). A pivot that is not positive is
+// either reported (smallest failing column kept) or replaced by a large value
+// (static pivoting) and counted. With pivot signs (dp.sgn, a quasi-definite
+// matrix) the block is factored as L S L^T: the pivot d_j must have the sign
+// s_j, L_jj = sqrt(s_j d_j), L_ij = a_ij / (s_j L_jj).
+//
+// What bounds it on GB300: an FP64 instruction occupies a quarter SM's unit for
+// 64 cycles whatever its active lanes (measured; results after 66), so the count of
+// FP64 warp instructions on each of the four warps is the time, and the chain of
+// 64 pivots is on it too. So the elimination runs on unscaled columns (a_ic -=
+// (a_ij / d_j) a_cj: no square root on the chain), all columns are scaled by 1 /
+// L_jj at the end, and the block goes in four panels of 16 columns: inside a panel
+// 2 to 8 threads share a row so that all four warps stay busy, each column is
+// published through shared memory (one barrier per column); past the panel a
+// rank-16 update over 8 x 8 blocks of the lower triangle. The loop over a panel's
+// columns stays rolled: straight-line code runs once per launch, from a cold
+// instruction cache (unrolled: 102 us a launch on the 32^3 grid's fronts, rolled: 82).
+constexpr int kPotrfThreads = 128;
+
+// Panel at column c0 of the block in S (rows c0 .. 63): PN threads per row,
+// thread h of a row holds the columns c0 + h + PN q.
+template <typename T, int PN>
+__device__ __forceinline__ void potrf_panel(T *S, int ls, int c0, T (*col)[64], const int8_t *neg, T *piv,
+                                            int32_t *status, int perturb, int first) {
+  constexpr int NQ = 16 / PN;
+  const int t = threadIdx.x, i = c0 + t / PN, h = t % PN;
+  const bool on = i < 64;
+  T x[NQ];
+#pragma unroll
+  for (int q = 0; q < NQ; q++) x[q] = on ? S[i * ls + c0 + h + PN * q] : T(0);
+  if (on && h == 0) col[0][i] = x[0];
+  __syncthreads();
+#pragma unroll 1
+  for (int j = 0; j < 16; j++) {
+    const T *cj = col[j & 1];
+    const bool ng = neg[c0 + j] != 0;
+    T d = flip(cj[c0 + j], ng);  // s_j d_j
+    if (!pivot_ok(d)) {  // (uniform over the block)
+      if (t == 0) {
+        if (perturb) atomicAdd(&status[ST_PERTURBED], 1);
+        else atomicMin(&status[ST_FAIL_COL], first + c0 + j);
+      }
+      d = perturb ? big_pivot<T>() : T(1);
+    }
+    if (t == 0) piv[c0 + j] = d;
+    if (j < 15) {
+      const T aij = on ? cj[i] : T(0), r0 = recip_start(d);
+      const T w0 = aij * r0;
+      T w = fma(w0, recip_err(d, r0), w0);
+      if (r0 == T(0)) w = aij / d;
+      w = flip(w, ng);  // a_ij / d_j
+#pragma unroll
+      for (int q = 0; q < NQ; q++)
+        if (PN * q + PN - 1 > j) {  // some column of this group lies past j
+          const int c = h + PN * q;
+          x[q] = fma(-w, c > j ? cj[c0 + c] : T(0), x[q]);
+          if (on && c == j + 1) col[(j + 1) & 1][i] = x[q];
+        }
+      __syncthreads();
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < NQ; q++)
+    if (on && c0 + h + PN * q <= i) S[i * ls + c0 + h + PN * q] = x[q];
+}
+
 template <typename T>
-__global__ void __launch_bounds__(256) potrf_kernel(DevPlan dp, const Task *__restrict__ tasks,
-                                                    int nb, T *__restrict__ L, int32_t *status,
-                                                    int perturb) {
+__global__ void __launch_bounds__(kPotrfThreads) potrf_kernel(DevPlan dp, const Task *__restrict__ tasks,
+                                                              T *__restrict__ L, int32_t *status,
+                                                              int perturb) {
+  constexpr int NB = 64, LS = NB + 1, NT = kPotrfThreads;
   const Task tk = tasks[blockIdx.x];
   const FrontInfo F = dp.fronts[tk.front];
-  const int k = tk.a, kb = min(nb, F.ncol - k), ls = nb + 1;
+  const int k = tk.a, kb = min(NB, F.ncol - k);
   T *A = L + F.loff + (int64_t)k * F.ld + k;
   const int8_t *sg = dp.sgn ? dp.sgn + F.first + k : nullptr;
-  extern __shared__ unsigned char smem_raw[];
-  T *Ad = reinterpret_cast<T *>(smem_raw);  // [nb][nb + 1]
+  __shared__ T S[NB * LS];  // the block; past kb: zero, with a unit diagonal
+  __shared__ T col[2][NB], piv[NB], rs[NB];
+  __shared__ int8_t neg[NB];
   const int tid = threadIdx.x;
-  for (int e = tid; e < kb * kb; e += blockDim.x) {
-    const int r = e / kb, c = e % kb;
-    if (r >= c) Ad[r * ls + c] = A[(int64_t)r * F.ld + c];
+#pragma unroll 16
+  for (int q = 0; q < NB * NB / NT; q++) {
+    const int e = tid + NT * q, r = e / NB, c = e % NB;
+    T v = r == c ? T(1) : T(0);
+    if (r < kb && c <= r) v = A[(int64_t)r * F.ld + c];
+    S[r * LS + c] = v;
   }
+  if (tid < NB) neg[tid] = sg && tid < kb && sg[tid] < 0;
   __syncthreads();
-  // FP64 Cholesky (no signs): the column below the pivot is multiplied by one
-  // reciprocal instead of divided entry by entry (an FP64 division is a long
-  // sequence on the FP64 pipe); FP32 and signed factors keep the division.
-  const bool recip = sizeof(T) == 8 && !sg;
-  __shared__ T rl;  // 1 / (s_j L_jj) of the current column
-  const int tx = tid % 16, ty = tid / 16;  // 16 x 16 grid over the trailing block
-  for (int j = 0; j < kb; j++) {
-    const T sj = (sg && sg[j] < 0) ? T(-1) : T(1);
-    if (tid == 0) {
-      T d = sj * Ad[j * ls + j];
-      if (!(d > T(0)) || !(d < big_pivot<T>() * big_pivot<T>())) {
-        if (perturb) {
-          d = big_pivot<T>();
-          atomicAdd(&status[ST_PERTURBED], 1);
-        } else {
-          atomicMin(&status[ST_FAIL_COL], F.first + k + j);
-          d = T(1);
+#pragma unroll 1
+  for (int p = 0; p < 4; p++) {
+    const int c0 = 16 * p;
+    if (c0 >= kb) break;
+    if (p < 2) potrf_panel<T, 2>(S, LS, c0, col, neg, piv, status, perturb, F.first + k);
+    else if (p == 2) potrf_panel<T, 4>(S, LS, c0, col, neg, piv, status, perturb, F.first + k);
+    else potrf_panel<T, 8>(S, LS, c0, col, neg, piv, status, perturb, F.first + k);
+    __syncthreads();
+    if (tid < 16) rs[c0 + tid] = inv_sqrt(piv[c0 + tid]);
+    __syncthreads();
+    {  // the panel's columns: s_j a_ij / L_jj, and L_jj = sqrt(d) from d and 1 / sqrt(d)
+      const int c = c0 + tid % 16;
+      const T r = rs[c];
+      for (int i = c0 + tid / 16; i < NB; i += NT / 16) {
+        if (i > c) {
+          S[i * LS + c] = flip(S[i * LS + c] * r, neg[c] != 0);
+        } else if (i == c) {
+          const T d = piv[c], l0 = d * r;
+          S[i * LS + c] = fma(fma(-l0, l0, d), T(0.5) * r, l0);
         }
       }
-      const T l = sqrt(d);
-      Ad[j * ls + j] = l;
-      if (recip) rl = T(1) / l;
     }
     __syncthreads();
-    if (recip) {
-      const T r = rl;
-      for (int i = j + 1 + tid; i < kb; i += blockDim.x) Ad[i * ls + j] *= r;
-    } else {
-      const T ljj = sj * Ad[j * ls + j];
-      for (int i = j + 1 + tid; i < kb; i += blockDim.x) Ad[i * ls + j] /= ljj;
-    }
-    __syncthreads();
-    for (int i = j + 1 + ty; i < kb; i += 16) {
-      const T lij = -sj * Ad[i * ls + j];
-      for (int c = j + 1 + tx; c <= i; c += 16) Ad[i * ls + c] = fma(lij, Ad[c * ls + j], Ad[i * ls + c]);
+    if (p == 3 || c0 + 16 >= kb) break;
+    // rows and columns past the panel: 8 x 8 blocks (bi >= bc) of the lower
+    // triangle, a block per warp, two outputs per lane
+    const int nb8 = (48 - c0) / 8, nblk = nb8 * (nb8 + 1) / 2, l = tid % 32;
+    for (int b = tid / 32; b < nblk; b += NT / 32) {
+      int bi = 0, rest = b;
+      while (rest > bi) rest -= ++bi;  // block row bi holds bi + 1 blocks
+      const int i = c0 + 16 + 8 * bi + l / 8, c = c0 + 16 + 8 * rest + l % 8;
+      const T *xi = S + i * LS + c0, *xk = xi + 4 * LS, *yc = S + c * LS + c0;
+      T s0 = T(0), s1 = T(0);
+#pragma unroll
+      for (int j = 0; j < 16; j++) {
+        const T y = flip(yc[j], neg[c0 + j] != 0);
+        s0 = fma(xi[j], y, s0);
+        s1 = fma(xk[j], y, s1);
+      }
+      if (c <= i) S[i * LS + c] -= s0;
+      if (c <= i + 4) S[(i + 4) * LS + c] -= s1;
     }
     __syncthreads();
   }
-  for (int e = tid; e < kb * kb; e += blockDim.x) {
-    const int r = e / kb, c = e % kb;
-    if (r >= c) A[(int64_t)r * F.ld + c] = Ad[r * ls + c];
+#pragma unroll 16
+  for (int q = 0; q < NB * NB / NT; q++) {
+    const int e = tid + NT * q, r = e / NB, c = e % NB;
+    if (r < kb && c <= r) A[(int64_t)r * F.ld + c] = S[r * LS + c];
   }
 }
 
-// Rows below the diagonal block: X <- X L_kk^{-T} (row-wise forward
-// substitution), kTrsmRows rows per block, kb <= nb <= 128; with pivot signs
-// X <- X L_kk^{-T} S_k.
+// Rows below the diagonal block: X <- X L_kk^{-T} (X L_kk^{-T} S_k with pivot
+// signs) by substitution, kb <= 64, 16 rows at a time on four warps. P = 8 lanes
+// share a row (lane h keeps the columns of residue h mod 8 in registers); with unit
+// columns u_c = L_:c / L_cc and z_c = x_c L_cc the substitution is z_c2 -= z_c
+// u_c2,c, and x = z / diag is formed once at the end, so a column costs its
+// multiply-adds and nothing else. Bound by the FP64 unit (64 cycles per warp
+// instruction on each quarter SM: 10 us per 16 rows and SM). A block takes `batches`
+// times 16 rows: more than one only when the rows exceed 16 per SM (trsm_batches),
+// so that a 3008-row front reaches every SM (128 rows a block, as before: 24
+// blocks, 169 us a launch on the 32^3 grid); the code of a batch is unrolled over
+// the columns and fits the instruction cache, which wider per-warp tiles (16
+// rows a warp, 56 KB of code run once) did not: 98 us against 55 us a launch on the
+// 40^3 grid.
+constexpr int kTrsmP = 8;
 template <typename T>
-__global__ void __launch_bounds__(kTrsmRows) trsm_kernel(DevPlan dp, const Task *__restrict__ tasks,
-                                                         int nb, T *__restrict__ L) {
-  const Task tk = tasks[blockIdx.x];
+__global__ void __launch_bounds__(128) trsm_kernel(DevPlan dp, const Task *__restrict__ ents, int nent,
+                                                   int batches, T *__restrict__ L) {
+  constexpr int NB = 64, LS = NB + 1, P = kTrsmP, NQ = NB / P;
+  static_assert(kTrsmRows == 4 * 32 / P, "rows per batch");
+  int lo = 0, hi = nent - 1;  // the front this block's rows belong to
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) / 2;
+    if (ents[mid].a <= (int)blockIdx.x) lo = mid;
+    else hi = mid - 1;
+  }
+  const Task tk = ents[lo];
   const FrontInfo F = dp.fronts[tk.front];
-  const int nf = F.ncol + F.nrow, i0 = tk.a, k = tk.b, ls = nb + 1;
-  const int kb = min(nb, F.ncol - k), rows = min(kTrsmRows, nf - i0);
-  extern __shared__ unsigned char smem_raw[];
-  T *Lk = reinterpret_cast<T *>(smem_raw);  // [nb][nb + 1]
-  T *X = Lk + nb * ls;                      // [kTrsmRows][nb + 1]
-  const T *A = L + F.loff + (int64_t)k * F.ld + k;
-  T *Xg = L + F.loff + (int64_t)i0 * F.ld + k;
-  const int tid = threadIdx.x;
-  for (int e = tid; e < kb * kb; e += blockDim.x) {
-    const int r = e / kb, c = e % kb;
-    Lk[r * ls + c] = (r >= c) ? A[(int64_t)r * F.ld + c] : T(0);
-  }
-  for (int e = tid; e < rows * kb; e += blockDim.x) {
-    const int r = e / kb, c = e % kb;
-    X[r * ls + c] = Xg[(int64_t)r * F.ld + c];
-  }
+  const int nf = F.ncol + F.nrow, k = tk.b, kb = min(NB, F.ncol - k);
+  const int tid = threadIdx.x, lane = tid % 32, h = lane % P;
+  int row = k + kb + batches * kTrsmRows * ((int)blockIdx.x - tk.a) + tid / P;
+  __shared__ T U[NB * LS];  // column c: u_c2,c at U[c * LS + c2]
+  __shared__ T rd[NB];      // s_c / L_cc
+  T *Xr = L + F.loff + (int64_t)row * F.ld + k;
+  T z[NQ];
+#pragma unroll
+  for (int q = 0; q < NQ; q++) z[q] = (row < nf && h + P * q < kb) ? Xr[h + P * q] : T(0);
   const int8_t *sg = dp.sgn ? dp.sgn + F.first + k : nullptr;
-  // FP64 without signs: the diagonal replaced by its reciprocal (no FP64
-  // division on the substitution's critical path); otherwise s_c L_cc, the
-  // signs also folded into the entries below the diagonal (s_c2 L_c,c2)
-  const bool recip = sizeof(T) == 8 && !sg;
+  const T *A = L + F.loff + (int64_t)k * F.ld + k;
+  if (tid < kb) {
+    const T d = A[(int64_t)tid * F.ld + tid];
+    rd[tid] = flip(recip(d), sg && sg[tid] < 0);
+  }
+  T u[NB * NB / 128];
+#pragma unroll
+  for (int q = 0; q < NB * NB / 128; q++) {
+    const int c2 = 2 * q + tid / NB, c = tid % NB;
+    u[q] = (c2 < kb && c < c2) ? A[(int64_t)c2 * F.ld + c] : T(0);
+  }
   __syncthreads();
-  for (int e = tid; e < kb * kb; e += blockDim.x) {
-    const int r = e / kb, c = e % kb;
-    if (r == c) {
-      const T d = (sg && sg[c] < 0) ? -Lk[r * ls + c] : Lk[r * ls + c];
-      Lk[r * ls + c] = recip ? T(1) / d : d;
-    } else if (r > c && sg && sg[c] < 0) {
-      Lk[r * ls + c] = -Lk[r * ls + c];
+  {
+    // column c of this thread: u = L_c2,c / L_cc (the signs of L and of the scale cancel)
+    const int c = tid % NB;
+    const T s = c < kb ? flip(rd[c], sg && sg[c] < 0) : T(0);
+#pragma unroll
+    for (int q = 0; q < NB * NB / 128; q++) {
+      const int c2 = 2 * q + tid / NB;
+      U[c * LS + c2] = 2 * q + 1 > (c & 32) ? u[q] * s : T(0);  // (uniform per warp)
     }
   }
   __syncthreads();
-  if (tid < rows) {  // column by column: the updates of one step are independent
-    T *x = X + tid * ls;
-    for (int c = 0; c < kb; c++) {
-      const T xc = recip ? x[c] * Lk[c * ls + c] : x[c] / Lk[c * ls + c];
-      x[c] = xc;
-      for (int c2 = c + 1; c2 < kb; c2++) x[c2] = fma(-xc, Lk[c2 * ls + c], x[c2]);
+#pragma unroll 1
+  for (int b = 0; b < batches && row - tid / P < nf; b++) {
+#pragma unroll
+    for (int c = 0; c < NB; c++) {
+      if (c >= kb) break;
+      const T zc = __shfl_sync(0xffffffffu, z[c / P], (lane & ~(P - 1)) | (c % P));
+#pragma unroll
+      for (int q = c / P; q < NQ; q++)  // (U is zero up to its own column)
+        if (P * q + P - 1 > c) z[q] = fma(-zc, U[c * LS + P * q + h], z[q]);
     }
-  }
-  __syncthreads();
-  for (int e = tid; e < rows * kb; e += blockDim.x) {
-    const int r = e / kb, c = e % kb;
-    Xg[(int64_t)r * F.ld + c] = X[r * ls + c];
-  }
-}
-
-// FP64 rows below a diagonal block without pivot signs: X <- X L_kk^{-T}. A
-// full 64-wide block keeps each thread's row in registers (64 values) and
-// reads the block by broadcast from shared memory, its diagonal replaced by
-// reciprocals; the 2080 multiply-adds of a row then issue back to back on the
-// FP64 pipe. A narrower last block takes the shared-memory loop of trsm_kernel.
-// Same arithmetic, in the same order, as trsm_kernel<double> on such a block.
-__global__ void __launch_bounds__(kTrsmRows) trsm_f64_kernel(DevPlan dp, const Task *__restrict__ tasks,
-                                                             double *__restrict__ L) {
-  constexpr int NB = 64, LS = NB + 1;
-  const Task tk = tasks[blockIdx.x];
-  const FrontInfo F = dp.fronts[tk.front];
-  const int nf = F.ncol + F.nrow, i0 = tk.a, k = tk.b;
-  const int kb = min(NB, F.ncol - k), rows = min(kTrsmRows, nf - i0);
-  extern __shared__ unsigned char smem_raw[];
-  double *Lk = reinterpret_cast<double *>(smem_raw);  // [NB][LS]
-  double *X = Lk + NB * LS;                           // [kTrsmRows][LS]
-  const double *A = L + F.loff + (int64_t)k * F.ld + k;
-  double *Xg = L + F.loff + (int64_t)i0 * F.ld + k;
-  const int tid = threadIdx.x;
-  for (int e = tid; e < kb * kb; e += blockDim.x) {
-    const int r = e / kb, c = e % kb;
-    const double v = A[(int64_t)r * F.ld + c];
-    Lk[r * LS + c] = r > c ? v : (r == c ? 1.0 / v : 0.0);
-  }
-  for (int e = tid; e < rows * kb; e += blockDim.x) {
-    const int r = e / kb, c = e % kb;
-    X[r * LS + c] = Xg[(int64_t)r * F.ld + c];
-  }
-  __syncthreads();
-  if (tid < rows) {
-    double *xs = X + tid * LS;
-    if (kb == NB) {
-      double x[NB];
 #pragma unroll
-      for (int c = 0; c < NB; c++) x[c] = xs[c];
+    for (int q = 0; q < NQ; q++)
+      if (row < nf && h + P * q < kb) Xr[h + P * q] = z[q] * rd[h + P * q];
+    row += kTrsmRows;
+    Xr += (int64_t)kTrsmRows * F.ld;
+    if (b + 1 < batches)
 #pragma unroll
-      for (int c = 0; c < NB; c++) {
-        x[c] *= Lk[c * LS + c];
-#pragma unroll
-        for (int c2 = c + 1; c2 < NB; c2++) x[c2] = fma(-x[c], Lk[c2 * LS + c], x[c2]);
-      }
-#pragma unroll
-      for (int c = 0; c < NB; c++) xs[c] = x[c];
-    } else {
-      for (int c = 0; c < kb; c++) {
-        const double xc = xs[c] * Lk[c * LS + c];
-        xs[c] = xc;
-        for (int c2 = c + 1; c2 < kb; c2++) xs[c2] = fma(-xc, Lk[c2 * LS + c], xs[c2]);
-      }
-    }
-  }
-  __syncthreads();
-  for (int e = tid; e < rows * kb; e += blockDim.x) {
-    const int r = e / kb, c = e % kb;
-    Xg[(int64_t)r * F.ld + c] = X[r * LS + c];
+      for (int q = 0; q < NQ; q++) z[q] = (row < nf && h + P * q < kb) ? Xr[h + P * q] : T(0);
   }
 }
 
@@ -463,45 +581,49 @@ void launch_build_level(const DevPlan &dp, const LevelPlan &LP, const double *kv
 }
 
 template <typename T>
-void launch_potrf(const DevPlan &dp, const Task *tasks, int ntasks, int nb, T *L, int32_t *status,
-                  bool perturb, cudaStream_t st) {
-  if (ntasks <= 0) return;
-  const size_t smem = (size_t)nb * (nb + 1) * sizeof(T);
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(potrf_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  { note_launch(); potrf_kernel<T><<<ntasks, 256, smem, st>>>(dp, tasks, nb, L, status, perturb ? 1 : 0); }
+void launch_potrf(const DevPlan &dp, const StepRange &S, T *L, int32_t *status, bool perturb,
+                  cudaStream_t st) {
+  if (S.potrf_e <= S.potrf_b) return;
+  note_launch();
+  potrf_kernel<T><<<S.potrf_e - S.potrf_b, kPotrfThreads, 0, st>>>(dp, dp.potrf + S.potrf_b, L, status,
+                                                                   perturb ? 1 : 0);
 }
 
 template <typename T>
-void launch_trsm(const DevPlan &dp, const Task *tasks, int ntasks, int nb, T *L, cudaStream_t st) {
-  if (ntasks <= 0) return;
-  const size_t smem = (size_t)(nb + kTrsmRows) * (nb + 1) * sizeof(T);
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(trsm_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  { note_launch(); trsm_kernel<T><<<ntasks, kTrsmRows, smem, st>>>(dp, tasks, nb, L); }
+void launch_trsm(const DevPlan &dp, const StepRange &S, T *L, cudaStream_t st) {
+  if (S.trsm_n <= 0) return;
+  note_launch();
+  trsm_kernel<T><<<S.trsm_n, 128, 0, st>>>(dp, dp.trsm + S.trsm_b, S.trsm_e - S.trsm_b, S.trsm_bat, L);
 }
 
-void launch_trsm_f64(const DevPlan &dp, const Task *tasks, int ntasks, double *L, cudaStream_t st) {
-  if (ntasks <= 0) return;
-  const size_t smem = (size_t)(64 + kTrsmRows) * 65 * sizeof(double);
-  cudaFuncSetAttribute(trsm_f64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  { note_launch(); trsm_f64_kernel<<<ntasks, kTrsmRows, smem, st>>>(dp, tasks, L); }
+static void launch_upd(const DevPlan &dp, const UpdRange &u, double *L, double *U, cudaStream_t st) {
+  if (u.n <= 0) return;
+  note_launch();
+  upd_kernel<double, kUpdTile64, 128, 64><<<u.n, 128, 0, st>>>(dp, dp.upd + u.b, u.e - u.b, u.k0, u.k1,
+                                                               u.clim, u.with_u, L, U);
+}
+static void launch_upd(const DevPlan &dp, const UpdRange &u, float *L, float *U, cudaStream_t st) {
+  if (u.n <= 0) return;
+  note_launch();
+  upd_kernel<float, kUpdTile32, 256, 32><<<u.n, 256, 0, st>>>(dp, dp.upd + u.b, u.e - u.b, u.k0, u.k1,
+                                                              u.clim, u.with_u, L, U);
 }
 
 template <typename T>
 void launch_factor_simt(const DevPlan &dp, const Plan &plan, const double *kval, T *L, T *U,
                         int32_t *status, bool perturb, cudaStream_t st) {
-  const int nb = plan.nb;
   for (const LevelPlan &LP : plan.levels) {
     launch_build_level<T>(dp, LP, kval, L, U, st);
     for (const StepRange &S : LP.steps) {
-      if (S.gemm_e > S.gemm_b)
-        { note_launch(); gemm_ll_kernel<T><<<S.gemm_e - S.gemm_b, 256, 0, st>>>(dp, S.gemm_b, nb, L); }
-      launch_potrf<T>(dp, dp.potrf + S.potrf_b, S.potrf_e - S.potrf_b, nb, L, status, perturb, st);
-      launch_trsm<T>(dp, dp.trsm + S.trsm_b, S.trsm_e - S.trsm_b, nb, L, st);
+      launch_potrf<T>(dp, S, L, status, perturb, st);
+      launch_trsm<T>(dp, S, L, st);
+      if (sizeof(T) == 8) {
+        launch_upd(dp, S.upd64, L, U, st);
+      } else {
+        launch_upd(dp, S.upd32, L, U, st);
+        launch_upd(dp, S.sup32, L, U, st);
+      }
     }
-    if (LP.syrk_e > LP.syrk_b)
-      { note_launch(); syrk_kernel<T><<<LP.syrk_e - LP.syrk_b, 256, 0, st>>>(dp, LP.syrk_b, L, U); }
   }
 }
 
@@ -517,12 +639,9 @@ template void launch_build_level<float>(const DevPlan &, const LevelPlan &, cons
                                         float *, float *, cudaStream_t);
 template void launch_build_level<double>(const DevPlan &, const LevelPlan &, const double *,
                                          double *, double *, cudaStream_t);
-template void launch_potrf<double>(const DevPlan &, const Task *, int, int, double *, int32_t *,
-                                   bool, cudaStream_t);
-template void launch_trsm<double>(const DevPlan &, const Task *, int, int, double *, cudaStream_t);
-template void launch_potrf<float>(const DevPlan &, const Task *, int, int, float *, int32_t *, bool,
-                                  cudaStream_t);
-template void launch_trsm<float>(const DevPlan &, const Task *, int, int, float *, cudaStream_t);
+template void launch_potrf<double>(const DevPlan &, const StepRange &, double *, int32_t *, bool,
+                                   cudaStream_t);
+template void launch_trsm<double>(const DevPlan &, const StepRange &, double *, cudaStream_t);
 template void launch_factor_simt<double>(const DevPlan &, const Plan &, const double *, double *,
                                          double *, int32_t *, bool, cudaStream_t);
 template void launch_factor_simt<float>(const DevPlan &, const Plan &, const double *, float *,

@@ -626,9 +626,8 @@ void OzPlan::factor(const DevPlan &dp, const Plan &plan, const double *kval, dou
       const StepRange &R = LP.steps[s];
       const Step &Z = V.steps[s];
       gemm(Z.gemm_b, Z.gemm_e);
-      launch_potrf<double>(dp, dp.potrf + R.potrf_b, R.potrf_e - R.potrf_b, plan.nb, L, status,
-                           false, st);
-      launch_trsm_f64(dp, dp.trsm + R.trsm_b, R.trsm_e - R.trsm_b, L, st);
+      launch_potrf<double>(dp, R, L, status, false, st);
+      launch_trsm<double>(dp, R, L, st);
       if (Z.slice_e > Z.slice_b) {
         note_launch();
         oz_slice_kernel<<<Z.slice_e - Z.slice_b, 256, 0, st>>>(dp, d_fr_, d_slice_ + Z.slice_b, L,

@@ -495,13 +495,11 @@ void build_plan(const Problem &P, const Symbolic &S, Plan &plan, int nb, int nbs
 
   // ---- task lists of every level -----------------------------------------
   const int BT = kBuildTile;  // front-assembly tile
-  const int GM = 64;        // GEMM / SYRK tile rows
-  const int TR = 128;       // TRSM rows per task
   const int GR = 256;       // solve gather positions per task
   const int SR = 128;       // solve forward-update rows per task
   const int SC = 256;       // solve backward-update columns per task
-  plan.build_tasks.clear(); plan.gemm_tasks.clear(); plan.potrf_tasks.clear();
-  plan.trsm_tasks.clear(); plan.syrk_tasks.clear(); plan.gath_tasks.clear();
+  plan.build_tasks.clear(); plan.potrf_tasks.clear(); plan.trsm_ents.clear();
+  plan.upd_ents.clear(); plan.gath_tasks.clear();
   plan.sdiag_tasks.clear(); plan.sgemv_tasks.clear(); plan.rgemv_tasks.clear();
   plan.toff.assign(ns, 0);
   plan.t_entries = 0;
@@ -532,42 +530,58 @@ void build_plan(const Problem &P, const Symbolic &S, Plan &plan, int nb, int nbs
     }
     LP.build_e = (int32_t)plan.build_tasks.size();
     LP.steps.clear();
+    // the level's fronts with more than `past` columns, numbered for one update launch
+    auto upd_range = [&](int32_t past, int32_t k0, int32_t k1, int32_t clim, int with_u, int TS) {
+      UpdRange u;
+      u.b = (int32_t)plan.upd_ents.size();
+      u.k0 = k0;
+      u.k1 = k1;
+      u.clim = clim;
+      u.with_u = with_u;
+      int64_t n = 0;
+      for (int32_t t = LP.front_b; t < LP.front_e; t++) {
+        const int32_t s = plan.level_fronts[t];
+        const FrontInfo &F = plan.fronts[s];
+        if (F.ncol <= past) continue;
+        const int64_t c = upd_tiles(F.ncol, F.nrow, k1, clim, with_u, TS);
+        if (c == 0) continue;
+        plan.upd_ents.push_back({s, (int32_t)n, k0, 0});
+        n += c;
+        if (n > INT32_MAX) throw std::runtime_error("plan: too many update tiles in one step");
+      }
+      u.e = (int32_t)plan.upd_ents.size();
+      u.n = (int32_t)n;
+      return u;
+    };
     for (int32_t k = 0; k < LP.max_ncol; k += nb) {
       StepRange st{};
-      st.gemm_b = (int32_t)plan.gemm_tasks.size();
-      if (k > 0)
-        for (int32_t t = LP.front_b; t < LP.front_e; t++) {
-          const int32_t s = plan.level_fronts[t];
-          const FrontInfo &F = plan.fronts[s];
-          if (F.ncol <= k) continue;
-          for (int32_t i0 = k; i0 < F.ncol + F.nrow; i0 += GM) plan.gemm_tasks.push_back({s, i0, k, 0});
-        }
-      st.gemm_e = (int32_t)plan.gemm_tasks.size();
       st.potrf_b = (int32_t)plan.potrf_tasks.size();
       for (int32_t t = LP.front_b; t < LP.front_e; t++) {
         const int32_t s = plan.level_fronts[t];
         if (plan.fronts[s].ncol > k) plan.potrf_tasks.push_back({s, k, 0, 0});
       }
       st.potrf_e = (int32_t)plan.potrf_tasks.size();
-      st.trsm_b = (int32_t)plan.trsm_tasks.size();
+      st.trsm_b = (int32_t)plan.trsm_ents.size();
+      auto below = [&](const FrontInfo &F) {
+        return F.ncol > k ? F.ncol + F.nrow - (k + std::min(nb, F.ncol - k)) : 0;
+      };
+      int64_t rows = 0;
+      for (int32_t t = LP.front_b; t < LP.front_e; t++) rows += below(plan.fronts[plan.level_fronts[t]]);
+      st.trsm_bat = trsm_batches(rows);
       for (int32_t t = LP.front_b; t < LP.front_e; t++) {
-        const int32_t s = plan.level_fronts[t];
-        const FrontInfo &F = plan.fronts[s];
-        if (F.ncol <= k) continue;
-        const int32_t kb = std::min(nb, F.ncol - k);
-        for (int32_t i0 = k + kb; i0 < F.ncol + F.nrow; i0 += TR) plan.trsm_tasks.push_back({s, i0, k, 0});
+        const int32_t s = plan.level_fronts[t], r = below(plan.fronts[s]);
+        if (r <= 0) continue;
+        plan.trsm_ents.push_back({s, st.trsm_n, k, 0});
+        st.trsm_n += (r + kTrsmRows * st.trsm_bat - 1) / (kTrsmRows * st.trsm_bat);
       }
-      st.trsm_e = (int32_t)plan.trsm_tasks.size();
+      st.trsm_e = (int32_t)plan.trsm_ents.size();
+      st.upd64 = upd_range(k, k, k + nb, INT32_MAX, 1, kUpdTile64);
+      // FP32: inside a super-step the columns up to its end, at its end the rest
+      const int32_t K0 = k / Plan::kSuper32 * Plan::kSuper32, K1 = K0 + Plan::kSuper32;
+      if (k + nb < K1) st.upd32 = upd_range(k + nb, k, k + nb, K1, 0, kUpdTile32);
+      if (k + nb == K1 || k + nb >= LP.max_ncol) st.sup32 = upd_range(K0, K0, K1, INT32_MAX, 1, kUpdTile32);
       LP.steps.push_back(st);
     }
-    LP.syrk_b = (int32_t)plan.syrk_tasks.size();
-    for (int32_t t = LP.front_b; t < LP.front_e; t++) {
-      const int32_t s = plan.level_fronts[t];
-      const FrontInfo &F = plan.fronts[s];
-      for (int32_t i0 = 0; i0 < F.nrow; i0 += GM)
-        for (int32_t j0 = 0; j0 <= i0; j0 += GM) plan.syrk_tasks.push_back({s, i0, j0, 0});
-    }
-    LP.syrk_e = (int32_t)plan.syrk_tasks.size();
     // solve: gather tasks cover every front (they also initialise its update vector)
     LP.gath_b = (int32_t)plan.gath_tasks.size();
     for (int32_t t = LP.front_b; t < LP.front_e; t++) {
@@ -708,19 +722,47 @@ void validate_plan(const Problem &P, const Symbolic &S, const Plan &pl) {
     }
     close_front();
   }
-  for (const Task &t : pl.gemm_tasks)
-    need(in_front(t) && t.b > 0 && t.b < pl.fronts[t.front].ncol && t.a >= t.b &&
-             t.a < nf(t.front), "gemm task");
   for (const Task &t : pl.potrf_tasks)
     need(in_front(t) && t.a >= 0 && t.a < pl.fronts[t.front].ncol, "potrf task");
-  for (const Task &t : pl.trsm_tasks) {
-    need(in_front(t) && t.b >= 0 && t.b < pl.fronts[t.front].ncol, "trsm task block");
-    const int32_t kb = std::min(pl.nb, pl.fronts[t.front].ncol - t.b);
-    need(t.a >= t.b + kb && t.a < nf(t.front), "trsm task rows");
-  }
-  for (const Task &t : pl.syrk_tasks)
-    need(in_front(t) && t.a >= 0 && t.a < pl.fronts[t.front].nrow && t.b >= 0 && t.b <= t.a,
-         "syrk task");
+  // block numbering of the panel solves and updates: ranges, consecutive
+  // numbers, and the first and last tile of every front inside the front
+  auto check_upd = [&](const UpdRange &u, int TS) {
+    need(0 <= u.b && u.b <= u.e && u.e <= (int32_t)pl.upd_ents.size(), "update range");
+    int64_t next = 0;
+    for (int32_t i = u.b; i < u.e; i++) {
+      const Task &t = pl.upd_ents[i];
+      need(in_front(t) && t.a == next && t.b == u.k0, "update entry");
+      const FrontInfo &F = pl.fronts[t.front];
+      need(u.k0 >= 0 && u.k0 < F.ncol && u.k0 < u.k1 && u.k0 % pl.nb == 0, "update columns");
+      const int64_t c = upd_tiles(F.ncol, F.nrow, u.k1, u.clim, u.with_u, TS);
+      need(c > 0, "update entry without tiles");
+      for (int64_t q : {(int64_t)0, c / 2, c - 1}) {
+        const UpdTile tl = upd_decode(F.ncol, F.nrow, u.k1, u.clim, u.with_u, TS, (int)q);
+        need(tl.c >= std::min(u.k1, F.ncol) && tl.c < tl.cend && tl.r >= tl.c && tl.r < nf(t.front) &&
+                 (tl.c < F.ncol ? tl.cend <= F.ncol : tl.cend == nf(t.front)),
+             "update tile");
+      }
+      next += c;
+    }
+    need(next == u.n, "update block count");
+  };
+  for (const LevelPlan &LP : pl.levels)
+    for (const StepRange &S2 : LP.steps) {
+      need(S2.trsm_bat >= 1 && S2.trsm_bat <= 4, "panel solve batches");
+      need(0 <= S2.trsm_b && S2.trsm_b <= S2.trsm_e && S2.trsm_e <= (int32_t)pl.trsm_ents.size(), "panel solve range");
+      int64_t next = 0;
+      for (int32_t i = S2.trsm_b; i < S2.trsm_e; i++) {
+        const Task &t = pl.trsm_ents[i];
+        need(in_front(t) && t.a == next && t.b >= 0 && t.b < pl.fronts[t.front].ncol, "panel solve entry");
+        const int64_t below = nf(t.front) - (t.b + std::min(pl.nb, pl.fronts[t.front].ncol - t.b));
+        need(below > 0, "panel solve rows");
+        next += (below + kTrsmRows * S2.trsm_bat - 1) / (kTrsmRows * S2.trsm_bat);
+      }
+      need(next == S2.trsm_n, "panel solve block count");
+      check_upd(S2.upd64, kUpdTile64);
+      check_upd(S2.upd32, kUpdTile32);
+      check_upd(S2.sup32, kUpdTile32);
+    }
   for (const Task &t : pl.gath_tasks)
     need(in_front(t) && t.a >= 0 && t.a < nf(t.front), "gather task");
   for (const Task &t : pl.sdiag_tasks)
@@ -746,7 +788,7 @@ void validate_plan(const Problem &P, const Symbolic &S, const Plan &pl) {
   for (const LevelPlan &LP : pl.levels) {
     need(LP.build_b <= LP.build_e && LP.build_e <= (int32_t)pl.build_tasks.size(), "build range");
     need(LP.k_b <= LP.k_e && LP.k_e <= (int64_t)pl.k_slot.size(), "K range");
-    need(LP.syrk_e <= (int32_t)pl.syrk_tasks.size() && LP.gath_e <= (int32_t)pl.gath_tasks.size() &&
+    need(LP.gath_e <= (int32_t)pl.gath_tasks.size() &&
              LP.rg_e <= (int32_t)pl.rgemv_tasks.size(), "level ranges");
   }
 }
