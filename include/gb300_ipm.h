@@ -592,7 +592,7 @@ IPM_API int32_t ipm_last_perturbed(const ipm_ctx *ctx);
  * kernels on the context's current data. kernel 0: the assembly kernel of
  * Eq. (5) on the inputs of the last kkt_assemble (rewrites the same K);
  * 1: the persistent FP32 triangular solve (both sweeps) with the current
- * FP32-storage factor; 2: the FP64 level-scheduled triangular solve with the
+ * FP32-storage factor; 2: the persistent FP64 triangular solve with the
  * current FP64 factor; 3 and 4: the persistent FP32 solve's forward sweep
  * alone and its backward sweep alone. The solves overwrite the context's
  * solve scratch only.

@@ -448,7 +448,7 @@ class IpmContext:
 
     def kkt_time_kernel(self, kernel: int, reps: int = 3) -> float:
         """Milliseconds per launch of one library kernel (0 assembly,
-        1 persistent FP32 solve, 2 FP64 level solve) on the current data."""
+        1 persistent FP32 solve, 2 persistent FP64 solve) on the current data."""
         ms = C.c_double()
         self._check(self._lib.kkt_time_kernel(self.handle, int(kernel), int(reps), C.byref(ms)))
         return ms.value

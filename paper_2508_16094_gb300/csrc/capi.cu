@@ -50,6 +50,7 @@ struct ipm_ctx {
   double *jv_copy = nullptr, *D_copy = nullptr, *wv_copy = nullptr;  // inputs kept for refinement
   float *Llo = nullptr;  // low parts of the split-TF32 factor
   float *dinv = nullptr, *fsa = nullptr, *fsb = nullptr, *fsx = nullptr;  // persistent FP32 solve
+  double *dinv64 = nullptr, *dsb = nullptr, *dsx = nullptr, *pspart64 = nullptr;  // FP64 (a: yv)
   unsigned *psflags = nullptr;  // its tickets, flags and counters
   float *pspart = nullptr;    // its partial sums
   // learned correction of a stale factor
@@ -188,14 +189,14 @@ void layout(ipm_ctx *c, char *base) {
   d.sgemv = upload(cv, pl.sgemv_tasks, st);
   d.rgemv = upload(cv, pl.rgemv_tasks, st);
   d.toff = upload(cv, pl.toff, st);
-  d.fs_inv = upload(cv, pl.fs_inv, st);
-  d.fs_first_slot = upload(cv, pl.fs_first_slot, st);
-  d.ps_tasks = upload(cv, pl.ps_tasks, st);
-  d.ps_pbase = upload(cv, pl.ps_pbase, st);
-  d.ps_kid_chunks = upload(cv, pl.ps_kid_chunks, st);
-  d.ps_recs = upload(cv, pl.ps_recs, st);
-  d.ps_parent_blocks = upload(cv, pl.ps_parent_blocks, st);
-  d.fs_dinv_off = upload(cv, pl.fs_dinv_off, st);
+  for (auto [ds, sp] : {std::pair<DevSolve *, const SolvePlan *>{&d.s32, &pl.s32}, {&d.s64, &pl.s64}}) {
+    *ds = DevSolve{};
+    if (sp->tasks.empty()) continue;
+    ds->inv = upload(cv, sp->inv, st);
+    ds->recs = upload(cv, sp->recs, st);
+    ds->dinv_off = upload(cv, sp->dinv_off, st);
+    ds->first_slot = upload(cv, sp->first_slot, st);
+  }
   d.k_slot = upload(cv, pl.k_slot, st);
   d.k_poff = upload(cv, pl.k_poff, st);
   d.k_w = upload(cv, pl.k_w, st);
@@ -276,12 +277,18 @@ void layout(ipm_ctx *c, char *base) {
   c->wv_copy = cv.take<double>(std::max<int64_t>(P.wp.empty() ? 0 : P.wp.back(), 1));
   c->vjx = cv.take<double>(m);
   c->vtA = cv.take<double>(m);
-  c->dinv = cv.take<float>(pl.fs_dinv_entries);
+  c->dinv = cv.take<float>(std::max<int64_t>(pl.s32.dinv_entries, 4));
   c->fsa = cv.take<float>(n);
   c->fsb = cv.take<float>(n);
   c->fsx = cv.take<float>(n);
-  c->psflags = cv.take<unsigned>(std::max<int64_t>(pl.ps_flag_words, 32));
-  c->pspart = cv.take<float>(std::max<int64_t>(pl.ps_part_entries, 1));
+  c->psflags = cv.take<unsigned>(std::max<int64_t>(std::max(pl.s32.flag_words, pl.s64.flag_words), 32));
+  c->pspart = cv.take<float>(std::max<int64_t>(pl.s32.part_entries, 1));
+  if (!pl.s64.tasks.empty()) {
+    c->dinv64 = cv.take<double>(pl.s64.dinv_entries);
+    c->dsb = cv.take<double>(n);
+    c->dsx = cv.take<double>(n);
+    c->pspart64 = cv.take<double>(pl.s64.part_entries);
+  }
   {  // learned-correction buffers (only when enabled)
     LearnedBufs &B = c->lb;
     const bool on = c->opts.learned != 0 || c->opts.learned_probes > 0;
@@ -359,8 +366,9 @@ ipm_status do_factor(ipm_ctx *c, int prec, int32_t *bad_col) {
     c->tcp.factor(c->dp, c->plan, c->kval, (float *)c->L, (float *)c->U, c->dinv, c->status,
                   prec == IPM_TF32X3 ? 3 : (prec == IPM_BF16 ? 16 : 1), c->st);
   }
-  if (prec == IPM_FP32)  // explicit inverses of the diagonal blocks for the persistent solve
-    launch_dinv(c->dp, c->plan, (const float *)c->L, c->dinv, c->st);  // (the TF32 paths write them)
+  // explicit inverses of the diagonal blocks for the persistent solve (the TF32 paths write them)
+  if (prec == IPM_FP32) launch_dinv(c->dp, c->plan, (const float *)c->L, c->dinv, c->st);
+  else if (prec == IPM_FP64) launch_dinv(c->dp, c->plan, (const double *)c->L, c->dinv64, c->st);
   CK(cudaGetLastError());
   int32_t out[ST_COUNT];
   CK(cudaMemcpyAsync(out, c->status, sizeof(out), cudaMemcpyDeviceToHost, c->st));
@@ -374,6 +382,7 @@ ipm_status do_factor(ipm_ctx *c, int prec, int32_t *bad_col) {
     CK(cudaMemcpyAsync(c->status, init, sizeof(init), cudaMemcpyHostToDevice, c->st));
     launch_factor_simt<double>(c->dp, c->plan, c->kval, (double *)c->L, (double *)c->U, c->status,
                                false, c->st);
+    launch_dinv(c->dp, c->plan, (const double *)c->L, c->dinv64, c->st);
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(out, c->status, sizeof(out), cudaMemcpyDeviceToHost, c->st));
     CK(cudaStreamSynchronize(c->st));
@@ -395,14 +404,31 @@ ipm_status do_factor(ipm_ctx *c, int prec, int32_t *bad_col) {
   return IPM_OK;
 }
 
-// One persistent FP32 solve launch over the workspace vectors: which = 0 both
-// sweeps (fsa -> fsx), 1 forward only (fsa -> fsb), 2 backward only (fsb -> fsx)
-void launch_fp32_solve(ipm_ctx *c, int which) {
-  launch_psolve(c->dp, c->plan, (const float *)c->L, c->dinv, c->fsa, c->fsb, c->fsx,
-                reinterpret_cast<float *>(c->tv), c->pspart, c->psflags, c->status, which != 2, which != 1,
-                c->st, c->test_spins, c->test_withhold);
+// One persistent solve launch over the workspace vectors: which = 0 both sweeps
+// (fsa -> fsx; FP64: yv -> dsx), 1 forward only (fsa -> fsb; yv -> dsb), 2 backward
+// only (fsb -> fsx; dsb -> dsx)
+template <typename T> void launch_held_solve(ipm_ctx *c, int which);
+template <> void launch_held_solve<float>(ipm_ctx *c, int which) {
+  launch_psolve<float>(c->dp, c->plan, (const float *)c->L, c->dinv, c->fsa, c->fsb, c->fsx,
+                       reinterpret_cast<float *>(c->tv), c->pspart, c->psflags, c->status, which != 2,
+                       which != 1, c->st, c->test_spins, c->test_withhold);
   c->test_spins = 0;
   c->test_withhold = -1;
+}
+template <> void launch_held_solve<double>(ipm_ctx *c, int which) {
+  launch_psolve<double>(c->dp, c->plan, (const double *)c->L, c->dinv64, c->yv, c->dsb, c->dsx, c->tv,
+                        c->pspart64, c->psflags, c->status, which != 2, which != 1, c->st, c->test_spins,
+                        c->test_withhold);
+  c->test_spins = 0;
+  c->test_withhold = -1;
+}
+void launch_fp32_solve(ipm_ctx *c, int which) { launch_held_solve<float>(c, which); }
+// Both sweeps, with K = L S L^T's signs between them for a quasi-definite system.
+template <typename T> void launch_both_sweeps(ipm_ctx *c, T *mid) {
+  if (!c->dp.sgn) return launch_held_solve<T>(c, 0);
+  launch_held_solve<T>(c, 1);
+  launch_sign<T>(c->dp, mid, c->st);
+  launch_held_solve<T>(c, 2);
 }
 
 // out = M^{-1} b with the current factor (b, out: original numbering, device)
@@ -421,20 +447,14 @@ void apply_factor(ipm_ctx *c, const double *b, double *out, bool accumulate) {
   }
   if (c->storage_bytes == 8 && c->factor_prec == IPM_FP64) {
     V.permute_in<double>(b, nullptr, c->yv);
-    launch_solve<double, double>(c->dp, c->plan, (const double *)c->L, c->yv, c->tv, c->st);
-    V.permute_out<double>(c->yv, nullptr, out, accumulate);
+    launch_both_sweeps<double>(c, c->dsb);
+    V.permute_out<double>(c->dsx, nullptr, out, accumulate);
   } else {
     double *scale = c->scal + 8, *amax = c->scal + 9;
     V.absmax(c->P.n, b, amax);
     V.inv_scale(amax, scale);
     V.permute_in<float>(b, scale, c->fsa);
-    if (c->dp.sgn) {  // K = L S L^T: forward sweep, S, backward sweep
-      launch_fp32_solve(c, 1);
-      launch_sign<float>(c->dp, c->fsb, c->st);
-      launch_fp32_solve(c, 2);
-    } else {
-      launch_fp32_solve(c, 0);
-    }
+    launch_both_sweeps<float>(c, c->fsb);
     V.permute_out<float>(c->fsx, scale, out, accumulate);
   }
 }
@@ -554,7 +574,7 @@ ipm_status do_solve(ipm_ctx *c, const double *b, double *x, int refine, ipm_solv
   }
   CK(cudaMemcpyAsync(x, xx, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
   CK(cudaGetLastError());
-  if (c->factor_prec != IPM_FP64) check_solve_barrier(c);
+  check_solve_barrier(c);
   if (c->bwd_measure) rel = bwd;
   c->last_rel = rel;
   if (info) *info = ipm_solve_info{iters, used_pcg, rel};
@@ -1027,13 +1047,15 @@ ipm_status kkt_analyze(ipm_ctx *c, const int32_t *perm, ipm_symbolic_info *info)
     analyze_symbolic(c->P, perm, c->S);
     build_plan(c->P, c->S, c->plan, 64, 64);
     validate_plan(c->P, c->S, c->plan);
-    build_fused_solve(c->plan);
+    build_fused_solve(c->plan, kSolveB32, c->plan.s32);
     c->tcp.build(c->plan);
     c->oz_on = c->opts.fp64_tc != 0 && c->sign_orig.empty();
     if (c->oz_on) c->ozp.build(c->plan);
     const int so = c->opts.storage_fp64;
     c->storage_bytes = (so == 1 || c->oz_on ||
                         (so < 0 && (c->opts.precision == IPM_FP64 || c->opts.fallback_fp64))) ? 8 : 4;
+    c->plan.s64 = SolvePlan{};
+    if (c->storage_bytes == 8) build_fused_solve(c->plan, kSolveB64, c->plan.s64);
     layout(c, nullptr);
     c->state = 1;
     if (info) {
@@ -1519,7 +1541,7 @@ ipm_status kkt_time_kernel(ipm_ctx *c, int32_t kernel, int32_t reps, double *ms)
     if ((kernel == 1 || kernel == 3 || kernel == 4) && c->factor_prec == IPM_FP64)
       throw Fail{IPM_ERR_STATE, "the persistent solve needs an FP32-storage factor"};
     if (kernel == 2 && c->factor_prec != IPM_FP64)
-      throw Fail{IPM_ERR_STATE, "the level solve is timed on an FP64 factor"};
+      throw Fail{IPM_ERR_STATE, "the FP64 solve is timed on an FP64 factor"};
     if (kernel < 0 || kernel > 4) throw Fail{IPM_ERR_ARG, "unknown kernel id"};
     // the solves' work does not depend on the values: zero right-hand sides
     if (kernel == 1 || kernel == 3) CK(cudaMemsetAsync(c->fsa, 0, c->P.n * sizeof(float), c->st));
@@ -1537,7 +1559,7 @@ ipm_status kkt_time_kernel(ipm_ctx *c, int32_t kernel, int32_t reps, double *ms)
       else if (kernel == 3 || kernel == 4)
         launch_fp32_solve(c, kernel == 3 ? 1 : 2);
       else
-        launch_solve<double, double>(c->dp, c->plan, (const double *)c->L, c->yv, c->tv, c->st);
+        launch_held_solve<double>(c, 0);
     }
     CK(cudaEventRecord(e1, c->st));
     CK(cudaEventSynchronize(e1));
@@ -1546,7 +1568,7 @@ ipm_status kkt_time_kernel(ipm_ctx *c, int32_t kernel, int32_t reps, double *ms)
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     CK(cudaGetLastError());
-    if (kernel == 1 || kernel >= 3) check_solve_barrier(c);
+    if (kernel != 0) check_solve_barrier(c);
     *ms = (double)t / reps;
     return IPM_OK;
   });

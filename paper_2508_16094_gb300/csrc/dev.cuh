@@ -9,19 +9,21 @@
 
 namespace gipm {
 
+// Device arrays of a SolvePlan.
+struct DevSolve {
+  const Task *inv;
+  const SolveRec *recs;       // per task: the task with its front's data
+  const int64_t *dinv_off;    // per slot
+  const int32_t *first_slot;  // per front: slot of its first diagonal block
+};
+
 // Device pointers of the plan and problem structure (all inside the caller's workspace).
 struct DevPlan {
   const FrontInfo *fronts;
   const int32_t *children, *inv, *relpos, *sri;
   const Task *build, *potrf, *trsm, *upd, *gath, *sdiag, *sgemv, *rgemv;
   const int64_t *toff;
-  const Task *fs_inv, *ps_tasks;  // persistent FP32 solve
-  const int64_t *ps_pbase;        // per front: first partial-sum row of its backward tasks
-  const int32_t *ps_kid_chunks;   // per front: below-front chunks of all its children
-  const SolveRec *ps_recs;        // per task: the task with its front's data
-  const int32_t *ps_parent_blocks;  // per front: diagonal blocks of its parent
-  const int64_t *fs_dinv_off;
-  const int32_t *fs_first_slot;  // per front: slot of its first diagonal block
+  DevSolve s32, s64;  // persistent solves (s64: null unless the storage is sized for FP64)
   const int64_t *k_slot, *k_poff, *k_w, *k_orig;
   const int32_t *k_pa, *k_pb, *k_diag;
   const int32_t *perm;  // final new -> old

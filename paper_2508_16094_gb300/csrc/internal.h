@@ -52,7 +52,7 @@ struct Task {
   int32_t front, a, b, c;
 };
 
-// One task of the persistent FP32 solve with everything it reads of its front,
+// One task of the persistent solve with everything it reads of its front,
 // so a CTA fetches what its next task needs in a single 112-byte copy.
 struct SolveRec {
   Task task;
@@ -66,10 +66,10 @@ struct SolveRec {
 };
 static_assert(sizeof(SolveRec) == 112 && sizeof(SolveRec) % 16 == 0, "SolveRec layout");
 
-// A task of the persistent FP32 solve. Tasks run in the order of the plan
+// A task of a persistent solve. Tasks run in the order of the plan
 // (a ticket taken from a global counter), and a task waits only for tasks
 // earlier in that order (flags and counters in device memory), so the solve
-// needs no grid barrier and cannot deadlock. Blocks are 128 wide.
+// needs no grid barrier and cannot deadlock. (Sizes below: FP32, 128-wide blocks.)
 enum SolveTaskKind : int32_t {
   WS_FWD_DIAG = 0,   // (front, a = block i): gather the children's update entries for
                      // the block's rows, subtract L_ij y_j for j < i as each y_j is
@@ -166,6 +166,29 @@ struct LevelPlan {
   int32_t max_ncol = 0;
 };
 
+// Persistent solve over blocks of `B` columns and chunks of `B` rows: inverses of
+// the diagonal blocks (slot s: jb rows of jb rounded up to 16 bytes at
+// dinv_off[s]; the slots of a front are consecutive from first_slot[front]) and
+// the task list, forward tasks first. Flags (32-bit words): [0, 32) tickets, then
+// per slot "y published", "x published", "partial sums done", per front
+// "update-vector chunks of its children done", "column blocks done".
+constexpr int kSolveB32 = 128, kSolveB64 = 64;  // block widths, FP32 and FP64
+struct SolvePlan {
+  int B = 0;
+  std::vector<Task> inv;                  // (front, first column, slot)
+  std::vector<int32_t> first_slot;        // per front: slot of block 0
+  std::vector<int64_t> dinv_off;
+  int64_t dinv_entries = 0;
+  std::vector<Task> tasks;                // (front, a, b, kind)
+  int32_t fwd_tasks = 0;
+  std::vector<int64_t> pbase;             // per front: first partial-sum row (B values each)
+  std::vector<SolveRec> recs;             // per task: the task and its front's data
+  std::vector<int32_t> kid_chunks;        // per front: below-front chunks of all its children
+  std::vector<int32_t> parent_blocks;     // per front: diagonal blocks of its parent (0 at roots)
+  int64_t part_entries = 0;               // values of partial sums
+  int64_t flag_words = 0;
+};
+
 // Numeric plan: everything the kernels need, built on the host by analysis.
 struct Plan {
   static constexpr int kSuper32 = 256;  // columns per super-step of the FP32 FMA-pipe factor
@@ -182,24 +205,7 @@ struct Plan {
   std::vector<Task> gath_tasks, sdiag_tasks, sgemv_tasks, rgemv_tasks;
   std::vector<int64_t> toff;         // per front: offset of its solve update vector (length nrow)
   int64_t t_entries = 0;
-  // persistent FP32 solve: inverses of the 128-wide diagonal blocks (slot s:
-  // jb rows of round_up(jb, 4) floats at fs_dinv_off[s]; the slots of a front
-  // are consecutive from fs_first_slot[front]) and its task list, forward
-  // tasks first. Flags (32-bit words): [0, 32) tickets, then per slot "y
-  // published", "x published", "partial sums done", per front "update-vector
-  // chunks of its children done", "column blocks done".
-  std::vector<Task> fs_inv;                  // (front, first column, slot)
-  std::vector<int32_t> fs_first_slot;        // per front: slot of block 0
-  std::vector<int64_t> fs_dinv_off;
-  int64_t fs_dinv_entries = 0;
-  std::vector<Task> ps_tasks;                // (front, a, b, kind)
-  int32_t ps_fwd_tasks = 0;
-  std::vector<int64_t> ps_pbase;             // per front: first partial-sum row (128 floats each)
-  std::vector<SolveRec> ps_recs;             // per task: the task and its front's data
-  std::vector<int32_t> ps_kid_chunks;        // per front: below-front chunks of all its children
-  std::vector<int32_t> ps_parent_blocks;     // per front: diagonal blocks of its parent (0 at roots)
-  int64_t ps_part_entries = 0;               // floats of partial sums
-  int64_t ps_flag_words = 0;
+  SolvePlan s32, s64;  // persistent solves (s64: when the storage is sized for FP64)
   // K entries in level-major order
   std::vector<int64_t> k_slot;   // element offset of L(i, j) in the factor storage
   std::vector<int64_t> k_poff;   // products [k_poff[q], k_poff[q+1])
@@ -231,7 +237,7 @@ struct Problem {
 void analyze_symbolic(const Problem &P, const int32_t *perm, Symbolic &S);
 void build_plan(const Problem &P, const Symbolic &S, Plan &plan, int nb, int nbs);
 void validate_plan(const Problem &P, const Symbolic &S, const Plan &plan);
-// Task lists of the fused FP32 solve (128-wide blocks), appended to the plan.
-void build_fused_solve(Plan &plan);
+// Task lists of a persistent solve with blocks of B columns (128 FP32, 64 FP64).
+void build_fused_solve(const Plan &plan, int B, SolvePlan &sp);
 
 }  // namespace gipm

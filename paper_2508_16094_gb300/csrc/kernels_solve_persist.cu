@@ -1,8 +1,9 @@
-// Persistent supernodal triangular solves for FP32 factors (TF32/TF32x3/BF16/FP32).
+// Persistent supernodal triangular solves (FP32 storage: TF32/TF32x3/BF16/FP32
+// factors, 128-wide blocks; FP64 storage: 64-wide blocks, so a lane reads 16
+// bytes of a row either way and a tile holds as many loads in flight).
 //
-// After each factorisation one launch inverts every 128-wide diagonal block of
-// L (explicit inverse, rows padded to a multiple of 4 floats). A solve is then
-// ONE launch of a persistent kernel whose CTAs take the tasks of the plan in
+// After each factorisation one launch inverts every diagonal block of L
+// (explicit inverse, rows padded to 16 bytes). A solve is then ONE launch of a persistent kernel whose CTAs take the tasks of the plan in
 // order from a global ticket counter (forward sweep leaves -> root, backward
 // sweep root -> leaves). Instead of grid barriers between phases, each task
 // waits only for the results it reads, published through flags and counters
@@ -28,9 +29,49 @@ namespace gipm {
 
 namespace {
 
-constexpr int kB = 128;                     // block width of the solve
 constexpr int kT = 256;                     // threads per CTA
 constexpr unsigned kBarrierSpins = 1u << 24;  // polls of >= 0.3 us each: seconds before giving up
+
+// Shapes of a solve over values of type T: blocks of B columns and chunks of B
+// rows, a warp takes RW rows and a lane the VW columns of one 16-byte load.
+template <typename T> struct Ps {
+  static constexpr int VW = 16 / (int)sizeof(T), B = 32 * VW, RW = B / (kT / 32);
+};
+static_assert(Ps<float>::B == kSolveB32 && Ps<double>::B == kSolveB64, "block widths of the plan");
+template <typename T> struct alignas(16) Vec {
+  T v[Ps<T>::VW];
+};
+template <typename T> __device__ __forceinline__ Vec<T> vzero() {
+  Vec<T> z;
+#pragma unroll
+  for (int h = 0; h < Ps<T>::VW; h++) z.v[h] = T(0);
+  return z;
+}
+// 16 bytes as one load or store (a copy of the struct is split into its members).
+__device__ __forceinline__ Vec<float> from16(float4 f) { return Vec<float>{{f.x, f.y, f.z, f.w}}; }
+__device__ __forceinline__ Vec<double> from16(double2 f) { return Vec<double>{{f.x, f.y}}; }
+__device__ __forceinline__ Vec<float> ldg16(const float *p) { return from16(__ldg(reinterpret_cast<const float4 *>(p))); }
+__device__ __forceinline__ Vec<double> ldg16(const double *p) { return from16(__ldg(reinterpret_cast<const double2 *>(p))); }
+__device__ __forceinline__ Vec<float> ld16(const float *p) { return from16(*reinterpret_cast<const float4 *>(p)); }
+__device__ __forceinline__ Vec<double> ld16(const double *p) { return from16(*reinterpret_cast<const double2 *>(p)); }
+__device__ __forceinline__ void st16(float *p, const Vec<float> &v) {
+  *reinterpret_cast<float4 *>(p) = make_float4(v.v[0], v.v[1], v.v[2], v.v[3]);
+}
+__device__ __forceinline__ void st16(double *p, const Vec<double> &v) {
+  *reinterpret_cast<double2 *>(p) = make_double2(v.v[0], v.v[1]);
+}
+// acc + <a, b>, the last component first
+template <typename T>
+__device__ __forceinline__ T vdot(const Vec<T> &a, const Vec<T> &b, T acc) {
+#pragma unroll
+  for (int h = Ps<T>::VW - 1; h >= 0; h--) acc = fma(a.v[h], b.v[h], acc);
+  return acc;
+}
+template <typename T> __device__ __forceinline__ Vec<T> vfma(const Vec<T> &l, T y, Vec<T> acc) {
+#pragma unroll
+  for (int h = 0; h < Ps<T>::VW; h++) acc.v[h] = fma(l.v[h], y, acc.v[h]);
+  return acc;
+}
 
 void ck(cudaError_t e, const char *what) {
   if (e != cudaSuccess) throw std::runtime_error(std::string(what) + ": " + cudaGetErrorString(e));
@@ -41,8 +82,8 @@ void ck(cudaError_t e, const char *what) {
 // floats with zeros above the diagonal and in the padding.
 __global__ void __launch_bounds__(128) dinv_kernel(DevPlan dp, const float *__restrict__ L,
                                                    float *__restrict__ Dinv) {
-  constexpr int LS = 129;
-  const Task tk = dp.fs_inv[blockIdx.x];
+  constexpr int LS = 129, kB = Ps<float>::B;
+  const Task tk = dp.s32.inv[blockIdx.x];
   const FrontInfo F = dp.fronts[tk.front];
   const int j = tk.a, jb = min(kB, F.ncol - j), ldi = (jb + 3) & ~3, tid = threadIdx.x;
   extern __shared__ float smd[];
@@ -63,19 +104,68 @@ __global__ void __launch_bounds__(128) dinv_kernel(DevPlan dp, const float *__re
     }
   }
   __syncthreads();
-  float *out = Dinv + dp.fs_dinv_off[tk.b];
+  float *out = Dinv + dp.s32.dinv_off[tk.b];
   for (int e = tid; e < jb * ldi; e += 128) {
     const int r = e / ldi, c = e % ldi;
     out[e] = (c <= r && c < jb) ? X[r * LS + c] : 0.f;
   }
 }
 
-struct PsArgs {
+// FP64: inverse of one diagonal block (jb <= 64), thread c builds column c in
+// registers, right-looking: x_m is finished, then every row below it takes its
+// multiple (independent multiply-adds, where a row's dot product would be one
+// chain). Warp 1's columns start at row 32, so it skips the rows above. Bound
+// by the FP64 pipe (2608 warp multiply-adds, 20 us of one SM per block).
+template <int N>
+__device__ __forceinline__ void inverse_columns(const double *A, const double *rd, int ls, int r0, int c,
+                                                int jb, double (&x)[N]) {
+#pragma unroll
+  for (int i = 0; i < N; i++) x[i] = r0 + i == c ? 1.0 : 0.0;
+#pragma unroll
+  for (int m = 0; m < N; m++) {
+    if (r0 + m >= jb) break;
+    x[m] *= rd[r0 + m];
+#pragma unroll
+    for (int i = m + 1; i < N; i++) x[i] = fma(-x[m], A[(r0 + m) * ls + r0 + i], x[i]);
+  }
+}
+__global__ void __launch_bounds__(64) dinv64_kernel(DevPlan dp, const double *__restrict__ L,
+                                                    double *__restrict__ Dinv) {
+  constexpr int kB = Ps<double>::B, LS = kB + 1;
+  const Task tk = dp.s64.inv[blockIdx.x];
+  const FrontInfo F = dp.fronts[tk.front];
+  const int j = tk.a, jb = min(kB, F.ncol - j), ldi = (jb + 1) & ~1, c = threadIdx.x;
+  __shared__ double A[kB * LS];  // column m of the block: A[m * LS + i], zero past jb
+  __shared__ double rd[kB];
+  const double *g = L + F.loff + (int64_t)j * F.ld + j;
+#pragma unroll 16
+  for (int i = 0; i < kB; i++) A[c * LS + i] = (i < jb && c <= i) ? g[(int64_t)i * F.ld + c] : 0.0;
+  __syncthreads();
+  if (c < jb) rd[c] = 1.0 / A[c * LS + c];
+  __syncthreads();
+  double *out = Dinv + dp.s64.dinv_off[tk.b];
+  if (c < 32) {
+    double x[kB];
+    inverse_columns<kB>(A, rd, LS, 0, c, jb, x);
+#pragma unroll
+    for (int i = 0; i < kB; i++)
+      if (i < jb && c < ldi) out[i * ldi + c] = c < jb ? x[i] : 0.0;
+  } else {
+    double x[kB / 2];
+    inverse_columns<kB / 2>(A, rd, LS, kB / 2, c, jb, x);
+#pragma unroll
+    for (int i = 0; i < kB; i++)
+      if (i < jb && c < ldi) out[i * ldi + c] = (i >= 32 && c < jb) ? x[i >= 32 ? i - 32 : 0] : 0.0;
+  }
+}
+
+template <typename T> struct PsArgs {
   DevPlan dp;
-  const float *L, *Dinv;
-  float *a, *b, *x, *t, *part;
+  DevSolve sv;
+  const T *L, *Dinv;
+  T *a, *b, *x, *t, *part;
   int32_t q0, q1;    // tasks [q0, q1) of the plan
-  unsigned *flags;   // plan.ps_flag_words words, zeroed before the launch
+  unsigned *flags;   // the solve plan's flag words, zeroed before the launch
   int32_t *status;   // ST_SOLVE_TIMEOUT
   unsigned spins;    // polls before a wait gives up
   int32_t withhold;  // test of the bounded wait: the task of this ticket is abandoned (-1: none)
@@ -83,19 +173,10 @@ struct PsArgs {
   int32_t fwd_here;  // the forward sweep runs in this launch: backward blocks wait for their y
 };
 
-constexpr int kRC = 128;  // rows below a front per task
 constexpr int kMaxKids = 32;  // children staged in shared memory for the gathers
 constexpr long long kCopySpinCycles = 2000000000ll;  // bounded wait on a staging copy (~1 s)
 
-__device__ __forceinline__ float ldcg(const float *p) { return __ldcg(p); }
-
-__device__ __forceinline__ float4 fma4(const float4 l, float y, float4 acc) {
-  acc.x = fmaf(l.x, y, acc.x);
-  acc.y = fmaf(l.y, y, acc.y);
-  acc.z = fmaf(l.z, y, acc.z);
-  acc.w = fmaf(l.w, y, acc.w);
-  return acc;
-}
+template <typename T> __device__ __forceinline__ T ldcg(const T *p) { return __ldcg(p); }
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -103,28 +184,36 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) {
 
 // Flag words (see Plan): tickets, then per slot y / x published and partial
 // sums done, per front update-vector chunks and column blocks done.
-__device__ __forceinline__ unsigned *f_ticket(const PsArgs &A) { return A.flags; }
-__device__ __forceinline__ unsigned *f_y(const PsArgs &A, int slot) { return A.flags + 32 + slot; }
-__device__ __forceinline__ unsigned *f_x(const PsArgs &A, int slot) { return A.flags + 32 + A.nslot + slot; }
-__device__ __forceinline__ unsigned *f_part(const PsArgs &A, int slot) {
+template <typename T>
+__device__ __forceinline__ unsigned *f_ticket(const PsArgs<T> &A) { return A.flags; }
+template <typename T>
+__device__ __forceinline__ unsigned *f_y(const PsArgs<T> &A, int slot) { return A.flags + 32 + slot; }
+template <typename T>
+__device__ __forceinline__ unsigned *f_x(const PsArgs<T> &A, int slot) { return A.flags + 32 + A.nslot + slot; }
+template <typename T>
+__device__ __forceinline__ unsigned *f_part(const PsArgs<T> &A, int slot) {
   return A.flags + 32 + 2 * A.nslot + slot;
 }
 // per front: chunks of rows below its children that are done (the children's
 // update vectors are complete once it reaches ps_kid_chunks[front])
-__device__ __forceinline__ unsigned *f_tvec(const PsArgs &A, int front) {
+template <typename T>
+__device__ __forceinline__ unsigned *f_tvec(const PsArgs<T> &A, int front) {
   return A.flags + 32 + 3 * A.nslot + front;
 }
-__device__ __forceinline__ unsigned *f_front(const PsArgs &A, int front) {
+template <typename T>
+__device__ __forceinline__ unsigned *f_front(const PsArgs<T> &A, int front) {
   return A.flags + 32 + 3 * A.nslot + A.nfr + front;
 }
 
 // Shared scratch of one CTA (dynamic shared memory).
-struct PsShared {
-  float di[kB * kB];            // staged inverse of a diagonal block (TMA bulk copy)
-  float sv[kB];                 // values handed to the diagonal-block solve
-  float xs[kRC];                // solution entries of the rows below a front
-  float red[kT / 32][16][33];   // per-warp transpose reduction of 16 row sums
-  float4 red4[kT / 32][32];     // per-row-group column sums
+template <typename T> struct PsShared {
+  static constexpr int B = Ps<T>::B;
+  T di[B * B];                  // staged inverse of a diagonal block (TMA bulk copy)
+  alignas(16) T sv[B];          // values handed to the diagonal-block solve
+  T xs[B];                      // solution entries of the rows below a front
+  T red[sizeof(T) == 4 ? kT / 32 : 1][Ps<T>::RW][33];  // FP32: per-warp transpose reduction of RW row sums
+  alignas(16) T ys[2][B];                   // FP64: the y block of the running product (double-buffered)
+  alignas(16) T red4[kT / 32][B];  // per-row-group column sums
   unsigned long long mbar;      // completion of the staging copy
   uint32_t parity;              // its phase
   int tk;                       // this CTA's current task
@@ -137,9 +226,11 @@ struct PsShared {
 };
 
 // Thread 0: start the bulk copy of a diagonal-block inverse into S.di.
-__device__ __forceinline__ void stage_dinv(const PsArgs &A, PsShared &S, int slot, int jb) {
-  const uint32_t bytes = (uint32_t)(jb * ((jb + 3) & ~3) * (int)sizeof(float));
-  const float *src = A.Dinv + A.dp.fs_dinv_off[slot];
+template <typename T>
+__device__ __forceinline__ void stage_dinv(const PsArgs<T> &A, PsShared<T> &S, int slot, int jb) {
+  constexpr int VW = Ps<T>::VW;
+  const uint32_t bytes = (uint32_t)(jb * ((jb + VW - 1) & ~(VW - 1)) * (int)sizeof(T));
+  const T *src = A.Dinv + A.sv.dinv_off[slot];
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&S.mbar)),
                "r"(bytes)
@@ -153,7 +244,8 @@ __device__ __forceinline__ void stage_dinv(const PsArgs &A, PsShared &S, int slo
 
 // All threads: bounded wait for the staging copy; false after a timeout (the
 // status word is set, and a second bounded wait lets the copy land first).
-__device__ bool wait_dinv(const PsArgs &A, PsShared &S) {
+template <typename T>
+__device__ bool wait_dinv(const PsArgs<T> &A, PsShared<T> &S) {
   const uint32_t par = S.parity;
   auto try_wait = [&]() {
     uint32_t done;
@@ -183,78 +275,218 @@ __device__ bool wait_dinv(const PsArgs &A, PsShared &S) {
   return ok;
 }
 
-// Row sums of 16 consecutive rows per warp: p[k] = <row k, v> for the lane's 4
-// columns; returns the full sum of row `lane` in lanes 0..15.
-__device__ __forceinline__ float rows16_reduce(PsShared &S, const float (&p)[16]) {
+// Row sums of RW consecutive rows per warp: p[k] = <row k, v> for the lane's VW
+// columns; returns the full sum of row `lane` in lanes 0 .. RW - 1.
+__device__ __forceinline__ float rows_reduce(PsShared<float> &S, const float (&p)[Ps<float>::RW]) {
+  constexpr int RW = Ps<float>::RW;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
 #pragma unroll
-  for (int k = 0; k < 16; k++) S.red[warp][k][lane] = p[k];
+  for (int k = 0; k < RW; k++) S.red[warp][k][lane] = p[k];
   __syncwarp();
   float s = 0.f;
-  if (lane < 16) {
+  if (lane < RW) {
 #pragma unroll 8
     for (int q = 0; q < 32; q++) s += S.red[warp][lane][q];
   }
   __syncwarp();
   return s;
 }
+// Sum over the four neighbouring lanes (valid in all of them).
+__device__ __forceinline__ double quad_sum(double v) {
+  v += __shfl_xor_sync(0xffffffffu, v, 1);
+  return v + __shfl_xor_sync(0xffffffffu, v, 2);
+}
+
+// Product of a B x B tile's rows (row stride ld) with a block of the forward
+// result, accumulated over tiles. The loads of a tile are issued by load(),
+// before the block is waited for.
+//  FP32: warp w takes rows 16w .. 16w + 15, lane: columns 4 lane ..; the row sums
+//  are reduced across the warp once, after the last tile.
+//  FP64: an addition costs as much as a multiply-add (64 cycles per warp on a
+//  quarter SM), so the cross-lane reduction is kept short: four threads share a
+//  row (thread h: columns 8m + 2h, 8m + 2h + 1) and y comes from shared memory.
+template <typename T> struct FwdTile;
+template <> struct FwdTile<float> {
+  static constexpr int RW = Ps<float>::RW;
+  float4 l[RW];
+  float acc[RW];
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int k = 0; k < RW; k++) acc[k] = 0.f;
+  }
+  // FULL: the block has all B columns
+  template <bool FULL>
+  __device__ __forceinline__ void load(const float *P, int64_t ld, int nr, int nc) {
+    const int c = 4 * (threadIdx.x % 32), rw = RW * (threadIdx.x / 32);
+    const float *row = P + (int64_t)rw * ld + c;
+#pragma unroll
+    for (int k = 0; k < RW; k++)
+      l[k] = ((FULL || c < nc) && rw + k < nr) ? __ldg(reinterpret_cast<const float4 *>(row + (int64_t)k * ld))
+                                               : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  // y: block of nc values; columns past nc (padding of a last block) never enter
+  template <bool FULL>
+  __device__ __forceinline__ void mul(PsShared<float> &, int, const float *y, int nc) {
+    const int c = 4 * (threadIdx.x % 32);
+    const float *yb = y + c;
+    const float4 y4 = FULL ? make_float4(ldcg(yb), ldcg(yb + 1), ldcg(yb + 2), ldcg(yb + 3))
+                           : make_float4(c < nc ? ldcg(yb) : 0.f, c + 1 < nc ? ldcg(yb + 1) : 0.f,
+                                         c + 2 < nc ? ldcg(yb + 2) : 0.f, c + 3 < nc ? ldcg(yb + 3) : 0.f);
+#pragma unroll
+    for (int k = 0; k < RW; k++) {
+      float4 v = l[k];
+      if (!FULL) {
+        if (c + 1 >= nc) v.y = 0.f;
+        if (c + 2 >= nc) v.z = 0.f;
+        if (c + 3 >= nc) v.w = 0.f;
+      }
+      acc[k] = fmaf(v.x, y4.x, fmaf(v.y, y4.y, fmaf(v.z, y4.z, fmaf(v.w, y4.w, acc[k]))));
+    }
+  }
+  // f(row, sum) once per row
+  template <typename F> __device__ __forceinline__ void finish(PsShared<float> &S, int nr, F f) {
+    const float s = rows_reduce(S, acc);
+    const int lane = threadIdx.x % 32, r = RW * (threadIdx.x / 32) + lane;
+    if (lane < RW && r < nr) f(r, s);
+  }
+};
+template <> struct FwdTile<double> {
+  static constexpr int NL = 8;
+  Vec<double> l[NL];
+  double acc;
+  __device__ __forceinline__ void clear() { acc = 0.0; }
+  template <bool FULL>
+  __device__ __forceinline__ void load(const double *P, int64_t ld, int nr, int nc) {
+    const int r = threadIdx.x / 4, c = 2 * (threadIdx.x % 4);
+    const double *row = P + (int64_t)r * ld + c;
+#pragma unroll
+    for (int m = 0; m < NL; m++)
+      l[m] = (r < nr && (FULL || 8 * m + c < nc)) ? ldg16(row + 8 * m) : vzero<double>();
+  }
+  template <bool FULL>
+  __device__ __forceinline__ void mul(PsShared<double> &S, int j, const double *y, int nc) {
+    double *ys = S.ys[j & 1];  // the other buffer may still be read by slower threads
+    if (threadIdx.x < Ps<double>::B) ys[threadIdx.x] = (int)threadIdx.x < nc ? ldcg(y + threadIdx.x) : 0.0;
+    __syncthreads();
+    const int c = 2 * (threadIdx.x % 4);
+#pragma unroll
+    for (int m = 0; m < NL; m++) {
+      Vec<double> x = l[m];
+      if (!FULL && 8 * m + c + 1 >= nc) x.v[1] = 0.0;
+      acc = vdot(x, ld16(ys + 8 * m + c), acc);
+    }
+  }
+  template <typename F> __device__ __forceinline__ void finish(PsShared<double> &, int nr, F f) {
+    const double s = quad_sum(acc);
+    const int r = threadIdx.x / 4;
+    if (threadIdx.x % 4 == 0 && r < nr) f(r, s);
+  }
+};
 
 // b[first + j + r] = sum_c Dinv[r][c] v[c]  (Dinv staged in S.di, v = S.sv
-// zero past jb); warp w takes rows 16w .. 16w + 15
-__device__ void diag_fwd(const PsArgs &A, PsShared &S, const FrontInfo &F, int j) {
-  const int jb = min(kB, F.ncol - j), ldi = (jb + 3) & ~3;
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, c = 4 * lane, rw = 16 * warp;
+// zero past jb); FP32: warp w takes rows 16w .. 16w + 15
+__device__ void diag_fwd(const PsArgs<float> &A, PsShared<float> &S, const FrontInfo &F, int j) {
+  constexpr int B = Ps<float>::B, RW = Ps<float>::RW;
+  const int jb = min(B, F.ncol - j), ldi = (jb + 3) & ~3;
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, c = 4 * lane, rw = RW * warp;
   if (rw >= jb) return;  // whole warp idle (uniform per warp)
   const float4 v4 = *reinterpret_cast<const float4 *>(S.sv + c);
-  float p[16];
+  float p[RW];
 #pragma unroll
-  for (int k = 0; k < 16; k++) {
+  for (int k = 0; k < RW; k++) {
     p[k] = 0.f;
     if (c < ldi && rw + k < jb) {
       const float4 d = *reinterpret_cast<const float4 *>(S.di + (rw + k) * ldi + c);
       p[k] = d.x * v4.x + d.y * v4.y + d.z * v4.z + d.w * v4.w;
     }
   }
-  const float s = rows16_reduce(S, p);
-  if (lane < 16 && rw + lane < jb) A.b[F.first + j + rw + lane] = s;
+  const float s = rows_reduce(S, p);
+  if (lane < RW && rw + lane < jb) A.b[F.first + j + rw + lane] = s;
+}
+// FP64: four threads per row, and a warp's eight rows stop at their diagonal
+__device__ void diag_fwd(const PsArgs<double> &A, PsShared<double> &S, const FrontInfo &F, int j) {
+  constexpr int B = Ps<double>::B;
+  const int jb = min(B, F.ncol - j), ldi = (jb + 1) & ~1, r = threadIdx.x / 4, c = 2 * (threadIdx.x % 4);
+  double s = 0.0;
+  for (int m = 0; m <= (int)threadIdx.x / 32; m++)
+    if (r < jb && 8 * m + c < ldi)
+      s = vdot(ld16(S.di + r * ldi + 8 * m + c), ld16(S.sv + 8 * m + c), s);
+  s = quad_sum(s);
+  if (threadIdx.x % 4 == 0 && r < jb) A.b[F.first + j + r] = s;
 }
 
+// Column sums over the row groups of S.red4: FP32 on the first warp, f(first of
+// four columns, their sums); FP64 with four threads per column, f(column, its sum).
+template <typename Fn> __device__ __forceinline__ void groups_sum(const PsShared<float> &S, Fn f) {
+  if (threadIdx.x >= 32) return;
+  const int q = threadIdx.x;
+  Vec<float> s = ld16(S.red4[0] + 4 * q);
+#pragma unroll
+  for (int g = 1; g < kT / 32; g++) {
+    const Vec<float> o = ld16(S.red4[g] + 4 * q);
+#pragma unroll
+    for (int h = 0; h < 4; h++) s.v[h] += o.v[h];
+  }
+  f(4 * q, s);
+}
+template <typename Fn> __device__ __forceinline__ void groups_sum(const PsShared<double> &S, Fn f) {
+  const int c = threadIdx.x / 4, g = 2 * (threadIdx.x % 4);
+  const double s = quad_sum(S.red4[g][c] + S.red4[g + 1][c]);
+  if (threadIdx.x % 4 == 0) f(c, s);
+}
+// f(column, sum) for each of them, and the store of all of them to a row
+template <typename Fn> __device__ __forceinline__ void each_sum(int c, const Vec<float> &s, Fn f) {
+#pragma unroll
+  for (int h = 0; h < 4; h++) f(c + h, s.v[h]);
+}
+template <typename Fn> __device__ __forceinline__ void each_sum(int c, double s, Fn f) { f(c, s); }
+__device__ __forceinline__ void put_sum(float *row, int c, const Vec<float> &s) {
+  st16(row + c, s);
+}
+__device__ __forceinline__ void put_sum(double *row, int c, double s) { row[c] = s; }
+
 // x[first + j + c] = sum_{r >= c} Dinv[r][c] v[r]  (Dinv staged in S.di, zero
-// above the diagonal; v = S.sv); thread (g, q): columns 4q .. 4q + 3, rows
-// 16g .. 16g + 15
-__device__ void diag_bwd(const PsArgs &A, PsShared &S, const FrontInfo &F, int j) {
-  const int jb = min(kB, F.ncol - j), ldi = (jb + 3) & ~3;
+// above the diagonal; v = S.sv). FP32: thread (g, q) takes columns 4q .. and rows
+// 16g ..; FP64: four threads per column, and a warp's eight columns start at their diagonal.
+__device__ void diag_bwd(const PsArgs<float> &A, PsShared<float> &S, const FrontInfo &F, int j) {
+  constexpr int B = Ps<float>::B, RW = Ps<float>::RW;
+  const int jb = min(B, F.ncol - j), ldi = (jb + 3) & ~3;
   const int q = threadIdx.x % 32, g = threadIdx.x / 32, c = 4 * q;
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  Vec<float> acc = vzero<float>();
   if (c < ldi) {
 #pragma unroll
-    for (int k = 0; k < 16; k++) {
-      const int r = 16 * g + k;
-      if (r < jb) acc = fma4(*reinterpret_cast<const float4 *>(S.di + r * ldi + c), S.sv[r], acc);
+    for (int k = 0; k < RW; k++) {
+      const int r = RW * g + k;
+      if (r < jb) acc = vfma(ld16(S.di + r * ldi + c), S.sv[r], acc);
     }
   }
-  S.red4[g][q] = acc;
+  st16(S.red4[g] + 4 * q, acc);
   __syncthreads();
-  if (threadIdx.x < 32) {
-    float4 s = S.red4[0][q];
-#pragma unroll
-    for (int h = 1; h < kT / 32; h++) {
-      const float4 o = S.red4[h][q];
-      s.x += o.x; s.y += o.y; s.z += o.z; s.w += o.w;
-    }
-    float *xo = A.x + F.first + j;
-    if (c + 0 < jb) xo[c + 0] = s.x;
-    if (c + 1 < jb) xo[c + 1] = s.y;
-    if (c + 2 < jb) xo[c + 2] = s.z;
-    if (c + 3 < jb) xo[c + 3] = s.w;
+  float *xo = A.x + F.first + j;
+  groups_sum(S, [&](int c0, auto s) {
+    each_sum(c0, s, [&](int cc, float v) {
+      if (cc < jb) xo[cc] = v;
+    });
+  });
+}
+__device__ void diag_bwd(const PsArgs<double> &A, PsShared<double> &S, const FrontInfo &F, int j) {
+  constexpr int B = Ps<double>::B;
+  const int jb = min(B, F.ncol - j), ldi = (jb + 1) & ~1, c = threadIdx.x / 4, h = threadIdx.x % 4;
+  double s = 0.0;
+  for (int m = 2 * (threadIdx.x / 32); m < B / 4; m++) {
+    const int r = 4 * m + h;
+    if (r < jb && c < jb) s = fma(S.di[r * ldi + c], S.sv[r], s);
   }
+  s = quad_sum(s);
+  if (h == 0 && c < jb) A.x[F.first + j + c] = s;
 }
 
 // Thread 0 polls *w until it reaches target (acquire), at most A.spins times
 // and only while no other wait of the launch has run out; the CTA then shares
 // the outcome (and, on success, S.ready = ready unless ready < -1). On expiry
 // the status word is set, and every later wait of the launch gives up at once.
-__device__ bool wait_flag(const PsArgs &A, PsShared &S, const unsigned *w, unsigned target,
+template <typename T>
+__device__ bool wait_flag(const PsArgs<T> &A, PsShared<T> &S, const unsigned *w, unsigned target,
                           int ready = -2) {
   __syncthreads();  // every thread has read the previous outcome
   if (threadIdx.x == 0) {
@@ -287,7 +519,8 @@ __device__ bool wait_flag(const PsArgs &A, PsShared &S, const unsigned *w, unsig
 // every earlier block visible, so a task behind the chain waits once and then
 // streams its blocks without polling. S.ready holds the highest block known
 // published (reset by the caller to -1).
-__device__ bool wait_chain(const PsArgs &A, PsShared &S, const unsigned *flags, int j, int last,
+template <typename T>
+__device__ bool wait_chain(const PsArgs<T> &A, PsShared<T> &S, const unsigned *flags, int j, int last,
                            int step) {
   if ((step > 0 ? j <= S.ready : j >= S.ready) && S.ready >= 0) return true;
   __syncthreads();  // every thread has read S.ready and the previous outcome
@@ -311,7 +544,8 @@ __device__ void signal(unsigned *w) {
 
 // Wait until the update vectors of all children of front s are complete (one
 // counter per front), and stage the children's map and vector offsets.
-__device__ bool wait_children(const PsArgs &A, PsShared &S, const FrontInfo &F, const SolveRec &R) {
+template <typename T>
+__device__ bool wait_children(const PsArgs<T> &A, PsShared<T> &S, const FrontInfo &F, const SolveRec &R) {
   const DevPlan &dp = A.dp;
   const int nk = F.child_end - F.child_begin;
   if (threadIdx.x < min(nk, kMaxKids)) {
@@ -330,7 +564,8 @@ __device__ bool wait_children(const PsArgs &A, PsShared &S, const FrontInfo &F, 
 // Sum of the children's update entries at front position p (after
 // wait_children), in child order; the map entries of two children are loaded
 // together, then their update entries.
-__device__ __forceinline__ float gather_children(const PsArgs &A, const PsShared &S,
+template <typename T>
+__device__ __forceinline__ T gather_children(const PsArgs<T> &A, const PsShared<T> &S,
                                                  const FrontInfo &F, int p) {
   const DevPlan &dp = A.dp;
   auto offs = [&](int k, int64_t &io, int64_t &to) {
@@ -343,7 +578,7 @@ __device__ __forceinline__ float gather_children(const PsArgs &A, const PsShared
       to = dp.toff[ch];
     }
   };
-  float v = 0.f;
+  T v = T(0);
   const int nk = S.nkids;
   int k = 0;
   for (; k + 1 < nk; k += 2) {
@@ -351,8 +586,8 @@ __device__ __forceinline__ float gather_children(const PsArgs &A, const PsShared
     offs(k, io0, to0);
     offs(k + 1, io1, to1);
     const int32_t q0 = dp.inv[io0 + p], q1 = dp.inv[io1 + p];
-    const float t0 = q0 >= 0 ? ldcg(A.t + to0 + q0) : 0.f;
-    const float t1 = q1 >= 0 ? ldcg(A.t + to1 + q1) : 0.f;
+    const T t0 = q0 >= 0 ? ldcg(A.t + to0 + q0) : T(0);
+    const T t1 = q1 >= 0 ? ldcg(A.t + to1 + q1) : T(0);
     if (q0 >= 0) v += t0;
     if (q1 >= 0) v += t1;
   }
@@ -374,7 +609,8 @@ struct Next {
   bool have;
 };
 
-__device__ __forceinline__ void take_next(const PsArgs &A, Next &N) {
+template <typename T>
+__device__ __forceinline__ void take_next(const PsArgs<T> &A, Next &N) {
   if (threadIdx.x == 32 && !N.have) {
     N.q = (int)atomicAdd(f_ticket(A), 1u) + A.q0;  // the result is first read after the task
     N.have = true;
@@ -383,9 +619,10 @@ __device__ __forceinline__ void take_next(const PsArgs &A, Next &N) {
 
 // Thread 32: start the asynchronous copy of record q into S.rec[buf], and
 // warm L2 with the record one grid further on.
-__device__ __forceinline__ void fetch_rec(const PsArgs &A, PsShared &S, int q, int buf) {
+template <typename T>
+__device__ __forceinline__ void fetch_rec(const PsArgs<T> &A, PsShared<T> &S, int q, int buf) {
   if (q >= A.q1) return;
-  const char *src = reinterpret_cast<const char *>(A.dp.ps_recs + q);
+  const char *src = reinterpret_cast<const char *>(A.sv.recs + q);
   const uint32_t dst = smem_u32(&S.rec[buf]);
 #pragma unroll
   for (int k = 0; k < (int)(sizeof(SolveRec) / 16); k++)
@@ -393,49 +630,35 @@ __device__ __forceinline__ void fetch_rec(const PsArgs &A, PsShared &S, int q, i
                  : "memory");
   asm volatile("cp.async.commit_group;" ::: "memory");
   const int ahead = min(q + (int)gridDim.x, A.q1 - 1);
-  asm volatile("prefetch.global.L2 [%0];" ::"l"(A.dp.ps_recs + ahead));
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(A.sv.recs + ahead));
 }
 
-// Forward, diagonal block i of front s: rows j0 .. j0 + jb of the front.
-// warp w: rows 16w .. 16w + 15, lane: columns 4 lane .. 4 lane + 3 of block j
-// (the loads of block j are issued before y_j is waited for).
-__device__ void fwd_diag(const PsArgs &A, PsShared &S, const SolveRec &R, Next &N) {
+// Forward, diagonal block i of front s: rows j0 .. j0 + jb of the front (the
+// loads of block j are issued before y_j is waited for).
+template <typename T>
+__device__ void fwd_diag(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R, Next &N) {
+  constexpr int B = Ps<T>::B;
   const Task &tk = R.task;
   const FrontInfo &F = R.front;
-  const DevPlan &dp = A.dp;
-  const int i = tk.a, j0 = kB * i, jb = min(kB, F.ncol - j0), slot0 = R.slot0;
+  const int i = tk.a, j0 = B * i, jb = min(B, F.ncol - j0), slot0 = R.slot0;
   if (threadIdx.x == 0) stage_dinv(A, S, slot0 + i, jb);
   bool ok = wait_children(A, S, F, R);
-  if (ok && threadIdx.x < kB)
+  if (ok && threadIdx.x < B)
     S.sv[threadIdx.x] = threadIdx.x < jb
                             ? ldcg(A.a + F.first + j0 + threadIdx.x) - gather_children(A, S, F, j0 + threadIdx.x)
-                            : 0.f;
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, c = 4 * lane, rw = 16 * warp;
-  // per-thread partial row sums over the lane's 4 columns of every block,
-  // reduced across the warp once after the last block
-  float acc[16];
-#pragma unroll
-  for (int k = 0; k < 16; k++) acc[k] = 0.f;
+                            : T(0);
+  FwdTile<T> tile;
+  tile.clear();
   if (threadIdx.x == 0) S.ready = -1;
   __syncthreads();  // no thread reads the previous task's value
-  for (int j = 0; j < i && ok; j++) {
-    float4 l[16];
-    const float *P = A.L + F.loff + (int64_t)(j0 + rw) * F.ld + kB * j + c;
-#pragma unroll
-    for (int k = 0; k < 16; k++)
-      l[k] = rw + k < jb ? __ldg(reinterpret_cast<const float4 *>(P + (int64_t)k * F.ld))
-                         : make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int j = 0; j < i && ok; j++) {  // block j < i is a full block
+    tile.template load<true>(A.L + F.loff + (int64_t)j0 * F.ld + B * j, F.ld, jb, B);
     ok = wait_chain(A, S, f_y(A, slot0), j, i - 1, 1);
     if (!ok) break;
-    const float *yb = A.b + F.first + kB * j + c;  // block j < i is a full block
-    const float4 y4 = make_float4(ldcg(yb), ldcg(yb + 1), ldcg(yb + 2), ldcg(yb + 3));
-#pragma unroll
-    for (int k = 0; k < 16; k++)
-      acc[k] = fmaf(l[k].x, y4.x, fmaf(l[k].y, y4.y, fmaf(l[k].z, y4.z, fmaf(l[k].w, y4.w, acc[k]))));
+    tile.template mul<true>(S, j, A.b + F.first + B * j, B);
   }
   take_next(A, N);
-  const float racc = rows16_reduce(S, acc);  // rows of this warp only
-  if (ok && lane < 16 && rw + lane < jb) S.sv[rw + lane] -= racc;
+  tile.finish(S, ok ? jb : 0, [&](int r, T v) { S.sv[r] -= v; });
   // the staged copy always lands before S.di is reused; the wait ends with a
   // barrier, after which every row of S.sv is final
   const bool got = wait_dinv(A, S);
@@ -447,75 +670,57 @@ __device__ void fwd_diag(const PsArgs &A, PsShared &S, const SolveRec &R, Next &
 
 // Forward, rows r0 .. r0 + nr below front s: the children's entries plus
 // L_rj y_j over every block j of the front, into the front's update vector.
-__device__ void fwd_below(const PsArgs &A, PsShared &S, const SolveRec &R, Next &N) {
+template <typename T>
+__device__ void fwd_below(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R, Next &N) {
+  constexpr int B = Ps<T>::B;
   const Task &tk = R.task;
   const FrontInfo &F = R.front;
-  const DevPlan &dp = A.dp;
-  const int r0 = tk.a, nr = min(kRC, F.nrow - r0), nb = (F.ncol + kB - 1) / kB;
+  const int r0 = tk.a, nr = min(B, F.nrow - r0), nb = (F.ncol + B - 1) / B;
   const int slot0 = R.slot0;
   bool ok = wait_children(A, S, F, R);
   if (ok && threadIdx.x < nr) S.xs[threadIdx.x] = gather_children(A, S, F, F.ncol + r0 + threadIdx.x);
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, c = 4 * lane, rw = 16 * warp;
-  float acc[16];  // partial row sums, reduced once after the last block
-#pragma unroll
-  for (int k = 0; k < 16; k++) acc[k] = 0.f;
+  FwdTile<T> tile;
+  tile.clear();
   if (threadIdx.x == 0) S.ready = -1;
   __syncthreads();  // no thread reads the previous task's value
   for (int j = 0; j < nb && ok; j++) {
-    const int jbj = min(kB, F.ncol - kB * j);
-    float4 l[16];
-    const float *P = A.L + F.loff + (int64_t)(F.ncol + r0 + rw) * F.ld + kB * j + c;
-#pragma unroll
-    for (int k = 0; k < 16; k++)
-      l[k] = (c < jbj && rw + k < nr) ? __ldg(reinterpret_cast<const float4 *>(P + (int64_t)k * F.ld))
-                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+    const int jbj = min(B, F.ncol - B * j);
+    const T *P = A.L + F.loff + (int64_t)(F.ncol + r0) * F.ld + B * j, *y = A.b + F.first + B * j;
+    if (jbj == B) tile.template load<true>(P, F.ld, nr, B);
+    else tile.template load<false>(P, F.ld, nr, jbj);
     ok = wait_chain(A, S, f_y(A, slot0), j, nb - 1, 1);
     if (!ok) break;
-    // columns past ncol (the padding of the last block) never enter the sums
-    const float *yb = A.b + F.first + kB * j + c;
-    const float4 y4 = make_float4(c < jbj ? ldcg(yb) : 0.f, c + 1 < jbj ? ldcg(yb + 1) : 0.f,
-                                  c + 2 < jbj ? ldcg(yb + 2) : 0.f, c + 3 < jbj ? ldcg(yb + 3) : 0.f);
-#pragma unroll
-    for (int k = 0; k < 16; k++) {
-      float4 v = l[k];
-      if (c + 1 >= jbj) v.y = 0.f;
-      if (c + 2 >= jbj) v.z = 0.f;
-      if (c + 3 >= jbj) v.w = 0.f;
-      acc[k] = fmaf(v.x, y4.x, fmaf(v.y, y4.y, fmaf(v.z, y4.z, fmaf(v.w, y4.w, acc[k]))));
-    }
+    if (jbj == B) tile.template mul<true>(S, j, y, B);
+    else tile.template mul<false>(S, j, y, jbj);
   }
   take_next(A, N);
-  const float racc = rows16_reduce(S, acc);
-  __syncthreads();
-  if (ok) {
-    if (lane < 16 && rw + lane < nr) A.t[R.toff + r0 + rw + lane] = S.xs[rw + lane] + racc;
-    signal(f_tvec(A, F.parent));  // rows below a front exist only below a parent
-  }
+  tile.finish(S, ok ? nr : 0, [&](int r, T v) { A.t[R.toff + r0 + r] = S.xs[r] + v; });
+  if (ok) signal(f_tvec(A, F.parent));  // rows below a front exist only below a parent
 }
 
 // Backward, rows r0 .. r0 + nr below front s: once the parent front (and so
 // every ancestor holding those rows) is solved, the partial sums
-// part[cb][c] = sum_r L[ncol + r0 + r, 128 cb + c] x[row r] of every column
+// part[cb][c] = sum_r L[ncol + r0 + r, B cb + c] x[row r] of every column
 // block, last block first (the order of the front's backward chain), each
-// published as it is written. Thread (g, q): columns 4q .. 4q + 3, rows
-// 16g .. 16g + 15; the loads of the next block are issued before the
-// reduction of the current one.
-__device__ void bwd_part(const PsArgs &A, PsShared &S, const SolveRec &R, Next &N) {
+// published as it is written. Thread (g, q): columns VW q .., rows RW g ..;
+// the loads of the next block are issued before the reduction of the current
+// one.
+template <typename T>
+__device__ void bwd_part(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R, Next &N) {
+  constexpr int B = Ps<T>::B, VW = Ps<T>::VW, RW = Ps<T>::RW;
   const Task &tk = R.task;
   const FrontInfo &F = R.front;
   const DevPlan &dp = A.dp;
-  const int r0 = tk.b, nr = min(kRC, F.nrow - r0), nb = (F.ncol + kB - 1) / kB;
-  const int nbl = (F.nrow + kRC - 1) / kRC;
+  const int r0 = tk.b, nr = min(B, F.nrow - r0), nb = (F.ncol + B - 1) / B;
+  const int nbl = (F.nrow + B - 1) / B;
   const int q = threadIdx.x % 32, g = threadIdx.x / 32;
-  const float *P = A.L + F.loff + (int64_t)(F.ncol + r0 + 16 * g) * F.ld + 4 * q;
-  float4 l[16];
+  const T *P = A.L + F.loff + (int64_t)(F.ncol + r0 + RW * g) * F.ld + VW * q;
+  Vec<T> l[RW];
   auto load = [&](int cb) {
-    const int c = kB * cb + 4 * q;
+    const int c = B * cb + VW * q;
 #pragma unroll
-    for (int k = 0; k < 16; k++)
-      l[k] = (c < F.ncol && 16 * g + k < nr)
-                 ? __ldg(reinterpret_cast<const float4 *>(P + (int64_t)k * F.ld + kB * cb))
-                 : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k = 0; k < RW; k++)
+      l[k] = (c < F.ncol && RW * g + k < nr) ? ldg16(P + (int64_t)k * F.ld + B * cb) : vzero<T>();
   };
   load(nb - 1);
   const int32_t xrow = threadIdx.x < nr ? dp.sri[F.rows_off + r0 + threadIdx.x] : 0;
@@ -525,23 +730,15 @@ __device__ void bwd_part(const PsArgs &A, PsShared &S, const SolveRec &R, Next &
   if (threadIdx.x < nr) S.xs[threadIdx.x] = ldcg(A.x + xrow);
   __syncthreads();
   for (int cb = nb - 1; cb >= 0; cb--) {
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    Vec<T> acc = vzero<T>();
 #pragma unroll
-    for (int k = 0; k < 16; k++)
-      if (16 * g + k < nr) acc = fma4(l[k], S.xs[16 * g + k], acc);
+    for (int k = 0; k < RW; k++)
+      if (RW * g + k < nr) acc = vfma(l[k], S.xs[RW * g + k], acc);
     if (cb > 0) load(cb - 1);
-    S.red4[g][q] = acc;
+    st16(S.red4[g] + VW * q, acc);
     __syncthreads();
-    if (threadIdx.x < 32) {
-      float4 sm = S.red4[0][q];
-#pragma unroll
-      for (int h = 1; h < kT / 32; h++) {
-        const float4 o = S.red4[h][q];
-        sm.x += o.x; sm.y += o.y; sm.z += o.z; sm.w += o.w;
-      }
-      const int64_t row = R.pbase + (int64_t)cb * nbl + r0 / kRC;
-      reinterpret_cast<float4 *>(A.part + row * kB)[q] = sm;
-    }
+    T *row = A.part + (R.pbase + (int64_t)cb * nbl + r0 / B) * B;
+    groups_sum(S, [&](int c, auto s) { put_sum(row, c, s); });
     signal(f_part(A, R.slot0 + cb));  // (its barrier also frees S.red4)
   }
 }
@@ -549,12 +746,13 @@ __device__ void bwd_part(const PsArgs &A, PsShared &S, const SolveRec &R, Next &
 // Backward, column block cb of front s: the partial sums in chunk order, then
 // L[block i, block cb]^T x_i for i > cb as each x_i is published, then
 // x_cb = L_cc^{-T} (.) with the staged inverse.
-__device__ void bwd_diag(const PsArgs &A, PsShared &S, const SolveRec &R, Next &N) {
+template <typename T>
+__device__ void bwd_diag(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R, Next &N) {
+  constexpr int B = Ps<T>::B, VW = Ps<T>::VW, RW = Ps<T>::RW;
   const Task &tk = R.task;
   const FrontInfo &F = R.front;
-  const DevPlan &dp = A.dp;
-  const int cb = tk.a, c0 = kB * cb, jb = min(kB, F.ncol - c0), nb = (F.ncol + kB - 1) / kB;
-  const int nbl = (F.nrow + kRC - 1) / kRC, slot0 = R.slot0;
+  const int cb = tk.a, c0 = B * cb, jb = min(B, F.ncol - c0), nb = (F.ncol + B - 1) / B;
+  const int nbl = (F.nrow + B - 1) / B, slot0 = R.slot0;
   if (threadIdx.x == 0) stage_dinv(A, S, slot0 + cb, jb);
   // b of this block is the forward result: published by this launch's forward
   // task of the block, or complete before a backward-only launch
@@ -562,50 +760,50 @@ __device__ void bwd_diag(const PsArgs &A, PsShared &S, const SolveRec &R, Next &
   if (ok && nbl > 0) ok = wait_flag(A, S, f_part(A, slot0 + cb), nbl);  // implies the parent is done
   else if (ok && F.parent >= 0)
     ok = wait_flag(A, S, f_front(A, F.parent), (unsigned)R.parent_blocks);
-  if (ok && threadIdx.x < kB) {
-    float v = 0.f;
+  if (ok && sizeof(T) == 8) {  // four threads per column (see quad_sum)
+    const int cc = threadIdx.x / 4;
+    const T *pp = A.part + (R.pbase + (int64_t)cb * nbl) * B + cc;
+    T ps = T(0);
+    for (int k = threadIdx.x % 4; k < nbl && cc < jb; k += 4) ps += ldcg(pp + (int64_t)k * B);
+    ps = quad_sum(ps);
+    if (threadIdx.x % 4 == 0) S.sv[cc] = cc < jb ? ldcg(A.b + F.first + c0 + cc) - ps : T(0);
+  } else if (ok && threadIdx.x < B) {
+    T v = T(0);
     if (threadIdx.x < jb) {
-      const float *pp = A.part + (R.pbase + (int64_t)cb * nbl) * kB + threadIdx.x;
-      float ps = 0.f;
-      for (int k = 0; k < nbl; k++) ps += ldcg(pp + (int64_t)k * kB);
+      const T *pp = A.part + (R.pbase + (int64_t)cb * nbl) * B + threadIdx.x;
+      T ps = T(0);
+      for (int k = 0; k < nbl; k++) ps += ldcg(pp + (int64_t)k * B);
       v = ldcg(A.b + F.first + c0 + threadIdx.x) - ps;
     }
     S.sv[threadIdx.x] = v;
   }
-  const int q = threadIdx.x % 32, g = threadIdx.x / 32, c = c0 + 4 * q;
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  const int q = threadIdx.x % 32, g = threadIdx.x / 32, c = c0 + VW * q;
+  Vec<T> acc = vzero<T>();
   if (threadIdx.x == 0) S.ready = -1;
   __syncthreads();  // no thread reads the previous task's value
   for (int i = nb - 1; i > cb && ok; i--) {
-    const int jbi = min(kB, F.ncol - kB * i);
-    float4 l[16];
-    const float *P = A.L + F.loff + (int64_t)(kB * i + 16 * g) * F.ld + c;
+    const int jbi = min(B, F.ncol - B * i);
+    Vec<T> l[RW];
+    const T *P = A.L + F.loff + (int64_t)(B * i + RW * g) * F.ld + c;
 #pragma unroll
-    for (int k = 0; k < 16; k++)
-      l[k] = (c < F.ncol && 16 * g + k < jbi) ? __ldg(reinterpret_cast<const float4 *>(P + (int64_t)k * F.ld))
-                                              : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k = 0; k < RW; k++)
+      l[k] = (c < F.ncol && RW * g + k < jbi) ? ldg16(P + (int64_t)k * F.ld) : vzero<T>();
     ok = wait_chain(A, S, f_x(A, slot0), i, cb + 1, -1);
     if (!ok) break;
-    // lane k < 16 loads x of row 16 g + k of block i; the warp shares them
-    const float xv = (q < 16 && 16 * g + q < jbi) ? ldcg(A.x + F.first + kB * i + 16 * g + q) : 0.f;
+    // lane k < RW loads x of row RW g + k of block i; the warp shares them
+    const T xv = (q < RW && RW * g + q < jbi) ? ldcg(A.x + F.first + B * i + RW * g + q) : T(0);
 #pragma unroll
-    for (int k = 0; k < 16; k++) acc = fma4(l[k], __shfl_sync(0xffffffffu, xv, k), acc);
+    for (int k = 0; k < RW; k++) acc = vfma(l[k], __shfl_sync(0xffffffffu, xv, k), acc);
   }
   take_next(A, N);
-  S.red4[g][q] = acc;
+  st16(S.red4[g] + VW * q, acc);
   __syncthreads();
-  if (ok && threadIdx.x < 32) {
-    float4 sm = S.red4[0][q];
-#pragma unroll
-    for (int h = 1; h < kT / 32; h++) {
-      const float4 o = S.red4[h][q];
-      sm.x += o.x; sm.y += o.y; sm.z += o.z; sm.w += o.w;
-    }
-    const float d[4] = {sm.x, sm.y, sm.z, sm.w};
-#pragma unroll
-    for (int k = 0; k < 4; k++)
-      if (4 * q + k < jb) S.sv[4 * q + k] -= d[k];
-  }
+  if (ok)
+    groups_sum(S, [&](int k0, auto s) {
+      each_sum(k0, s, [&](int k, T v) {
+        if (k < jb) S.sv[k] -= v;
+      });
+    });
   const bool got = wait_dinv(A, S);  // (ends with a barrier)
   if (ok && got) {
     diag_bwd(A, S, F, c0);
@@ -617,9 +815,9 @@ __device__ void bwd_diag(const PsArgs &A, PsShared &S, const SolveRec &R, Next &
 
 // Persistent solve: every CTA takes tasks in plan order from the global ticket
 // counter until the range is exhausted.
-__global__ void __launch_bounds__(kT, 2) psolve_kernel(PsArgs A) {
+template <typename T> __global__ void __launch_bounds__(kT, 2) psolve_kernel(PsArgs<T> A) {
   extern __shared__ __align__(128) unsigned char ps_smem[];
-  PsShared &S = *reinterpret_cast<PsShared *>(ps_smem);
+  PsShared<T> &S = *reinterpret_cast<PsShared<T> *>(ps_smem);
   // Thread 32 takes the tickets: the first here, each next one inside the
   // running task once it has passed its last wait (take_next), or right after
   // a task that ended early; the next task's record is copied into the other
@@ -663,18 +861,18 @@ __global__ void __launch_bounds__(kT, 2) psolve_kernel(PsArgs A) {
   }
 }
 
-int psolve_grid(int ntask) {
+template <typename T> int psolve_grid(int ntask) {
   static int per_device[64] = {0};
   int dev = 0;
   ck(cudaGetDevice(&dev), "cudaGetDevice");
   int &g = per_device[dev & 63];
   if (g == 0) {
     int sms = 0, nb = 0;
-    ck(cudaFuncSetAttribute(psolve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                            (int)sizeof(PsShared)),
+    ck(cudaFuncSetAttribute(psolve_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                            (int)sizeof(PsShared<T>)),
        "solve shared-memory attribute");
     ck(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
-    ck(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, psolve_kernel, kT, sizeof(PsShared)),
+    ck(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, psolve_kernel<T>, kT, sizeof(PsShared<T>)),
        "occupancy");
     g = std::max(1, sms * std::min(nb, 2));
   }
@@ -685,7 +883,7 @@ int psolve_grid(int ntask) {
 
 void launch_dinv(const DevPlan &dp, const Plan &plan, const float *L, float *Dinv,
                  cudaStream_t st) {
-  const int n = (int)plan.fs_inv.size();
+  const int n = (int)plan.s32.inv.size();
   if (n == 0) return;
   const int smem = 2 * 128 * 129 * (int)sizeof(float);
   static bool attr = false;
@@ -697,20 +895,36 @@ void launch_dinv(const DevPlan &dp, const Plan &plan, const float *L, float *Din
   dinv_kernel<<<n, 128, smem, st>>>(dp, L, Dinv);
 }
 
-void launch_psolve(const DevPlan &dp, const Plan &plan, const float *L, const float *Dinv, float *a,
-                   float *b, float *x, float *t, float *part, unsigned *flags, int32_t *status,
-                   bool fwd, bool bwd, cudaStream_t st, unsigned test_spins, int test_withhold) {
-  const int32_t q0 = fwd ? 0 : plan.ps_fwd_tasks;
-  const int32_t q1 = bwd ? (int32_t)plan.ps_tasks.size() : plan.ps_fwd_tasks;
-  if (q1 <= q0) return;
-  ck(cudaMemsetAsync(flags, 0, (size_t)plan.ps_flag_words * sizeof(unsigned), st), "solve flags");
-  const int grid = psolve_grid(q1 - q0);
-  PsArgs A{dp, L, Dinv, a, b, x, t, part, q0, q1, flags, status,
-           test_spins ? test_spins : kBarrierSpins, test_withhold,
-           (int32_t)plan.fs_dinv_off.size(), (int32_t)plan.fronts.size(), fwd && bwd ? 1 : 0};
+void launch_dinv(const DevPlan &dp, const Plan &plan, const double *L, double *Dinv,
+                 cudaStream_t st) {
+  const int n = (int)plan.s64.inv.size();
+  if (n == 0) return;
   note_launch();
-  psolve_kernel<<<grid, kT, sizeof(PsShared), st>>>(A);
+  dinv64_kernel<<<n, 64, 0, st>>>(dp, L, Dinv);
+}
+
+template <typename T>
+void launch_psolve(const DevPlan &dp, const Plan &plan, const T *L, const T *Dinv, T *a, T *b, T *x, T *t,
+                   T *part, unsigned *flags, int32_t *status, bool fwd, bool bwd, cudaStream_t st,
+                   unsigned test_spins, int test_withhold) {
+  const SolvePlan &sp = sizeof(T) == 8 ? plan.s64 : plan.s32;
+  const int32_t q0 = fwd ? 0 : sp.fwd_tasks;
+  const int32_t q1 = bwd ? (int32_t)sp.tasks.size() : sp.fwd_tasks;
+  if (q1 <= q0) return;
+  ck(cudaMemsetAsync(flags, 0, (size_t)sp.flag_words * sizeof(unsigned), st), "solve flags");
+  const int grid = psolve_grid<T>(q1 - q0);
+  PsArgs<T> A{dp, sizeof(T) == 8 ? dp.s64 : dp.s32, L, Dinv, a, b, x, t, part, q0, q1, flags, status,
+              test_spins ? test_spins : kBarrierSpins, test_withhold,
+              (int32_t)sp.dinv_off.size(), (int32_t)plan.fronts.size(), fwd && bwd ? 1 : 0};
+  note_launch();
+  psolve_kernel<T><<<grid, kT, sizeof(PsShared<T>), st>>>(A);
   ck(cudaGetLastError(), "solve launch");
 }
+template void launch_psolve<float>(const DevPlan &, const Plan &, const float *, const float *, float *,
+                                   float *, float *, float *, float *, unsigned *, int32_t *, bool, bool,
+                                   cudaStream_t, unsigned, int);
+template void launch_psolve<double>(const DevPlan &, const Plan &, const double *, const double *, double *,
+                                    double *, double *, double *, double *, unsigned *, int32_t *, bool,
+                                    bool, cudaStream_t, unsigned, int);
 
 }  // namespace gipm

@@ -42,19 +42,21 @@ void launch_sign(const DevPlan &dp, V *y, cudaStream_t st);
 // commits no device memory (lazy module loading); used by the allocation-free solve.
 cudaError_t preload_level_solve();
 
-// Persistent FP32 solve: inverses of the 128-wide diagonal blocks (after each
-// FP32 factorisation), then x = L^{-T} L^{-1} a in one launch, with b the
-// forward result and t the update vectors. fwd/bwd select the sweeps: forward
+// Persistent solve: inverses of the diagonal blocks (after each factorisation
+// that does not write them itself), then x = L^{-T} L^{-1} a in one launch, with b
+// the forward result and t the update vectors. fwd/bwd select the sweeps: forward
 // only maps a to b = L^{-1} a; backward only maps b to x = L^{-T} b. part:
-// plan.ps_part_entries floats of scratch; flags: plan.ps_flag_words words
-// (zeroed by the launch). A wait that runs out sets status[ST_SOLVE_TIMEOUT]
-// and the launch drains. test_spins (0: the default of seconds) bounds each
-// wait; test_withhold >= 0 abandons the task of that ticket (tests of
-// the bounded wait).
+// part_entries values of scratch; flags: flag_words words (zeroed by the launch),
+// both from the solve plan of the storage type. A wait that runs out sets
+// status[ST_SOLVE_TIMEOUT] and the launch drains. test_spins (0: the default of
+// seconds) bounds each wait; test_withhold >= 0 abandons the task of that ticket
+// (tests of the bounded wait).
 void launch_dinv(const DevPlan &dp, const Plan &plan, const float *L, float *Dinv, cudaStream_t st);
-void launch_psolve(const DevPlan &dp, const Plan &plan, const float *L, const float *Dinv, float *a,
-                   float *b, float *x, float *t, float *part, unsigned *bar, int32_t *status, bool fwd,
-                   bool bwd, cudaStream_t st, unsigned test_spins = 0, int test_withhold = -1);
+void launch_dinv(const DevPlan &dp, const Plan &plan, const double *L, double *Dinv, cudaStream_t st);
+template <typename T>
+void launch_psolve(const DevPlan &dp, const Plan &plan, const T *L, const T *Dinv, T *a, T *b, T *x, T *t,
+                   T *part, unsigned *flags, int32_t *status, bool fwd, bool bwd, cudaStream_t st,
+                   unsigned test_spins = 0, int test_withhold = -1);
 
 // Sampled entries of L (final numbering).
 template <typename T>

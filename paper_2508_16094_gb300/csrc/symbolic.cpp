@@ -797,97 +797,96 @@ void validate_plan(const Problem &P, const Symbolic &S, const Plan &pl) {
 
 namespace gipm {
 
-// Fused FP32 solve: for every front and 128-wide block column j, one inverse
-// task (the diagonal block's inverse, jb x jb, at fs_dinv_off[slot]), forward
-// tasks over the rows [j, nf) in chunks of 128 (the chunk starting at j also
-// publishes the solved block), backward tasks over the columns [0, j) in
-// chunks of 256 (at least one, which publishes the solved block).
-void build_fused_solve(Plan &pl) {
-  constexpr int B = 128, RC = 128;
+// Persistent solve: for every front and B-wide block column, one inverse task,
+// one forward and one backward task, and per B-row chunk below the front one
+// forward and one backward task (SolveTaskKind).
+void build_fused_solve(const Plan &pl, int B, SolvePlan &sp) {
+  const int RC = B, vw = B / 32;  // values per 16 bytes
+  sp.B = B;
   const int32_t nfr = (int32_t)pl.fronts.size();
-  pl.fs_inv.clear();
-  pl.fs_dinv_off.clear();
-  pl.fs_dinv_entries = 0;
-  pl.ps_tasks.clear();
-  pl.fs_first_slot.assign(nfr, 0);
+  sp.inv.clear();
+  sp.dinv_off.clear();
+  sp.dinv_entries = 0;
+  sp.tasks.clear();
+  sp.first_slot.assign(nfr, 0);
   for (int32_t s = 0; s < nfr; s++) {
     const FrontInfo &F = pl.fronts[s];
-    pl.fs_first_slot[s] = (int32_t)pl.fs_dinv_off.size();
+    sp.first_slot[s] = (int32_t)sp.dinv_off.size();
     for (int32_t j = 0; j < F.ncol; j += B) {
       const int32_t jb = std::min(B, F.ncol - j);
-      const int32_t slot = (int32_t)pl.fs_dinv_off.size();
-      pl.fs_dinv_off.push_back(pl.fs_dinv_entries);
-      pl.fs_dinv_entries += (int64_t)jb * round_up(jb, 4);  // keeps every slot 16-byte aligned
-      pl.fs_inv.push_back({s, j, slot, 0});
+      const int32_t slot = (int32_t)sp.dinv_off.size();
+      sp.dinv_off.push_back(sp.dinv_entries);
+      sp.dinv_entries += (int64_t)jb * round_up(jb, vw);  // keeps every slot 16-byte aligned
+      sp.inv.push_back({s, j, slot, 0});
     }
   }
-  pl.fs_dinv_entries = std::max<int64_t>(pl.fs_dinv_entries, 4);
+  sp.dinv_entries = std::max<int64_t>(sp.dinv_entries, 4);
   auto nblk = [&](int32_t s) { return (pl.fronts[s].ncol + B - 1) / B; };
   // forward, leaves to root, level by level: the diagonal chunks of every front
   // of the level (ascending), then the chunks of rows below the fronts
   for (const LevelPlan &LP : pl.levels) {
     for (int32_t t = LP.front_b; t < LP.front_e; t++) {
       const int32_t s = pl.level_fronts[t];
-      for (int32_t i = 0; i < nblk(s); i++) pl.ps_tasks.push_back({s, i, 0, WS_FWD_DIAG});
+      for (int32_t i = 0; i < nblk(s); i++) sp.tasks.push_back({s, i, 0, WS_FWD_DIAG});
     }
     for (int32_t t = LP.front_b; t < LP.front_e; t++) {
       const int32_t s = pl.level_fronts[t];
-      for (int32_t r0 = 0; r0 < pl.fronts[s].nrow; r0 += RC) pl.ps_tasks.push_back({s, r0, 0, WS_FWD_BELOW});
+      for (int32_t r0 = 0; r0 < pl.fronts[s].nrow; r0 += RC) sp.tasks.push_back({s, r0, 0, WS_FWD_BELOW});
     }
   }
-  pl.ps_fwd_tasks = (int32_t)pl.ps_tasks.size();
+  sp.fwd_tasks = (int32_t)sp.tasks.size();
   // backward, root to leaves, level by level: the partial sums of every
-  // 128-row chunk below every front of the level (one task per chunk, all
+  // B-row chunk below every front of the level (one task per chunk, all
   // column blocks), then the column blocks (last to first)
-  pl.ps_pbase.assign(nfr, 0);
+  sp.pbase.assign(nfr, 0);
   int64_t prow = 0;
   for (int32_t s = 0; s < nfr; s++) {
-    pl.ps_pbase[s] = prow;
+    sp.pbase[s] = prow;
     prow += (int64_t)nblk(s) * ((pl.fronts[s].nrow + RC - 1) / RC);
   }
-  pl.ps_part_entries = std::max<int64_t>(prow, 1) * B;
+  sp.part_entries = std::max<int64_t>(prow, 1) * B;
   for (int32_t li = (int32_t)pl.levels.size() - 1; li >= 0; li--) {
     const LevelPlan &LP = pl.levels[li];
     for (int32_t t = LP.front_b; t < LP.front_e; t++) {
       const int32_t s = pl.level_fronts[t];
-      for (int32_t r0 = 0; r0 < pl.fronts[s].nrow; r0 += RC) pl.ps_tasks.push_back({s, 0, r0, WS_BWD_PART});
+      for (int32_t r0 = 0; r0 < pl.fronts[s].nrow; r0 += RC) sp.tasks.push_back({s, 0, r0, WS_BWD_PART});
     }
     for (int32_t t = LP.front_b; t < LP.front_e; t++) {
       const int32_t s = pl.level_fronts[t];
-      for (int32_t cb = nblk(s) - 1; cb >= 0; cb--) pl.ps_tasks.push_back({s, cb, 0, WS_BWD_DIAG});
+      for (int32_t cb = nblk(s) - 1; cb >= 0; cb--) sp.tasks.push_back({s, cb, 0, WS_BWD_DIAG});
     }
   }
-  pl.ps_kid_chunks.assign(nfr, 0);
-  pl.ps_parent_blocks.assign(nfr, 0);
+  sp.kid_chunks.assign(nfr, 0);
+  sp.parent_blocks.assign(nfr, 0);
   for (int32_t s = 0; s < nfr; s++) {
     const int32_t par = pl.fronts[s].parent;
     if (par >= 0) {
-      pl.ps_kid_chunks[par] += (pl.fronts[s].nrow + RC - 1) / RC;
-      pl.ps_parent_blocks[s] = nblk(par);
+      sp.kid_chunks[par] += (pl.fronts[s].nrow + RC - 1) / RC;
+      sp.parent_blocks[s] = nblk(par);
     }
   }
-  const int64_t nslot = (int64_t)pl.fs_dinv_off.size();
-  pl.ps_flag_words = 32 + 3 * nslot + 2 * (int64_t)nfr;
+  const int64_t nslot = (int64_t)sp.dinv_off.size();
+  sp.flag_words = 32 + 3 * nslot + 2 * (int64_t)nfr;
   // range checks (the kernel masks only the chunk edges), and the order every
   // wait of the kernel relies on: a task waits only for earlier tasks
   auto need = [](bool ok, const char *w) {
     if (!ok) throw std::runtime_error(std::string("solve plan check failed: ") + w);
   };
-  for (const Task &t : pl.fs_inv)
-    need(t.b >= 0 && t.b < nslot && t.b == pl.fs_first_slot[t.front] + t.a / B &&
-             pl.fs_dinv_off[t.b] % 4 == 0,
+  for (const Task &t : sp.inv)
+    need(t.b >= 0 && t.b < nslot && t.b == sp.first_slot[t.front] + t.a / B &&
+             sp.dinv_off[t.b] % vw == 0,
          "inverse task");
   std::vector<int32_t> fwd_diag_seen(nfr, 0), fwd_below_seen(nfr, 0), bwd_diag_seen(nfr, 0);
   std::vector<int32_t> bwd_part_seen(nfr, 0), level_of(nfr, -1);
   for (size_t li = 0; li < pl.levels.size(); li++)
     for (int32_t t = pl.levels[li].front_b; t < pl.levels[li].front_e; t++) level_of[pl.level_fronts[t]] = (int32_t)li;
   auto nbelow = [&](int32_t s) { return (pl.fronts[s].nrow + RC - 1) / RC; };
-  for (size_t q = 0; q < pl.ps_tasks.size(); q++) {
-    const Task &t = pl.ps_tasks[q];
+  for (size_t q = 0; q < sp.tasks.size(); q++) {
+    const Task &t = sp.tasks[q];
     need(t.front >= 0 && t.front < nfr, "task front");
     const FrontInfo &F = pl.fronts[t.front];
-    need(F.ld % 4 == 0 && F.loff % 4 == 0, "panel alignment");
-    need((q < (size_t)pl.ps_fwd_tasks) == (t.c <= WS_FWD_BELOW) && t.c >= 0 && t.c <= WS_BWD_DIAG,
+    need(F.ld % vw == 0 && F.loff % vw == 0, "panel alignment");
+    need((q < (size_t)sp.fwd_tasks) == (t.c <= WS_FWD_BELOW) && t.c >= 0 && t.c <= WS_BWD_DIAG,
          "task order");
     const int32_t s = t.front;
     switch (t.c) {
@@ -905,7 +904,7 @@ void build_fused_solve(Plan &pl) {
       case WS_BWD_PART:
         need(t.a == 0 && t.b == RC * bwd_part_seen[s] && t.b < F.nrow &&
                  (F.parent < 0 || bwd_diag_seen[F.parent] == nblk(F.parent)) &&
-                 pl.ps_pbase[s] + (int64_t)(nblk(s) - 1) * nbelow(s) + t.b / RC < pl.ps_part_entries / B,
+                 sp.pbase[s] + (int64_t)(nblk(s) - 1) * nbelow(s) + t.b / RC < sp.part_entries / B,
              "backward partial task");
         bwd_part_seen[s]++;
         break;
@@ -924,13 +923,13 @@ void build_fused_solve(Plan &pl) {
       need(pl.fronts[pl.children[ci]].parent == s, "child list");
       kids += nbelow(pl.children[ci]);
     }
-    need(kids == pl.ps_kid_chunks[s], "children's chunk count");
+    need(kids == sp.kid_chunks[s], "children's chunk count");
   }
-  pl.ps_recs.resize(pl.ps_tasks.size());
-  for (size_t q = 0; q < pl.ps_tasks.size(); q++) {
-    const int32_t s = pl.ps_tasks[q].front;
-    pl.ps_recs[q] = SolveRec{pl.ps_tasks[q], pl.fronts[s], pl.toff[s], pl.ps_pbase[s],
-                             pl.fs_first_slot[s], pl.ps_kid_chunks[s], pl.ps_parent_blocks[s], 0};
+  sp.recs.resize(sp.tasks.size());
+  for (size_t q = 0; q < sp.tasks.size(); q++) {
+    const int32_t s = sp.tasks[q].front;
+    sp.recs[q] = SolveRec{sp.tasks[q], pl.fronts[s], pl.toff[s], sp.pbase[s],
+                             sp.first_slot[s], sp.kid_chunks[s], sp.parent_blocks[s], 0};
   }
 }
 

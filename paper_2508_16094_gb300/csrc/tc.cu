@@ -815,7 +815,7 @@ __global__ void __launch_bounds__(256, 1) potrf_inv_kernel(DevPlan dp, const Tas
   }
   float *out = Linv + (int64_t)slot * 128 * 128;
   const int ldi = (kb + 3) & ~3;
-  float *o2 = Dinv ? Dinv + dp.fs_dinv_off[dp.fs_first_slot[tk.front] + k / TcPlan::kNb] : nullptr;
+  float *o2 = Dinv ? Dinv + dp.s32.dinv_off[dp.s32.first_slot[tk.front] + k / TcPlan::kNb] : nullptr;
 #pragma unroll
   for (int a = 0; a < 8; a++)
 #pragma unroll
