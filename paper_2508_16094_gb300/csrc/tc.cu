@@ -706,130 +706,305 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(192, 1)
 // of its factor, written row-major (128 x 128, zero outside the lower kb x kb
 // triangle) to scratch slot `b` for the triangular solve of the rows below as
 // a tensor-core product, and (when Dinv is given) in the layout of the
-// persistent solve. One right-looking step per column j does both: the rank-1
-// update of the trailing block with column j of the factor, and the update of
-// Y (which starts as I and ends as L^{-1} up to row scaling) with the same
-// column and row j of the inverse, Y_j / L_jj. Thread (ty, tx) of a 16 x 16
-// grid holds rows ty + 16a and columns tx + 16b of the lower tiles a >= b of
-// both matrices in registers; the column of the factor, the row of Y and the
-// next pivot's 1 / L_jj (computed by its owner before the barrier) are
-// published in shared memory, double-buffered, so a step costs one barrier.
-// The loop over the 16 columns of a tile column stays rolled, which keeps the
-// code that runs once per launch small. A non-positive pivot is replaced by a
-// large value (static pivoting) and counted.
-__global__ void __launch_bounds__(256, 1) potrf_inv_kernel(DevPlan dp, const Task *__restrict__ tasks,
-                                                        float *__restrict__ L,
-                                                        float *__restrict__ Linv,
-                                                        float *__restrict__ Dinv, int32_t *status) {
-  const Task tk = tasks[blockIdx.x];
-  const FrontInfo F = dp.fronts[tk.front];
-  const int k = tk.a, slot = tk.b, kb = min(TcPlan::kNb, F.ncol - k);
-  __shared__ float cbuf[2][128];  // column j of the factor (unscaled, updated through step j - 1)
-  __shared__ float ybuf[2][128];  // row j of Y
-  __shared__ float rdv[128];      // 1 / L_jj
-  __shared__ float sqv[128];      // L_jj
-  float *g = L + F.loff + (int64_t)k * F.ld + k;
-  const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
-  // the pivot of column j, owned by the thread holding entry (j, j)
-  auto pivot = [&](int j, float d) {
-    const bool bad = !(d > 0.f) || !(d < 3.0e38f);
-    if (bad) {
-      d = 1e30f;
-      atomicAdd(&status[ST_PERTURBED], 1);
-    }
-    // 1 / sqrt(d) from the hardware estimate and one Newton step for
-    // r^-2 = d (r' = r + r (1 - d r^2) / 2, error ~1 ulp), instead of a
-    // correctly rounded square root and division on the step's critical path
-    float r = d >= 1e-30f ? rsqrtf(d) : 1.f / sqrtf(d);
-    r = fmaf(0.5f * r, fmaf(-d * r, r, 1.f), r);
-    sqv[j] = d * r;
-    rdv[j] = r;
-  };
-  float acc[8][8], y[8][8];  // entries a >= b only
+// persistent solve. A non-positive pivot is replaced by a large value (static
+// pivoting) and counted.
+//
+// Bound by the chain of 128 pivots (one launch is a step of a front's chain): what
+// counts is the latency of one column. So a step takes two columns and touches 16
+// only (panels of 16 on warps 0-7, two threads per row, eight columns each in
+// registers, unscaled columns: a_ic -= (a_ij / d_j) a_cj; the next pair is published
+// through shared memory before the one barrier of a step, the rest of the panel
+// updated after it beside the next pivots). Past the panel a rank-16
+// update on all warps, 16 x 16 blocks with 16-byte shared-memory reads. Meanwhile
+// warps 8-15 write the finished columns out and take the inverse further by block
+// substitution (Y_b = X_bb R_b with a 16 x 16 inverse, then R_i -= L_ib Y_b; a product of
+// larger inverses has no residual bound), one and two block rows behind the panel.
+// One right-looking loop that updated the whole block and the inverse per column
+// took 60 us a launch.
+//
+// Shared block, row stride kLs: L in the lower triangle, the inverse X in the
+// rest, X[r][c] at [c][r + 4] (r >= c, so always right of the diagonal, and four
+// consecutive rows of X are one aligned 16-byte read).
+constexpr int kLs = 132, kPiThreads = 512, kXdLs = 20;
+constexpr int kPiSmem = (128 * kLs + 2 * 16 * kXdLs) * 4;
+
+// acc[ii][jj] = sum_{k < 16} A[i][k] B[j][k], rows i = l / 4 + 8 ii of A (stride lda) and
+// j = l % 4 + 4 jj of B (stride kLs), 16-byte aligned rows.
+__device__ __forceinline__ void blk_nt(const float *A, int lda, const float *B, float (&acc)[2][4]) {
+  const int l = threadIdx.x % 32;
+  const float *pa = A + (l / 4) * lda, *pb = B + (l % 4) * kLs;
 #pragma unroll
-  for (int a = 0; a < 8; a++)
+  for (int ii = 0; ii < 2; ii++)
 #pragma unroll
-    for (int b = 0; b <= a; b++) {
-      const int r = ty + 16 * a, c = tx + 16 * b;
-      acc[a][b] = (r < kb && c <= r) ? g[(int64_t)r * F.ld + c] : 0.f;
-      y[a][b] = (a == b && tx == ty) ? 1.f : 0.f;
-    }
-  if (tx == 0)
+    for (int jj = 0; jj < 4; jj++) acc[ii][jj] = 0.f;
 #pragma unroll
-    for (int a = 0; a < 8; a++) cbuf[0][ty + 16 * a] = acc[a][0];
-  if (ty == 0) ybuf[0][tx] = y[0][0];
-  if (tid == 0) pivot(0, acc[0][0]);
-  __syncthreads();
+  for (int k = 0; k < 16; k += 4) {
+    float4 a[2], b[4];
 #pragma unroll
-  for (int jb = 0; jb < 8; jb++) {
-    if (16 * jb < kb) {
-#pragma unroll 1
-      for (int jj = 0; jj < 16; jj++) {
-        const int j = 16 * jb + jj;
-        if (j >= kb) break;
-        const float *cb = cbuf[j & 1], *yb = ybuf[j & 1];
-        const float rs = rdv[j];
-        float u[8], v[8], x[8];
+    for (int ii = 0; ii < 2; ii++) a[ii] = *reinterpret_cast<const float4 *>(pa + 8 * ii * lda + k);
 #pragma unroll
-        for (int a = jb; a < 8; a++) {
-          const int r = ty + 16 * a, c = tx + 16 * a;
-          u[a] = r > j ? cb[r] * rs : 0.f;  // L_rj below the diagonal
-          v[a] = c > j ? cb[c] * rs : 0.f;
-        }
+    for (int jj = 0; jj < 4; jj++) b[jj] = *reinterpret_cast<const float4 *>(pb + 4 * jj * kLs + k);
 #pragma unroll
-        for (int b = 0; b <= jb; b++) x[b] = yb[tx + 16 * b] * rs;  // row j of L^{-1}
+    for (int ii = 0; ii < 2; ii++)
 #pragma unroll
-        for (int a = jb; a < 8; a++)
-#pragma unroll
-          for (int b = jb; b <= a; b++) acc[a][b] = fmaf(-u[a], v[b], acc[a][b]);
-#pragma unroll
-        for (int a = jb; a < 8; a++)
-#pragma unroll
-          for (int b = 0; b <= jb && b <= a; b++) y[a][b] = fmaf(-u[a], x[b], y[a][b]);
-        const int jn = j + 1;
-        if (jn < kb) {
-          float *nc = cbuf[jn & 1], *ny = ybuf[jn & 1];
-          if (jj < 15) {
-            if (tx == jj + 1) {
-#pragma unroll
-              for (int a = jb; a < 8; a++) nc[ty + 16 * a] = acc[a][jb];
-              if (ty == jj + 1) pivot(jn, acc[jb][jb]);
-            }
-            if (ty == jj + 1)
-#pragma unroll
-              for (int b = 0; b <= jb; b++) ny[tx + 16 * b] = y[jb][b];
-          } else if (jb < 7) {
-            if (tx == 0) {
-#pragma unroll
-              for (int a = jb + 1; a < 8; a++) nc[ty + 16 * a] = acc[a][jb + 1];
-              if (ty == 0) pivot(jn, acc[jb + 1][jb + 1]);
-            }
-            if (ty == 0)
-#pragma unroll
-              for (int b = 0; b <= jb + 1; b++) ny[tx + 16 * b] = y[jb + 1][b];
-          }
-        }
-        __syncthreads();
-      }
+      for (int jj = 0; jj < 4; jj++)
+        acc[ii][jj] = fmaf(a[ii].x, b[jj].x, fmaf(a[ii].y, b[jj].y, fmaf(a[ii].z, b[jj].z,
+                      fmaf(a[ii].w, b[jj].w, acc[ii][jj]))));
+  }
+}
+
+// 1 / d of a pivot (reciprocal estimate and one Newton step); one that is not
+// positive is replaced and counted (by thread 0: the branch is uniform).
+__device__ __forceinline__ float pivot_inverse(float &d, int32_t *status) {
+  if (d >= 1e-37f && d <= 8e37f) {
+    const float i = __fdividef(1.f, d);
+    return fmaf(i, fmaf(-d, i, 1.f), i);
+  }
+  if (!(d > 0.f) || !(d < 3.0e38f)) {
+    d = 1e30f;
+    if (threadIdx.x == 0) atomicAdd(&status[ST_PERTURBED], 1);
+  }
+  return 1.f / d;
+}
+
+// Barrier over `threads` threads (whole warps) of the block; id 0 is __syncthreads.
+__device__ __forceinline__ void bar_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// Rows r0, r0 + step, .. < r1 of column block b0 of L to global memory (four lanes per
+// row, rows r0 + l / 4 of a warp); entries past the diagonal are kept.
+__device__ __forceinline__ void put_columns(const float *S, float *g, int64_t ld, int b0, int r0, int step,
+                                            int r1) {
+  const int l = threadIdx.x % 32, c = b0 + 4 * (l % 4);
+  for (int r = r0 + l / 4; r < r1; r += step) {
+    if (c > r) continue;
+    const float4 v = *reinterpret_cast<const float4 *>(S + r * kLs + c);
+    float *o = g + (int64_t)r * ld + c;
+    if (c + 3 <= r) {
+      *reinterpret_cast<float4 *>(o) = v;
+    } else {
+      o[0] = v.x;
+      if (c + 1 <= r) o[1] = v.y;
+      if (c + 2 <= r) o[2] = v.z;
     }
   }
+}
+
+// On one warp: the 16 rows of the diagonal block at b0 out, then X_bb (lane c < 16
+// its column c) in X's place, where its zeros fall on the block's own L entries,
+// and row-major in XD.
+__device__ __forceinline__ void inverse_diag(float *S, float *XD, const float *rsv, float *g, int64_t ld, int kb,
+                                             int b0) {
+  const int l = threadIdx.x % 32;
+  put_columns(S, g, ld, b0, b0, 8, min(kb, b0 + 16));
+  float x[16];
+  const float *B = S + b0 * kLs + b0;
+#pragma unroll
+  for (int i = 0; i < 16; i++) x[i] = i == l ? 1.f : 0.f;
+#pragma unroll
+  for (int m = 0; m < 16; m++) {
+    x[m] *= rsv[b0 + m];
+#pragma unroll
+    for (int i = m + 1; i < 16; i++) x[i] = fmaf(-x[m], B[i * kLs + m], x[i]);
+  }
+  __syncwarp();
+  if (l >= 16) return;
+  float *o = S + (b0 + l) * kLs + b0 + 4, *xd = XD + l;
+#pragma unroll
+  for (int i = 0; i < 16; i++) {
+    const float v = i >= l ? x[i] : 0.f;
+    o[i] = v;
+    xd[i * kXdLs] = v;
+  }
+}
+
+// Y_b = X_bb R_b, the column block `w` on one warp, in place.
+__device__ __forceinline__ void inverse_row(float *S, const float *XD, int b0, int w) {
+  const int l = threadIdx.x % 32;
+  float acc[2][4];
+  blk_nt(XD, kXdLs, S + 16 * w * kLs + b0 + 4, acc);
+  __syncwarp();
+#pragma unroll
+  for (int ii = 0; ii < 2; ii++)
+#pragma unroll
+    for (int jj = 0; jj < 4; jj++)
+      S[(16 * w + l % 4 + 4 * jj) * kLs + b0 + l / 4 + 8 * ii + 4] = acc[ii][jj];
+}
+
+// R_i(c) -= L_ib Y_b(c) for every block row i below b0, on nw warps (w: number of this one).
+__device__ __forceinline__ void inverse_update(float *S, int KB, int b0, int w, int nw) {
+  const int l = threadIdx.x % 32, nb = b0 / 16, below = KB / 16 - nb - 1;
+  for (int u = w; u < below * (nb + 1); u += nw) {
+    const int i0 = b0 + 16 + 16 * (u / (nb + 1)), cb = 16 * (u % (nb + 1));
+    float acc[2][4];
+    blk_nt(S + i0 * kLs + b0, kLs, S + cb * kLs + b0 + 4, acc);
+#pragma unroll
+    for (int ii = 0; ii < 2; ii++)
+#pragma unroll
+      for (int jj = 0; jj < 4; jj++) {
+        float *o = S + (cb + l % 4 + 4 * jj) * kLs + i0 + l / 4 + 8 * ii + 4;
+        *o = (cb < b0 ? *o : 0.f) - acc[ii][jj];
+      }
+  }
+}
+
+// What warps 8 .. 15 do beside the panel at c0 (or, c0 = KB, after the last one): warp 8
+// the diagonal block before it, the others the rows below that block out and the
+// inverse's block row before that.
+__device__ __forceinline__ void inverse_behind(float *S, float *XD, const float *rsv, float *g, int64_t ld, int kb,
+                                               int KB, int c0, int w) {
+  if (c0 < 16) return;
+  float *xd = XD + (c0 / 16 & 1) * 16 * kXdLs, *xd_old = XD + (c0 / 16 - 1 & 1) * 16 * kXdLs;
+  if (w == 0) {
+    inverse_diag(S, xd, rsv, g, ld, kb, c0 - 16);
+    return;
+  }
+  constexpr int NW = kPiThreads / 64 - 1;
+  put_columns(S, g, ld, c0 - 16, c0 + 8 * (w - 1), 8 * NW, kb);
+  if (c0 < 32) return;
+  if (w - 1 < c0 / 16 - 2) inverse_row(S, xd_old, c0 - 32, w - 1);
+  bar_sync(2, 32 * NW);
+  inverse_update(S, KB, c0 - 32, w - 1, NW);
+}
+
+__global__ void __launch_bounds__(kPiThreads, 1) potrf_inv_kernel(DevPlan dp, const Task *__restrict__ tasks,
+                                                                float *__restrict__ L,
+                                                                float *__restrict__ Linv,
+                                                                float *__restrict__ Dinv, int32_t *status) {
+  extern __shared__ __align__(16) float S[];
+  float *XD = S + 128 * kLs;  // 16 x 16 inverses of the last two diagonal blocks, row-major
+  __shared__ float cp[3][2][128], piv[128], rsv[128];  // column pairs of the running panel
+  constexpr int kPanel = kPiThreads / 2;
+  const Task tk = tasks[blockIdx.x];
+  const FrontInfo F = dp.fronts[tk.front];
+  const int k = tk.a, slot = tk.b, kb = min(TcPlan::kNb, F.ncol - k), KB = (kb + 15) & ~15;
+  float *g = L + F.loff + (int64_t)k * F.ld + k;
+  const int tid = threadIdx.x, warp = tid / 32, l = tid % 32;
+  // the block (rows of 16-byte reads: ld and k are multiples of 4); past kb a
+  // unit diagonal
+  {
+    float4 v[8];
+    const int c = 4 * l;
+#pragma unroll
+    for (int q = 0; q < 8; q++) {
+      const int r = warp + 16 * q;
+      v[q] = (r < kb && c <= r) ? *reinterpret_cast<const float4 *>(g + (int64_t)r * F.ld + c)
+                                : make_float4(r == c, r == c + 1, r == c + 2, r == c + 3);
+    }
+#pragma unroll
+    for (int q = 0; q < 8; q++) {
+      const int r = warp + 16 * q;
+      if (c <= r) *reinterpret_cast<float4 *>(S + r * kLs + c) = v[q];
+    }
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int c0 = 0; c0 < KB; c0 += 16) {
+    const int act = ((KB - c0) * 2 + 31) & ~31;  // threads of the panel: whole warps with rows
+    if (tid < act) {
+      const int i = c0 + tid / 2, h = tid % 2;  // (KB is a multiple of 16: every row exists)
+      float x[8];                               // columns c0 + h + 2 q of row i
+#pragma unroll
+      for (int q = 0; q < 8; q++) x[q] = S[i * kLs + c0 + h + 2 * q];
+      cp[0][h][i] = x[0];
+      bar_sync(1, act);
+#pragma unroll
+      for (int q = 0; q < 8; q++) {  // columns j = 2 q and j + 1 of the panel
+        const float *p0 = cp[q % 3][0] + c0, *p1 = cp[q % 3][1] + c0;
+        float d1 = p0[2 * q], d2 = p1[2 * q + 1];
+        const float a21 = p0[2 * q + 1], a1 = p0[i - c0], a2 = p1[i - c0];
+        float v1[8], v2[8];
+#pragma unroll
+        for (int r = q + 1; r < 8; r++) {
+          v1[r] = p0[h + 2 * r];
+          v2[r] = p1[h + 2 * r];
+        }
+        const float i1 = pivot_inverse(d1, status);
+        const float t = a21 * i1;
+        d2 = fmaf(-t, a21, d2);
+        const float i2 = pivot_inverse(d2, status);
+        if (tid == 0) {
+          piv[c0 + 2 * q] = d1;
+          piv[c0 + 2 * q + 1] = d2;
+        }
+        const float w1 = a1 * i1, a2p = fmaf(-w1, a21, a2), w2 = a2p * i2;
+        if (h == 1) x[q] = a2p;
+        if (q == 7) break;
+        // the next pair first
+        x[q + 1] = fmaf(-w1, v1[q + 1], fmaf(-w2, fmaf(-t, v1[q + 1], v2[q + 1]), x[q + 1]));
+        cp[(q + 1) % 3][h][i] = x[q + 1];
+        bar_sync(1, act);
+#pragma unroll
+        for (int r = q + 2; r < 8; r++)
+          x[r] = fmaf(-w1, v1[r], fmaf(-w2, fmaf(-t, v1[r], v2[r]), x[r]));
+      }
+      bar_sync(1, act);
+#pragma unroll
+      for (int q = 0; q < 8; q++) {  // 1 / L_cc: hardware estimate and one Newton step
+        const int c = c0 + h + 2 * q;
+        const float d = piv[c];
+        float r = rsqrtf(d);
+        r = fmaf(0.5f * r, fmaf(-d * r, r, 1.f), r);
+        if (c <= i) S[i * kLs + c] = c == i ? d * r : x[q] * r;
+        if (c == i) rsv[c] = r;
+      }
+    } else if (tid >= kPanel) {
+      inverse_behind(S, XD, rsv, g, F.ld, kb, KB, c0, warp - kPanel / 32);
+    }
+    __syncthreads();
+    // rank-16 update of the lower triangle past the panel, a 16 x 16 block per warp
+    const int n16 = (KB - c0 - 16) / 16, nblk = n16 * (n16 + 1) / 2;
+    for (int u = warp; u < nblk; u += kPiThreads / 32) {
+      int bi = 0, rest = u;
+      while (rest > bi) rest -= ++bi;  // block row bi holds bi + 1 blocks
+      const int i0 = c0 + 16 + 16 * bi, j0 = c0 + 16 + 16 * rest;
+      float acc[2][4];
+      blk_nt(S + i0 * kLs + c0, kLs, S + j0 * kLs + c0, acc);
+#pragma unroll
+      for (int ii = 0; ii < 2; ii++)
+#pragma unroll
+        for (int jj = 0; jj < 4; jj++) {
+          const int r = i0 + l / 4 + 8 * ii, c = j0 + l % 4 + 4 * jj;
+          if (c <= r) S[r * kLs + c] -= acc[ii][jj];
+        }
+    }
+    __syncthreads();
+  }
+  if (tid >= kPanel) inverse_behind(S, XD, rsv, g, F.ld, kb, KB, KB, warp - kPanel / 32);
+  __syncthreads();
+  if (warp < KB / 16 - 1) inverse_row(S, XD + (KB / 16 & 1) * 16 * kXdLs, KB - 16, warp);
+  __syncthreads();
+  // X out, 4 x 4 entries per thread and pass: four consecutive rows of X are one
+  // 16-byte read, four lanes write 64 consecutive bytes of a row
   float *out = Linv + (int64_t)slot * 128 * 128;
   const int ldi = (kb + 3) & ~3;
   float *o2 = Dinv ? Dinv + dp.s32.dinv_off[dp.s32.first_slot[tk.front] + k / TcPlan::kNb] : nullptr;
 #pragma unroll
-  for (int a = 0; a < 8; a++)
+  for (int q = 0; q < 2; q++) {
+    const int u = warp + 16 * q;  // 32 (row, column) tiles of 32 x 16
+    const int r0 = 32 * (u / 8) + 4 * (l / 4), c = 16 * (u % 8) + 4 * (l % 4);
+    float v[4][4];  // [column][row]
 #pragma unroll
-    for (int b = 0; b < 8; b++) {
-      const int r = ty + 16 * a, c = tx + 16 * b;
-      float xv = 0.f;
-      if (b <= a) {
-        if (r < kb && c < r) g[(int64_t)r * F.ld + c] = acc[a][b] * rdv[c];
-        if (r < kb && c == r) g[(int64_t)r * F.ld + c] = sqv[c];
-        if (r < kb && c <= r) xv = y[a][b] * rdv[r];
-      }
-      out[r * 128 + c] = xv;
-      if (o2 && r < kb && c < ldi) o2[r * ldi + c] = xv;
+    for (int h = 0; h < 4; h++) {
+      float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (c <= r0 + 3 && c + h < KB && r0 < KB) f = *reinterpret_cast<const float4 *>(S + (c + h) * kLs + r0 + 4);
+      v[h][0] = f.x;
+      v[h][1] = f.y;
+      v[h][2] = f.z;
+      v[h][3] = f.w;
     }
+#pragma unroll
+    for (int ii = 0; ii < 4; ii++) {
+      const int r = r0 + ii;
+      float t[4];
+#pragma unroll
+      for (int h = 0; h < 4; h++) t[h] = (r < kb && c + h <= r) ? v[h][ii] : 0.f;
+      const float4 o = make_float4(t[0], t[1], t[2], t[3]);
+      *reinterpret_cast<float4 *>(out + r * 128 + c) = o;
+      if (o2 && r < kb && c < ldi) *reinterpret_cast<float4 *>(o2 + r * ldi + c) = o;
+    }
+  }
 }
 
 }  // namespace
@@ -1116,6 +1291,7 @@ void TcPlan::encode(const Plan &plan, float *L, float *Llo, float *U, cudaStream
                         cudaMemcpyHostToDevice, st) != cudaSuccess)
       throw std::runtime_error("tensor map upload failed");
   if (cudaStreamSynchronize(st) != cudaSuccess) throw std::runtime_error("tensor map upload failed");
+  cudaFuncSetAttribute(potrf_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPiSmem);
   cudaFuncSetAttribute(tc_gemm_kernel<1, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<1, 128>::smem);
   cudaFuncSetAttribute(tc_gemm_kernel<3, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<3, 128>::smem);
   cudaFuncSetAttribute(tc_pair_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<1, kSyrkN>::smem);
@@ -1210,7 +1386,7 @@ void TcPlan::factor(const DevPlan &dp, const Plan &plan, const double *kval, flo
         const Step &s = lv.steps[i];
         if (s.gemm_e > s.gemm_b) gemm(d_gemm_ + s.gemm_b, s.gemm_e - s.gemm_b, ctas, st);
         if (s.potrf_e > s.potrf_b)
-          { note_launch(); potrf_inv_kernel<<<s.potrf_e - s.potrf_b, 256, 0, st>>>(dp, d_potrf_ + s.potrf_b, L, d_inv_, Dinv, status); }
+          { note_launch(); potrf_inv_kernel<<<s.potrf_e - s.potrf_b, kPiThreads, kPiSmem, st>>>(dp, d_potrf_ + s.potrf_b, L, d_inv_, Dinv, status); }
         if (s.trsm_e > s.trsm_b) gemm(d_trsm_ + s.trsm_b, s.trsm_e - s.trsm_b, ctas, st);
       }
     }
