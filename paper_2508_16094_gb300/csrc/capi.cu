@@ -67,6 +67,7 @@ struct ipm_ctx {
   int test_withhold = -1;    // ... and the ticket of the task it abandons
   double *lb_loss = nullptr;
   double *scal = nullptr, *partial = nullptr;
+  unsigned *ticket = nullptr;  // of the reductions (VecOps), zeroed when the workspace is set
   IpmScalars *sc = nullptr;
   int32_t *status = nullptr, *col2s = nullptr;
   TcPlan tcp;
@@ -95,7 +96,7 @@ struct ipm_ctx {
   int32_t last_perturbed = 0;
   int64_t refine_steps = 0, pcg_steps = 0;
   double last_rel = 0.0;
-  VecOps vec() const { return VecOps{dp, st, partial}; }
+  VecOps vec() const { return VecOps{dp, st, partial, ticket}; }
   ~ipm_ctx() { delete sys; }
 };
 
@@ -322,6 +323,7 @@ void layout(ipm_ctx *c, char *base) {
   }
   c->scal = cv.take<double>(64);
   c->partial = cv.take<double>(kRedBlocks * 8);
+  c->ticket = cv.take<unsigned>(32);
   c->sc = cv.take<IpmScalars>(1);
   c->status = cv.take<int32_t>(ST_COUNT);
   c->L = cv.take<char>((size_t)pl.l_entries * c->storage_bytes);
@@ -431,45 +433,54 @@ template <typename T> void launch_both_sweeps(ipm_ctx *c, T *mid) {
   launch_held_solve<T>(c, 2);
 }
 
-// out = M^{-1} b with the current factor (b, out: original numbering, device)
-void apply_factor(ipm_ctx *c, const double *b, double *out, bool accumulate) {
+// The preconditioner up to the final numbering's result: P b (times scale[0] for an
+// FP32-storage factor), the sweeps; y points to the result.
+bool factor_is_fp64(const ipm_ctx *c) { return c->storage_bytes == 8 && c->factor_prec == IPM_FP64; }
+void sweeps(ipm_ctx *c, const double *b, const double *scale) {
   VecOps V = c->vec();
+  if (factor_is_fp64(c)) {
+    V.permute_in<double>(b, nullptr, c->yv);
+    launch_both_sweeps<double>(c, c->dsb);
+    return;
+  }
+  V.permute_in<float>(b, scale, c->fsa);
   if (c->learned_active) {  // P^T L_s^{-T} (Delta + U U^T)^{-1} L_s^{-1} P b
-    double *scale = c->scal + 8, *amax = c->scal + 9;
-    V.absmax(c->P.n, b, amax);
-    V.inv_scale(amax, scale);
-    V.permute_in<float>(b, scale, c->fsa);
     launch_fp32_solve(c, 1);
     learned_apply(c->lb, c->fsb, c->st);
     launch_fp32_solve(c, 2);
-    V.permute_out<float>(c->fsx, scale, out, accumulate);
-    return;
-  }
-  if (c->storage_bytes == 8 && c->factor_prec == IPM_FP64) {
-    V.permute_in<double>(b, nullptr, c->yv);
-    launch_both_sweeps<double>(c, c->dsb);
-    V.permute_out<double>(c->dsx, nullptr, out, accumulate);
   } else {
-    double *scale = c->scal + 8, *amax = c->scal + 9;
-    V.absmax(c->P.n, b, amax);
-    V.inv_scale(amax, scale);
-    V.permute_in<float>(b, scale, c->fsa);
     launch_both_sweeps<float>(c, c->fsb);
-    V.permute_out<float>(c->fsx, scale, out, accumulate);
   }
+}
+// out = M^{-1} b with the current factor (b, out: original numbering, device; scale:
+// 1 / max |b|)
+void apply_factor(ipm_ctx *c, const double *b, const double *scale, double *out, bool accumulate) {
+  VecOps V = c->vec();
+  sweeps(c, b, scale);
+  if (factor_is_fp64(c)) V.permute_out<double>(c->dsx, nullptr, out, accumulate);
+  else V.permute_out<float>(c->fsx, scale, out, accumulate);
+}
+// z = M^{-1} r, rz = r . z, beta = rz / rz_old (when given)
+void apply_factor_dot(ipm_ctx *c, const double *r, const double *scale, double *z, const double *rz_old,
+                      double *rz, double *beta) {
+  VecOps V = c->vec();
+  sweeps(c, r, scale);
+  if (factor_is_fp64(c)) V.permute_out_dot<double>(c->dsx, nullptr, r, z, rz_old, rz, beta);
+  else V.permute_out_dot<float>(c->fsx, scale, r, z, rz_old, rz, beta);
 }
 
 // A wait of the persistent solve that ran out of time: the launch drained and
 // its result is invalid; clear the word (each launch zeroes its own flags) and
 // report the timeout.
+void report_solve_timeout(ipm_ctx *c) {
+  CK(cudaMemsetAsync(c->status + ST_SOLVE_TIMEOUT, 0, sizeof(int32_t), c->st));
+  throw Fail{IPM_ERR_TIMEOUT, "a bounded wait of the persistent solve ran out of time"};
+}
 void check_solve_barrier(ipm_ctx *c) {
   int32_t flag = 0;
   CK(cudaMemcpyAsync(&flag, c->status + ST_SOLVE_TIMEOUT, sizeof(flag), cudaMemcpyDeviceToHost, c->st));
   CK(cudaStreamSynchronize(c->st));
-  if (flag) {
-    CK(cudaMemsetAsync(c->status + ST_SOLVE_TIMEOUT, 0, sizeof(int32_t), c->st));
-    throw Fail{IPM_ERR_TIMEOUT, "a bounded wait of the persistent solve ran out of time"};
-  }
+  if (flag) report_solve_timeout(c);
 }
 
 // ---- solve with refinement / PCG ----------------------------------------------
@@ -478,51 +489,59 @@ ipm_status do_solve(ipm_ctx *c, const double *b, double *x, int refine, ipm_solv
   VecOps V = c->vec();
   const int64_t n = c->P.n;
   const ipm_options &o = c->opts;
-  double *bb = c->vb, *r = c->vr, *z = c->vz, *p = c->vp, *q = c->vq, *xx = c->vx;
-  CK(cudaMemcpyAsync(bb, b, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
-  double *sN = c->scal;  // scalars: 0 |b|, 1 |r|, 2 rz, 3 pq, 4 rz_new
-  const int pcg_max = c->pcg_override >= 0 ? c->pcg_override : o.pcg_max;
-  V.absmax(n, bb, sN + 0);
-  const double bn = d2h_scalar(c, sN + 0);
-  if (info) *info = ipm_solve_info{0, 0, 0.0};
-  if (bn == 0.0) {
-    CK(cudaMemsetAsync(x, 0, n * sizeof(double), c->st));
-    c->last_rel = 0.0;
-    return IPM_OK;
+  double *r = c->vr, *z = c->vz, *p = c->vp, *q = c->vq;
+  // x is the running solution; b is copied only where the two overlap
+  const double *bb = b;
+  if (b < x + n && x < b + n) {
+    CK(cudaMemcpyAsync(c->vb, b, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
+    bb = c->vb;
   }
+  // scalars: 0, 1 |b| and its scale; 2, 3 |r| and its scale, 4 the solve's timeout word, 5 |x|
+  // (bwd_measure); 6, 7 rz of alternating iterations; 8 alpha, 9 beta
+  double *sN = c->scal, *sR = sN + 2;
+  const int pcg_max = c->pcg_override >= 0 ? c->pcg_override : o.pcg_max;
+  V.absmax(n, bb, sN, true);
+  if (info) *info = ipm_solve_info{0, 0, 0.0};
   // ||b - K x|| / ||b|| drives refinement. For a badly scaled matrix (the grid
   // NLP: entries up to (nx+1)^4 times D) its floor is about eps ||K|| ||x|| / ||b||,
   // so with bwd_measure the solve is accepted on the normwise backward error
   // ||b - K x|| / (||K|| ||x|| + ||b||) instead (refinement still runs until it stalls).
-  double bwd = 0.0;
+  double bwd = 0.0, bn = 0.0;
+  bool timed_out = false;
   auto residual = [&](const double *xv) {
-    V.residual(c->cur_jvals, c->cur_D, c->cur_wvals, c->cur_delta_p, xv, bb, r, c->vtA);
-    V.absmax(n, r, sN + 1);
-    if (!c->bwd_measure) return d2h_scalar(c, sN + 1) / bn;
-    V.absmax(n, xv, sN + 5);
-    double h2[5];
-    CK(cudaMemcpyAsync(h2, sN + 1, 5 * sizeof(double), cudaMemcpyDeviceToHost, c->st));
+    V.residual(c->cur_jvals, c->cur_D, c->cur_wvals, c->cur_delta_p, xv, bb, r, c->vtA, sR,
+               c->status + ST_SOLVE_TIMEOUT);
+    if (c->bwd_measure) V.absmax(n, xv, sN + 5);
+    double h[6];
+    CK(cudaMemcpyAsync(h, sN, sizeof(h), cudaMemcpyDeviceToHost, c->st));
     CK(cudaStreamSynchronize(c->st));
-    bwd = h2[0] / (c->knorm * h2[4] + bn);
-    return h2[0] / bn;
+    bn = h[0];
+    timed_out = h[4] != 0.0;
+    if (c->bwd_measure) bwd = h[2] / (c->knorm * h[5] + bn);
+    return h[2] / bn;
   };
   double rel;
   if (c->warm_x) {  // x holds a nearby solution (the predictor's direction)
-    CK(cudaMemcpyAsync(xx, x, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
-    residual(xx);
-    apply_factor(c, r, xx, true);
+    residual(x);
+    if (bn > 0.0) apply_factor(c, r, sR + 1, x, true);
   } else {
-    apply_factor(c, bb, xx, false);
+    apply_factor(c, bb, sN + 1, x, false);
   }
-  rel = residual(xx);
+  rel = residual(x);
+  if (bn == 0.0) {
+    CK(cudaMemsetAsync(x, 0, n * sizeof(double), c->st));
+    if (timed_out) report_solve_timeout(c);
+    c->last_rel = 0.0;
+    return IPM_OK;
+  }
   int iters = 0, used_pcg = 0;
   if (refine != IPM_REFINE_NONE && refine != IPM_REFINE_PCG) {
     double prev = rel;
     int slow = 0;
     while (rel > o.ir_tol && iters < o.ir_max) {
-      apply_factor(c, r, xx, true);
+      apply_factor(c, r, sR + 1, x, true);
       iters++;
-      rel = residual(xx);
+      rel = residual(x);
       if (!(rel < 0.5 * prev)) slow++;
       else slow = 0;
       prev = std::min(prev, rel);
@@ -534,25 +553,18 @@ ipm_status do_solve(ipm_ctx *c, const double *b, double *x, int refine, ipm_solv
       !(c->bwd_measure && bwd <= o.ir_tol && std::isfinite(rel))) {
     // PCG on K x = b preconditioned by the factor, from the current x
     if (!std::isfinite(rel)) {
-      CK(cudaMemsetAsync(xx, 0, n * sizeof(double), c->st));
-      rel = residual(xx);
+      CK(cudaMemsetAsync(x, 0, n * sizeof(double), c->st));
+      rel = residual(x);
     }
     used_pcg = 1;
-    CK(cudaMemsetAsync(c->vc, 0, n * sizeof(double), c->st));  // zero right-hand side for q = K p
-    apply_factor(c, r, z, false);
-    CK(cudaMemcpyAsync(p, z, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
-    V.dot(n, r, z, sN + 2);
+    double *rz = sN + 6, *rz_next = sN + 7, *alpha = sN + 8, *beta = sN + 9;
+    apply_factor_dot(c, r, sR + 1, p, nullptr, rz, nullptr);  // p = z
     const double rel0 = rel;
     int k = 0;
     for (; k < pcg_max && rel > o.ir_tol; k++) {
-      // q = K p  (residual of b = 0 gives -K p)
-      V.residual(c->cur_jvals, c->cur_D, c->cur_wvals, c->cur_delta_p, p, c->vc, q, c->vtA);
-      V.negate(n, q);
-      V.dot(n, p, q, sN + 3);
-      V.axpy_ratio(n, sN + 2, sN + 3, +1, p, xx);
-      V.axpy_ratio(n, sN + 2, sN + 3, -1, q, r);
-      V.absmax(n, r, sN + 1);
-      rel = d2h_scalar(c, sN + 1) / bn;
+      V.kp_dot(c->cur_jvals, c->cur_D, c->cur_wvals, c->cur_delta_p, p, q, c->vtA, rz, alpha);
+      V.cg_step(n, alpha, p, q, x, r, sR);
+      rel = d2h_scalar(c, sR) / bn;
       if (rel <= o.ir_tol || !std::isfinite(rel)) { k++; break; }
       // a corrected stale factor is only worth keeping if PCG converges
       // within the budget: from the fifth iteration on, give up once the mean
@@ -563,18 +575,16 @@ ipm_status do_solve(ipm_ctx *c, const double *b, double *x, int refine, ipm_solv
         const double need = (k + 1) + std::log(o.ir_tol / rel) / rate;
         if (need > pcg_max) { k++; break; }
       }
-      apply_factor(c, r, z, false);
-      V.dot(n, r, z, sN + 4);
-      V.xpby_ratio(n, sN + 4, sN + 2, z, p);
-      CK(cudaMemcpyAsync(sN + 2, sN + 4, sizeof(double), cudaMemcpyDeviceToDevice, c->st));
+      apply_factor_dot(c, r, sR + 1, z, rz, rz_next, beta);
+      V.cg_direction(n, beta, z, p);
+      std::swap(rz, rz_next);
     }
     c->pcg_steps += k;
     iters += k;
-    rel = residual(xx);  // true residual of the returned iterate
+    rel = residual(x);  // true residual of the returned iterate
   }
-  CK(cudaMemcpyAsync(x, xx, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
   CK(cudaGetLastError());
-  check_solve_barrier(c);
+  if (timed_out) report_solve_timeout(c);
   if (c->bwd_measure) rel = bwd;
   c->last_rel = rel;
   if (info) *info = ipm_solve_info{iters, used_pcg, rel};
@@ -1090,6 +1100,7 @@ ipm_status ipm_set_workspace(ipm_ctx *c, void *buf, size_t bytes) {
     CK(cudaGetDevice(&c->device));
     const size_t total = c->ws_need;
     layout(c, base);
+    CK(cudaMemsetAsync(c->ticket, 0, sizeof(unsigned), c->st));
     CK(cudaStreamSynchronize(c->st));
     if (c->sys) {  // the formulation's system takes the rest of the buffer
       c->ws_need = total;
@@ -1260,7 +1271,7 @@ ipm_status ipm_solve(ipm_ctx *c, const double *jv, const double *b, const double
       eval_g(c, jv, b, x);
       V.jtv(jv, lam, -1.0, wv, x, cc, c->vrd);  // rd = c + W x - J^T lambda
       if (wv) V.jtv(jv, lam, 0.0, wv, x, nullptr, c->vwx);  // W x
-      V.kkt(c->vg, s, lam, c->vrd, cc, wv ? c->vwx : nullptr, x, c->scal + 24, c->sc);
+      V.kkt(c->vg, s, lam, c->vrd, cc, wv ? c->vwx : nullptr, x, c->sc);
       IpmScalars h;
       CK(cudaMemcpyAsync(&h, c->sc, sizeof(h), cudaMemcpyDeviceToHost, c->st));
       CK(cudaStreamSynchronize(c->st));
@@ -1367,8 +1378,8 @@ ipm_status ipm_solve(ipm_ctx *c, const double *jv, const double *b, const double
           stt = direction(c, jv, b, cc, wv, x, s, lam, nullptr, c->vdx, c->vds, c->vdl, &si);
       }
       if (stt != IPM_OK) { res.status = stt; c->learned_active = false; break; }
-      V.ftb(s, c->vds, lam, c->vdl, c->scal + 32, c->sc, true);
-      V.muaff(s, c->vds, lam, c->vdl, c->scal + 34, c->sc);
+      V.ftb(s, c->vds, lam, c->vdl, c->sc, true);
+      V.muaff(s, c->vds, lam, c->vdl, c->sc);
       // corrector: w = sigma mu - ds_aff .* dl_aff
       V.corrector_target(c->vds, c->vdl, c->sc, c->vw);
       {
@@ -1412,7 +1423,7 @@ ipm_status ipm_solve(ipm_ctx *c, const double *jv, const double *b, const double
         low_step = c->factor_prec != IPM_FP64 && c->factor_prec != fb_prec;
         prev_kkt = res.kkt;
       }
-      V.ftb(s, c->vds, lam, c->vdl, c->scal + 32, c->sc, false);
+      V.ftb(s, c->vds, lam, c->vdl, c->sc, false);
       V.update(c->sc, x, c->vdx, s, c->vds, lam, c->vdl);
       {  // cost-driven escalation (cg_escalate): CG steps of this iteration's two solves
         const int64_t cg_now = c->pcg_steps + (c->sys ? c->sys->pcg_steps : 0);
@@ -1612,13 +1623,11 @@ ipm_status ipm_learned_sample(ipm_ctx *c, const double *jv, const double *x, con
     learned_diag(c->dp, jv, c->vD, c->cur_delta_p, B.diag_new, c->st);
     learned_features(c->dp, B, jv, c->vD, x, c->st);
     CK(cudaMemcpyAsync(feat, B.feat, n * kNF * sizeof(float), cudaMemcpyDeviceToDevice, c->st));
-    CK(cudaMemsetAsync(c->vc, 0, n * sizeof(double), c->st));
     for (int p = 0; p < B.P; p++) {  // w_p = L^{-1} P K P^T L^{-T} z_p
       CK(cudaMemcpyAsync(c->fsb, z + (int64_t)p * n, n * sizeof(float), cudaMemcpyDeviceToDevice, c->st));
       launch_fp32_solve(c, 2);
       V.permute_out<float>(c->fsx, nullptr, c->vz, false);
-      V.residual(jv, c->vD, c->cur_wvals, c->cur_delta_p, c->vz, c->vc, c->vq, c->vtA);
-      V.negate(n, c->vq);
+      V.kx(jv, c->vD, c->cur_wvals, c->cur_delta_p, c->vz, c->vq, c->vtA);
       V.permute_in<float>(c->vq, nullptr, c->fsa);
       launch_fp32_solve(c, 1);
       CK(cudaMemcpyAsync(w + (int64_t)p * n, c->fsb, n * sizeof(float), cudaMemcpyDeviceToDevice, c->st));
@@ -1804,7 +1813,7 @@ ipm_status nlp_solve(ipm_ctx *c, const NlpFns &F, double *x, double *s, double *
     for (it = 0; it <= o.max_iter; it++) {
       const double f = eval_at(x, c->vg);
       V.jtv(jv, lam, -1.0, nullptr, nullptr, grad, c->vrd);  // grad f - J^T lambda
-      V.kkt(c->vg, s, lam, c->vrd, zero, nullptr, x, c->scal + 24, c->sc);
+      V.kkt(c->vg, s, lam, c->vrd, zero, nullptr, x, c->sc);
       IpmScalars h;
       CK(cudaMemcpyAsync(&h, c->sc, sizeof(h), cudaMemcpyDeviceToHost, c->st));
       CK(cudaStreamSynchronize(c->st));
@@ -1896,7 +1905,7 @@ ipm_status nlp_solve(ipm_ctx *c, const NlpFns &F, double *x, double *s, double *
       if (stt != IPM_OK) { res.status = stt; break; }
       // common step from the fraction to the boundary, then backtracking on the merit
       set_sc(offsetof(IpmScalars, mu), mu);
-      V.ftb(s, c->vds, lam, c->vdl, c->scal + 32, c->sc, false);
+      V.ftb(s, c->vds, lam, c->vdl, c->sc, false);
       CK(cudaMemcpyAsync(&h, c->sc, sizeof(h), cudaMemcpyDeviceToHost, c->st));
       CK(cudaStreamSynchronize(c->st));
       double alpha = std::min(h.alpha_p, h.alpha_d);
@@ -2092,18 +2101,18 @@ ipm_status kkt_solve_noalloc(ipm_ctx *c, const double *b, double *x) {
     double *t = y + std::max<int32_t>(c->P.n, 1);
     // every entry of y and t is written before it is read (permutation in,
     // then the gathers initialise each front's update vector): nothing to clear
-    VecOps V{c->dp, c->st, partial};
+    VecOps V{c->dp, c->st, partial, reinterpret_cast<unsigned *>(scal + 8)};
+    CK(cudaMemsetAsync(scal + 8, 0, sizeof(unsigned), c->st));  // the reduction's ticket
     if (c->factor_prec == IPM_FP64) {
       V.permute_in<double>(b, nullptr, y);
       launch_solve<double, double>(c->dp, c->plan, (const double *)c->L, y, t, c->st);
       V.permute_out<double>(y, nullptr, x, false);
     } else {
-      V.absmax(c->P.n, b, scal + 1);
-      V.inv_scale(scal + 1, scal);
+      V.absmax(c->P.n, b, scal, true);  // scal[1]: its scale
       float *yf = reinterpret_cast<float *>(y), *tf = reinterpret_cast<float *>(t);
-      V.permute_in<float>(b, scal, yf);
+      V.permute_in<float>(b, scal + 1, yf);
       launch_solve<float, float>(c->dp, c->plan, (const float *)c->L, yf, tf, c->st);
-      V.permute_out<float>(yf, scal, x, false);
+      V.permute_out<float>(yf, scal + 1, x, false);
     }
     CK(cudaGetLastError());
     return IPM_OK;

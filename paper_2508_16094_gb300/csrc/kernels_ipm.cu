@@ -1,8 +1,10 @@
 // FP64 map/reduce kernels of the interior-point iteration (Sec. 1: line search
 // and barrier updates are map or reduce operations) and of the matrix-free
-// residual used by iterative refinement. Reductions are two-pass with a fixed
-// grid, so every result is bit-reproducible.
+// residual used by iterative refinement. A reduction's grid depends on the length
+// alone and its partial results are combined in block order, so every result is
+// bit-reproducible.
 #include <cfloat>
+#include <type_traits>
 
 #include "ipm_kernels.h"
 
@@ -12,55 +14,73 @@ namespace {
 
 constexpr int kRedBlock = 256;
 
-__device__ __forceinline__ double red_combine(double a, double b, int op) {
-  return op == RED_SUM ? a + b : (op == RED_MAX ? fmax(a, b) : fmin(a, b));
+// |v| on the integer pipe, NaN as zero (the maxima skip NaN): an FP64 comparison
+// occupies GB300's FP64 unit as long as a multiply-add.
+__device__ __forceinline__ double abs_or_zero(double v) {
+  const long long b = __double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFll;
+  return b > 0x7FF0000000000000ll ? 0.0 : __longlong_as_double(b);
 }
-__device__ __forceinline__ double red_identity(int op) {
-  return op == RED_SUM ? 0.0 : (op == RED_MAX ? -DBL_MAX : DBL_MAX);
+__device__ __forceinline__ double max_nonneg(double a, double b) {
+  return __double_as_longlong(a) > __double_as_longlong(b) ? a : b;
 }
+// RED_MAX combines values >= 0 (identity 0)
+template <int OP> __device__ __forceinline__ double red_combine(double a, double b) {
+  return OP == RED_SUM ? a + b : (OP == RED_MAX ? max_nonneg(a, b) : fmin(a, b));
+}
+template <int OP> __device__ __forceinline__ double red_identity() { return OP == RED_MIN ? DBL_MAX : 0.0; }
 
-// Block-level reduction of NS slots; thread 0 writes partial[blockIdx.x * NS + k].
-template <int NS>
-__device__ void block_reduce_store(double (&v)[NS], const RedOps &ops, double *partial) {
-  __shared__ double sh[NS][kRedBlock / 32];
+template <int OP> __device__ __forceinline__ double warp_reduce(double x, int from) {
+  for (int o = from; o > 0; o >>= 1) x = red_combine<OP>(x, __shfl_xor_sync(0xffffffffu, x, o));
+  return x;
+}
+// Reduction over a block, the result in thread 0.
+template <int OP> __device__ __forceinline__ double block_reduce(double x, double *sh) {
   const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
-#pragma unroll
-  for (int k = 0; k < NS; k++) {
-    double x = v[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x = red_combine(x, __shfl_xor_sync(0xffffffffu, x, o), ops.op[k]);
-    if (lane == 0) sh[k][warp] = x;
-  }
+  x = warp_reduce<OP>(x, 16);
+  if (lane == 0) sh[warp] = x;
   __syncthreads();
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int k = 0; k < NS; k++) {
-      double x = sh[k][0];
-      for (int w = 1; w < kRedBlock / 32; w++) x = red_combine(x, sh[k][w], ops.op[k]);
-      partial[blockIdx.x * NS + k] = x;
-    }
-  }
+  if (warp == 0) x = warp_reduce<OP>(lane < kRedBlock / 32 ? sh[lane] : red_identity<OP>(), 4);
+  return x;
 }
 
-template <int NS>
-__global__ void final_reduce_kernel(const double *partial, int nblocks, RedOps ops, double *out) {
-  double v[NS];
-#pragma unroll
-  for (int k = 0; k < NS; k++) v[k] = red_identity(ops.op[k]);
-  for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-#pragma unroll
-    for (int k = 0; k < NS; k++) v[k] = red_combine(v[k], partial[b * NS + k], ops.op[k]);
-  __shared__ double sh[NS][kRedBlock];
-#pragma unroll
-  for (int k = 0; k < NS; k++) sh[k][threadIdx.x] = v[k];
-  __syncthreads();
+// Reduction over the grid in one launch: every block stores its partial results,
+// the last one to finish combines them (in block order, so results do not
+// depend on which block that is) and calls fin(results) on one thread. `ticket`
+// is zero before the launch and zero again after it. A second launch whose one
+// thread added 256 values, as before, took 17 us.
+template <int... OPS, typename Fin>
+__device__ __forceinline__ void grid_reduce(double (&v)[sizeof...(OPS)], double *partial, unsigned *ticket,
+                                            Fin fin) {
+  constexpr int NS = sizeof...(OPS);
+  __shared__ double sh[NS][kRedBlock / 32];
+  __shared__ bool last;
+  {
+    int k = 0;
+    ((v[k] = block_reduce<OPS>(v[k], sh[k]), k++), ...);
+  }
   if (threadIdx.x == 0) {
 #pragma unroll
-    for (int k = 0; k < NS; k++) {
-      double x = sh[k][0];
-      for (int t = 1; t < kRedBlock; t++) x = red_combine(x, sh[k][t], ops.op[k]);
-      out[k] = x;
-    }
+    for (int k = 0; k < NS; k++) partial[blockIdx.x * NS + k] = v[k];
+    __threadfence();
+    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  {
+    int k = 0;
+    auto one = [&](auto op) {
+      constexpr int OP = decltype(op)::value;
+      double x = red_identity<OP>();
+      for (int b = threadIdx.x; b < (int)gridDim.x; b += kRedBlock)
+        x = red_combine<OP>(x, __ldcg(partial + b * NS + k));
+      v[k] = block_reduce<OP>(x, sh[k]);
+      k++;
+    };
+    (one(std::integral_constant<int, OPS>{}), ...);
+  }
+  if (threadIdx.x == 0) {
+    fin(v);
+    *ticket = 0u;
   }
 }
 
@@ -68,6 +88,11 @@ __global__ void final_reduce_kernel(const double *partial, int nblocks, RedOps o
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (n);             \
        i += (int64_t)gridDim.x * blockDim.x)
 
+// Blocks of a reduction over n values: at most kRedBlocks, a function of n alone.
+inline int red_grid(int64_t n) {
+  const int64_t g = (n + kRedBlock - 1) / kRedBlock;
+  return (int)(g < 1 ? 1 : (g > kRedBlocks ? kRedBlocks : g));
+}
 inline int grid_of(int64_t n) {
   int64_t g = (n + 255) / 256;
   return (int)(g < 1 ? 1 : (g > 152 * 16 ? 152 * 16 : g));
@@ -132,25 +157,62 @@ __global__ void resid_rows_kernel(DevPlan dp, const double *__restrict__ jv,
     tA[r] = D[r] * a;
   }
 }
-__global__ void resid_cols_kernel(DevPlan dp, const double *__restrict__ jv,
-                                  const double *__restrict__ D, const double *__restrict__ wv,
-                                  double delta_p, const double *__restrict__ tA,
-                                  const double *__restrict__ x, const double *__restrict__ b,
-                                  double *__restrict__ r) {
-  GRID_STRIDE(j, dp.n) {
-    double a = 0.0;
-    for (int64_t t = dp.jtp[j]; t < dp.jtp[j + 1]; t++) {
-      const int32_t e = dp.jtpos[t];
-      a = fma(jv[e], tA[dp.jrow[e]], a);
-    }
-    double d = delta_p;
-    if (dp.lpos[j] >= 0) d += D[dp.lpos[j]];
-    if (dp.upos[j] >= 0) d += D[dp.upos[j]];
-    a = fma(d, x[j], a);
-    if (wv)
-      for (int64_t e = dp.wfp[j]; e < dp.wfp[j + 1]; e++) a = fma(wv[dp.wfsrc[e]], x[dp.wfi[e]], a);
-    r[j] = b[j] - a;
+// (K x)_j from tA = D_A J x
+__device__ __forceinline__ double kx_col(const DevPlan &dp, const double *jv, const double *D,
+                                         const double *wv, double delta_p, const double *tA,
+                                         const double *x, int64_t j) {
+  double a = 0.0;
+  for (int64_t t = dp.jtp[j]; t < dp.jtp[j + 1]; t++) {
+    const int32_t e = dp.jtpos[t];
+    a = fma(jv[e], tA[dp.jrow[e]], a);
   }
+  double d = delta_p;
+  if (dp.lpos[j] >= 0) d += D[dp.lpos[j]];
+  if (dp.upos[j] >= 0) d += D[dp.upos[j]];
+  a = fma(d, x[j], a);
+  if (wv)
+    for (int64_t e = dp.wfp[j]; e < dp.wfp[j + 1]; e++) a = fma(wv[dp.wfsrc[e]], x[dp.wfi[e]], a);
+  return a;
+}
+// 1 / m, the scale that keeps a right-hand side of largest entry m in FP32's range
+__device__ __forceinline__ double scale_of(double m) { return (m > 0.0 && m < DBL_MAX) ? 1.0 / m : 1.0; }
+
+// r = b - K x, and its largest entry and scale (`flag`: a status word copied out beside them)
+__global__ void __launch_bounds__(kRedBlock) resid_cols_kernel(
+    DevPlan dp, const double *__restrict__ jv, const double *__restrict__ D, const double *__restrict__ wv,
+    double delta_p, const double *__restrict__ tA, const double *__restrict__ x,
+    const double *__restrict__ b, double *__restrict__ r, const int32_t *flag, double *out,
+    double *partial, unsigned *ticket) {
+  double m[1] = {0.0};
+  GRID_STRIDE(j, dp.n) {
+    const double v = b[j] - kx_col(dp, jv, D, wv, delta_p, tA, x, j);
+    r[j] = v;
+    m[0] = max_nonneg(m[0], abs_or_zero(v));
+  }
+  grid_reduce<RED_MAX>(m, partial, ticket, [&](double (&v)[1]) {
+    out[0] = v[0];
+    out[1] = scale_of(v[0]);
+    if (flag) out[2] = (double)*flag;
+  });
+}
+// q = K p, p . q and the step length alpha = rz / (p . q) (0 if that is 0)
+__global__ void __launch_bounds__(kRedBlock) kp_dot_kernel(
+    DevPlan dp, const double *__restrict__ jv, const double *__restrict__ D, const double *__restrict__ wv,
+    double delta_p, const double *__restrict__ tA, const double *__restrict__ p, double *__restrict__ q,
+    const double *rz, double *alpha, double *partial, unsigned *ticket) {
+  double s[1] = {0.0};
+  GRID_STRIDE(j, dp.n) {
+    const double v = kx_col(dp, jv, D, wv, delta_p, tA, p, j);
+    q[j] = v;
+    s[0] = fma(p[j], v, s[0]);
+  }
+  grid_reduce<RED_SUM>(s, partial, ticket,
+                       [&](double (&v)[1]) { alpha[0] = v[0] != 0.0 ? rz[0] / v[0] : 0.0; });
+}
+__global__ void kx_kernel(DevPlan dp, const double *__restrict__ jv, const double *__restrict__ D,
+                          const double *__restrict__ wv, double delta_p, const double *__restrict__ tA,
+                          const double *__restrict__ x, double *__restrict__ q) {
+  GRID_STRIDE(j, dp.n) q[j] = kx_col(dp, jv, D, wv, delta_p, tA, x, j);
 }
 
 // row sums of |K|: |W| 1 + |J_A|^T D_A |J_A| 1 + D_l + D_u + delta_p (D >= 0)
@@ -200,70 +262,102 @@ __global__ void permute_out_kernel(int32_t n, const int32_t *__restrict__ perm,
   }
 }
 
-// ---- reductions -----------------------------------------------------------
-__global__ void absmax_kernel(int64_t n, const double *__restrict__ v, double *partial) {
-  double a[1] = {0.0};
-  GRID_STRIDE(i, n) a[0] = fmax(a[0], fabs(v[i]));
-  RedOps ops{{RED_MAX}};
-  block_reduce_store<1>(a, ops, partial);
-}
-__global__ void dot_kernel(int64_t n, const double *__restrict__ a, const double *__restrict__ b,
-                           double *partial) {
-  double v[1] = {0.0};
-  GRID_STRIDE(i, n) v[0] = fma(a[i], b[i], v[0]);
-  RedOps ops{{RED_SUM}};
-  block_reduce_store<1>(v, ops, partial);
-}
-__global__ void inv_scale_kernel(const double *absmax, double *scale) {
-  // scale = 1 / max|v| (1 if zero): keeps low-precision right-hand sides in range
-  const double m = absmax[0];
-  scale[0] = (m > 0.0 && m < DBL_MAX) ? 1.0 / m : 1.0;
+// z = P^T y / scale, r . z, and beta = (r . z) / rz_old (without it: only r . z)
+template <typename V>
+__global__ void __launch_bounds__(kRedBlock) permute_out_dot_kernel(
+    int32_t n, const int32_t *__restrict__ perm, const V *__restrict__ y, const double *__restrict__ scale,
+    const double *__restrict__ r, double *__restrict__ z, const double *rz_old, double *rz, double *beta,
+    double *partial, unsigned *ticket) {
+  const double s = scale ? 1.0 / scale[0] : 1.0;
+  double d[1] = {0.0};
+  GRID_STRIDE(k, n) {
+    const int32_t i = perm[k];
+    const double v = (double)y[k] * s;
+    z[i] = v;
+    d[0] = fma(r[i], v, d[0]);
+  }
+  grid_reduce<RED_SUM>(d, partial, ticket, [&](double (&v)[1]) {
+    if (rz_old) beta[0] = rz_old[0] != 0.0 ? v[0] / rz_old[0] : 0.0;
+    rz[0] = v[0];
+  });
 }
 
-// KKT quantities: slots 0 sum s.lambda, 1 max|g - s|, 2 max|s.lambda|, 3 max|rd|, 4 f(x)
-__global__ void kkt_reduce_kernel(DevPlan dp, const double *__restrict__ g,
-                                  const double *__restrict__ s, const double *__restrict__ lam,
-                                  const double *__restrict__ rd, const double *__restrict__ c,
-                                  const double *__restrict__ wx, const double *__restrict__ x,
-                                  double *partial) {
+// ---- reductions -----------------------------------------------------------
+// out[0] = max |v|, out[1] = its scale (see scale_of)
+__global__ void __launch_bounds__(kRedBlock) absmax_kernel(int64_t n, const double *__restrict__ v, double *out,
+                                                           int with_scale, double *partial, unsigned *ticket) {
+  double a[1] = {0.0};
+  GRID_STRIDE(i, n) a[0] = max_nonneg(a[0], abs_or_zero(v[i]));
+  grid_reduce<RED_MAX>(a, partial, ticket, [&](double (&m)[1]) {
+    out[0] = m[0];
+    if (with_scale) out[1] = scale_of(m[0]);
+  });
+}
+__global__ void __launch_bounds__(kRedBlock) dot_kernel(int64_t n, const double *__restrict__ a,
+                                                        const double *__restrict__ b, double *out,
+                                                        double *partial, unsigned *ticket) {
+  double v[1] = {0.0};
+  GRID_STRIDE(i, n) v[0] = fma(a[i], b[i], v[0]);
+  grid_reduce<RED_SUM>(v, partial, ticket, [&](double (&d)[1]) { out[0] = d[0]; });
+}
+
+// KKT quantities: sum s.lambda, max|g - s|, max|s.lambda|, max|rd|, f(x)
+__global__ void __launch_bounds__(kRedBlock) kkt_reduce_kernel(
+    DevPlan dp, const double *__restrict__ g, const double *__restrict__ s, const double *__restrict__ lam,
+    const double *__restrict__ rd, const double *__restrict__ c, const double *__restrict__ wx,
+    const double *__restrict__ x, IpmScalars *sc, double *partial, unsigned *ticket) {
   double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
   GRID_STRIDE(i, dp.mt + dp.n) {
     if (i < dp.mt) {
       const double sl = s[i] * lam[i];
       v[0] += sl;
-      v[1] = fmax(v[1], fabs(g[i] - s[i]));
-      v[2] = fmax(v[2], fabs(sl));
+      v[1] = max_nonneg(v[1], abs_or_zero(g[i] - s[i]));
+      v[2] = max_nonneg(v[2], abs_or_zero(sl));
     } else {
       const int64_t j = i - dp.mt;
-      v[3] = fmax(v[3], fabs(rd[j]));
+      v[3] = max_nonneg(v[3], abs_or_zero(rd[j]));
       v[4] = fma(c[j] + (wx ? 0.5 * wx[j] : 0.0), x[j], v[4]);
     }
   }
-  RedOps ops{{RED_SUM, RED_MAX, RED_MAX, RED_MAX, RED_SUM}};
-  block_reduce_store<5>(v, ops, partial);
+  const int64_t mt = dp.mt;
+  grid_reduce<RED_SUM, RED_MAX, RED_MAX, RED_MAX, RED_SUM>(v, partial, ticket, [&](double (&red)[5]) {
+    sc->mu = red[0] / (double)(mt > 0 ? mt : 1);
+    sc->primal_inf = red[1];
+    sc->compl_inf = red[2];
+    sc->dual_inf = red[3];
+    sc->fx = red[4];
+  });
 }
 
-// fraction to the boundary: slot 0 min over ds<0 of -s/ds, slot 1 min over dl<0 of -lam/dl
-__global__ void ftb_kernel(int64_t mt, const double *__restrict__ s, const double *__restrict__ ds,
-                           const double *__restrict__ lam, const double *__restrict__ dl,
-                           double *partial) {
+// fraction to the boundary: min over ds<0 of -s/ds, min over dl<0 of -lam/dl
+__global__ void __launch_bounds__(kRedBlock) ftb_kernel(
+    int64_t mt, const double *__restrict__ s, const double *__restrict__ ds, const double *__restrict__ lam,
+    const double *__restrict__ dl, IpmScalars *sc, int affine, double *partial, unsigned *ticket) {
   double v[2] = {DBL_MAX, DBL_MAX};
   GRID_STRIDE(i, mt) {
     if (ds[i] < 0.0) v[0] = fmin(v[0], -s[i] / ds[i]);
     if (dl[i] < 0.0) v[1] = fmin(v[1], -lam[i] / dl[i]);
   }
-  RedOps ops{{RED_MIN, RED_MIN}};
-  block_reduce_store<2>(v, ops, partial);
+  grid_reduce<RED_MIN, RED_MIN>(v, partial, ticket, [&](double (&red)[2]) {
+    if (affine) {
+      sc->alpha_aff_p = fmin(1.0, red[0]);
+      sc->alpha_aff_d = fmin(1.0, red[1]);
+    } else {
+      const double tau = fmax(0.99, 1.0 - sc->mu);
+      sc->alpha_p = fmin(1.0, tau * red[0]);
+      sc->alpha_d = fmin(1.0, tau * red[1]);
+    }
+  });
 }
 
-__global__ void muaff_kernel(int64_t mt, const double *__restrict__ s, const double *__restrict__ ds,
-                             const double *__restrict__ lam, const double *__restrict__ dl,
-                             const IpmScalars *sc, double *partial) {
+__global__ void __launch_bounds__(kRedBlock) muaff_kernel(
+    int64_t mt, const double *__restrict__ s, const double *__restrict__ ds, const double *__restrict__ lam,
+    const double *__restrict__ dl, IpmScalars *sc, double *partial, unsigned *ticket) {
   const double ap = sc->alpha_aff_p, ad = sc->alpha_aff_d;
   double v[1] = {0.0};
   GRID_STRIDE(i, mt) v[0] = fma(fma(ap, ds[i], s[i]), fma(ad, dl[i], lam[i]), v[0]);
-  RedOps ops{{RED_SUM}};
-  block_reduce_store<1>(v, ops, partial);
+  grid_reduce<RED_SUM>(v, partial, ticket,
+                       [&](double (&red)[1]) { sc->mu_aff = red[0] / (double)(mt > 0 ? mt : 1); });
 }
 
 // ---- elementwise steps ---------------------------------------------------
@@ -331,38 +425,29 @@ __global__ void update_kernel(int64_t n, int64_t mt, const IpmScalars *sc, doubl
     }
   }
 }
-// scalar bookkeeping after reductions
-__global__ void finish_kkt_kernel(const double *red, int64_t mt, IpmScalars *sc) {
-  sc->mu = red[0] / (double)(mt > 0 ? mt : 1);
-  sc->primal_inf = red[1];
-  sc->compl_inf = red[2];
-  sc->dual_inf = red[3];
-  sc->fx = red[4];
-}
-__global__ void finish_ftb_kernel(const double *red, IpmScalars *sc, int affine) {
-  if (affine) {
-    sc->alpha_aff_p = fmin(1.0, red[0]);
-    sc->alpha_aff_d = fmin(1.0, red[1]);
-  } else {
-    const double tau = fmax(0.99, 1.0 - sc->mu);
-    sc->alpha_p = fmin(1.0, tau * red[0]);
-    sc->alpha_d = fmin(1.0, tau * red[1]);
-  }
-}
-__global__ void finish_muaff_kernel(const double *red, int64_t mt, IpmScalars *sc) {
-  sc->mu_aff = red[0] / (double)(mt > 0 ? mt : 1);
-}
-
 // ---- vector updates used by refinement / PCG ------------------------------
-__global__ void axpy_dev_kernel(int64_t n, const double *alpha_num, const double *alpha_den,
-                                int sign, const double *__restrict__ xv, double *__restrict__ yv) {
-  const double a = (alpha_den[0] != 0.0) ? sign * alpha_num[0] / alpha_den[0] : 0.0;
-  GRID_STRIDE(i, n) yv[i] = fma(a, xv[i], yv[i]);
+// x += alpha p, r -= alpha q, and the largest entry of the new r with its scale
+__global__ void __launch_bounds__(kRedBlock) cg_step_kernel(
+    int64_t n, const double *alpha, const double *__restrict__ p, const double *__restrict__ q,
+    double *__restrict__ x, double *__restrict__ r, double *out, double *partial, unsigned *ticket) {
+  const double a = alpha[0];
+  double m[1] = {0.0};
+  GRID_STRIDE(i, n) {
+    x[i] = fma(a, p[i], x[i]);
+    const double v = fma(-a, q[i], r[i]);
+    r[i] = v;
+    m[0] = max_nonneg(m[0], abs_or_zero(v));
+  }
+  grid_reduce<RED_MAX>(m, partial, ticket, [&](double (&v)[1]) {
+    out[0] = v[0];
+    out[1] = scale_of(v[0]);
+  });
 }
-__global__ void xpby_dev_kernel(int64_t n, const double *num, const double *den,
-                                const double *__restrict__ xv, double *__restrict__ p) {
-  const double b = (den[0] != 0.0) ? num[0] / den[0] : 0.0;
-  GRID_STRIDE(i, n) p[i] = fma(b, p[i], xv[i]);
+// p = z + beta p
+__global__ void cg_direction_kernel(int64_t n, const double *beta, const double *__restrict__ z,
+                                    double *__restrict__ p) {
+  const double b = beta[0];
+  GRID_STRIDE(i, n) p[i] = fma(b, p[i], z[i]);
 }
 
 }  // namespace
@@ -379,29 +464,16 @@ cudaError_t preload_vec_kernels() {
   q((const void *)permute_out_kernel<double>);
   q((const void *)permute_out_kernel<float>);
   q((const void *)absmax_kernel);
-  q((const void *)inv_scale_kernel);
-  q((const void *)final_reduce_kernel<1>);
   return e;
 }
 
-void VecOps::reduce_final(int ns, const RedOps &ops, double *out) const {
-  switch (ns) {
-    case 1: { note_launch(); final_reduce_kernel<1><<<1, kRedBlock, 0, st>>>(partial, kRedBlocks, ops, out); } break;
-    case 2: { note_launch(); final_reduce_kernel<2><<<1, kRedBlock, 0, st>>>(partial, kRedBlocks, ops, out); } break;
-    case 5: { note_launch(); final_reduce_kernel<5><<<1, kRedBlock, 0, st>>>(partial, kRedBlocks, ops, out); } break;
-    default: break;
-  }
-}
-void VecOps::absmax(int64_t n, const double *v, double *out) const {
-  { note_launch(); absmax_kernel<<<kRedBlocks, kRedBlock, 0, st>>>(n, v, partial); }
-  reduce_final(1, RedOps{{RED_MAX}}, out);
+void VecOps::absmax(int64_t n, const double *v, double *out, bool with_scale) const {
+  note_launch();
+  absmax_kernel<<<red_grid(n), kRedBlock, 0, st>>>(n, v, out, with_scale ? 1 : 0, partial, ticket);
 }
 void VecOps::dot(int64_t n, const double *a, const double *b, double *out) const {
-  { note_launch(); dot_kernel<<<kRedBlocks, kRedBlock, 0, st>>>(n, a, b, partial); }
-  reduce_final(1, RedOps{{RED_SUM}}, out);
-}
-void VecOps::inv_scale(const double *absmax_v, double *scale) const {
-  { note_launch(); inv_scale_kernel<<<1, 1, 0, st>>>(absmax_v, scale); }
+  note_launch();
+  dot_kernel<<<red_grid(n), kRedBlock, 0, st>>>(n, a, b, out, partial, ticket);
 }
 void VecOps::jv(const double *jvals, const double *x, double *out) const {
   if (dp.m > 0) { note_launch(); jv_kernel<<<grid_of(dp.m), 256, 0, st>>>(dp, jvals, x, out); }
@@ -416,10 +488,38 @@ void VecOps::jtv(const double *jvals, const double *v, double sgn, const double 
 void VecOps::init_slack(const double *gv, double *s, double *lam) const {
   if (dp.mt > 0) { note_launch(); init_slack_kernel<<<grid_of(dp.mt), 256, 0, st>>>(dp.mt, gv, s, lam); }
 }
-void VecOps::residual(const double *jvals, const double *D, const double *wv, double delta_p,
-                      const double *x, const double *b, double *r, double *tA) const {
+void VecOps::rows_product(const double *jvals, const double *D, const double *x, double *tA) const {
   if (dp.m > 0) { note_launch(); resid_rows_kernel<<<grid_of(dp.m), 256, 0, st>>>(dp, jvals, D, x, tA); }
-  { note_launch(); resid_cols_kernel<<<grid_of(dp.n), 256, 0, st>>>(dp, jvals, D, wv, delta_p, tA, x, b, r); }
+}
+void VecOps::residual(const double *jvals, const double *D, const double *wv, double delta_p,
+                      const double *x, const double *b, double *r, double *tA, double *out,
+                      const int32_t *flag) const {
+  rows_product(jvals, D, x, tA);
+  note_launch();
+  resid_cols_kernel<<<red_grid(dp.n), kRedBlock, 0, st>>>(dp, jvals, D, wv, delta_p, tA, x, b, r, flag, out,
+                                                          partial, ticket);
+}
+void VecOps::kx(const double *jvals, const double *D, const double *wv, double delta_p, const double *x,
+                double *q, double *tA) const {
+  rows_product(jvals, D, x, tA);
+  note_launch();
+  kx_kernel<<<grid_of(dp.n), 256, 0, st>>>(dp, jvals, D, wv, delta_p, tA, x, q);
+}
+void VecOps::kp_dot(const double *jvals, const double *D, const double *wv, double delta_p, const double *p,
+                    double *q, double *tA, const double *rz, double *alpha) const {
+  rows_product(jvals, D, p, tA);
+  note_launch();
+  kp_dot_kernel<<<red_grid(dp.n), kRedBlock, 0, st>>>(dp, jvals, D, wv, delta_p, tA, p, q, rz, alpha, partial,
+                                                      ticket);
+}
+void VecOps::cg_step(int64_t n, const double *alpha, const double *p, const double *q, double *x, double *r,
+                     double *out) const {
+  note_launch();
+  cg_step_kernel<<<red_grid(n), kRedBlock, 0, st>>>(n, alpha, p, q, x, r, out, partial, ticket);
+}
+void VecOps::cg_direction(int64_t n, const double *beta, const double *z, double *p) const {
+  note_launch();
+  cg_direction_kernel<<<grid_of(n), 256, 0, st>>>(n, beta, z, p);
 }
 void VecOps::abs_rowsum(const double *jvals, const double *D, const double *wv, double delta_p,
                         double *out, double *tA) const {
@@ -434,17 +534,26 @@ template <typename V>
 void VecOps::permute_out(const V *y, const double *scale, double *x, bool accumulate) const {
   { note_launch(); permute_out_kernel<V><<<grid_of(dp.n), 256, 0, st>>>(dp.n, dp.perm, y, scale, x, accumulate); }
 }
+template <typename V>
+void VecOps::permute_out_dot(const V *y, const double *scale, const double *r, double *z, const double *rz_old,
+                             double *rz, double *beta) const {
+  note_launch();
+  permute_out_dot_kernel<V><<<red_grid(dp.n), kRedBlock, 0, st>>>(dp.n, dp.perm, y, scale, r, z, rz_old, rz, beta,
+                                                                  partial, ticket);
+}
+template void VecOps::permute_out_dot<double>(const double *, const double *, const double *, double *,
+                                              const double *, double *, double *) const;
+template void VecOps::permute_out_dot<float>(const float *, const double *, const double *, double *,
+                                             const double *, double *, double *) const;
 template void VecOps::permute_in<double>(const double *, const double *, double *) const;
 template void VecOps::permute_in<float>(const double *, const double *, float *) const;
 template void VecOps::permute_out<double>(const double *, const double *, double *, bool) const;
 template void VecOps::permute_out<float>(const float *, const double *, double *, bool) const;
 
 void VecOps::kkt(const double *g, const double *s, const double *lam, const double *rd,
-                 const double *c, const double *wx, const double *x, double *red5,
-                 IpmScalars *sc) const {
-  { note_launch(); kkt_reduce_kernel<<<kRedBlocks, kRedBlock, 0, st>>>(dp, g, s, lam, rd, c, wx, x, partial); }
-  reduce_final(5, RedOps{{RED_SUM, RED_MAX, RED_MAX, RED_MAX, RED_SUM}}, red5);
-  { note_launch(); finish_kkt_kernel<<<1, 1, 0, st>>>(red5, dp.mt, sc); }
+                 const double *c, const double *wx, const double *x, IpmScalars *sc) const {
+  note_launch();
+  kkt_reduce_kernel<<<red_grid(dp.mt + dp.n), kRedBlock, 0, st>>>(dp, g, s, lam, rd, c, wx, x, sc, partial, ticket);
 }
 void VecOps::g(const double *jx, const double *x, const double *b, const double *l,
                const double *u, double *gout) const {
@@ -465,17 +574,15 @@ void VecOps::recover(const double *D, const double *gv, const double *w, const d
   if (dp.mt > 0)
     { note_launch(); recover_kernel<<<grid_of(dp.mt), 256, 0, st>>>(dp.mt, D, gv, w, s, lam, jdx, ds, dl); }
 }
-void VecOps::ftb(const double *s, const double *ds, const double *lam, const double *dl,
-                 double *red2, IpmScalars *sc, bool affine) const {
-  { note_launch(); ftb_kernel<<<kRedBlocks, kRedBlock, 0, st>>>(dp.mt, s, ds, lam, dl, partial); }
-  reduce_final(2, RedOps{{RED_MIN, RED_MIN}}, red2);
-  { note_launch(); finish_ftb_kernel<<<1, 1, 0, st>>>(red2, sc, affine ? 1 : 0); }
+void VecOps::ftb(const double *s, const double *ds, const double *lam, const double *dl, IpmScalars *sc,
+                 bool affine) const {
+  note_launch();
+  ftb_kernel<<<red_grid(dp.mt), kRedBlock, 0, st>>>(dp.mt, s, ds, lam, dl, sc, affine ? 1 : 0, partial, ticket);
 }
 void VecOps::muaff(const double *s, const double *ds, const double *lam, const double *dl,
-                   double *red1, IpmScalars *sc) const {
-  { note_launch(); muaff_kernel<<<kRedBlocks, kRedBlock, 0, st>>>(dp.mt, s, ds, lam, dl, sc, partial); }
-  reduce_final(1, RedOps{{RED_SUM}}, red1);
-  { note_launch(); finish_muaff_kernel<<<1, 1, 0, st>>>(red1, dp.mt, sc); }
+                   IpmScalars *sc) const {
+  note_launch();
+  muaff_kernel<<<red_grid(dp.mt), kRedBlock, 0, st>>>(dp.mt, s, ds, lam, dl, sc, partial, ticket);
 }
 void VecOps::corrector_target(const double *ds, const double *dl, IpmScalars *sc,
                               double *w) const {
@@ -484,14 +591,6 @@ void VecOps::corrector_target(const double *ds, const double *dl, IpmScalars *sc
 void VecOps::update(const IpmScalars *sc, double *x, const double *dx, double *s,
                     const double *ds, double *lam, const double *dl) const {
   { note_launch(); update_kernel<<<grid_of(dp.n + dp.mt), 256, 0, st>>>(dp.n, dp.mt, sc, x, dx, s, ds, lam, dl); }
-}
-void VecOps::axpy_ratio(int64_t n, const double *num, const double *den, int sign,
-                        const double *x, double *y) const {
-  { note_launch(); axpy_dev_kernel<<<grid_of(n), 256, 0, st>>>(n, num, den, sign, x, y); }
-}
-void VecOps::xpby_ratio(int64_t n, const double *num, const double *den, const double *x,
-                        double *p) const {
-  { note_launch(); xpby_dev_kernel<<<grid_of(n), 256, 0, st>>>(n, num, den, x, p); }
 }
 
 }  // namespace gipm
