@@ -149,6 +149,25 @@ __global__ void kadd_kernel(DevPlan dp, int64_t q0, int64_t q1, const double *__
   }
 }
 
+// 16 bytes as one load or store (a copy of the struct is split into its members).
+template <typename T> struct Vec16 {
+  T v[16 / sizeof(T)];
+};
+__device__ __forceinline__ Vec16<float> ld16(const float *p) {
+  const float4 f = *reinterpret_cast<const float4 *>(p);
+  return Vec16<float>{{f.x, f.y, f.z, f.w}};
+}
+__device__ __forceinline__ Vec16<double> ld16(const double *p) {
+  const double2 f = *reinterpret_cast<const double2 *>(p);
+  return Vec16<double>{{f.x, f.y}};
+}
+__device__ __forceinline__ void st16(float *p, const Vec16<float> &v) {
+  *reinterpret_cast<float4 *>(p) = make_float4(v.v[0], v.v[1], v.v[2], v.v[3]);
+}
+__device__ __forceinline__ void st16(double *p, const Vec16<double> &v) {
+  *reinterpret_cast<double2 *>(p) = make_double2(v.v[0], v.v[1]);
+}
+
 // Trailing update of a level's fronts by the finished columns [k0, k1) (C -= A S
 // B^T, A and B rows of a front's panel, S = diag(pivot signs), nullptr: I): one
 // TS x TS tile of the columns [min(k1, ncol), min(clim, ncol)) of a panel, or,
@@ -196,7 +215,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 3 : 2) upd_kernel(DevPlan
   }
   const int8_t *sk = dp.sgn ? dp.sgn + F.first + k0 : nullptr;
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-  struct __align__(16) V { T v[VW]; };
+  using V = Vec16<T>;
   V reg[PER];
   auto load = [&](int kc) {  // chunk [kc, kc + BK) of both operands (zero past K, M, N)
 #pragma unroll
@@ -207,7 +226,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 3 : 2) upd_kernel(DevPlan
 #pragma unroll
       for (int h = 0; h < VW; h++) x.v[h] = T(0);
       if (r < (isb ? N : M) && kk < K) {
-        x = *reinterpret_cast<const V *>((isb ? B : A) + (int64_t)r * F.ld + kk);
+        x = ld16((isb ? B : A) + (int64_t)r * F.ld + kk);
 #pragma unroll
         for (int h = 0; h < VW; h++) {
           if (kk + h >= K) x.v[h] = T(0);
@@ -233,7 +252,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 3 : 2) upd_kernel(DevPlan
     for (int q = 0; q < PER; q++) {
       const bool isb = q >= PER / 2;
       const int e = tid + NT * (isb ? q - PER / 2 : q);
-      *reinterpret_cast<V *>((isb ? sB : sA) + (e / NV) * LD + VW * (e % NV)) = reg[q];
+      st16((isb ? sB : sA) + (e / NV) * LD + VW * (e % NV), reg[q]);
     }
     __syncthreads();
     if (sizeof(T) == 4 && kc + BK < K) load(kc + BK);  // (FP64: one chunk)
@@ -242,9 +261,9 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 3 : 2) upd_kernel(DevPlan
     for (int kk = 0; kk < kn; kk += VW) {
       V a[MI], b[NJ];
 #pragma unroll
-      for (int i = 0; i < MI; i++) a[i] = *reinterpret_cast<const V *>(sA + (ty + TY * i) * LD + kk);
+      for (int i = 0; i < MI; i++) a[i] = ld16(sA + (ty + TY * i) * LD + kk);
 #pragma unroll
-      for (int j = 0; j < NJ; j++) b[j] = *reinterpret_cast<const V *>(sB + (tx + 16 * j) * LD + kk);
+      for (int j = 0; j < NJ; j++) b[j] = ld16(sB + (tx + 16 * j) * LD + kk);
 #pragma unroll
       for (int h = 0; h < VW; h++)
 #pragma unroll
@@ -266,12 +285,27 @@ template <typename T> __device__ __forceinline__ T big_pivot();
 template <> __device__ __forceinline__ float big_pivot<float>() { return 1e30f; }
 template <> __device__ __forceinline__ double big_pivot<double>() { return 1e64; }
 
-// 1 / sqrt(d) for d > 0: the FP32 estimate and one third-order step,
-// r (1 + e/2 + 3 e^2 / 8) with e = 1 - d r^2 (|e| < 2^-21: the step's own error
-// is below 2^-62). Values outside FP32's normal range take the library functions.
+// Out of line, so that the division is not evaluated beside the usual path.
+template <typename T> __device__ __noinline__ T slow_div(T a, T b) { return a / b; }
+
+// Estimates of 1 / d and 1 / sqrt(d) in FP32 for a double d > 0 within FP32's
+// normal range (in_fp32), converted by moving bits: GB300's FP64 unit takes about
+// 90 cycles for a conversion or a comparison, as for a multiply-add.
+__device__ __forceinline__ bool in_fp32(double d) {  // 2^-119 <= d < 2^120
+  return ((unsigned)__double2hiint(d) >> 20) - 904u < 239u;  // (false for d < 0 and NaN)
+}
+__device__ __forceinline__ float low_float(double d) {  // d cut to 24 bits
+  return __int_as_float(((__double2hiint(d) - (896 << 20)) << 3) | ((unsigned)__double2loint(d) >> 29));
+}
+__device__ __forceinline__ double widen(float f) {  // normal f > 0
+  const int b = __float_as_int(f);
+  return __hiloint2double((b >> 3) + (896 << 20), b << 29);
+}
+// 1 / sqrt(d): one third-order step from the estimate, r (1 + e/2 + 3 e^2 / 8) with e =
+// 1 - d r^2 (|e| < 2^-20: the step's own error is below 2^-58).
 __device__ __forceinline__ double inv_sqrt(double d) {
-  if (!(d > 1e-36 && d < 1e36)) return 1.0 / sqrt(d);
-  const double r = (double)rsqrtf((float)d);
+  if (!in_fp32(d)) return slow_div(1.0, sqrt(d));
+  const double r = widen(rsqrtf(low_float(d)));
   const double e = fma(-(d * r), r, 1.0);
   return fma(r * e, fma(0.375, e, 0.5), r);
 }
@@ -280,23 +314,19 @@ __device__ __forceinline__ float inv_sqrt(float d) {
   const float r = rsqrtf(d);
   return fmaf(0.5f * r, fmaf(-d * r, r, 1.f), r);
 }
-// 1 / d for d > 0 is r0 (1 + e + e^2), r0 an FP32 reciprocal and e = 1 - d r0 (|e| <
-// 2^-21); a / d is a r0 plus (e + e^2) of it, a chain of three FP64 operations. r0 = 0
-// tells that d is outside FP32's normal range (the callers then divide).
-__device__ __forceinline__ double recip_start(double d) {
-  const unsigned ex = ((unsigned)__double2hiint(d) >> 20) & 0x7FFu;  // 2^-119 .. 2^119
-  return ex - 904u < 239u ? (double)__fdividef(1.f, (float)d) : 0.0;
-}
-__device__ __forceinline__ float recip_start(float d) { return 1.f / d; }
+// 1 / d is r0 (1 + e + e^2), r0 the estimate and e = 1 - d r0 (|e| < 2^-20), and a / d
+// is a r0 plus (e + e^2) of it: a chain of three FP64 operations.
+__device__ __forceinline__ double recip_start(double d) { return widen(__fdividef(1.f, low_float(d))); }
 __device__ __forceinline__ double recip_err(double d, double r0) {
   const double e = fma(-d, r0, 1.0);
   return fma(e, e, e);
 }
-__device__ __forceinline__ float recip_err(float, float) { return 0.f; }
-template <typename T> __device__ __forceinline__ T recip(T d) {
-  const T r0 = recip_start(d);
-  return r0 != T(0) ? fma(r0, recip_err(d, r0), r0) : T(1) / d;
+__device__ __forceinline__ double quotient(double a, double d) {
+  if (!in_fp32(d)) return slow_div(a, d);
+  const double r0 = recip_start(d), w0 = a * r0;
+  return fma(w0, recip_err(d, r0), w0);
 }
+__device__ __forceinline__ float quotient(float a, float d) { return a * (1.f / d); }
 // s v for s = +-1 and 0 < d < big_pivot^2 (false for NaN) on the integer pipe:
 // an FP64 multiplication or comparison costs as much as a multiply-add.
 __device__ __forceinline__ double flip(double v, bool neg) {
@@ -316,37 +346,41 @@ __device__ __forceinline__ bool pivot_ok(float d) { return d > 0.f && d < INFINI
 // s_j, L_jj = sqrt(s_j d_j), L_ij = a_ij / (s_j L_jj).
 //
 // What bounds it on GB300: an FP64 instruction occupies a quarter SM's unit for
-// 64 cycles whatever its active lanes (measured; results after 66), so the count of
-// FP64 warp instructions on each of the four warps is the time, and the chain of
-// 64 pivots is on it too. So the elimination runs on unscaled columns (a_ic -=
-// (a_ij / d_j) a_cj: no square root on the chain), all columns are scaled by 1 /
-// L_jj at the end, and the block goes in four panels of 16 columns: inside a panel
-// 2 to 8 threads share a row so that all four warps stay busy, each column is
-// published through shared memory (one barrier per column); past the panel a
-// rank-16 update over 8 x 8 blocks of the lower triangle. The loop over a panel's
-// columns stays rolled: straight-line code runs once per launch, from a cold
-// instruction cache (unrolled: 102 us a launch on the 32^3 grid's fronts, rolled: 82).
+// 64 cycles whatever its active lanes (measured; results after 66; a conversion or
+// comparison more), so the count of FP64 warp instructions on each of the four
+// warps is the time, and the chain of 64 pivots is on it too. So the elimination
+// runs on unscaled columns (a_ic -= (a_ij / d_j) a_cj: no square root on the chain),
+// all columns are scaled by 1 / L_jj at the end of their panel, and the block goes in
+// four panels of 16 columns, two threads per row, each column published through
+// shared memory (one barrier per column); past the panel a rank-16 update over 8 x 8
+// blocks of the lower triangle.
 constexpr int kPotrfThreads = 128;
 
-// Panel at column c0 of the block in S (rows c0 .. 63): PN threads per row,
-// thread h of a row holds the columns c0 + h + PN q.
-template <typename T, int PN>
+// Barrier 1 over the first `threads` threads of the block (whole warps).
+__device__ __forceinline__ void bar1(int threads) {
+  asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
+}
+
+// Panel at column c0 of the block in S (rows c0 .. 63) on 2 (64 - c0) threads: two
+// per row, thread h of a row holds the columns c0 + h + 2 q.
+template <typename T>
 __device__ __forceinline__ void potrf_panel(T *S, int ls, int c0, T (*col)[64], const int8_t *neg, T *piv,
                                             int32_t *status, int perturb, int first) {
-  constexpr int NQ = 16 / PN;
-  const int t = threadIdx.x, i = c0 + t / PN, h = t % PN;
-  const bool on = i < 64;
-  T x[NQ];
+  const int t = threadIdx.x, i = t / 2, h = t % 2, act = 2 * (64 - c0);  // row c0 + i
+  T x[8];
 #pragma unroll
-  for (int q = 0; q < NQ; q++) x[q] = on ? S[i * ls + c0 + h + PN * q] : T(0);
-  if (on && h == 0) col[0][i] = x[0];
-  __syncthreads();
-#pragma unroll 1
+  for (int q = 0; q < 8; q++) x[q] = S[(c0 + i) * ls + c0 + h + 2 * q];
+  if (h == 0) col[0][i] = x[0];
+  bar1(act);
+#pragma unroll
   for (int j = 0; j < 16; j++) {
-    const T *cj = col[j & 1];
+    const T *cj = col[j % 3];
     const bool ng = neg[c0 + j] != 0;
-    T d = flip(cj[c0 + j], ng);  // s_j d_j
-    if (!pivot_ok(d)) {  // (uniform over the block)
+    T d = flip(cj[j], ng), v[8];  // s_j d_j; the column's entries at this thread's columns
+    const T aij = cj[i];
+#pragma unroll
+    for (int q = (j + 1) / 2; q < 8; q++) v[q] = cj[h + 2 * q];
+    if (!pivot_ok(d)) {  // (uniform over the panel)
       if (t == 0) {
         if (perturb) atomicAdd(&status[ST_PERTURBED], 1);
         else atomicMin(&status[ST_FAIL_COL], first + c0 + j);
@@ -354,25 +388,33 @@ __device__ __forceinline__ void potrf_panel(T *S, int ls, int c0, T (*col)[64], 
       d = perturb ? big_pivot<T>() : T(1);
     }
     if (t == 0) piv[c0 + j] = d;
-    if (j < 15) {
-      const T aij = on ? cj[i] : T(0), r0 = recip_start(d);
-      const T w0 = aij * r0;
-      T w = fma(w0, recip_err(d, r0), w0);
-      if (r0 == T(0)) w = aij / d;
-      w = flip(w, ng);  // a_ij / d_j
+    if (j == 15) break;
+    const T w = flip(quotient(aij, d), ng);  // a_ij / d_j
+    // column j + 1 first: published before the barrier, the other columns after it,
+    // beside the next pivot's chain (three buffers: the next column but one is
+    // written while slower warps still read column j); column j itself is final
+    const int qn = (j + 1) / 2;
+    if (j % 2 == 1 || h == 1) x[qn] = fma(-w, v[qn], x[qn]);
+    if (h == (j + 1) % 2) col[(j + 1) % 3][i] = x[qn];
+    bar1(act);
 #pragma unroll
-      for (int q = 0; q < NQ; q++)
-        if (PN * q + PN - 1 > j) {  // some column of this group lies past j
-          const int c = h + PN * q;
-          x[q] = fma(-w, c > j ? cj[c0 + c] : T(0), x[q]);
-          if (on && c == j + 1) col[(j + 1) & 1][i] = x[q];
-        }
-      __syncthreads();
-    }
+    for (int q = (j + 1) / 2 + 1; q < 8; q++) x[q] = fma(-w, v[q], x[q]);
   }
 #pragma unroll
-  for (int q = 0; q < NQ; q++)
-    if (on && c0 + h + PN * q <= i) S[i * ls + c0 + h + PN * q] = x[q];
+  for (int q = 0; q < 8; q++)
+    if (h + 2 * q <= i) S[(c0 + i) * ls + c0 + h + 2 * q] = x[q];
+}
+
+// s0, s1 = sum_j x0_j (s_j) y_j, sum_j x1_j (s_j) y_j over a panel's 16 columns
+template <typename T, bool SIGNED>
+__device__ __forceinline__ void panel_dots(const T *x0, const T *x1, const T *y, const int8_t *neg, T &s0, T &s1) {
+  s0 = s1 = T(0);
+#pragma unroll
+  for (int j = 0; j < 16; j++) {
+    const T v = SIGNED ? flip(y[j], neg[j] != 0) : y[j];
+    s0 = fma(x0[j], v, s0);
+    s1 = fma(x1[j], v, s1);
+  }
 }
 
 template <typename T>
@@ -386,7 +428,7 @@ __global__ void __launch_bounds__(kPotrfThreads) potrf_kernel(DevPlan dp, const 
   T *A = L + F.loff + (int64_t)k * F.ld + k;
   const int8_t *sg = dp.sgn ? dp.sgn + F.first + k : nullptr;
   __shared__ T S[NB * LS];  // the block; past kb: zero, with a unit diagonal
-  __shared__ T col[2][NB], piv[NB], rs[NB];
+  __shared__ T col[3][NB], piv[NB], rs[NB];
   __shared__ int8_t neg[NB];
   const int tid = threadIdx.x;
 #pragma unroll 16
@@ -402,22 +444,22 @@ __global__ void __launch_bounds__(kPotrfThreads) potrf_kernel(DevPlan dp, const 
   for (int p = 0; p < 4; p++) {
     const int c0 = 16 * p;
     if (c0 >= kb) break;
-    if (p < 2) potrf_panel<T, 2>(S, LS, c0, col, neg, piv, status, perturb, F.first + k);
-    else if (p == 2) potrf_panel<T, 4>(S, LS, c0, col, neg, piv, status, perturb, F.first + k);
-    else potrf_panel<T, 8>(S, LS, c0, col, neg, piv, status, perturb, F.first + k);
+    if (tid < 2 * (NB - c0)) potrf_panel<T>(S, LS, c0, col, neg, piv, status, perturb, F.first + k);
     __syncthreads();
     if (tid < 16) rs[c0 + tid] = inv_sqrt(piv[c0 + tid]);
     __syncthreads();
     {  // the panel's columns: s_j a_ij / L_jj, and L_jj = sqrt(d) from d and 1 / sqrt(d)
       const int c = c0 + tid % 16;
       const T r = rs[c];
-      for (int i = c0 + tid / 16; i < NB; i += NT / 16) {
-        if (i > c) {
-          S[i * LS + c] = flip(S[i * LS + c] * r, neg[c] != 0);
-        } else if (i == c) {
-          const T d = piv[c], l0 = d * r;
-          S[i * LS + c] = fma(fma(-l0, l0, d), T(0.5) * r, l0);
-        }
+      const bool ng = neg[c] != 0;
+#pragma unroll
+      for (int q = 0; q < 8; q++) {
+        const int i = c0 + tid / 16 + 8 * q;
+        if (i < NB && i > c) S[i * LS + c] = flip(S[i * LS + c] * r, ng);
+      }
+      if (tid < 16) {
+        const T d = piv[c], l0 = d * r;
+        S[c * LS + c] = fma(fma(-l0, l0, d), T(0.5) * r, l0);
       }
     }
     __syncthreads();
@@ -429,16 +471,12 @@ __global__ void __launch_bounds__(kPotrfThreads) potrf_kernel(DevPlan dp, const 
       int bi = 0, rest = b;
       while (rest > bi) rest -= ++bi;  // block row bi holds bi + 1 blocks
       const int i = c0 + 16 + 8 * bi + l / 8, c = c0 + 16 + 8 * rest + l % 8;
-      const T *xi = S + i * LS + c0, *xk = xi + 4 * LS, *yc = S + c * LS + c0;
-      T s0 = T(0), s1 = T(0);
-#pragma unroll
-      for (int j = 0; j < 16; j++) {
-        const T y = flip(yc[j], neg[c0 + j] != 0);
-        s0 = fma(xi[j], y, s0);
-        s1 = fma(xk[j], y, s1);
-      }
-      if (c <= i) S[i * LS + c] -= s0;
-      if (c <= i + 4) S[(i + 4) * LS + c] -= s1;
+      const T *x = S + i * LS + c0, *y = S + c * LS + c0;
+      T *o = S + i * LS + c, s0, s1;
+      if (sg) panel_dots<T, true>(x, x + 4 * LS, y, neg + c0, s0, s1);
+      else panel_dots<T, false>(x, x + 4 * LS, y, neg + c0, s0, s1);
+      if (c <= i) o[0] -= s0;
+      if (c <= i + 4) o[4 * LS] -= s1;
     }
     __syncthreads();
   }
@@ -489,7 +527,7 @@ __global__ void __launch_bounds__(128) trsm_kernel(DevPlan dp, const Task *__res
   const T *A = L + F.loff + (int64_t)k * F.ld + k;
   if (tid < kb) {
     const T d = A[(int64_t)tid * F.ld + tid];
-    rd[tid] = flip(recip(d), sg && sg[tid] < 0);
+    rd[tid] = flip(quotient(T(1), d), sg && sg[tid] < 0);
   }
   T u[NB * NB / 128];
 #pragma unroll
