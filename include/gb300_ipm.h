@@ -333,8 +333,11 @@ typedef struct {
 typedef struct {
   int32_t precision;          /* IPM_FP64, or IPM_FP32: FP32 block factor and solves with
                                  two FP64 refinement steps per solve */
-  int32_t instances_per_cta;  /* 2, 4, 8 or 16 (16 lanes per instance) */
-  int32_t ctas;               /* persistent grid size, 0 = automatic */
+  int32_t instances_per_cta;  /* 2, 4, 8 or 16. IPM_FP32: instances of one CTA (16 lanes
+                                 each). IPM_FP64: one CTA per instance, and
+                                 instances_per_cta * ctas instances in flight */
+  int32_t ctas;               /* persistent grid size, 0 = automatic (IPM_FP64: as many
+                                 instances in flight as the GPU holds) */
 } ipm_mpc_config;
 
 /* Workspace bytes for a batch (host only). */

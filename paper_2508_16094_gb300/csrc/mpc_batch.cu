@@ -17,6 +17,7 @@
 // The FP32 variant assembles, factors and solves in FP32 and refines in FP64
 // on a residual evaluated matrix-free from A, B and D (J v, scaled by D, J^T),
 // so the FP64 pipe only carries the refinement.
+#include <algorithm>
 #include <cfloat>
 #include <cmath>
 #include <stdexcept>
@@ -466,13 +467,13 @@ __device__ void step_lengths(const Group &G, const Inst<double> &I, double tau, 
   ad = fmin(1.0, tau * md);
 }
 
-__device__ void solve_instance(const Group &G, const MpcArgs &a, int inst, bool mixed) {
+__device__ void solve_instance(const Group &G, const MpcArgs &a, int inst) {
   Views V{make_inst<double>(a, inst), make_inst<float>(a, inst)};
   const Inst<double> &I = V.d;
   const int i = G.lane;
   const int T = I.T;
   const double mt = (double)T * 56.0;
-  bool f32 = mixed;
+  bool f32 = true;  // until a solve misses its tolerance
   // starting point: z at the middle of its box (0), s = max(g, 1), lambda = 1
   for (int k = 0; k < T; k++) I.z[k * NS + i] = 0.0;
   __syncwarp(G.mask);
@@ -603,13 +604,13 @@ __device__ void solve_instance(const Group &G, const MpcArgs &a, int inst, bool 
     a.kkt[inst] = kkt;
     a.iters[inst] = it;
     a.status[inst] = status;
-    if (a.fp64_used) a.fp64_used[inst] = (mixed && !f32) ? 1 : 0;
+    if (a.fp64_used) a.fp64_used[inst] = f32 ? 0 : 1;
   }
   if (a.zout)
     for (int k = 0; k < T; k++) a.zout[(a.soff[inst] + k) * NS + i] = I.z[k * NS + i];
 }
 
-__global__ void __launch_bounds__(256) mpc_ipm_kernel(MpcArgs a, int mixed) {
+__global__ void __launch_bounds__(256) mpc_ipm_kernel(MpcArgs a) {
   Group G;
   G.lane = threadIdx.x % 16;
   G.mask = 0xFFFFu << (((threadIdx.x % 32) / 16) * 16);
@@ -618,7 +619,7 @@ __global__ void __launch_bounds__(256) mpc_ipm_kernel(MpcArgs a, int mixed) {
     if (G.lane == 0) q = atomicAdd(a.counter, 1);
     q = __shfl_sync(G.mask, q, 0, 16);
     if (q >= a.count) break;
-    solve_instance(G, a, a.order[q], mixed != 0);
+    solve_instance(G, a, a.order[q]);
   }
 }
 
@@ -627,10 +628,15 @@ __global__ void reset_counter_kernel(int *c) { *c = 0; }
 }  // namespace
 
 void launch_mpc(const MpcArgs &a, int precision, int instances_per_cta, int ctas, cudaStream_t st) {
-  const int threads = 16 * instances_per_cta;
   { note_launch(); reset_counter_kernel<<<1, 1, 0, st>>>(a.counter); }
+  if (precision == 0) {
+    const int64_t slots = ctas > 0 ? (int64_t)ctas * instances_per_cta : mpc_cta_slots();
+    launch_mpc_cta(a, (int)std::min<int64_t>(a.count, slots), st);
+    return;
+  }
+  if (ctas <= 0) ctas = 152 * std::max(1, 64 / instances_per_cta);
   note_launch();
-  mpc_ipm_kernel<<<ctas, threads, 0, st>>>(a, precision == 0 ? 0 : 1);
+  mpc_ipm_kernel<<<ctas, 16 * instances_per_cta, 0, st>>>(a);
 }
 
 }  // namespace gipm

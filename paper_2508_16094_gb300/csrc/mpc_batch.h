@@ -26,8 +26,12 @@ struct MpcArgs {
   int32_t *fp64_used;  // per instance: 1 if the FP32 factor was replaced by FP64 (or nullptr)
 };
 
-// precision 0: FP64 factor and solves; 1: FP32 factor/solves + 2 FP64
-// refinement steps per solve. instances_per_cta in {2, 4, 8, 16}.
+// precision 0: FP64 factor and solves, one CTA per instance in flight (mpc_cta.cu);
+// 1: FP32 factor/solves + 2 FP64 refinement steps per solve, 16 lanes per instance.
+// instances_per_cta in {2, 4, 8, 16}; instances_per_cta * ctas instances in flight
+// (ctas = 0: as many as the GPU holds at once).
 void launch_mpc(const MpcArgs &a, int precision, int instances_per_cta, int ctas, cudaStream_t st);
+int mpc_cta_slots();
+void launch_mpc_cta(const MpcArgs &a, int ctas, cudaStream_t st);
 
 }  // namespace gipm

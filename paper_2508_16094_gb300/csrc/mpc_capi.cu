@@ -112,9 +112,7 @@ ipm_status ipm_solve_batched(const ipm_mpc_batch *b, const ipm_mpc_config *cfg, 
   a.kkt = d_kkt;
   a.iters = d_iters;
   a.status = d_status;
-  int ctas = cfg->ctas;
-  if (ctas <= 0) ctas = 152 * std::max(1, 64 / ipc);
-  launch_mpc(a, cfg->precision == IPM_FP64 ? 0 : 1, ipc, ctas, (cudaStream_t)stream);
+  launch_mpc(a, cfg->precision == IPM_FP64 ? 0 : 1, ipc, cfg->ctas, (cudaStream_t)stream);
   return cudaGetLastError() == cudaSuccess ? IPM_OK : IPM_ERR_CUDA;
 }
 
