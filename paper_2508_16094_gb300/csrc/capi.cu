@@ -53,6 +53,7 @@ struct ipm_ctx {
   double *dinv64 = nullptr, *dsb = nullptr, *dsx = nullptr, *pspart64 = nullptr;  // FP64 (a: yv)
   unsigned *psflags = nullptr;  // its tickets, flags and counters
   float *pspart = nullptr;    // its partial sums
+  SolveWords psw32, psw64;    // its published entries
   // learned correction of a stale factor
   LearnedBufs lb;
   bool learned_active = false;  // PCG preconditioner = corrected stale factor
@@ -284,11 +285,16 @@ void layout(ipm_ctx *c, char *base) {
   c->fsx = cv.take<float>(n);
   c->psflags = cv.take<unsigned>(std::max<int64_t>(std::max(pl.s32.flag_words, pl.s64.flag_words), 32));
   c->pspart = cv.take<float>(std::max<int64_t>(pl.s32.part_entries, 1));
+  const int64_t nw32 = solve_words(pl.s32), nw64 = solve_words(pl.s64);
+  c->psw32.y = cv.take<uint2>(nw32);
+  c->psw32.x = cv.take<uint2>(nw32);
   if (!pl.s64.tasks.empty()) {
     c->dinv64 = cv.take<double>(pl.s64.dinv_entries);
     c->dsb = cv.take<double>(n);
     c->dsx = cv.take<double>(n);
     c->pspart64 = cv.take<double>(pl.s64.part_entries);
+    c->psw64.y = cv.take<uint2>(nw64);
+    c->psw64.x = cv.take<uint2>(nw64);
   }
   {  // learned-correction buffers (only when enabled)
     LearnedBufs &B = c->lb;
@@ -412,14 +418,14 @@ ipm_status do_factor(ipm_ctx *c, int prec, int32_t *bad_col) {
 template <typename T> void launch_held_solve(ipm_ctx *c, int which);
 template <> void launch_held_solve<float>(ipm_ctx *c, int which) {
   launch_psolve<float>(c->dp, c->plan, (const float *)c->L, c->dinv, c->fsa, c->fsb, c->fsx,
-                       reinterpret_cast<float *>(c->tv), c->pspart, c->psflags, c->status, which != 2,
+                       reinterpret_cast<float *>(c->tv), c->pspart, c->psflags, c->psw32, c->status, which != 2,
                        which != 1, c->st, c->test_spins, c->test_withhold);
   c->test_spins = 0;
   c->test_withhold = -1;
 }
 template <> void launch_held_solve<double>(ipm_ctx *c, int which) {
   launch_psolve<double>(c->dp, c->plan, (const double *)c->L, c->dinv64, c->yv, c->dsb, c->dsx, c->tv,
-                        c->pspart64, c->psflags, c->status, which != 2, which != 1, c->st, c->test_spins,
+                        c->pspart64, c->psflags, c->psw64, c->status, which != 2, which != 1, c->st, c->test_spins,
                         c->test_withhold);
   c->test_spins = 0;
   c->test_withhold = -1;
@@ -1101,6 +1107,13 @@ ipm_status ipm_set_workspace(ipm_ctx *c, void *buf, size_t bytes) {
     const size_t total = c->ws_need;
     layout(c, base);
     CK(cudaMemsetAsync(c->ticket, 0, sizeof(unsigned), c->st));
+    for (auto [w, sp] : {std::pair<SolveWords *, const SolvePlan *>{&c->psw32, &c->plan.s32},
+                         {&c->psw64, &c->plan.s64}}) {
+      w->epoch = 0;  // no word carries a tag yet
+      if (sp->tasks.empty()) continue;
+      CK(cudaMemsetAsync(w->y, 0, solve_words(*sp) * sizeof(uint2), c->st));
+      CK(cudaMemsetAsync(w->x, 0, solve_words(*sp) * sizeof(uint2), c->st));
+    }
     CK(cudaStreamSynchronize(c->st));
     if (c->sys) {  // the formulation's system takes the rest of the buffer
       c->ws_need = total;

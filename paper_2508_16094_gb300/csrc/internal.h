@@ -170,8 +170,8 @@ struct LevelPlan {
 // the diagonal blocks (slot s: jb rows of jb rounded up to 16 bytes at
 // dinv_off[s]; the slots of a front are consecutive from first_slot[front]) and
 // the task list, forward tasks first. Flags (32-bit words): [0, 32) tickets, then
-// per slot "y published", "x published", "partial sums done", per front
-// "update-vector chunks of its children done", "column blocks done".
+// per slot "partial sums done", per front "update-vector chunks of its children
+// done", "column blocks done".
 constexpr int kSolveB32 = 128, kSolveB64 = 64;  // block widths, FP32 and FP64
 struct SolvePlan {
   int B = 0;

@@ -6,14 +6,20 @@
 // (explicit inverse, rows padded to 16 bytes). A solve is then ONE launch of a persistent kernel whose CTAs take the tasks of the plan in
 // order from a global ticket counter (forward sweep leaves -> root, backward
 // sweep root -> leaves). Instead of grid barriers between phases, each task
-// waits only for the results it reads, published through flags and counters
-// in device memory: a diagonal block of the forward sweep subtracts
-// L_ij y_j as each y_j of its front appears (a wavefront down the front's
-// blocks), rows below a front take every y_j and then count towards the
-// front's update vector, which the parent's gathers wait for; the backward
-// sweep mirrors this with partial sums over the rows below a front (waiting
-// for the parent front) and x_i published block by block. A task waits only
-// for earlier tasks, so the schedule cannot deadlock, and every wait is
+// waits only for the results it reads. Along the diagonal blocks of a front, whose
+// chain is the time of a solve, the entries of y and x carry their own flag: each
+// 32-bit half is stored with the launch's tag in one 8-byte word, and a
+// consumer reads the words until all of them have the tag, so a block costs one
+// trip through L2 and no fence (a counter behind a release, polled and
+// acquired before the values are read, takes three: 2.6 us a block of the root
+// against 1.8; a whole solve, TF32x3: 834 -> 666 us at 48^3, 1845 -> 1548 at
+// 64^3, FP64 1484 -> 1302 at 40^3). A
+// diagonal block of the forward sweep subtracts L_ij y_j as each y_j of its front
+// appears (a wavefront down the front's blocks), rows below a front take every
+// y_j and then count towards the front's update vector, which the parent's gathers
+// wait for; the backward sweep mirrors this with partial sums over the rows below
+// a front (waiting for the parent front) and x_i published block by block. A task
+// waits only for earlier tasks, so the schedule cannot deadlock, and every wait is
 // bounded: on expiry the status word is set and the whole launch drains.
 // Three vectors keep reads disjoint from writes: a (right-hand side), b
 // (forward result) and x (solution); t holds the fronts' update vectors.
@@ -166,6 +172,8 @@ template <typename T> struct PsArgs {
   T *a, *b, *x, *t, *part;
   int32_t q0, q1;    // tasks [q0, q1) of the plan
   unsigned *flags;   // the solve plan's flag words, zeroed before the launch
+  uint2 *ly, *lx;    // published entries of y and x (see LL words), B per slot (FP64: 2 B)
+  unsigned epoch;    // tag of this launch's entries
   int32_t *status;   // ST_SOLVE_TIMEOUT
   unsigned spins;    // polls before a wait gives up
   int32_t withhold;  // test of the bounded wait: the task of this ticket is abandoned (-1: none)
@@ -182,27 +190,23 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-// Flag words (see Plan): tickets, then per slot y / x published and partial
-// sums done, per front update-vector chunks and column blocks done.
+// Flag words (see SolvePlan): tickets, then per slot partial sums done, per front
+// update-vector chunks and column blocks done.
 template <typename T>
 __device__ __forceinline__ unsigned *f_ticket(const PsArgs<T> &A) { return A.flags; }
 template <typename T>
-__device__ __forceinline__ unsigned *f_y(const PsArgs<T> &A, int slot) { return A.flags + 32 + slot; }
-template <typename T>
-__device__ __forceinline__ unsigned *f_x(const PsArgs<T> &A, int slot) { return A.flags + 32 + A.nslot + slot; }
-template <typename T>
 __device__ __forceinline__ unsigned *f_part(const PsArgs<T> &A, int slot) {
-  return A.flags + 32 + 2 * A.nslot + slot;
+  return A.flags + 32 + slot;
 }
 // per front: chunks of rows below its children that are done (the children's
 // update vectors are complete once it reaches ps_kid_chunks[front])
 template <typename T>
 __device__ __forceinline__ unsigned *f_tvec(const PsArgs<T> &A, int front) {
-  return A.flags + 32 + 3 * A.nslot + front;
+  return A.flags + 32 + A.nslot + front;
 }
 template <typename T>
 __device__ __forceinline__ unsigned *f_front(const PsArgs<T> &A, int front) {
-  return A.flags + 32 + 3 * A.nslot + A.nfr + front;
+  return A.flags + 32 + A.nslot + A.nfr + front;
 }
 
 // Shared scratch of one CTA (dynamic shared memory).
@@ -211,14 +215,12 @@ template <typename T> struct PsShared {
   T di[B * B];                  // staged inverse of a diagonal block (TMA bulk copy)
   alignas(16) T sv[B];          // values handed to the diagonal-block solve
   T xs[B];                      // solution entries of the rows below a front
-  T red[sizeof(T) == 4 ? kT / 32 : 1][Ps<T>::RW][33];  // FP32: per-warp transpose reduction of RW row sums
-  alignas(16) T ys[2][B];                   // FP64: the y block of the running product (double-buffered)
+  alignas(16) T ys[sizeof(T) == 8 ? kT / 32 : 1][B];  // FP64: a warp's copy of the running y block
   alignas(16) T red4[kT / 32][B];  // per-row-group column sums
   unsigned long long mbar;      // completion of the staging copy
   uint32_t parity;              // its phase
   int tk;                       // this CTA's current task
   int ok;                       // outcome of the last wait
-  int ready;                    // blocks of the running chain known to be published
   int nkids;                    // children of the task's front staged below
   int64_t kid_inv[kMaxKids];    // their child -> front map offsets
   int64_t kid_toff[kMaxKids];   // their update-vector offsets
@@ -243,9 +245,10 @@ __device__ __forceinline__ void stage_dinv(const PsArgs<T> &A, PsShared<T> &S, i
 }
 
 // All threads: bounded wait for the staging copy; false after a timeout (the
-// status word is set, and a second bounded wait lets the copy land first).
+// status word is set, and a second bounded wait lets the copy land first) or if
+// ok_in was false in any thread.
 template <typename T>
-__device__ bool wait_dinv(const PsArgs<T> &A, PsShared<T> &S) {
+__device__ bool wait_dinv(const PsArgs<T> &A, PsShared<T> &S, bool ok_in) {
   const uint32_t par = S.parity;
   auto try_wait = [&]() {
     uint32_t done;
@@ -270,42 +273,112 @@ __device__ bool wait_dinv(const PsArgs<T> &A, PsShared<T> &S) {
       break;
     }
   }
-  ok = __syncthreads_and(ok) != 0;  // one outcome for the whole CTA
+  ok = __syncthreads_and(ok && ok_in) != 0;  // one outcome for the whole CTA
   if (threadIdx.x == 0) S.parity = par ^ 1u;
   return ok;
 }
 
-// Row sums of RW consecutive rows per warp: p[k] = <row k, v> for the lane's VW
-// columns; returns the full sum of row `lane` in lanes 0 .. RW - 1.
-__device__ __forceinline__ float rows_reduce(PsShared<float> &S, const float (&p)[Ps<float>::RW]) {
-  constexpr int RW = Ps<float>::RW;
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-#pragma unroll
-  for (int k = 0; k < RW; k++) S.red[warp][k][lane] = p[k];
-  __syncwarp();
-  float s = 0.f;
-  if (lane < RW) {
-#pragma unroll 8
-    for (int q = 0; q < 32; q++) s += S.red[warp][lane][q];
-  }
-  __syncwarp();
-  return s;
+// Words of published entries: value bits and the launch's tag in one 8-byte access
+// (FP64: two words, low and high half), so a word with the tag holds its value.
+__device__ __forceinline__ uint2 split_word(unsigned long long w) { return make_uint2((unsigned)w, (unsigned)(w >> 32)); }
+__device__ __forceinline__ unsigned long long make_word(unsigned bits, unsigned tag) {
+  return (unsigned long long)tag << 32 | bits;
 }
+__device__ __forceinline__ uint4 ld_words(const uint2 *p) {
+  unsigned long long a, b;
+  asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+  const uint2 u = split_word(a), v = split_word(b);
+  return make_uint4(u.x, u.y, v.x, v.y);
+}
+__device__ __forceinline__ uint2 ld_word(const uint2 *p) {
+  unsigned long long a;
+  asm volatile("ld.volatile.global.u64 %0, [%1];" : "=l"(a) : "l"(p) : "memory");
+  return split_word(a);
+}
+__device__ __forceinline__ void publish(uint2 *slot, int r, float v, unsigned tag) {
+  asm volatile("st.volatile.global.u64 [%0], %1;" ::"l"(slot + r), "l"(make_word(__float_as_uint(v), tag)) : "memory");
+}
+__device__ __forceinline__ void publish(uint2 *slot, int r, double v, unsigned tag) {
+  asm volatile("st.volatile.global.v2.u64 [%0], {%1, %2};" ::"l"(slot + 2 * r),
+               "l"(make_word((unsigned)__double2loint(v), tag)), "l"(make_word((unsigned)__double2hiint(v), tag))
+               : "memory");
+}
+__device__ __forceinline__ double word_double(unsigned lo, unsigned hi) { return __hiloint2double((int)hi, (int)lo); }
+template <typename T> __device__ __forceinline__ uint2 *slot_words(uint2 *base, int slot) {
+  return base + (int64_t)slot * (Ps<T>::B * (int)(sizeof(T) / 4));
+}
+
+// One warp: until load() holds in every lane (it reads the lane's words and tells
+// whether they carry the tag), at most A.spins polls and only while no other wait
+// of the launch has run out. The block next in a chain (critical) polls all its
+// words; the others watch the block's first word, to leave L2 to the chain.
+template <typename T, typename Load>
+__device__ __forceinline__ bool wait_words(const PsArgs<T> &A, const uint2 *first, bool critical, Load load) {
+  if (__all_sync(0xffffffffu, load())) return true;
+  const int lane = threadIdx.x % 32;
+  for (unsigned spins = 0;; spins++) {
+    bool look = true;
+    if (!critical) {
+      unsigned seen = 0;
+      if (lane == 0) seen = ld_word(first).y == A.epoch;
+      look = __shfl_sync(0xffffffffu, seen, 0) != 0;
+      if (!look) __nanosleep(64);
+    }
+    if (look && __all_sync(0xffffffffu, load())) return true;
+    int stop = 0;
+    if (lane == 0 && (spins & 63u) == 0) stop = *(volatile int32_t *)(A.status + ST_SOLVE_TIMEOUT) != 0;
+    if (lane == 0 && spins >= A.spins) {
+      atomicExch(A.status + ST_SOLVE_TIMEOUT, 1);
+      stop = 1;
+    }
+    if (__shfl_sync(0xffffffffu, stop, 0)) return false;
+  }
+}
+
+// Row sums of 16 consecutive rows per warp: p[k] = <row k, v> for the lane's
+// columns; returns the full sum of row lane / 2 (each lane keeps half of its rows
+// at every exchange).
+__device__ __forceinline__ float rows_reduce(const float (&p)[16]) {
+  const int lane = threadIdx.x % 32;
+  float a[8], b[4], c[2], d;
+  const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4, h1 = lane & 2;
+#pragma unroll
+  for (int k = 0; k < 8; k++) a[k] = (h4 ? p[k + 8] : p[k]) + __shfl_xor_sync(0xffffffffu, h4 ? p[k] : p[k + 8], 16);
+#pragma unroll
+  for (int k = 0; k < 4; k++) b[k] = (h3 ? a[k + 4] : a[k]) + __shfl_xor_sync(0xffffffffu, h3 ? a[k] : a[k + 4], 8);
+#pragma unroll
+  for (int k = 0; k < 2; k++) c[k] = (h2 ? b[k + 2] : b[k]) + __shfl_xor_sync(0xffffffffu, h2 ? b[k] : b[k + 2], 4);
+  d = (h1 ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, h1 ? c[0] : c[1], 2);
+  return d + __shfl_xor_sync(0xffffffffu, d, 1);
+}
+// Entry r of a published block; false while its words lack the tag.
+__device__ __forceinline__ bool read_word(const uint2 *slot, int r, unsigned tag, float &v) {
+  const uint2 w = ld_word(slot + r);
+  v = __uint_as_float(w.x);
+  return w.y == tag;
+}
+__device__ __forceinline__ bool read_word(const uint2 *slot, int r, unsigned tag, double &v) {
+  const uint4 w = ld_words(slot + 2 * r);
+  v = word_double(w.x, w.z);
+  return w.y == tag && w.w == tag;
+}
+
 // Sum over the four neighbouring lanes (valid in all of them).
-__device__ __forceinline__ double quad_sum(double v) {
+template <typename T> __device__ __forceinline__ T quad_sum(T v) {
   v += __shfl_xor_sync(0xffffffffu, v, 1);
   return v + __shfl_xor_sync(0xffffffffu, v, 2);
 }
 
 // Product of a B x B tile's rows (row stride ld) with a block of the forward
 // result, accumulated over tiles. The loads of a tile are issued by load(),
-// before the block is waited for.
+// before the block's words are waited for (wait_y, per warp).
 //  FP32: warp w takes rows 16w .. 16w + 15, lane: columns 4 lane ..; the row sums
 //  are reduced across the warp once, after the last tile.
 //  FP64: an addition costs as much as a multiply-add (64 cycles per warp on a
 //  quarter SM), so the cross-lane reduction is kept short: four threads share a
 //  row (thread h: columns 8m + 2h, 8m + 2h + 1) and y comes from shared memory.
 template <typename T> struct FwdTile;
+
 template <> struct FwdTile<float> {
   static constexpr int RW = Ps<float>::RW;
   float4 l[RW];
@@ -325,13 +398,24 @@ template <> struct FwdTile<float> {
                                                : make_float4(0.f, 0.f, 0.f, 0.f);
   }
   // y: block of nc values; columns past nc (padding of a last block) never enter
-  template <bool FULL>
-  __device__ __forceinline__ void mul(PsShared<float> &, int, const float *y, int nc) {
+  uint4 w0, w1;
+  __device__ __forceinline__ bool wait_y(const PsArgs<float> &A, const uint2 *words, int nc, bool critical) {
     const int c = 4 * (threadIdx.x % 32);
-    const float *yb = y + c;
-    const float4 y4 = FULL ? make_float4(ldcg(yb), ldcg(yb + 1), ldcg(yb + 2), ldcg(yb + 3))
-                           : make_float4(c < nc ? ldcg(yb) : 0.f, c + 1 < nc ? ldcg(yb + 1) : 0.f,
-                                         c + 2 < nc ? ldcg(yb + 2) : 0.f, c + 3 < nc ? ldcg(yb + 3) : 0.f);
+    return wait_words(A, words, critical, [&]() {
+      if (c >= nc) return true;
+      w0 = ld_words(words + c);
+      w1 = ld_words(words + c + 2);
+      return w0.y == A.epoch && (c + 1 >= nc || w0.w == A.epoch) && (c + 2 >= nc || w1.y == A.epoch) &&
+             (c + 3 >= nc || w1.w == A.epoch);
+    });
+  }
+  template <bool FULL>
+  __device__ __forceinline__ void mul(PsShared<float> &, int nc) {
+    const int c = 4 * (threadIdx.x % 32);
+    const float4 y4 = make_float4(FULL || c < nc ? __uint_as_float(w0.x) : 0.f,
+                                  FULL || c + 1 < nc ? __uint_as_float(w0.z) : 0.f,
+                                  FULL || c + 2 < nc ? __uint_as_float(w1.x) : 0.f,
+                                  FULL || c + 3 < nc ? __uint_as_float(w1.z) : 0.f);
 #pragma unroll
     for (int k = 0; k < RW; k++) {
       float4 v = l[k];
@@ -344,10 +428,10 @@ template <> struct FwdTile<float> {
     }
   }
   // f(row, sum) once per row
-  template <typename F> __device__ __forceinline__ void finish(PsShared<float> &S, int nr, F f) {
-    const float s = rows_reduce(S, acc);
-    const int lane = threadIdx.x % 32, r = RW * (threadIdx.x / 32) + lane;
-    if (lane < RW && r < nr) f(r, s);
+  template <typename F> __device__ __forceinline__ void finish(int nr, F f) {
+    const float s = rows_reduce(acc);
+    const int lane = threadIdx.x % 32, r = RW * (threadIdx.x / 32) + lane / 2;
+    if (lane % 2 == 0 && r < nr) f(r, s);
   }
 };
 template <> struct FwdTile<double> {
@@ -363,11 +447,24 @@ template <> struct FwdTile<double> {
     for (int m = 0; m < NL; m++)
       l[m] = (r < nr && (FULL || 8 * m + c < nc)) ? ldg16(row + 8 * m) : vzero<double>();
   }
+  uint4 w0, w1;  // the lane's two entries of y
+  __device__ __forceinline__ bool wait_y(const PsArgs<double> &A, const uint2 *words, int nc, bool critical) {
+    const int v = 2 * (threadIdx.x % 32);
+    return wait_words(A, words, critical, [&]() {
+      if (v >= nc) return true;
+      w0 = ld_words(words + 2 * v);
+      w1 = ld_words(words + 2 * v + 2);
+      return w0.y == A.epoch && w0.w == A.epoch && (v + 1 >= nc || (w1.y == A.epoch && w1.w == A.epoch));
+    });
+  }
   template <bool FULL>
-  __device__ __forceinline__ void mul(PsShared<double> &S, int j, const double *y, int nc) {
-    double *ys = S.ys[j & 1];  // the other buffer may still be read by slower threads
-    if (threadIdx.x < Ps<double>::B) ys[threadIdx.x] = (int)threadIdx.x < nc ? ldcg(y + threadIdx.x) : 0.0;
-    __syncthreads();
+  __device__ __forceinline__ void mul(PsShared<double> &S, int nc) {
+    const int v = 2 * (threadIdx.x % 32);
+    double *ys = S.ys[threadIdx.x / 32];
+    __syncwarp();  // the previous block has been read
+    st16(ys + v, Vec<double>{{FULL || v < nc ? word_double(w0.x, w0.z) : 0.0,
+                              FULL || v + 1 < nc ? word_double(w1.x, w1.z) : 0.0}});
+    __syncwarp();
     const int c = 2 * (threadIdx.x % 4);
 #pragma unroll
     for (int m = 0; m < NL; m++) {
@@ -376,16 +473,17 @@ template <> struct FwdTile<double> {
       acc = vdot(x, ld16(ys + 8 * m + c), acc);
     }
   }
-  template <typename F> __device__ __forceinline__ void finish(PsShared<double> &, int nr, F f) {
+  template <typename F> __device__ __forceinline__ void finish(int nr, F f) {
     const double s = quad_sum(acc);
     const int r = threadIdx.x / 4;
     if (threadIdx.x % 4 == 0 && r < nr) f(r, s);
   }
 };
 
-// b[first + j + r] = sum_c Dinv[r][c] v[c]  (Dinv staged in S.di, v = S.sv
-// zero past jb); FP32: warp w takes rows 16w .. 16w + 15
-__device__ void diag_fwd(const PsArgs<float> &A, PsShared<float> &S, const FrontInfo &F, int j) {
+// y = b[first + j + r] = sum_c Dinv[r][c] v[c]  (Dinv staged in S.di, v = S.sv
+// zero past jb), published in the slot's words; a warp's rows stop at their diagonal.
+// FP32: warp w takes rows 16w .. 16w + 15
+__device__ void diag_fwd(const PsArgs<float> &A, PsShared<float> &S, const FrontInfo &F, int j, int slot) {
   constexpr int B = Ps<float>::B, RW = Ps<float>::RW;
   const int jb = min(B, F.ncol - j), ldi = (jb + 3) & ~3;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, c = 4 * lane, rw = RW * warp;
@@ -395,16 +493,20 @@ __device__ void diag_fwd(const PsArgs<float> &A, PsShared<float> &S, const Front
 #pragma unroll
   for (int k = 0; k < RW; k++) {
     p[k] = 0.f;
-    if (c < ldi && rw + k < jb) {
+    if (c <= rw + k && rw + k < jb) {  // (zero above the diagonal)
       const float4 d = *reinterpret_cast<const float4 *>(S.di + (rw + k) * ldi + c);
       p[k] = d.x * v4.x + d.y * v4.y + d.z * v4.z + d.w * v4.w;
     }
   }
-  const float s = rows_reduce(S, p);
-  if (lane < RW && rw + lane < jb) A.b[F.first + j + rw + lane] = s;
+  const float s = rows_reduce(p);
+  const int r = rw + lane / 2;
+  if (lane % 2 == 0 && r < jb) {
+    publish(slot_words<float>(A.ly, slot), r, s, A.epoch);
+    A.b[F.first + j + r] = s;
+  }
 }
-// FP64: four threads per row, and a warp's eight rows stop at their diagonal
-__device__ void diag_fwd(const PsArgs<double> &A, PsShared<double> &S, const FrontInfo &F, int j) {
+// FP64: four threads per row
+__device__ void diag_fwd(const PsArgs<double> &A, PsShared<double> &S, const FrontInfo &F, int j, int slot) {
   constexpr int B = Ps<double>::B;
   const int jb = min(B, F.ncol - j), ldi = (jb + 1) & ~1, r = threadIdx.x / 4, c = 2 * (threadIdx.x % 4);
   double s = 0.0;
@@ -412,7 +514,10 @@ __device__ void diag_fwd(const PsArgs<double> &A, PsShared<double> &S, const Fro
     if (r < jb && 8 * m + c < ldi)
       s = vdot(ld16(S.di + r * ldi + 8 * m + c), ld16(S.sv + 8 * m + c), s);
   s = quad_sum(s);
-  if (threadIdx.x % 4 == 0 && r < jb) A.b[F.first + j + r] = s;
+  if (threadIdx.x % 4 == 0 && r < jb) {
+    publish(slot_words<double>(A.ly, slot), r, s, A.epoch);
+    A.b[F.first + j + r] = s;
+  }
 }
 
 // Column sums over the row groups of S.red4: FP32 on the first warp, f(first of
@@ -446,14 +551,14 @@ __device__ __forceinline__ void put_sum(float *row, int c, const Vec<float> &s) 
 __device__ __forceinline__ void put_sum(double *row, int c, double s) { row[c] = s; }
 
 // x[first + j + c] = sum_{r >= c} Dinv[r][c] v[r]  (Dinv staged in S.di, zero
-// above the diagonal; v = S.sv). FP32: thread (g, q) takes columns 4q .. and rows
+// above the diagonal; v = S.sv), published in the slot's words. FP32: thread (g, q) takes columns 4q .. and rows
 // 16g ..; FP64: four threads per column, and a warp's eight columns start at their diagonal.
-__device__ void diag_bwd(const PsArgs<float> &A, PsShared<float> &S, const FrontInfo &F, int j) {
+__device__ void diag_bwd(const PsArgs<float> &A, PsShared<float> &S, const FrontInfo &F, int j, int slot) {
   constexpr int B = Ps<float>::B, RW = Ps<float>::RW;
   const int jb = min(B, F.ncol - j), ldi = (jb + 3) & ~3;
   const int q = threadIdx.x % 32, g = threadIdx.x / 32, c = 4 * q;
   Vec<float> acc = vzero<float>();
-  if (c < ldi) {
+  if (c < ldi && c < RW * (g + 1)) {  // (zero above the diagonal)
 #pragma unroll
     for (int k = 0; k < RW; k++) {
       const int r = RW * g + k;
@@ -465,11 +570,13 @@ __device__ void diag_bwd(const PsArgs<float> &A, PsShared<float> &S, const Front
   float *xo = A.x + F.first + j;
   groups_sum(S, [&](int c0, auto s) {
     each_sum(c0, s, [&](int cc, float v) {
-      if (cc < jb) xo[cc] = v;
+      if (cc >= jb) return;
+      publish(slot_words<float>(A.lx, slot), cc, v, A.epoch);
+      xo[cc] = v;
     });
   });
 }
-__device__ void diag_bwd(const PsArgs<double> &A, PsShared<double> &S, const FrontInfo &F, int j) {
+__device__ void diag_bwd(const PsArgs<double> &A, PsShared<double> &S, const FrontInfo &F, int j, int slot) {
   constexpr int B = Ps<double>::B;
   const int jb = min(B, F.ncol - j), ldi = (jb + 1) & ~1, c = threadIdx.x / 4, h = threadIdx.x % 4;
   double s = 0.0;
@@ -478,16 +585,18 @@ __device__ void diag_bwd(const PsArgs<double> &A, PsShared<double> &S, const Fro
     if (r < jb && c < jb) s = fma(S.di[r * ldi + c], S.sv[r], s);
   }
   s = quad_sum(s);
-  if (h == 0 && c < jb) A.x[F.first + j + c] = s;
+  if (h == 0 && c < jb) {
+    publish(slot_words<double>(A.lx, slot), c, s, A.epoch);
+    A.x[F.first + j + c] = s;
+  }
 }
 
 // Thread 0 polls *w until it reaches target (acquire), at most A.spins times
 // and only while no other wait of the launch has run out; the CTA then shares
-// the outcome (and, on success, S.ready = ready unless ready < -1). On expiry
-// the status word is set, and every later wait of the launch gives up at once.
+// the outcome. On expiry the status word is set, and every later wait of the
+// launch gives up at once.
 template <typename T>
-__device__ bool wait_flag(const PsArgs<T> &A, PsShared<T> &S, const unsigned *w, unsigned target,
-                          int ready = -2) {
+__device__ bool wait_flag(const PsArgs<T> &A, PsShared<T> &S, const unsigned *w, unsigned target) {
   __syncthreads();  // every thread has read the previous outcome
   if (threadIdx.x == 0) {
     unsigned v, spins = 0;
@@ -507,31 +616,9 @@ __device__ bool wait_flag(const PsArgs<T> &A, PsShared<T> &S, const unsigned *w,
       __nanosleep(32);
     }
     S.ok = ok;
-    if (ok && ready >= -1) S.ready = ready;
   }
   __syncthreads();
   return S.ok != 0;
-}
-
-// Wait for block j of a chain whose flags are published in order (each
-// producer acquired its predecessor's flag before releasing its own), with
-// `last` the last block this task needs: one acquire of the last flag makes
-// every earlier block visible, so a task behind the chain waits once and then
-// streams its blocks without polling. S.ready holds the highest block known
-// published (reset by the caller to -1).
-template <typename T>
-__device__ bool wait_chain(const PsArgs<T> &A, PsShared<T> &S, const unsigned *flags, int j, int last,
-                           int step) {
-  if ((step > 0 ? j <= S.ready : j >= S.ready) && S.ready >= 0) return true;
-  __syncthreads();  // every thread has read S.ready and the previous outcome
-  if (threadIdx.x == 0) {
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(flags + last) : "memory");
-    if (v >= 1u) S.ready = last;
-  }
-  __syncthreads();
-  if (S.ready == last) return true;
-  return wait_flag(A, S, flags + j, 1, j);
 }
 
 // After this CTA's writes: count one more on *w. The barrier orders every
@@ -649,23 +736,18 @@ __device__ void fwd_diag(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R, 
                             : T(0);
   FwdTile<T> tile;
   tile.clear();
-  if (threadIdx.x == 0) S.ready = -1;
-  __syncthreads();  // no thread reads the previous task's value
+  __syncthreads();  // S.sv is written
+  const T *row = A.L + F.loff + (int64_t)j0 * F.ld;
   for (int j = 0; j < i && ok; j++) {  // block j < i is a full block
-    tile.template load<true>(A.L + F.loff + (int64_t)j0 * F.ld + B * j, F.ld, jb, B);
-    ok = wait_chain(A, S, f_y(A, slot0), j, i - 1, 1);
-    if (!ok) break;
-    tile.template mul<true>(S, j, A.b + F.first + B * j, B);
+    tile.template load<true>(row + B * j, F.ld, jb, B);
+    ok = tile.wait_y(A, slot_words<T>(A.ly, slot0 + j), B, j == i - 1);
+    if (ok) tile.template mul<true>(S, B);
   }
   take_next(A, N);
-  tile.finish(S, ok ? jb : 0, [&](int r, T v) { S.sv[r] -= v; });
+  tile.finish(ok ? jb : 0, [&](int r, T v) { S.sv[r] -= v; });
   // the staged copy always lands before S.di is reused; the wait ends with a
   // barrier, after which every row of S.sv is final
-  const bool got = wait_dinv(A, S);
-  if (ok && got) {
-    diag_fwd(A, S, F, j0);
-    signal(f_y(A, slot0 + i));
-  }
+  if (wait_dinv(A, S, ok)) diag_fwd(A, S, F, j0, slot0 + i);
 }
 
 // Forward, rows r0 .. r0 + nr below front s: the children's entries plus
@@ -681,21 +763,21 @@ __device__ void fwd_below(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R,
   if (ok && threadIdx.x < nr) S.xs[threadIdx.x] = gather_children(A, S, F, F.ncol + r0 + threadIdx.x);
   FwdTile<T> tile;
   tile.clear();
-  if (threadIdx.x == 0) S.ready = -1;
-  __syncthreads();  // no thread reads the previous task's value
+  __syncthreads();  // S.xs is written
+  const T *row = A.L + F.loff + (int64_t)(F.ncol + r0) * F.ld;
   for (int j = 0; j < nb && ok; j++) {
     const int jbj = min(B, F.ncol - B * j);
-    const T *P = A.L + F.loff + (int64_t)(F.ncol + r0) * F.ld + B * j, *y = A.b + F.first + B * j;
+    const T *P = row + B * j;
     if (jbj == B) tile.template load<true>(P, F.ld, nr, B);
     else tile.template load<false>(P, F.ld, nr, jbj);
-    ok = wait_chain(A, S, f_y(A, slot0), j, nb - 1, 1);
+    ok = tile.wait_y(A, slot_words<T>(A.ly, slot0 + j), jbj, false);
     if (!ok) break;
-    if (jbj == B) tile.template mul<true>(S, j, y, B);
-    else tile.template mul<false>(S, j, y, jbj);
+    if (jbj == B) tile.template mul<true>(S, B);
+    else tile.template mul<false>(S, jbj);
   }
   take_next(A, N);
-  tile.finish(S, ok ? nr : 0, [&](int r, T v) { A.t[R.toff + r0 + r] = S.xs[r] + v; });
-  if (ok) signal(f_tvec(A, F.parent));  // rows below a front exist only below a parent
+  tile.finish(ok ? nr : 0, [&](int r, T v) { A.t[R.toff + r0 + r] = S.xs[r] + v; });
+  if (__syncthreads_and(ok)) signal(f_tvec(A, F.parent));  // rows below a front exist only below a parent
 }
 
 // Backward, rows r0 .. r0 + nr below front s: once the parent front (and so
@@ -743,6 +825,18 @@ __device__ void bwd_part(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R, 
   }
 }
 
+// Brings a warp's RW rows of a tile (512 bytes each; nr rows in the tile) into L2
+// ahead of their loads: a tile's registers allow one in flight, and DRAM's latency
+// is as long as a chain's step.
+template <typename T> __device__ __forceinline__ void prefetch_tile(const T *P, int64_t ld, int nr) {
+  constexpr int RW = Ps<T>::RW, PER = RW / 8, EL = 128 / (int)sizeof(T);  // lines per lane, values per line
+  const int lane = threadIdx.x % 32, r = RW * (threadIdx.x / 32) + lane * PER / 4;
+  if (r >= nr) return;
+#pragma unroll
+  for (int h = 0; h < PER; h++)
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(P + (int64_t)r * ld + (lane * PER % 4 + h) * EL));
+}
+
 // Backward, column block cb of front s: the partial sums in chunk order, then
 // L[block i, block cb]^T x_i for i > cb as each x_i is published, then
 // x_cb = L_cc^{-T} (.) with the staged inverse.
@@ -754,62 +848,62 @@ __device__ void bwd_diag(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R, 
   const int cb = tk.a, c0 = B * cb, jb = min(B, F.ncol - c0), nb = (F.ncol + B - 1) / B;
   const int nbl = (F.nrow + B - 1) / B, slot0 = R.slot0;
   if (threadIdx.x == 0) stage_dinv(A, S, slot0 + cb, jb);
-  // b of this block is the forward result: published by this launch's forward
-  // task of the block, or complete before a backward-only launch
-  bool ok = !A.fwd_here || wait_flag(A, S, f_y(A, slot0 + cb), 1);
-  if (ok && nbl > 0) ok = wait_flag(A, S, f_part(A, slot0 + cb), nbl);  // implies the parent is done
+  bool ok = true;
+  if (nbl > 0) ok = wait_flag(A, S, f_part(A, slot0 + cb), nbl);  // implies the parent is done
   else if (ok && F.parent >= 0)
     ok = wait_flag(A, S, f_front(A, F.parent), (unsigned)R.parent_blocks);
-  if (ok && sizeof(T) == 8) {  // four threads per column (see quad_sum)
-    const int cc = threadIdx.x / 4;
-    const T *pp = A.part + (R.pbase + (int64_t)cb * nbl) * B + cc;
+  // b of this block is the forward result: the words of this launch's forward
+  // task of the block, or complete before a backward-only launch
+  if (ok) {
+    // FP64: four threads per column (see quad_sum), the first holds the result
+    constexpr int TPC = sizeof(T) == 8 ? 4 : 1;
+    const int cc = threadIdx.x / TPC;
+    const bool mine = threadIdx.x % TPC == 0 && cc < jb;
+    T bv = T(0);
+    const uint2 *words = slot_words<T>(A.ly, slot0 + cb);
+    if (A.fwd_here)
+      ok = wait_words(A, words, false, [&]() { return !mine || read_word(words, cc, A.epoch, bv); });
+    else if (mine)
+      bv = ldcg(A.b + F.first + c0 + cc);
     T ps = T(0);
-    for (int k = threadIdx.x % 4; k < nbl && cc < jb; k += 4) ps += ldcg(pp + (int64_t)k * B);
-    ps = quad_sum(ps);
-    if (threadIdx.x % 4 == 0) S.sv[cc] = cc < jb ? ldcg(A.b + F.first + c0 + cc) - ps : T(0);
-  } else if (ok && threadIdx.x < B) {
-    T v = T(0);
-    if (threadIdx.x < jb) {
-      const T *pp = A.part + (R.pbase + (int64_t)cb * nbl) * B + threadIdx.x;
-      T ps = T(0);
-      for (int k = 0; k < nbl; k++) ps += ldcg(pp + (int64_t)k * B);
-      v = ldcg(A.b + F.first + c0 + threadIdx.x) - ps;
-    }
-    S.sv[threadIdx.x] = v;
+    const T *pp = A.part + (R.pbase + (int64_t)cb * nbl) * B + cc;
+    for (int k = threadIdx.x % TPC; k < nbl && cc < jb; k += TPC) ps += ldcg(pp + (int64_t)k * B);
+    if (TPC == 4) ps = quad_sum(ps);
+    if (threadIdx.x % TPC == 0 && cc < B) S.sv[cc] = bv - ps;  // (zero past jb)
   }
   const int q = threadIdx.x % 32, g = threadIdx.x / 32, c = c0 + VW * q;
   Vec<T> acc = vzero<T>();
-  if (threadIdx.x == 0) S.ready = -1;
-  __syncthreads();  // no thread reads the previous task's value
+  const bool wide = c0 + B <= F.ncol;  // (a block with blocks after it is a whole one)
+  if (wide && nb - 2 > cb) prefetch_tile(A.L + F.loff + (int64_t)(B * (nb - 2)) * F.ld + c0, F.ld, B);
   for (int i = nb - 1; i > cb && ok; i--) {
     const int jbi = min(B, F.ncol - B * i);
+    if (wide && i - 2 > cb) prefetch_tile(A.L + F.loff + (int64_t)(B * (i - 2)) * F.ld + c0, F.ld, B);
     Vec<T> l[RW];
     const T *P = A.L + F.loff + (int64_t)(B * i + RW * g) * F.ld + c;
 #pragma unroll
     for (int k = 0; k < RW; k++)
       l[k] = (c < F.ncol && RW * g + k < jbi) ? ldg16(P + (int64_t)k * F.ld) : vzero<T>();
-    ok = wait_chain(A, S, f_x(A, slot0), i, cb + 1, -1);
+    // lane k < RW reads x of row RW g + k of block i; the warp shares them
+    T xv = T(0);
+    const bool mine = q < RW && RW * g + q < jbi;
+    const uint2 *words = slot_words<T>(A.lx, slot0 + i);
+    ok = wait_words(A, words, i == cb + 1, [&]() { return !mine || read_word(words, RW * g + q, A.epoch, xv); });
     if (!ok) break;
-    // lane k < RW loads x of row RW g + k of block i; the warp shares them
-    const T xv = (q < RW && RW * g + q < jbi) ? ldcg(A.x + F.first + B * i + RW * g + q) : T(0);
 #pragma unroll
     for (int k = 0; k < RW; k++) acc = vfma(l[k], __shfl_sync(0xffffffffu, xv, k), acc);
   }
   take_next(A, N);
   st16(S.red4[g] + VW * q, acc);
-  __syncthreads();
+  ok = __syncthreads_and(ok) != 0;
   if (ok)
     groups_sum(S, [&](int k0, auto s) {
       each_sum(k0, s, [&](int k, T v) {
         if (k < jb) S.sv[k] -= v;
       });
     });
-  const bool got = wait_dinv(A, S);  // (ends with a barrier)
-  if (ok && got) {
-    diag_bwd(A, S, F, c0);
-    signal(f_x(A, slot0 + cb));
-    if (threadIdx.x == 0)  // the release of signal() above already ordered the writes
-      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(f_front(A, tk.front)) : "memory");
+  if (wait_dinv(A, S, ok)) {  // (ends with a barrier)
+    diag_bwd(A, S, F, c0, slot0 + cb);
+    signal(f_front(A, tk.front));
   }
 }
 
@@ -903,17 +997,28 @@ void launch_dinv(const DevPlan &dp, const Plan &plan, const double *L, double *D
   dinv64_kernel<<<n, 64, 0, st>>>(dp, L, Dinv);
 }
 
+int64_t solve_words(const SolvePlan &sp) {  // one per FP32 value, two per FP64 value
+  return std::max<int64_t>((int64_t)sp.dinv_off.size() * sp.B * (sp.B == kSolveB64 ? 2 : 1), 2);
+}
+
 template <typename T>
 void launch_psolve(const DevPlan &dp, const Plan &plan, const T *L, const T *Dinv, T *a, T *b, T *x, T *t,
-                   T *part, unsigned *flags, int32_t *status, bool fwd, bool bwd, cudaStream_t st,
-                   unsigned test_spins, int test_withhold) {
+                   T *part, unsigned *flags, SolveWords &words, int32_t *status, bool fwd, bool bwd,
+                   cudaStream_t st, unsigned test_spins, int test_withhold) {
   const SolvePlan &sp = sizeof(T) == 8 ? plan.s64 : plan.s32;
   const int32_t q0 = fwd ? 0 : sp.fwd_tasks;
   const int32_t q1 = bwd ? (int32_t)sp.tasks.size() : sp.fwd_tasks;
   if (q1 <= q0) return;
   ck(cudaMemsetAsync(flags, 0, (size_t)sp.flag_words * sizeof(unsigned), st), "solve flags");
   const int grid = psolve_grid<T>(q1 - q0);
-  PsArgs<T> A{dp, sizeof(T) == 8 ? dp.s64 : dp.s32, L, Dinv, a, b, x, t, part, q0, q1, flags, status,
+  if (++words.epoch == 0) {  // the tags start over
+    const size_t bytes = solve_words(sp) * sizeof(uint2);
+    ck(cudaMemsetAsync(words.y, 0, bytes, st), "solve words");
+    ck(cudaMemsetAsync(words.x, 0, bytes, st), "solve words");
+    words.epoch = 1;
+  }
+  PsArgs<T> A{dp, sizeof(T) == 8 ? dp.s64 : dp.s32, L, Dinv, a, b, x, t, part, q0, q1, flags, words.y, words.x,
+              words.epoch, status,
               test_spins ? test_spins : kBarrierSpins, test_withhold,
               (int32_t)sp.dinv_off.size(), (int32_t)plan.fronts.size(), fwd && bwd ? 1 : 0};
   note_launch();
@@ -921,10 +1026,10 @@ void launch_psolve(const DevPlan &dp, const Plan &plan, const T *L, const T *Din
   ck(cudaGetLastError(), "solve launch");
 }
 template void launch_psolve<float>(const DevPlan &, const Plan &, const float *, const float *, float *,
-                                   float *, float *, float *, float *, unsigned *, int32_t *, bool, bool,
-                                   cudaStream_t, unsigned, int);
+                                   float *, float *, float *, float *, unsigned *, SolveWords &, int32_t *,
+                                   bool, bool, cudaStream_t, unsigned, int);
 template void launch_psolve<double>(const DevPlan &, const Plan &, const double *, const double *, double *,
-                                    double *, double *, double *, double *, unsigned *, int32_t *, bool,
-                                    bool, cudaStream_t, unsigned, int);
+                                    double *, double *, double *, double *, unsigned *, SolveWords &,
+                                    int32_t *, bool, bool, cudaStream_t, unsigned, int);
 
 }  // namespace gipm

@@ -42,6 +42,14 @@ void launch_sign(const DevPlan &dp, V *y, cudaStream_t st);
 // commits no device memory (lazy module loading); used by the allocation-free solve.
 cudaError_t preload_level_solve();
 
+// Tagged entries the persistent solve hands from block to block (zeroed once, before
+// the first launch; each launch takes the next tag): solve_words(plan) each.
+struct SolveWords {
+  uint2 *y = nullptr, *x = nullptr;
+  unsigned epoch = 0;
+};
+int64_t solve_words(const SolvePlan &sp);
+
 // Persistent solve: inverses of the diagonal blocks (after each factorisation
 // that does not write them itself), then x = L^{-T} L^{-1} a in one launch, with b
 // the forward result and t the update vectors. fwd/bwd select the sweeps: forward
@@ -55,8 +63,8 @@ void launch_dinv(const DevPlan &dp, const Plan &plan, const float *L, float *Din
 void launch_dinv(const DevPlan &dp, const Plan &plan, const double *L, double *Dinv, cudaStream_t st);
 template <typename T>
 void launch_psolve(const DevPlan &dp, const Plan &plan, const T *L, const T *Dinv, T *a, T *b, T *x, T *t,
-                   T *part, unsigned *flags, int32_t *status, bool fwd, bool bwd, cudaStream_t st,
-                   unsigned test_spins = 0, int test_withhold = -1);
+                   T *part, unsigned *flags, SolveWords &words, int32_t *status, bool fwd, bool bwd,
+                   cudaStream_t st, unsigned test_spins = 0, int test_withhold = -1);
 
 // Sampled entries of L (final numbering).
 template <typename T>

@@ -866,7 +866,7 @@ void build_fused_solve(const Plan &pl, int B, SolvePlan &sp) {
     }
   }
   const int64_t nslot = (int64_t)sp.dinv_off.size();
-  sp.flag_words = 32 + 3 * nslot + 2 * (int64_t)nfr;
+  sp.flag_words = 32 + nslot + 2 * (int64_t)nfr;
   // range checks (the kernel masks only the chunk edges), and the order every
   // wait of the kernel relies on: a task waits only for earlier tasks
   auto need = [](bool ok, const char *w) {
