@@ -25,6 +25,8 @@
 
 using namespace gipm;
 
+constexpr int kRhsScal = 16;  // device scalars of one right-hand side (see RhsRun)
+
 struct ipm_ctx {
   Problem P;
   Symbolic S;
@@ -41,7 +43,7 @@ struct ipm_ctx {
   DevPlan dp{};
   double *kval = nullptr;
   void *L = nullptr, *U = nullptr;
-  double *yv = nullptr, *tv = nullptr;  // solve scratch (doubles; float views)
+  double *yv = nullptr, *tv = nullptr;  // solve scratch (doubles; float views), kSolveRhs of each
   double *vx = nullptr, *vr = nullptr, *vc = nullptr, *vz = nullptr, *vp = nullptr,
          *vq = nullptr, *vb = nullptr, *vdx = nullptr, *vrd = nullptr, *vwx = nullptr;
   double *vg = nullptr, *vD = nullptr, *vw = nullptr, *vds = nullptr, *vdl = nullptr,
@@ -54,6 +56,8 @@ struct ipm_ctx {
   unsigned *psflags = nullptr;  // its tickets, flags and counters
   float *pspart = nullptr;    // its partial sums
   SolveWords psw32, psw64;    // its published entries
+  // do_solves: r, z, p, q of right-hand sides 1 .. (four n each), and the scalars of all (kRhsScal each)
+  double *vrk = nullptr, *rscal = nullptr;
   // learned correction of a stale factor
   LearnedBufs lb;
   bool learned_active = false;  // PCG preconditioner = corrected stale factor
@@ -267,8 +271,11 @@ void layout(ipm_ctx *c, char *base) {
   const size_t n = std::max<int64_t>(P.n, 1), mt = std::max<int64_t>(P.mt, 1),
                m = std::max<int32_t>(P.m, 1);
   c->kval = cv.take<double>(std::max<int64_t>(d.nk, 1));
-  c->yv = cv.take<double>(n);
-  c->tv = cv.take<double>(pl.t_entries);
+  constexpr size_t R = kSolveRhs;  // right-hand sides of one persistent solve
+  c->yv = cv.take<double>(R * n);
+  c->tv = cv.take<double>(R * pl.t_entries);
+  c->vrk = cv.take<double>(4 * (R - 1) * n);
+  c->rscal = cv.take<double>(kRhsScal * R);
   for (double **v : {&c->vx, &c->vr, &c->vc, &c->vz, &c->vp, &c->vq, &c->vb, &c->vdx, &c->vrd,
                      &c->vwx})
     *v = cv.take<double>(n);
@@ -280,19 +287,19 @@ void layout(ipm_ctx *c, char *base) {
   c->vjx = cv.take<double>(m);
   c->vtA = cv.take<double>(m);
   c->dinv = cv.take<float>(std::max<int64_t>(pl.s32.dinv_entries, 4));
-  c->fsa = cv.take<float>(n);
-  c->fsb = cv.take<float>(n);
-  c->fsx = cv.take<float>(n);
-  c->psflags = cv.take<unsigned>(std::max<int64_t>(std::max(pl.s32.flag_words, pl.s64.flag_words), 32));
-  c->pspart = cv.take<float>(std::max<int64_t>(pl.s32.part_entries, 1));
-  const int64_t nw32 = solve_words(pl.s32), nw64 = solve_words(pl.s64);
+  c->fsa = cv.take<float>(R * n);
+  c->fsb = cv.take<float>(R * n);
+  c->fsx = cv.take<float>(R * n);
+  c->psflags = cv.take<unsigned>(R * std::max<int64_t>(std::max(pl.s32.flag_words, pl.s64.flag_words), 32));
+  c->pspart = cv.take<float>(R * std::max<int64_t>(pl.s32.part_entries, 1));
+  const int64_t nw32 = R * solve_words(pl.s32), nw64 = R * solve_words(pl.s64);
   c->psw32.y = cv.take<uint2>(nw32);
   c->psw32.x = cv.take<uint2>(nw32);
   if (!pl.s64.tasks.empty()) {
     c->dinv64 = cv.take<double>(pl.s64.dinv_entries);
-    c->dsb = cv.take<double>(n);
-    c->dsx = cv.take<double>(n);
-    c->pspart64 = cv.take<double>(pl.s64.part_entries);
+    c->dsb = cv.take<double>(R * n);
+    c->dsx = cv.take<double>(R * n);
+    c->pspart64 = cv.take<double>(R * pl.s64.part_entries);
     c->psw64.y = cv.take<uint2>(nw64);
     c->psw64.x = cv.take<uint2>(nw64);
   }
@@ -414,65 +421,69 @@ ipm_status do_factor(ipm_ctx *c, int prec, int32_t *bad_col) {
 
 // One persistent solve launch over the workspace vectors: which = 0 both sweeps
 // (fsa -> fsx; FP64: yv -> dsx), 1 forward only (fsa -> fsb; yv -> dsb), 2 backward
-// only (fsb -> fsx; dsb -> dsx)
-template <typename T> void launch_held_solve(ipm_ctx *c, int which);
-template <> void launch_held_solve<float>(ipm_ctx *c, int which) {
-  launch_psolve<float>(c->dp, c->plan, (const float *)c->L, c->dinv, c->fsa, c->fsb, c->fsx,
-                       reinterpret_cast<float *>(c->tv), c->pspart, c->psflags, c->psw32, c->status, which != 2,
-                       which != 1, c->st, c->test_spins, c->test_withhold);
+// only (fsb -> fsx; dsb -> dsx), of the first nrhs right-hand sides there
+template <typename T> void launch_held_solve(ipm_ctx *c, int which, int nrhs) {
+  constexpr bool f64 = sizeof(T) == 8;
+  const SolvePlan &sp = f64 ? c->plan.s64 : c->plan.s32;
+  SolveWords &words = f64 ? c->psw64 : c->psw32;
+  SolveBufs<T> v;
+  if constexpr (f64) {
+    v.a = c->yv, v.b = c->dsb, v.x = c->dsx, v.t = c->tv, v.part = c->pspart64;
+  } else {
+    v.a = c->fsa, v.b = c->fsb, v.x = c->fsx, v.t = reinterpret_cast<float *>(c->tv), v.part = c->pspart;
+  }
+  v.flags = c->psflags;
+  v.sd = SolveStride{std::max<int64_t>(c->P.n, 1), c->plan.t_entries, sp.part_entries, sp.flag_words,
+                     solve_words(sp)};
+  const T *Dinv;
+  if constexpr (f64) Dinv = c->dinv64;
+  else Dinv = c->dinv;
+  launch_psolve<T>(c->dp, c->plan, (const T *)c->L, Dinv, v, nrhs, words, c->status, which != 2, which != 1,
+                   c->st, c->test_spins, c->test_withhold);
   c->test_spins = 0;
   c->test_withhold = -1;
 }
-template <> void launch_held_solve<double>(ipm_ctx *c, int which) {
-  launch_psolve<double>(c->dp, c->plan, (const double *)c->L, c->dinv64, c->yv, c->dsb, c->dsx, c->tv,
-                        c->pspart64, c->psflags, c->psw64, c->status, which != 2, which != 1, c->st, c->test_spins,
-                        c->test_withhold);
-  c->test_spins = 0;
-  c->test_withhold = -1;
-}
-void launch_fp32_solve(ipm_ctx *c, int which) { launch_held_solve<float>(c, which); }
+void launch_fp32_solve(ipm_ctx *c, int which) { launch_held_solve<float>(c, which, 1); }
 // Both sweeps, with K = L S L^T's signs between them for a quasi-definite system.
-template <typename T> void launch_both_sweeps(ipm_ctx *c, T *mid) {
-  if (!c->dp.sgn) return launch_held_solve<T>(c, 0);
-  launch_held_solve<T>(c, 1);
-  launch_sign<T>(c->dp, mid, c->st);
-  launch_held_solve<T>(c, 2);
+template <typename T> void launch_both_sweeps(ipm_ctx *c, T *mid, int nrhs) {
+  if (!c->dp.sgn) return launch_held_solve<T>(c, 0, nrhs);
+  launch_held_solve<T>(c, 1, nrhs);
+  for (int k = 0; k < nrhs; k++) launch_sign<T>(c->dp, mid + (int64_t)k * c->P.n, c->st);
+  launch_held_solve<T>(c, 2, nrhs);
 }
 
 // The preconditioner up to the final numbering's result: P b (times scale[0] for an
-// FP32-storage factor), the sweeps; y points to the result.
+// FP32-storage factor) into right-hand side k of the sweeps' vectors, the sweeps.
 bool factor_is_fp64(const ipm_ctx *c) { return c->storage_bytes == 8 && c->factor_prec == IPM_FP64; }
-void sweeps(ipm_ctx *c, const double *b, const double *scale) {
+void sweeps_in(ipm_ctx *c, const double *b, const double *scale, int k) {
   VecOps V = c->vec();
-  if (factor_is_fp64(c)) {
-    V.permute_in<double>(b, nullptr, c->yv);
-    launch_both_sweeps<double>(c, c->dsb);
-    return;
-  }
-  V.permute_in<float>(b, scale, c->fsa);
-  if (c->learned_active) {  // P^T L_s^{-T} (Delta + U U^T)^{-1} L_s^{-1} P b
+  const int64_t off = (int64_t)k * c->P.n;
+  if (factor_is_fp64(c)) V.permute_in<double>(b, nullptr, c->yv + off);
+  else V.permute_in<float>(b, scale, c->fsa + off);
+}
+void sweeps_run(ipm_ctx *c, int nrhs) {
+  if (factor_is_fp64(c)) return launch_both_sweeps<double>(c, c->dsb, nrhs);
+  if (c->learned_active) {  // P^T L_s^{-T} (Delta + U U^T)^{-1} L_s^{-1} P b (one right-hand side)
     launch_fp32_solve(c, 1);
     learned_apply(c->lb, c->fsb, c->st);
     launch_fp32_solve(c, 2);
   } else {
-    launch_both_sweeps<float>(c, c->fsb);
+    launch_both_sweeps<float>(c, c->fsb, nrhs);
   }
 }
-// out = M^{-1} b with the current factor (b, out: original numbering, device; scale:
-// 1 / max |b|)
-void apply_factor(ipm_ctx *c, const double *b, const double *scale, double *out, bool accumulate) {
+void sweeps_out(ipm_ctx *c, const double *scale, int k, double *out, bool accumulate) {
   VecOps V = c->vec();
-  sweeps(c, b, scale);
-  if (factor_is_fp64(c)) V.permute_out<double>(c->dsx, nullptr, out, accumulate);
-  else V.permute_out<float>(c->fsx, scale, out, accumulate);
+  const int64_t off = (int64_t)k * c->P.n;
+  if (factor_is_fp64(c)) V.permute_out<double>(c->dsx + off, nullptr, out, accumulate);
+  else V.permute_out<float>(c->fsx + off, scale, out, accumulate);
 }
-// z = M^{-1} r, rz = r . z, beta = rz / rz_old (when given)
-void apply_factor_dot(ipm_ctx *c, const double *r, const double *scale, double *z, const double *rz_old,
-                      double *rz, double *beta) {
+// As sweeps_out, with rz = r . out and beta = rz / rz_old (when given).
+void sweeps_out_dot(ipm_ctx *c, const double *scale, int k, const double *r, double *out, const double *rz_old,
+                    double *rz, double *beta) {
   VecOps V = c->vec();
-  sweeps(c, r, scale);
-  if (factor_is_fp64(c)) V.permute_out_dot<double>(c->dsx, nullptr, r, z, rz_old, rz, beta);
-  else V.permute_out_dot<float>(c->fsx, scale, r, z, rz_old, rz, beta);
+  const int64_t off = (int64_t)k * c->P.n;
+  if (factor_is_fp64(c)) V.permute_out_dot<double>(c->dsx + off, nullptr, r, out, rz_old, rz, beta);
+  else V.permute_out_dot<float>(c->fsx + off, scale, r, out, rz_old, rz, beta);
 }
 
 // A wait of the persistent solve that ran out of time: the launch drained and
@@ -490,115 +501,208 @@ void check_solve_barrier(ipm_ctx *c) {
 }
 
 // ---- solve with refinement / PCG ----------------------------------------------
-ipm_status do_solve(ipm_ctx *c, const double *b, double *x, int refine, ipm_solve_info *info) {
+// One right-hand side of do_solves. s: device scalars; 0, 1 |b| and its scale; 2, 3
+// |r| and its scale, 4 the solve's timeout word, 5 |x|; 8, 9 r . z of alternating PCG
+// iterations, 10 alpha, 11 beta.
+struct RhsRun {
+  const double *b;
+  double *x, *r, *z, *p, *q, *s;
+  double bn = 0.0, rel = 0.0, bwd = 0.0, prev = 0.0, rel0 = 0.0;
+  int iters = 0, used_pcg = 0, slow = 0, it = 0;
+  bool going = false;  // in the loop that runs
+};
+
+// Solves with K <= kSolveRhs right-hand sides, b[k n ..] -> x[k n ..] (K > 1: b and x
+// apart, no learned correction or warm start). They go through refinement and PCG side
+// by side: the triangular solves of a step are one launch, its residuals one
+// synchronisation, and who has converged drops out. info, status: K entries each.
+void do_solves(ipm_ctx *c, int K, const double *b, double *x, int refine, ipm_solve_info *info,
+               ipm_status *status) {
   if (c->state < 4) throw Fail{IPM_ERR_STATE, "kkt_solve before kkt_factor"};
   VecOps V = c->vec();
   const int64_t n = c->P.n;
   const ipm_options &o = c->opts;
-  double *r = c->vr, *z = c->vz, *p = c->vp, *q = c->vq;
-  // x is the running solution; b is copied only where the two overlap
-  const double *bb = b;
-  if (b < x + n && x < b + n) {
-    CK(cudaMemcpyAsync(c->vb, b, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
-    bb = c->vb;
+  RhsRun run[kSolveRhs];
+  for (int k = 0; k < K; k++) {
+    RhsRun &u = run[k];
+    u.b = b + k * n;
+    u.x = x + k * n;
+    double *v = c->vrk + 4 * (k - 1) * n;
+    u.r = k == 0 ? c->vr : v;
+    u.z = k == 0 ? c->vz : v + n;
+    u.p = k == 0 ? c->vp : v + 2 * n;
+    u.q = k == 0 ? c->vq : v + 3 * n;
+    u.s = c->rscal + kRhsScal * k;
   }
-  // scalars: 0, 1 |b| and its scale; 2, 3 |r| and its scale, 4 the solve's timeout word, 5 |x|
-  // (bwd_measure); 6, 7 rz of alternating iterations; 8 alpha, 9 beta
-  double *sN = c->scal, *sR = sN + 2;
+  // x is the running solution; b is copied only where the two overlap
+  if (b < x + K * n && x < b + K * n) {
+    CK(cudaMemcpyAsync(c->vb, b, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
+    run[0].b = c->vb;
+  }
   const int pcg_max = c->pcg_override >= 0 ? c->pcg_override : o.pcg_max;
-  V.absmax(n, bb, sN, true);
-  if (info) *info = ipm_solve_info{0, 0, 0.0};
+  for (int k = 0; k < K; k++) V.absmax(n, run[k].b, run[k].s, true);
+  // the right-hand sides a step is for
+  RhsRun *act[kSolveRhs];
+  int na = 0;
+  auto collect = [&](auto want) {
+    na = 0;
+    for (int k = 0; k < K; k++)
+      if (want(run[k])) act[na++] = &run[k];
+    return na > 0;
+  };
+  auto going = [](const RhsRun &u) { return u.going; };
+  double h[kRhsScal * kSolveRhs];
+  auto scalars = [&]() {  // to the host
+    CK(cudaMemcpyAsync(h, c->rscal, kRhsScal * K * sizeof(double), cudaMemcpyDeviceToHost, c->st));
+    CK(cudaStreamSynchronize(c->st));
+  };
+  auto host = [&](const RhsRun &u) { return h + (u.s - c->rscal); };
   // ||b - K x|| / ||b|| drives refinement. For a badly scaled matrix (the grid
   // NLP: entries up to (nx+1)^4 times D) its floor is about eps ||K|| ||x|| / ||b||,
   // so with bwd_measure the solve is accepted on the normwise backward error
   // ||b - K x|| / (||K|| ||x|| + ||b||) instead (refinement still runs until it stalls).
-  double bwd = 0.0, bn = 0.0;
   bool timed_out = false;
-  auto residual = [&](const double *xv) {
-    V.residual(c->cur_jvals, c->cur_D, c->cur_wvals, c->cur_delta_p, xv, bb, r, c->vtA, sR,
-               c->status + ST_SOLVE_TIMEOUT);
-    if (c->bwd_measure) V.absmax(n, xv, sN + 5);
-    double h[6];
-    CK(cudaMemcpyAsync(h, sN, sizeof(h), cudaMemcpyDeviceToHost, c->st));
-    CK(cudaStreamSynchronize(c->st));
-    bn = h[0];
-    timed_out = h[4] != 0.0;
-    if (c->bwd_measure) bwd = h[2] / (c->knorm * h[5] + bn);
-    return h[2] / bn;
+  auto residuals = [&]() {
+    for (int k = 0; k < na; k++) {
+      RhsRun &u = *act[k];
+      V.residual(c->cur_jvals, c->cur_D, c->cur_wvals, c->cur_delta_p, u.x, u.b, u.r, c->vtA, u.s + 2,
+                 c->status + ST_SOLVE_TIMEOUT);
+      if (c->bwd_measure) V.absmax(n, u.x, u.s + 5);
+    }
+    scalars();
+    for (int k = 0; k < na; k++) {
+      RhsRun &u = *act[k];
+      const double *hs = host(u);
+      u.bn = hs[0];
+      timed_out = timed_out || hs[4] != 0.0;
+      if (c->bwd_measure) u.bwd = hs[2] / (c->knorm * hs[5] + u.bn);
+      u.rel = hs[2] / u.bn;
+    }
   };
-  double rel;
+  // x (+)= M^{-1} (b, or its residual) with the current factor
+  auto apply = [&](bool from_b, bool accumulate) {
+    const int sc = from_b ? 1 : 3;
+    for (int k = 0; k < na; k++) sweeps_in(c, from_b ? act[k]->b : act[k]->r, act[k]->s + sc, k);
+    sweeps_run(c, na);
+    for (int k = 0; k < na; k++) sweeps_out(c, act[k]->s + sc, k, act[k]->x, accumulate);
+  };
+  // PCG: z (first: p) = M^{-1} r, r . z and beta
+  auto precondition = [&](bool first) {
+    for (int k = 0; k < na; k++) sweeps_in(c, act[k]->r, act[k]->s + 3, k);
+    sweeps_run(c, na);
+    for (int k = 0; k < na; k++) {
+      RhsRun &u = *act[k];
+      double *now = u.s + 8 + u.it % 2, *old = u.s + 8 + (u.it + 1) % 2;
+      sweeps_out_dot(c, u.s + 3, k, u.r, first ? u.p : u.z, first ? nullptr : old, now, first ? nullptr : u.s + 11);
+    }
+  };
+  collect([](const RhsRun &) { return true; });
   if (c->warm_x) {  // x holds a nearby solution (the predictor's direction)
-    residual(x);
-    if (bn > 0.0) apply_factor(c, r, sR + 1, x, true);
+    residuals();
+    if (run[0].bn > 0.0) apply(false, true);
   } else {
-    apply_factor(c, bb, sN + 1, x, false);
+    apply(true, false);
   }
-  rel = residual(x);
-  if (bn == 0.0) {
-    CK(cudaMemsetAsync(x, 0, n * sizeof(double), c->st));
-    if (timed_out) report_solve_timeout(c);
-    c->last_rel = 0.0;
-    return IPM_OK;
+  residuals();
+  for (int k = 0; k < K; k++) {
+    RhsRun &u = run[k];
+    u.prev = u.rel;
+    u.going = refine != IPM_REFINE_NONE && refine != IPM_REFINE_PCG && u.bn != 0.0 && u.rel > o.ir_tol && o.ir_max > 0;
   }
-  int iters = 0, used_pcg = 0;
-  if (refine != IPM_REFINE_NONE && refine != IPM_REFINE_PCG) {
-    double prev = rel;
-    int slow = 0;
-    while (rel > o.ir_tol && iters < o.ir_max) {
-      apply_factor(c, r, sR + 1, x, true);
-      iters++;
-      rel = residual(x);
-      if (!(rel < 0.5 * prev)) slow++;
-      else slow = 0;
-      prev = std::min(prev, rel);
-      if (slow >= 2 || !std::isfinite(rel)) break;
+  while (collect(going)) {
+    apply(false, true);
+    residuals();
+    for (int k = 0; k < na; k++) {
+      RhsRun &u = *act[k];
+      u.iters++;
+      c->refine_steps++;
+      if (!(u.rel < 0.5 * u.prev)) u.slow++;
+      else u.slow = 0;
+      u.prev = std::min(u.prev, u.rel);
+      u.going = u.slow < 2 && u.rel > o.ir_tol && u.iters < o.ir_max;  // (a residual that is not finite ends it)
+      if (!std::isfinite(u.rel)) u.going = false;
     }
-    c->refine_steps += iters;
   }
-  if ((refine == IPM_REFINE_PCG || refine == IPM_REFINE_IR) && (rel > o.ir_tol || !std::isfinite(rel)) &&
-      !(c->bwd_measure && bwd <= o.ir_tol && std::isfinite(rel))) {
-    // PCG on K x = b preconditioned by the factor, from the current x
-    if (!std::isfinite(rel)) {
-      CK(cudaMemsetAsync(x, 0, n * sizeof(double), c->st));
-      rel = residual(x);
+  auto pcg = [&](const RhsRun &u) {
+    return u.bn != 0.0 && (refine == IPM_REFINE_PCG || refine == IPM_REFINE_IR) &&
+           (u.rel > o.ir_tol || !std::isfinite(u.rel)) &&
+           !(c->bwd_measure && u.bwd <= o.ir_tol && std::isfinite(u.rel));
+  };
+  // PCG on K x = b preconditioned by the factor, from the current x
+  if (collect(pcg)) {
+    for (int k = 0; k < na; k++) act[k]->used_pcg = 1;
+    auto restart = [](const RhsRun &u) { return u.used_pcg && !std::isfinite(u.rel); };
+    if (collect(restart)) {
+      for (int k = 0; k < na; k++) CK(cudaMemsetAsync(act[k]->x, 0, n * sizeof(double), c->st));
+      residuals();
     }
-    used_pcg = 1;
-    double *rz = sN + 6, *rz_next = sN + 7, *alpha = sN + 8, *beta = sN + 9;
-    apply_factor_dot(c, r, sR + 1, p, nullptr, rz, nullptr);  // p = z
-    const double rel0 = rel;
-    int k = 0;
-    for (; k < pcg_max && rel > o.ir_tol; k++) {
-      V.kp_dot(c->cur_jvals, c->cur_D, c->cur_wvals, c->cur_delta_p, p, q, c->vtA, rz, alpha);
-      V.cg_step(n, alpha, p, q, x, r, sR);
-      rel = d2h_scalar(c, sR) / bn;
-      if (rel <= o.ir_tol || !std::isfinite(rel)) { k++; break; }
-      // a corrected stale factor is only worth keeping if PCG converges
-      // within the budget: from the fifth iteration on, give up once the mean
-      // contraction so far projects past pcg_max
-      if (c->learned_active && k + 1 >= 5) {
-        if (!(rel < rel0)) { k++; break; }
-        const double rate = std::log(rel / rel0) / (k + 1);  // < 0
-        const double need = (k + 1) + std::log(o.ir_tol / rel) / rate;
-        if (need > pcg_max) { k++; break; }
+    auto used = [](const RhsRun &u) { return u.used_pcg != 0; };
+    collect(used);
+    precondition(true);  // p = z
+    for (int k = 0; k < na; k++) {
+      RhsRun &u = *act[k];
+      u.rel0 = u.rel;
+      u.going = u.it < pcg_max && u.rel > o.ir_tol;
+    }
+    while (collect(going)) {
+      for (int k = 0; k < na; k++) {
+        RhsRun &u = *act[k];
+        V.kp_dot(c->cur_jvals, c->cur_D, c->cur_wvals, c->cur_delta_p, u.p, u.q, c->vtA, u.s + 8 + u.it % 2, u.s + 10);
+        V.cg_step(n, u.s + 10, u.p, u.q, u.x, u.r, u.s + 2);
       }
-      apply_factor_dot(c, r, sR + 1, z, rz, rz_next, beta);
-      V.cg_direction(n, beta, z, p);
-      std::swap(rz, rz_next);
+      scalars();
+      for (int k = 0; k < na; k++) {
+        RhsRun &u = *act[k];
+        u.rel = host(u)[2] / u.bn;
+        u.it++;
+        if (u.rel <= o.ir_tol || !std::isfinite(u.rel) || u.it >= pcg_max) u.going = false;
+        // a corrected stale factor is only worth keeping if PCG converges
+        // within the budget: from the fifth iteration on, give up once the mean
+        // contraction so far projects past pcg_max
+        if (u.going && c->learned_active && u.it >= 5) {
+          const double rate = std::log(u.rel / u.rel0) / u.it;  // < 0
+          const double need = u.it + std::log(o.ir_tol / u.rel) / rate;
+          if (!(u.rel < u.rel0) || need > pcg_max) u.going = false;
+        }
+      }
+      if (!collect(going)) break;
+      precondition(false);
+      for (int k = 0; k < na; k++) V.cg_direction(n, act[k]->s + 11, act[k]->z, act[k]->p);
     }
-    c->pcg_steps += k;
-    iters += k;
-    rel = residual(x);  // true residual of the returned iterate
+    collect(used);
+    for (int k = 0; k < na; k++) {
+      c->pcg_steps += act[k]->it;
+      act[k]->iters += act[k]->it;
+    }
+    residuals();  // true residuals of the returned iterates
   }
+  for (int k = 0; k < K; k++)
+    if (run[k].bn == 0.0) CK(cudaMemsetAsync(run[k].x, 0, n * sizeof(double), c->st));
   CK(cudaGetLastError());
   if (timed_out) report_solve_timeout(c);
-  if (c->bwd_measure) rel = bwd;
-  c->last_rel = rel;
-  if (info) *info = ipm_solve_info{iters, used_pcg, rel};
-  if (!(rel <= o.accept_tol)) {
-    c->err = "linear solve residual " + std::to_string(rel) + " above accept_tol";
-    return IPM_ERR_NUMERIC;
+  for (int k = 0; k < K; k++) {
+    RhsRun &u = run[k];
+    status[k] = IPM_OK;
+    if (u.bn == 0.0) {
+      info[k] = ipm_solve_info{0, 0, 0.0};
+      c->last_rel = 0.0;
+      continue;
+    }
+    const double rel = c->bwd_measure ? u.bwd : u.rel;
+    c->last_rel = rel;
+    info[k] = ipm_solve_info{u.iters, u.used_pcg, rel};
+    if (!(rel <= o.accept_tol)) {
+      c->err = "linear solve residual " + std::to_string(rel) + " above accept_tol";
+      status[k] = IPM_ERR_NUMERIC;
+    }
   }
-  return IPM_OK;
+}
+ipm_status do_solve(ipm_ctx *c, const double *b, double *x, int refine, ipm_solve_info *info) {
+  ipm_solve_info one{};
+  ipm_status st = IPM_OK;
+  do_solves(c, 1, b, x, refine, &one, &st);
+  if (info) *info = one;
+  return st;
 }
 
 void set_assembly(ipm_ctx *c, const double *wv, const double *jv, const double *D, double dp) {
@@ -1111,8 +1215,8 @@ ipm_status ipm_set_workspace(ipm_ctx *c, void *buf, size_t bytes) {
                          {&c->psw64, &c->plan.s64}}) {
       w->epoch = 0;  // no word carries a tag yet
       if (sp->tasks.empty()) continue;
-      CK(cudaMemsetAsync(w->y, 0, solve_words(*sp) * sizeof(uint2), c->st));
-      CK(cudaMemsetAsync(w->x, 0, solve_words(*sp) * sizeof(uint2), c->st));
+      CK(cudaMemsetAsync(w->y, 0, kSolveRhs * solve_words(*sp) * sizeof(uint2), c->st));
+      CK(cudaMemsetAsync(w->x, 0, kSolveRhs * solve_words(*sp) * sizeof(uint2), c->st));
     }
     CK(cudaStreamSynchronize(c->st));
     if (c->sys) {  // the formulation's system takes the rest of the buffer
@@ -1178,14 +1282,22 @@ ipm_status kkt_solve(ipm_ctx *c, const double *b, double *x, int32_t nrhs, int32
     const int64_t n = t->P.n;
     ipm_solve_info all{0, 0, 0.0};
     ipm_status worst = IPM_OK;
-    for (int32_t k = 0; k < nrhs; k++) {
-      ipm_solve_info one{};
-      const ipm_status st = do_solve(t, b + k * n, x + k * n, refine, &one);
-      if (st != IPM_OK && t != c) c->err = t->err;
-      all.iterations += one.iterations;
-      all.used_pcg = std::max(all.used_pcg, one.used_pcg);
-      all.rel_residual = std::max(all.rel_residual, one.rel_residual);
-      if (st != IPM_OK && worst == IPM_OK) worst = st;
+    // in groups that share the sweeps; one by one where b and x overlap (a solve may
+    // then overwrite the next right-hand side)
+    const bool apart = !(b < x + nrhs * n && x < b + nrhs * n) && !t->learned_active && !t->warm_x;
+    for (int32_t k = 0; k < nrhs;) {
+      const int K = apart ? std::min(nrhs - k, kSolveRhs) : 1;
+      ipm_solve_info one[kSolveRhs];
+      ipm_status st[kSolveRhs];
+      do_solves(t, K, b + k * n, x + k * n, refine, one, st);
+      for (int q = 0; q < K; q++) {
+        if (st[q] != IPM_OK && t != c) c->err = t->err;
+        all.iterations += one[q].iterations;
+        all.used_pcg = std::max(all.used_pcg, one[q].used_pcg);
+        all.rel_residual = std::max(all.rel_residual, one[q].rel_residual);
+        if (st[q] != IPM_OK && worst == IPM_OK) worst = st[q];
+      }
+      k += K;
     }
     if (info) *info = all;
     return worst;
@@ -1583,7 +1695,7 @@ ipm_status kkt_time_kernel(ipm_ctx *c, int32_t kernel, int32_t reps, double *ms)
       else if (kernel == 3 || kernel == 4)
         launch_fp32_solve(c, kernel == 3 ? 1 : 2);
       else
-        launch_held_solve<double>(c, 0);
+        launch_held_solve<double>(c, 0, 1);
     }
     CK(cudaEventRecord(e1, c->st));
     CK(cudaEventSynchronize(e1));

@@ -171,7 +171,8 @@ template <typename T> struct PsArgs {
   const T *L, *Dinv;
   T *a, *b, *x, *t, *part;
   int32_t q0, q1;    // tasks [q0, q1) of the plan
-  unsigned *flags;   // the solve plan's flag words, zeroed before the launch
+  unsigned *ticket;  // ticket counter, and the solve plan's flag words, zeroed before the launch
+  unsigned *flags;
   uint2 *ly, *lx;    // published entries of y and x (see LL words), B per slot (FP64: 2 B)
   unsigned epoch;    // tag of this launch's entries
   int32_t *status;   // ST_SOLVE_TIMEOUT
@@ -179,7 +180,21 @@ template <typename T> struct PsArgs {
   int32_t withhold;  // test of the bounded wait: the task of this ticket is abandoned (-1: none)
   int32_t nslot, nfr;
   int32_t fwd_here;  // the forward sweep runs in this launch: backward blocks wait for their y
+  int32_t nrhs;      // right-hand sides; ticket k is task k / nrhs of right-hand side k % nrhs
+  SolveStride sd;    // from one right-hand side's vectors, flags and words to the next
 };
+
+// The vectors, flags and words of right-hand side k.
+template <typename T> __device__ __forceinline__ void shift_rhs(PsArgs<T> &A, int k) {
+  A.a += k * A.sd.n;
+  A.b += k * A.sd.n;
+  A.x += k * A.sd.n;
+  A.t += k * A.sd.t;
+  A.part += k * A.sd.part;
+  A.flags += k * A.sd.flags;
+  A.ly += k * A.sd.words;
+  A.lx += k * A.sd.words;
+}
 
 constexpr int kMaxKids = 32;  // children staged in shared memory for the gathers
 constexpr long long kCopySpinCycles = 2000000000ll;  // bounded wait on a staging copy (~1 s)
@@ -192,8 +207,6 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) {
 
 // Flag words (see SolvePlan): tickets, then per slot partial sums done, per front
 // update-vector chunks and column blocks done.
-template <typename T>
-__device__ __forceinline__ unsigned *f_ticket(const PsArgs<T> &A) { return A.flags; }
 template <typename T>
 __device__ __forceinline__ unsigned *f_part(const PsArgs<T> &A, int slot) {
   return A.flags + 32 + slot;
@@ -220,6 +233,7 @@ template <typename T> struct PsShared {
   unsigned long long mbar;      // completion of the staging copy
   uint32_t parity;              // its phase
   int tk;                       // this CTA's current task
+  int rhs;                      // and its right-hand side
   int ok;                       // outcome of the last wait
   int nkids;                    // children of the task's front staged below
   int64_t kid_inv[kMaxKids];    // their child -> front map offsets
@@ -692,14 +706,14 @@ __device__ __forceinline__ T gather_children(const PsArgs<T> &A, const PsShared<
 // the record then overlap the task's remaining work, and no CTA ever holds a
 // ticket while it waits, so the smallest unfinished ticket is always running.
 struct Next {
-  int q;
+  int q;  // ticket
   bool have;
 };
 
 template <typename T>
 __device__ __forceinline__ void take_next(const PsArgs<T> &A, Next &N) {
   if (threadIdx.x == 32 && !N.have) {
-    N.q = (int)atomicAdd(f_ticket(A), 1u) + A.q0;  // the result is first read after the task
+    N.q = (int)atomicAdd(A.ticket, 1u);  // the result is first read after the task
     N.have = true;
   }
 }
@@ -907,9 +921,21 @@ __device__ void bwd_diag(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R, 
   }
 }
 
+template <typename T> __device__ __forceinline__ void run_task(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R, Next &N) {
+  switch (R.task.c) {
+    case WS_FWD_DIAG: fwd_diag(A, S, R, N); break;
+    case WS_FWD_BELOW: fwd_below(A, S, R, N); break;
+    case WS_BWD_PART: bwd_part(A, S, R, N); break;
+    default: bwd_diag(A, S, R, N); break;
+  }
+}
+
 // Persistent solve: every CTA takes tasks in plan order from the global ticket
-// counter until the range is exhausted.
-template <typename T> __global__ void __launch_bounds__(kT, 2) psolve_kernel(PsArgs<T> A) {
+// counter until the range is exhausted. With several right-hand sides (MANY) each
+// task comes once per right-hand side, next to each other: their chains of blocks,
+// which leave most of the chip waiting, run side by side, and a tile of L is read
+// from DRAM once for all of them.
+template <typename T, bool MANY> __global__ void __launch_bounds__(kT, 2) psolve_kernel(PsArgs<T> A) {
   extern __shared__ __align__(128) unsigned char ps_smem[];
   PsShared<T> &S = *reinterpret_cast<PsShared<T> *>(ps_smem);
   // Thread 32 takes the tickets: the first here, each next one inside the
@@ -918,17 +944,19 @@ template <typename T> __global__ void __launch_bounds__(kT, 2) psolve_kernel(PsA
   // shared buffer while the CTA finishes the current one.
   Next N{0, false};
   int cur = 0;
+  auto fetch = [&](int ticket, int buf) {  // thread 32: the ticket's task
+    const int q = A.q0 + (MANY ? ticket / A.nrhs : ticket);
+    fetch_rec(A, S, q, buf);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    S.tk = q;
+    if (MANY) S.rhs = ticket % A.nrhs;
+  };
   if (threadIdx.x == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&S.mbar)), "r"(1u));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     S.parity = 0;
   }
-  if (threadIdx.x == 32) {
-    const int q = (int)atomicAdd(f_ticket(A), 1u) + A.q0;
-    fetch_rec(A, S, q, 0);
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    S.tk = q;
-  }
+  if (threadIdx.x == 32) fetch((int)atomicAdd(A.ticket, 1u), 0);
   __syncthreads();
   while (true) {
     const int qt = S.tk;
@@ -938,39 +966,35 @@ template <typename T> __global__ void __launch_bounds__(kT, 2) psolve_kernel(PsA
     if (qt == A.withhold) {
       // abandoned (test of the bounded waits): the tasks that need its result
       // run out of time
-    } else switch (R.task.c) {
-      case WS_FWD_DIAG: fwd_diag(A, S, R, N); break;
-      case WS_FWD_BELOW: fwd_below(A, S, R, N); break;
-      case WS_BWD_PART: bwd_part(A, S, R, N); break;
-      default: bwd_diag(A, S, R, N); break;
+    } else if (MANY) {
+      PsArgs<T> Ak = A;
+      shift_rhs(Ak, S.rhs);
+      run_task(Ak, S, R, N);
+    } else {
+      run_task(A, S, R, N);
     }
     take_next(A, N);  // a task that gave up early
-    if (threadIdx.x == 32) {
-      fetch_rec(A, S, N.q, cur ^ 1);
-      asm volatile("cp.async.wait_all;" ::: "memory");
-      S.tk = N.q;
-    }
+    if (threadIdx.x == 32) fetch(N.q, cur ^ 1);
     __syncthreads();  // the next record has landed; the shared scratch is free
     cur ^= 1;
   }
 }
 
-template <typename T> int psolve_grid(int ntask) {
+template <typename T, bool MANY> int psolve_grid(int64_t ntask) {
   static int per_device[64] = {0};
   int dev = 0;
   ck(cudaGetDevice(&dev), "cudaGetDevice");
   int &g = per_device[dev & 63];
   if (g == 0) {
     int sms = 0, nb = 0;
-    ck(cudaFuncSetAttribute(psolve_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                            (int)sizeof(PsShared<T>)),
+    auto kernel = psolve_kernel<T, MANY>;
+    ck(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PsShared<T>)),
        "solve shared-memory attribute");
     ck(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
-    ck(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, psolve_kernel<T>, kT, sizeof(PsShared<T>)),
-       "occupancy");
+    ck(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, kT, sizeof(PsShared<T>)), "occupancy");
     g = std::max(1, sms * std::min(nb, 2));
   }
-  return std::max(1, std::min(g, ntask));
+  return (int)std::max<int64_t>(1, std::min<int64_t>(g, ntask));
 }
 
 }  // namespace
@@ -1002,34 +1026,34 @@ int64_t solve_words(const SolvePlan &sp) {  // one per FP32 value, two per FP64 
 }
 
 template <typename T>
-void launch_psolve(const DevPlan &dp, const Plan &plan, const T *L, const T *Dinv, T *a, T *b, T *x, T *t,
-                   T *part, unsigned *flags, SolveWords &words, int32_t *status, bool fwd, bool bwd,
-                   cudaStream_t st, unsigned test_spins, int test_withhold) {
+void launch_psolve(const DevPlan &dp, const Plan &plan, const T *L, const T *Dinv, const SolveBufs<T> &v,
+                   int nrhs, SolveWords &words, int32_t *status, bool fwd, bool bwd, cudaStream_t st,
+                   unsigned test_spins, int test_withhold) {
   const SolvePlan &sp = sizeof(T) == 8 ? plan.s64 : plan.s32;
   const int32_t q0 = fwd ? 0 : sp.fwd_tasks;
   const int32_t q1 = bwd ? (int32_t)sp.tasks.size() : sp.fwd_tasks;
   if (q1 <= q0) return;
-  ck(cudaMemsetAsync(flags, 0, (size_t)sp.flag_words * sizeof(unsigned), st), "solve flags");
-  const int grid = psolve_grid<T>(q1 - q0);
+  ck(cudaMemsetAsync(v.flags, 0, (size_t)(nrhs * v.sd.flags) * sizeof(unsigned), st), "solve flags");
   if (++words.epoch == 0) {  // the tags start over
-    const size_t bytes = solve_words(sp) * sizeof(uint2);
+    const size_t bytes = (size_t)(kSolveRhs * v.sd.words) * sizeof(uint2);
     ck(cudaMemsetAsync(words.y, 0, bytes, st), "solve words");
     ck(cudaMemsetAsync(words.x, 0, bytes, st), "solve words");
     words.epoch = 1;
   }
-  PsArgs<T> A{dp, sizeof(T) == 8 ? dp.s64 : dp.s32, L, Dinv, a, b, x, t, part, q0, q1, flags, words.y, words.x,
-              words.epoch, status,
-              test_spins ? test_spins : kBarrierSpins, test_withhold,
-              (int32_t)sp.dinv_off.size(), (int32_t)plan.fronts.size(), fwd && bwd ? 1 : 0};
+  PsArgs<T> A{dp, sizeof(T) == 8 ? dp.s64 : dp.s32, L, Dinv, v.a, v.b, v.x, v.t, v.part, q0, q1, v.flags, v.flags,
+              words.y, words.x, words.epoch, status, test_spins ? test_spins : kBarrierSpins, test_withhold,
+              (int32_t)sp.dinv_off.size(), (int32_t)plan.fronts.size(), fwd && bwd ? 1 : 0, nrhs, v.sd};
+  const int64_t tickets = (int64_t)(q1 - q0) * nrhs;
   note_launch();
-  psolve_kernel<T><<<grid, kT, sizeof(PsShared<T>), st>>>(A);
+  if (nrhs == 1) psolve_kernel<T, false><<<psolve_grid<T, false>(tickets), kT, sizeof(PsShared<T>), st>>>(A);
+  else psolve_kernel<T, true><<<psolve_grid<T, true>(tickets), kT, sizeof(PsShared<T>), st>>>(A);
   ck(cudaGetLastError(), "solve launch");
 }
-template void launch_psolve<float>(const DevPlan &, const Plan &, const float *, const float *, float *,
-                                   float *, float *, float *, float *, unsigned *, SolveWords &, int32_t *,
-                                   bool, bool, cudaStream_t, unsigned, int);
-template void launch_psolve<double>(const DevPlan &, const Plan &, const double *, const double *, double *,
-                                    double *, double *, double *, double *, unsigned *, SolveWords &,
-                                    int32_t *, bool, bool, cudaStream_t, unsigned, int);
+template void launch_psolve<float>(const DevPlan &, const Plan &, const float *, const float *,
+                                   const SolveBufs<float> &, int, SolveWords &, int32_t *, bool, bool,
+                                   cudaStream_t, unsigned, int);
+template void launch_psolve<double>(const DevPlan &, const Plan &, const double *, const double *,
+                                    const SolveBufs<double> &, int, SolveWords &, int32_t *, bool, bool,
+                                    cudaStream_t, unsigned, int);
 
 }  // namespace gipm

@@ -50,6 +50,22 @@ struct SolveWords {
 };
 int64_t solve_words(const SolvePlan &sp);
 
+// The vectors of a persistent solve: right-hand sides, forward results, solutions,
+// update vectors, partial sums and flags of up to kSolveRhs right-hand sides, each
+// kind `sd` apart from one to the next (t in values of T). A solve is bound by its
+// chain of diagonal blocks, so right-hand sides side by side cost little until they
+// fill the chip: 56^3 TF32x3, eight right-hand sides with PCG: 27.4 ms one by one,
+// 16.6 in fours, 15.2 as eight.
+constexpr int kSolveRhs = 8;
+struct SolveStride {
+  int64_t n = 0, t = 0, part = 0, flags = 0, words = 0;
+};
+template <typename T> struct SolveBufs {
+  T *a = nullptr, *b = nullptr, *x = nullptr, *t = nullptr, *part = nullptr;
+  unsigned *flags = nullptr;
+  SolveStride sd;
+};
+
 // Persistent solve: inverses of the diagonal blocks (after each factorisation
 // that does not write them itself), then x = L^{-T} L^{-1} a in one launch, with b
 // the forward result and t the update vectors. fwd/bwd select the sweeps: forward
@@ -62,9 +78,9 @@ int64_t solve_words(const SolvePlan &sp);
 void launch_dinv(const DevPlan &dp, const Plan &plan, const float *L, float *Dinv, cudaStream_t st);
 void launch_dinv(const DevPlan &dp, const Plan &plan, const double *L, double *Dinv, cudaStream_t st);
 template <typename T>
-void launch_psolve(const DevPlan &dp, const Plan &plan, const T *L, const T *Dinv, T *a, T *b, T *x, T *t,
-                   T *part, unsigned *flags, SolveWords &words, int32_t *status, bool fwd, bool bwd,
-                   cudaStream_t st, unsigned test_spins = 0, int test_withhold = -1);
+void launch_psolve(const DevPlan &dp, const Plan &plan, const T *L, const T *Dinv, const SolveBufs<T> &v,
+                   int nrhs, SolveWords &words, int32_t *status, bool fwd, bool bwd, cudaStream_t st,
+                   unsigned test_spins = 0, int test_withhold = -1);
 
 // Sampled entries of L (final numbering).
 template <typename T>
