@@ -75,6 +75,7 @@ struct ipm_ctx {
   unsigned *ticket = nullptr;  // of the reductions (VecOps), zeroed when the workspace is set
   IpmScalars *sc = nullptr;
   int32_t *status = nullptr, *col2s = nullptr;
+  ChainStream chain;   // of the FMA-pipe FP64 factor
   TcPlan tcp;
   OzPlan ozp;          // FP64 factor on tensor cores (Ozaki slices), with options.fp64_tc
   bool oz_on = false;  // its task lists and slice storage were sized by kkt_analyze
@@ -372,10 +373,10 @@ ipm_status do_factor(ipm_ctx *c, int prec, int32_t *bad_col) {
     c->ozp.factor(c->dp, c->plan, c->kval, (double *)c->L, (double *)c->U, c->status, c->st);
   } else if (prec == IPM_FP64) {
     launch_factor_simt<double>(c->dp, c->plan, c->kval, (double *)c->L, (double *)c->U, c->status,
-                               false, c->st);
+                               false, c->chain, c->st);
   } else if (prec == IPM_FP32) {
     launch_factor_simt<float>(c->dp, c->plan, c->kval, (float *)c->L, (float *)c->U, c->status,
-                              true, c->st);
+                              true, c->chain, c->st);
   } else {
     if (!c->tcp.ready()) throw Fail{IPM_ERR_UNSUPPORTED, "tensor-core factor not prepared"};
     c->tcp.factor(c->dp, c->plan, c->kval, (float *)c->L, (float *)c->U, c->dinv, c->status,
@@ -396,7 +397,7 @@ ipm_status do_factor(ipm_ctx *c, int prec, int32_t *bad_col) {
     // FP64 factor of the same matrix decides before the caller regularises.
     CK(cudaMemcpyAsync(c->status, init, sizeof(init), cudaMemcpyHostToDevice, c->st));
     launch_factor_simt<double>(c->dp, c->plan, c->kval, (double *)c->L, (double *)c->U, c->status,
-                               false, c->st);
+                               false, c->chain, c->st);
     launch_dinv(c->dp, c->plan, (const double *)c->L, c->dinv64, c->st);
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(out, c->status, sizeof(out), cudaMemcpyDeviceToHost, c->st));
@@ -1233,6 +1234,7 @@ ipm_status ipm_set_workspace(ipm_ctx *c, void *buf, size_t bytes) {
     CK(preload_vec_kernels());
     c->have_stale = false;
     if (c->lb_on) learned_init_weights(c);
+    if (!c->sys) c->chain.create();
     try {  // tensor maps of the FP32 panels for the tensor-core path
       if (!c->sys) c->tcp.encode(c->plan, (float *)c->L, c->Llo, (float *)c->U, c->st);
     } catch (const std::exception &e) {

@@ -90,26 +90,26 @@ enum SolveTaskKind : int32_t {
 // front's first block of the launch, b = first column of the step} per front,
 // and a block finds its front by bisection, so a front's O((nf / tile)^2)
 // update tiles need no list.
+constexpr int64_t kSms = 152;  // SMs the schedules are made for
 constexpr int kTrsmRows = 16;  // rows per batch of a panel solve's blocks
 // Batches per block, for `rows` rows in the launch: one while every block has an
 // SM of its own (a launch then lasts one batch), up to four beyond that, which
 // read the diagonal block once per 64 rows.
 inline int trsm_batches(int64_t rows) {
-  constexpr int64_t kSms = 152;
   const int64_t b = (rows + kTrsmRows * kSms - 1) / (kTrsmRows * kSms);
   return (int)(b < 1 ? 1 : b > 4 ? 4 : b);
 }
 constexpr int kUpdTile64 = 32;  // update tile, FP64
 constexpr int kUpdTile32 = 64;  // update tile, FP32
-// One trailing-update launch: columns from min(k1, ncol) to min(clim, ncol) of
+// One trailing-update launch: columns from min(c0, ncol) to min(clim, ncol) of
 // the panels, and with_u the update matrices, by the columns [k0, min(k1, ncol)).
 struct UpdRange {
   int32_t b = 0, e = 0, n = 0;  // entries, blocks
-  int32_t k0 = 0, k1 = 0, clim = 0, with_u = 0;
+  int32_t k0 = 0, k1 = 0, c0 = 0, clim = 0, with_u = 0;
 };
 struct StepRange {
   int32_t potrf_b = 0, potrf_e = 0, trsm_b = 0, trsm_e = 0, trsm_n = 0, trsm_bat = 1;
-  UpdRange upd64;         // FP64: everything right of the step's columns
+  UpdRange next64, rest64;  // FP64: the next step's columns (with look-ahead), everything past them
   UpdRange upd32, sup32;  // FP32: the rest of the super-step; at its end everything past it
 };
 
@@ -161,6 +161,7 @@ struct LevelPlan {
   int32_t rg_b = 0, rg_e = 0;        // backward-solve tasks on the rows below the block
   int32_t sdiag_b = 0, sdiag_e = 0;  // solve diagonal-block tasks, by step: see solve_steps
   std::vector<StepRange> steps;      // factor steps (block columns)
+  bool ahead64 = false;              // FP64: look-ahead (see factor_steps64)
   std::vector<int32_t> sstep_b;      // solve steps: [sstep_b[j], sstep_b[j+1]) in stasks
   std::vector<int32_t> sgemv_b;      // solve update tasks per step
   int32_t max_ncol = 0;

@@ -10,6 +10,7 @@
 // U = F22 - L21 L21^T. No atomics on values: results are bit-reproducible.
 #include <cfloat>
 #include <climits>
+#include <stdexcept>
 
 #include "launch.h"
 
@@ -170,7 +171,7 @@ __device__ __forceinline__ void st16(double *p, const Vec16<double> &v) {
 
 // Trailing update of a level's fronts by the finished columns [k0, k1) (C -= A S
 // B^T, A and B rows of a front's panel, S = diag(pivot signs), nullptr: I): one
-// TS x TS tile of the columns [min(k1, ncol), min(clim, ncol)) of a panel, or,
+// TS x TS tile of the columns [min(c0, ncol), min(clim, ncol)) of a panel, or,
 // with_u, also of the update matrix, per block (tile numbering: upd_decode).
 //
 // FP64 (32 x 32 tiles, 64 columns per launch, right-looking): GB300's FP64 pipe
@@ -183,7 +184,7 @@ __device__ __forceinline__ void st16(double *p, const Vec16<double> &v) {
 // (columns of a super-step: see Plan::kSuper32).
 template <typename T, int TS, int NT, int BK>
 __global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 3 : 2) upd_kernel(DevPlan dp, const Task *__restrict__ ents, int nent,
-                                                 int k0, int k1, int clim, int with_u,
+                                                 int k0, int k1, int c0, int clim, int with_u,
                                                  T *__restrict__ L, T *__restrict__ U) {
   constexpr int TY = NT / 16, MI = TS / TY, NJ = TS / 16;
   constexpr int VW = 16 / (int)sizeof(T), LD = BK + VW, NV = BK / VW;  // rows of BK values, 16-byte padded
@@ -200,7 +201,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 3 : 2) upd_kernel(DevPlan
   const Task tk = ents[lo];
   const FrontInfo F = dp.fronts[tk.front];
   const int nf = F.ncol + F.nrow, K = min(k1, F.ncol) - k0;
-  const UpdTile tl = upd_decode(F.ncol, F.nrow, k1, clim, with_u, TS, (int)blockIdx.x - tk.a);
+  const UpdTile tl = upd_decode(F.ncol, F.nrow, c0, clim, with_u, TS, (int)blockIdx.x - tk.a);
   const int M = min(TS, nf - tl.r), N = min(TS, tl.cend - tl.c);
   T *P = L + F.loff;
   const T *A = P + (int64_t)tl.r * F.ld + k0, *B = P + (int64_t)tl.c * F.ld + k0;
@@ -637,26 +638,70 @@ void launch_trsm(const DevPlan &dp, const StepRange &S, T *L, cudaStream_t st) {
 static void launch_upd(const DevPlan &dp, const UpdRange &u, double *L, double *U, cudaStream_t st) {
   if (u.n <= 0) return;
   note_launch();
-  upd_kernel<double, kUpdTile64, 128, 64><<<u.n, 128, 0, st>>>(dp, dp.upd + u.b, u.e - u.b, u.k0, u.k1,
+  upd_kernel<double, kUpdTile64, 128, 64><<<u.n, 128, 0, st>>>(dp, dp.upd + u.b, u.e - u.b, u.k0, u.k1, u.c0,
                                                                u.clim, u.with_u, L, U);
 }
 static void launch_upd(const DevPlan &dp, const UpdRange &u, float *L, float *U, cudaStream_t st) {
   if (u.n <= 0) return;
   note_launch();
-  upd_kernel<float, kUpdTile32, 256, 32><<<u.n, 256, 0, st>>>(dp, dp.upd + u.b, u.e - u.b, u.k0, u.k1,
+  upd_kernel<float, kUpdTile32, 256, 32><<<u.n, 256, 0, st>>>(dp, dp.upd + u.b, u.e - u.b, u.k0, u.k1, u.c0,
                                                               u.clim, u.with_u, L, U);
+}
+
+void ChainStream::create() {
+  if (s) return;
+  int lo = 0, hi = 0;
+  if (cudaDeviceGetStreamPriorityRange(&lo, &hi) != cudaSuccess ||
+      cudaStreamCreateWithPriority(&s, cudaStreamNonBlocking, hi) != cudaSuccess ||
+      cudaEventCreateWithFlags(&solved, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&updated, cudaEventDisableTiming) != cudaSuccess)
+    throw std::runtime_error("cannot create the factorisation's chain stream");
+}
+ChainStream::~ChainStream() {
+  if (solved) cudaEventDestroy(solved);
+  if (updated) cudaEventDestroy(updated);
+  if (s) cudaStreamDestroy(s);
+}
+
+// FP64 with look-ahead: the chain (diagonal block, panel solve, update of the
+// next step's columns) goes on its own stream ahead of the update of everything past
+// them, whose blocks it would otherwise wait for; it has the higher priority, so its
+// blocks start as soon as an SM has room. The columns of step s + 1 take the updates of
+// steps 0 .. s in order: rest(s - 1) is complete before next(s) starts. 32^3 grid LP
+// (FP64): 47.2 -> 43.7 ms a system.
+static void factor_steps64(const DevPlan &dp, const LevelPlan &LP, double *L, double *U, int32_t *status, bool perturb,
+                           const ChainStream &ch, cudaStream_t st) {
+  cudaEventRecord(ch.updated, st);  // the level's fronts are built
+  cudaStreamWaitEvent(ch.s, ch.updated, 0);
+  for (size_t k = 0; k < LP.steps.size(); k++) {
+    const StepRange &S = LP.steps[k];
+    launch_potrf<double>(dp, S, L, status, perturb, ch.s);
+    launch_trsm<double>(dp, S, L, ch.s);
+    cudaEventRecord(ch.solved, ch.s);
+    if (k > 0) cudaStreamWaitEvent(ch.s, ch.updated, 0);
+    launch_upd(dp, S.next64, L, U, ch.s);
+    cudaStreamWaitEvent(st, ch.solved, 0);
+    launch_upd(dp, S.rest64, L, U, st);
+    if (k + 1 < LP.steps.size()) cudaEventRecord(ch.updated, st);
+  }
 }
 
 template <typename T>
 void launch_factor_simt(const DevPlan &dp, const Plan &plan, const double *kval, T *L, T *U,
-                        int32_t *status, bool perturb, cudaStream_t st) {
+                        int32_t *status, bool perturb, const ChainStream &ch, cudaStream_t st) {
   for (const LevelPlan &LP : plan.levels) {
     launch_build_level<T>(dp, LP, kval, L, U, st);
+    if constexpr (sizeof(T) == 8) {
+      if (LP.ahead64) {
+        factor_steps64(dp, LP, L, U, status, perturb, ch, st);
+        continue;
+      }
+    }
     for (const StepRange &S : LP.steps) {
       launch_potrf<T>(dp, S, L, status, perturb, st);
       launch_trsm<T>(dp, S, L, st);
       if (sizeof(T) == 8) {
-        launch_upd(dp, S.upd64, L, U, st);
+        launch_upd(dp, S.rest64, L, U, st);
       } else {
         launch_upd(dp, S.upd32, L, U, st);
         launch_upd(dp, S.sup32, L, U, st);
@@ -681,9 +726,9 @@ template void launch_potrf<double>(const DevPlan &, const StepRange &, double *,
                                    cudaStream_t);
 template void launch_trsm<double>(const DevPlan &, const StepRange &, double *, cudaStream_t);
 template void launch_factor_simt<double>(const DevPlan &, const Plan &, const double *, double *,
-                                         double *, int32_t *, bool, cudaStream_t);
+                                         double *, int32_t *, bool, const ChainStream &, cudaStream_t);
 template void launch_factor_simt<float>(const DevPlan &, const Plan &, const double *, float *,
-                                        float *, int32_t *, bool, cudaStream_t);
+                                        float *, int32_t *, bool, const ChainStream &, cudaStream_t);
 template void launch_factor_entries<double>(const DevPlan &, const double *, const int32_t *,
                                             int64_t, const int32_t *, const int32_t *, double *,
                                             cudaStream_t);

@@ -12,9 +12,20 @@ void launch_assemble(const DevPlan &dp, const double *jv, const double *D, const
 
 // Multifrontal factorisation of all levels with SIMT FMA kernels. status must
 // be initialised by the caller (ST_FAIL_COL = INT32_MAX, ST_PERTURBED = 0).
+// Stream and events of the FP64 factor's look-ahead (one per context; see
+// factor_steps64).
+struct ChainStream {
+  cudaStream_t s = nullptr;                         // highest priority
+  cudaEvent_t solved = nullptr, updated = nullptr;  // fork / join
+  ChainStream() = default;
+  ChainStream(const ChainStream &) = delete;
+  ChainStream &operator=(const ChainStream &) = delete;
+  ~ChainStream();
+  void create();
+};
 template <typename T>
 void launch_factor_simt(const DevPlan &dp, const Plan &plan, const double *kval, T *L, T *U,
-                        int32_t *status, bool perturb, cudaStream_t st);
+                        int32_t *status, bool perturb, const ChainStream &ch, cudaStream_t st);
 
 // Pieces of a level of the factorisation, shared with the tensor-core path:
 // front assembly (+ K entries), diagonal-block Cholesky (64 wide) and the

@@ -531,11 +531,12 @@ void build_plan(const Problem &P, const Symbolic &S, Plan &plan, int nb, int nbs
     LP.build_e = (int32_t)plan.build_tasks.size();
     LP.steps.clear();
     // the level's fronts with more than `past` columns, numbered for one update launch
-    auto upd_range = [&](int32_t past, int32_t k0, int32_t k1, int32_t clim, int with_u, int TS) {
+    auto upd_range = [&](int32_t past, int32_t k0, int32_t k1, int32_t c0, int32_t clim, int with_u, int TS) {
       UpdRange u;
       u.b = (int32_t)plan.upd_ents.size();
       u.k0 = k0;
       u.k1 = k1;
+      u.c0 = c0;
       u.clim = clim;
       u.with_u = with_u;
       int64_t n = 0;
@@ -543,7 +544,7 @@ void build_plan(const Problem &P, const Symbolic &S, Plan &plan, int nb, int nbs
         const int32_t s = plan.level_fronts[t];
         const FrontInfo &F = plan.fronts[s];
         if (F.ncol <= past) continue;
-        const int64_t c = upd_tiles(F.ncol, F.nrow, k1, clim, with_u, TS);
+        const int64_t c = upd_tiles(F.ncol, F.nrow, c0, clim, with_u, TS);
         if (c == 0) continue;
         plan.upd_ents.push_back({s, (int32_t)n, k0, 0});
         n += c;
@@ -553,6 +554,17 @@ void build_plan(const Problem &P, const Symbolic &S, Plan &plan, int nb, int nbs
       u.n = (int32_t)n;
       return u;
     };
+    // Look-ahead in a level of several steps where what can run beside the chain is at
+    // least a block per SM: less is over before the chain needs its SMs, and the events
+    // between the streams cost about 2 us a step (a 639-column root with 136 such blocks:
+    // 23.5 ms an LP solve without, 23.7 with; the 32^3 grid, with thousands: 47.2 ms a
+    // system without, 43.7 with).
+    int64_t beside = 0;
+    for (int32_t t = LP.front_b; t < LP.front_e; t++) {
+      const FrontInfo &F = plan.fronts[plan.level_fronts[t]];
+      beside += upd_tiles(F.ncol, F.nrow, 2 * nb, INT32_MAX, 1, kUpdTile64);
+    }
+    LP.ahead64 = LP.max_ncol > nb && beside >= kSms;
     for (int32_t k = 0; k < LP.max_ncol; k += nb) {
       StepRange st{};
       st.potrf_b = (int32_t)plan.potrf_tasks.size();
@@ -575,11 +587,12 @@ void build_plan(const Problem &P, const Symbolic &S, Plan &plan, int nb, int nbs
         st.trsm_n += (r + kTrsmRows * st.trsm_bat - 1) / (kTrsmRows * st.trsm_bat);
       }
       st.trsm_e = (int32_t)plan.trsm_ents.size();
-      st.upd64 = upd_range(k, k, k + nb, INT32_MAX, 1, kUpdTile64);
+      if (LP.ahead64 && k + nb < LP.max_ncol) st.next64 = upd_range(k + nb, k, k + nb, k + nb, k + 2 * nb, 0, kUpdTile64);
+      st.rest64 = upd_range(k, k, k + nb, LP.ahead64 ? k + 2 * nb : k + nb, INT32_MAX, 1, kUpdTile64);
       // FP32: inside a super-step the columns up to its end, at its end the rest
       const int32_t K0 = k / Plan::kSuper32 * Plan::kSuper32, K1 = K0 + Plan::kSuper32;
-      if (k + nb < K1) st.upd32 = upd_range(k + nb, k, k + nb, K1, 0, kUpdTile32);
-      if (k + nb == K1 || k + nb >= LP.max_ncol) st.sup32 = upd_range(K0, K0, K1, INT32_MAX, 1, kUpdTile32);
+      if (k + nb < K1) st.upd32 = upd_range(k + nb, k, k + nb, k + nb, K1, 0, kUpdTile32);
+      if (k + nb == K1 || k + nb >= LP.max_ncol) st.sup32 = upd_range(K0, K0, K1, K1, INT32_MAX, 1, kUpdTile32);
       LP.steps.push_back(st);
     }
     // solve: gather tasks cover every front (they also initialise its update vector)
@@ -733,12 +746,12 @@ void validate_plan(const Problem &P, const Symbolic &S, const Plan &pl) {
       const Task &t = pl.upd_ents[i];
       need(in_front(t) && t.a == next && t.b == u.k0, "update entry");
       const FrontInfo &F = pl.fronts[t.front];
-      need(u.k0 >= 0 && u.k0 < F.ncol && u.k0 < u.k1 && u.k0 % pl.nb == 0, "update columns");
-      const int64_t c = upd_tiles(F.ncol, F.nrow, u.k1, u.clim, u.with_u, TS);
+      need(u.k0 >= 0 && u.k0 < F.ncol && u.k0 < u.k1 && u.k1 <= u.c0 && u.k0 % pl.nb == 0, "update columns");
+      const int64_t c = upd_tiles(F.ncol, F.nrow, u.c0, u.clim, u.with_u, TS);
       need(c > 0, "update entry without tiles");
       for (int64_t q : {(int64_t)0, c / 2, c - 1}) {
-        const UpdTile tl = upd_decode(F.ncol, F.nrow, u.k1, u.clim, u.with_u, TS, (int)q);
-        need(tl.c >= std::min(u.k1, F.ncol) && tl.c < tl.cend && tl.r >= tl.c && tl.r < nf(t.front) &&
+        const UpdTile tl = upd_decode(F.ncol, F.nrow, u.c0, u.clim, u.with_u, TS, (int)q);
+        need(tl.c >= std::min(u.c0, F.ncol) && tl.c < tl.cend && tl.r >= tl.c && tl.r < nf(t.front) &&
                  (tl.c < F.ncol ? tl.cend <= F.ncol : tl.cend == nf(t.front)),
              "update tile");
       }
@@ -759,7 +772,15 @@ void validate_plan(const Problem &P, const Symbolic &S, const Plan &pl) {
         next += (below + kTrsmRows * S2.trsm_bat - 1) / (kTrsmRows * S2.trsm_bat);
       }
       need(next == S2.trsm_n, "panel solve block count");
-      check_upd(S2.upd64, kUpdTile64);
+      check_upd(S2.next64, kUpdTile64);
+      check_upd(S2.rest64, kUpdTile64);
+      const int32_t c0 = S2.rest64.k1;  // columns past the step's, each in one of the two
+      if (S2.next64.n > 0)
+        need(S2.next64.c0 == c0 && S2.next64.clim == S2.rest64.c0 && S2.next64.k0 == S2.rest64.k0 &&
+                 S2.next64.k1 == c0,
+             "update halves");
+      else
+        need(S2.rest64.c0 == c0 || c0 >= LP.max_ncol, "update columns left out");
       check_upd(S2.upd32, kUpdTile32);
       check_upd(S2.sup32, kUpdTile32);
     }
