@@ -64,7 +64,8 @@ constexpr int kTmemCols = 512;
 constexpr int kSmem = kStages * kStageBytes + 1024 /*barriers*/ + 1024 /*alignment*/;
 constexpr int kThreads = 320;  // warp 0 TMA, warp 1 MMA, warps 2-9 epilogue
 constexpr int kEpiWarps = 8;
-constexpr int kTargetCtas = 2 * 152;  // split long K ranges until a launch has about this many CTAs
+constexpr int kTargetCtas = 2 * 152;  // split long K ranges until a launch has about this many tasks
+constexpr int kMainCtas = 24;         // SMs the look-ahead work leaves to the chain
 constexpr int kMinSplitWin = 4;       // windows per CTA at least
 constexpr int16_t kZeroExp = -32768;  // window of zeros (or rows past the front)
 constexpr int16_t kNanExp = 32767;    // window holding an Inf or NaN
@@ -146,8 +147,11 @@ __device__ __forceinline__ long long scaled_int(unsigned long long b, int mx) {
 
 // Slices of one window of a front: columns [b, b + c) (a finished 64-column
 // block, or that block and the one before it, sliced again with one
-// exponent), rows [a, a + 128) below the window's last diagonal block: one
-// warp per row.
+// exponent), rows [a, a + kSliceRows) below the window's last diagonal block: one
+// warp per row. A row is a chain of a load, a reduction and the digits, 1 us that
+// nothing hides, so a warp takes two rows and no more: with 128 rows a block (16 to a
+// warp) a step waited 19 us for its slices, 30.6 ms a 40^3 system against 28.4 now.
+constexpr int kSliceRows = 16;
 __global__ void __launch_bounds__(256) oz_slice_kernel(DevPlan dp, const OzFront *__restrict__ ozf,
                                                        const Task *__restrict__ tasks,
                                                        const double *__restrict__ L,
@@ -159,7 +163,7 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(DevPlan dp, const OzFront
   const int nf = F.ncol + F.nrow, c0 = tk.b, width = tk.c, blk = c0 / kBlk;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int64_t plane = (int64_t)nf * Z.lds;
-  const int rend = min(nf, tk.a + 128);
+  const int rend = min(nf, tk.a + kSliceRows);
   const float pw[kP] = {1.f, 0x1p-8f, 0x1p-16f, 0x1p-24f, 0x1p-32f, 0x1p-40f, 0x1p-48f};
   for (int row = tk.a + warp; row < rend; row += 8) {
     const double *xr = L + F.loff + (int64_t)row * F.ld + c0;
@@ -197,7 +201,7 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(DevPlan dp, const OzFront
   }
 }
 
-// One task: a 128 x 64 tile of C -= A B^T over the windows [wb, we).
+// The tasks of one launch: 128 x 64 tiles of C -= A B^T over the windows [wb, we).
 //  Mode 0 (left-looking update of block column k = b): C = panel rows a..,
 //    columns k..k+64; A = panel rows a.., B = panel rows k.., K = columns [0, k).
 //  Mode 1 (update-matrix SYRK): C = U rows a.., columns b..; A = panel rows
@@ -205,8 +209,24 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(DevPlan dp, const OzFront
 // Window w of the K range covers columns [128 w, 128 w + 128), the last one
 // only 64 when the range has an odd number of blocks; its exponent is that of
 // block 2 w. c = mode | wb << 2 | we << 17.
+struct OzTile {
+  int front, a, b, mode, wb, we, nf, arow, brow, npair;  // operand rows are front-local
+  __device__ __forceinline__ OzTile(const DevPlan &dp, const Task &tk) {
+    const FrontInfo &F = dp.fronts[tk.front];
+    front = tk.front, a = tk.a, b = tk.b;
+    mode = tk.c & 3;
+    wb = (tk.c >> 2) & 0x7FFF, we = (tk.c >> 17) & 0x7FFF;
+    nf = F.ncol + F.nrow;
+    arow = mode == 0 ? a : F.ncol + a;
+    brow = mode == 0 ? b : F.ncol + b;
+    npair = (mode == 0 ? b / kBlk : (F.ncol + kBlk - 1) / kBlk) / 2;  // windows of two blocks
+  }
+};
+// Persistent: CTA c takes tasks c, c + grid, ..; the copies and products of its next
+// task start while the epilogue still adds up the one before, and a launch can leave
+// SMs to a concurrent one.
 __global__ void __launch_bounds__(kThreads, 1)
-    oz_gemm_kernel(DevPlan dp, const OzFront *__restrict__ ozf, const Task *__restrict__ tasks,
+    oz_gemm_kernel(DevPlan dp, const OzFront *__restrict__ ozf, const Task *__restrict__ tasks, int ntask,
                    const CUtensorMap *__restrict__ maps, const int16_t *__restrict__ E,
                    double *__restrict__ L, double *__restrict__ U, int32_t *status) {
   extern __shared__ uint8_t smem_raw[];
@@ -215,21 +235,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t *full = reinterpret_cast<uint64_t *>(base + kStages * kStageBytes);
   uint64_t *empty = full + kStages;
   uint64_t *accfull = empty + kStages;  // the window's sums are in tensor memory
-  uint64_t *accempty = accfull + 1;     // the epilogue has read them
-  uint64_t *drain = accempty + 1;       // all products issued by this CTA complete
+  uint64_t *accempty = accfull + 1;     // [kSlots] the epilogue has read this sum
+  uint64_t *drain = accempty + kSlots;  // all products issued by this CTA complete
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drain + 1);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-
-  const Task tk = tasks[blockIdx.x];
-  const FrontInfo F = dp.fronts[tk.front];
-  const int mode = tk.c & 3;
-  const int wb = (tk.c >> 2) & 0x7FFF, we = (tk.c >> 17) & 0x7FFF;
-  const int nf = F.ncol + F.nrow;
-  const int arow = mode == 0 ? tk.a : F.ncol + tk.a;  // operand rows (front-local)
-  const int brow = mode == 0 ? tk.b : F.ncol + tk.b;
-  const int nblk = mode == 0 ? tk.b / kBlk : (F.ncol + kBlk - 1) / kBlk;  // blocks of K
-  const int npair = nblk / 2;  // windows of two blocks
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; s++) {
@@ -237,7 +247,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&empty[s], 1);
     }
     mbar_init(accfull, 1);
-    mbar_init(accempty, kEpiWarps);
+    for (int d = 0; d < kSlots; d++) mbar_init(&accempty[d], kEpiWarps);
     mbar_init(drain, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -256,19 +266,22 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   if (warp == 0) {
     if (lane == 0) {  // TMA producer: all 7 slices of a 32-column step of A and B
-      const CUtensorMap *ma = maps + 2 * tk.front, *mb = ma + 1;
       uint32_t g = 0;
-      for (int w = wb; w < we && !*abort_flag; w++)
-        for (int sub = 0; sub < (w < npair ? 4 : 2); sub++, g++) {
-          const int s = g % kStages;
-          const uint32_t round = g / kStages;
-          if (!mbar_wait(&empty[s], (round & 1) ^ 1, status)) { *abort_flag = 1; break; }
-          mbar_arrive_expect_tx(&full[s], kStageBytes);
-          uint8_t *st = base + s * kStageBytes;
-          const int x = w * 2 * kBlk + sub * kKs;
-          tma_load_3d(st, ma, &full[s], x, arow, 0);
-          tma_load_3d(st + kABytes, mb, &full[s], x, brow, 0);
-        }
+      for (int t = blockIdx.x; t < ntask && !*abort_flag; t += gridDim.x) {
+        const OzTile T(dp, tasks[t]);
+        const CUtensorMap *ma = maps + 2 * T.front, *mb = ma + 1;
+        for (int w = T.wb; w < T.we && !*abort_flag; w++)
+          for (int sub = 0; sub < (w < T.npair ? 4 : 2); sub++, g++) {
+            const int s = g % kStages;
+            const uint32_t round = g / kStages;
+            if (!mbar_wait(&empty[s], (round & 1) ^ 1, status)) { *abort_flag = 1; break; }
+            mbar_arrive_expect_tx(&full[s], kStageBytes);
+            uint8_t *st = base + s * kStageBytes;
+            const int x = w * 2 * kBlk + sub * kKs;
+            tma_load_3d(st, ma, &full[s], x, T.arow, 0);
+            tma_load_3d(st + kABytes, mb, &full[s], x, T.brow, 0);
+          }
+      }
       if (*abort_flag)  // let the copies already issued land before the CTA exits
         for (uint32_t q = g > (uint32_t)kStages ? g - kStages : 0; q < g; q++)
           mbar_wait(&full[q % kStages], (q / kStages) & 1, status);
@@ -277,33 +290,39 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) {  // MMA issuer
       uint32_t g = 0;
       int wi = 0;
-      for (int w = wb; w < we && !*abort_flag; w++, wi++) {
-        if (!mbar_wait(accempty, (wi & 1) ^ 1, status)) { *abort_flag = 1; break; }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        bool fail = false;
-        for (int sub = 0; sub < (w < npair ? 4 : 2); sub++, g++) {
-          const int s = g % kStages;
-          const uint32_t round = g / kStages;
-          if (!mbar_wait(&full[s], round & 1, status)) { *abort_flag = 1; fail = true; break; }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t a0 = smem_u32(base + s * kStageBytes), b0 = a0 + kABytes;
+      bool fail = false;
+      for (int t = blockIdx.x; t < ntask && !fail && !*abort_flag; t += gridDim.x) {
+        const OzTile T(dp, tasks[t]);
+        for (int w = T.wb; w < T.we && !fail && !*abort_flag; w++, wi++) {
+          for (int sub = 0; sub < (w < T.npair ? 4 : 2); sub++, g++) {
+            const int s = g % kStages;
+            const uint32_t round = g / kStages;
+            if (!mbar_wait(&full[s], round & 1, status)) { *abort_flag = 1; fail = true; break; }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t a0 = smem_u32(base + s * kStageBytes), b0 = a0 + kABytes;
 #pragma unroll
-          for (int d = 0; d <= 6; d++) {
-            const uint32_t acc = tmem + (uint32_t)((d < 5 ? d : 5) * kN);
+            for (int d = 0; d <= 6; d++) {
+              if (sub == 0 && d < kSlots) {  // the epilogue is done with this sum of the window before
+                if (!mbar_wait(&accempty[d], (wi & 1) ^ 1, status)) { *abort_flag = 1; fail = true; break; }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+              }
+              const uint32_t acc = tmem + (uint32_t)((d < 5 ? d : 5) * kN);
 #pragma unroll
-            for (int i = 0; i <= d; i++) {
-              const uint64_t ad = sw64_desc(a0 + i * kAPlane), bd = sw64_desc(b0 + (d - i) * kBPlane);
+              for (int i = 0; i <= d; i++) {
+                const uint64_t ad = sw64_desc(a0 + i * kAPlane), bd = sw64_desc(b0 + (d - i) * kBPlane);
 #pragma unroll
-              for (int kk = 0; kk < 2; kk++) {  // 16 BF16 (32 bytes) of K per product
-                const bool first = sub == 0 && kk == 0 && i == 0 && d <= 5;
-                mma_bf16(acc, ad + 2 * kk, bd + 2 * kk, kIdesc, first ? 0u : 1u);
+                for (int kk = 0; kk < 2; kk++) {  // 16 BF16 (32 bytes) of K per product
+                  const bool first = sub == 0 && kk == 0 && i == 0 && d <= 5;
+                  mma_bf16(acc, ad + 2 * kk, bd + 2 * kk, kIdesc, first ? 0u : 1u);
+                }
               }
             }
+            if (fail) break;
+            mma_commit(&empty[s]);
           }
-          mma_commit(&empty[s]);
+          if (fail) break;
+          mma_commit(accfull);
         }
-        if (fail) break;
-        mma_commit(accfull);
       }
       mma_commit(drain);  // tensor memory is released only after every product landed
       mbar_wait(drain, 0, status);
@@ -312,85 +331,68 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int q = warp & 3;         // tensor-memory lane quarter this warp may access
     const int c0 = 32 * ((warp - 2) >> 2);  // this thread's 32 columns of the tile
     const int r = 32 * q + lane;    // its row of the tile
-    const OzFront Z = ozf[tk.front];
-    const bool arow_ok = arow + r < nf;
-    const int16_t *ea_row = E + Z.eoff + (int64_t)(arow + r) * Z.nblk;
-    const int16_t *eb_col = E + Z.eoff + (int64_t)(brow + c0) * Z.nblk;
-    const int nb_rows = nf - (brow + c0);  // B rows of this thread's columns inside the front
-    double acc[32];
-#pragma unroll
-    for (int c = 0; c < 32; c++) acc[c] = 0.0;
     int wi = 0;
-    for (int w = wb; w < we && !*abort_flag; w++, wi++) {
-      const int ea = arow_ok ? ea_row[2 * w] : kZeroExp;
-      // lane c holds the exponent of this thread's column c0 + c (one load per
-      // lane; the additions below take it by shuffle)
-      const int eb_lane = lane < nb_rows ? eb_col[(int64_t)lane * Z.nblk + 2 * w] : kZeroExp;
-      if (!mbar_wait(accfull, wi & 1, status)) { *abort_flag = 1; break; }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      // W of all 32 entries first (cheap FP32/INT work), then free the
-      // accumulators for the next window, then the FP64 additions
-      long long Wv[32];
+    for (int t = blockIdx.x; t < ntask && !*abort_flag; t += gridDim.x) {
+      const OzTile T(dp, tasks[t]);
+      const OzFront Z = ozf[T.front];
+      const bool arow_ok = T.arow + r < T.nf;
+      const int16_t *ea_row = E + Z.eoff + (int64_t)(T.arow + r) * Z.nblk;
+      const int16_t *eb_col = E + Z.eoff + (int64_t)(T.brow + c0) * Z.nblk;
+      const int nb_rows = T.nf - (T.brow + c0);  // B rows of this thread's columns inside the front
+      double acc[32];
 #pragma unroll
-      for (int sub = 0; sub < 4; sub++) {  // 8 columns at a time, one sum at a time
-        const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(c0 + 8 * sub);
-        uint32_t v[8];
-        int hi[8];
-        tmem_ld8(ta, v);  // diagonal 0
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      for (int c = 0; c < 32; c++) acc[c] = 0.0;
+      for (int w = T.wb; w < T.we && !*abort_flag; w++, wi++) {
+        const int ea = arow_ok ? ea_row[2 * w] : kZeroExp;
+        // lane c holds the exponent of this thread's column c0 + c (one load per
+        // lane; the additions below take it by shuffle)
+        const int eb_lane = lane < nb_rows ? eb_col[(int64_t)lane * Z.nblk + 2 * w] : kZeroExp;
+        if (!mbar_wait(accfull, wi & 1, status)) { *abort_flag = 1; break; }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        // W of all 32 entries, one sum after the other: each is handed back as soon as
+        // it is read, so the next window's products follow one sum behind. The FP64
+        // additions come last.
+        const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c0;
+        auto sum = [&](int d, auto f) {
 #pragma unroll
-        for (int c = 0; c < 8; c++) hi[c] = exact_int(v[c], 1.f) * 256;
-        tmem_ld8(ta + kN, v);  // diagonal 1
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          for (int h = 0; h < 4; h++) {
+            uint32_t v[8];
+            tmem_ld8(ta + (uint32_t)(d * kN + 8 * h), v);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-        for (int c = 0; c < 8; c++) Wv[8 * sub + c] = (long long)(hi[c] + wide_int(v[c], 0x1p8f)) << 32;
-        tmem_ld8(ta + 2 * kN, v);  // diagonal 2
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            for (int c = 0; c < 8; c++) f(8 * h + c, v[c]);
+          }
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&accempty[d]);
+        };
+        int hi[32];  // of W's upper word
+        long long Wv[32];
+        sum(0, [&](int c, uint32_t v) { hi[c] = exact_int(v, 1.f) * 256; });
+        sum(1, [&](int c, uint32_t v) { hi[c] += wide_int(v, 0x1p8f); });
+        sum(2, [&](int c, uint32_t v) { Wv[c] = ((long long)hi[c] << 32) + ((long long)wide_int(v, 0x1p16f) << 24); });
+        sum(3, [&](int c, uint32_t v) { Wv[c] += (long long)wide_int(v, 0x1p24f) << 16; });
+        sum(4, [&](int c, uint32_t v) { Wv[c] += (long long)wide_int(v, 0x1p32f) << 8; });
+        sum(5, [&](int c, uint32_t v) { Wv[c] += wide_int(v, 0x1p40f); });  // diagonals 5 and 6 (rounded), |.| < 2^24 units
 #pragma unroll
-        for (int c = 0; c < 8; c++) Wv[8 * sub + c] += (long long)wide_int(v[c], 0x1p16f) << 24;
-        tmem_ld8(ta + 3 * kN, v);  // diagonal 3
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-        for (int c = 0; c < 8; c++) hi[c] = wide_int(v[c], 0x1p24f);
-        tmem_ld8(ta + 4 * kN, v);  // diagonal 4
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-        for (int c = 0; c < 8; c++)
-          Wv[8 * sub + c] += ((long long)hi[c] << 16) + ((long long)wide_int(v[c], 0x1p32f) << 8);
-        tmem_ld8(ta + 5 * kN, v);  // diagonals 5 and 6 (rounded), |.| < 2^24 units
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-        for (int c = 0; c < 8; c++) Wv[8 * sub + c] += wide_int(v[c], 0x1p40f);
+        for (int c = 0; c < 32; c++) {
+          const int eb = __shfl_sync(0xFFFFFFFFu, eb_lane, c);
+          acc[c] += scaled_double(Wv[c], ea, eb);
+        }
       }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) mbar_arrive(accempty);
+      if (!*abort_flag) {
+        const FrontInfo &F = dp.fronts[T.front];
+        const bool upd = T.mode == 0;
+        const int M = min(kM, upd ? T.nf - T.a : F.nrow - T.a);
+        const int N = min(kN, upd ? F.ncol - T.b : F.nrow - T.b);
+        const int64_t ldc = upd ? F.ld : F.uld;
+        double *C = (upd ? L + F.loff : U + F.uoff) + (int64_t)T.a * ldc + T.b;
+        if (r < M) {
+          double *crow = C + (int64_t)r * ldc + c0;
 #pragma unroll
-      for (int c = 0; c < 32; c++) {
-        const int eb = __shfl_sync(0xFFFFFFFFu, eb_lane, c);
-        acc[c] += scaled_double(Wv[c], ea, eb);
-      }
-    }
-    if (!*abort_flag) {
-      int M, N;
-      double *C;
-      int64_t ldc;
-      if (mode == 0) {
-        M = min(kM, nf - tk.a);
-        N = min(kBlk, F.ncol - tk.b);
-        C = L + F.loff + (int64_t)tk.a * F.ld + tk.b;
-        ldc = F.ld;
-      } else {
-        M = min(kM, F.nrow - tk.a);
-        N = min(kN, F.nrow - tk.b);
-        C = U + F.uoff + (int64_t)tk.a * F.uld + tk.b;
-        ldc = F.uld;
-      }
-      if (r < M) {
-        double *crow = C + (int64_t)r * ldc + c0;
-#pragma unroll
-        for (int c = 0; c < 32; c++)
-          if (c0 + c < N) atomicAdd(crow + c, -acc[c]);
+          for (int c = 0; c < 32; c++)
+            if (c0 + c < N) atomicAdd(crow + c, -acc[c]);
+        }
       }
     }
   }
@@ -401,6 +403,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                  "r"(kTmemCols));
 }
 
+// Windows of block column j's K range that are complete one step ahead, when block
+// j - 1 is still to be finished (the rest is one window, see windows).
+int ahead_windows(int j) { return j > 0 ? (j - 1) / 2 : 0; }
+
 // Chunks of the K range of each tile: enough CTAs for the launch, at least
 // kMinSplitWin windows each.
 int split_for(int64_t tiles, int nwin) {
@@ -409,16 +415,24 @@ int split_for(int64_t tiles, int nwin) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(want, nwin / kMinSplitWin));
 }
 
-void push_split(std::vector<Task> &out, int32_t front, int32_t a, int32_t b, int mode, int nwin,
+void push_split(std::vector<Task> &out, int32_t front, int32_t a, int32_t b, int mode, int first, int nwin,
                 int split) {
   for (int c = 0; c < split; c++) {
-    const int w0 = (int)((int64_t)nwin * c / split), w1 = (int)((int64_t)nwin * (c + 1) / split);
+    const int w0 = first + (int)((int64_t)nwin * c / split), w1 = first + (int)((int64_t)nwin * (c + 1) / split);
     if (w1 > w0) out.push_back({front, a, b, mode | (w0 << 2) | (w1 << 17)});
   }
 }
 
 // Windows of a K range of nblk blocks: pairs, and a last single block.
 int windows(int nblk) { return nblk / 2 + nblk % 2; }
+
+int sm_count() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
+    throw std::runtime_error("FP64 tensor-core factor: SM count");
+  return n;
+}
 
 }  // namespace
 
@@ -448,23 +462,27 @@ void OzPlan::build(const Plan &plan) {
     Level &V = levels_[l];
     for (int32_t k = 0; k < LP.max_ncol; k += kBlk) {
       Step st{};
-      st.gemm_b = (int)gemm_.size();
-      if (k > 0) {
+      // windows [w0, w1) of block column c, every front and row tile
+      auto update = [&](int32_t c, int w0, int w1) {
         int64_t tiles = 0;
         for (int32_t t = LP.front_b; t < LP.front_e; t++) {
           const FrontInfo &F = plan.fronts[plan.level_fronts[t]];
-          if (F.ncol > k) tiles += (F.ncol + F.nrow - k + kM - 1) / kM;
+          if (F.ncol > c) tiles += (F.ncol + F.nrow - c + kM - 1) / kM;
         }
-        const int nw = windows(k / kBlk);
-        const int split = split_for(tiles, nw);
-        for (int32_t t = LP.front_b; t < LP.front_e; t++) {
+        const int split = split_for(tiles, w1 - w0);
+        for (int32_t t = LP.front_b; t < LP.front_e && w1 > w0; t++) {
           const int32_t s = plan.level_fronts[t];
           const FrontInfo &F = plan.fronts[s];
-          if (F.ncol <= k) continue;
-          for (int32_t i0 = k; i0 < F.ncol + F.nrow; i0 += kM) push_split(gemm_, s, i0, k, 0, nw, split);
+          if (F.ncol <= c) continue;
+          for (int32_t i0 = c; i0 < F.ncol + F.nrow; i0 += kM) push_split(gemm_, s, i0, c, 0, w0, w1 - w0, split);
         }
-      }
-      st.gemm_e = (int)gemm_.size();
+      };
+      const int j = k / kBlk;
+      st.gemm_b = (int)gemm_.size();
+      update(k, ahead_windows(j), windows(j));
+      st.gemm_e = st.ahead_b = (int)gemm_.size();
+      update(k + kBlk, 0, ahead_windows(j + 1));
+      st.ahead_e = (int)gemm_.size();
       // the finished block (an even block alone, an odd block with the one
       // before it), rows below it
       st.slice_b = (int)slice_.size();
@@ -475,7 +493,7 @@ void OzPlan::build(const Plan &plan) {
         if (F.ncol <= k) continue;
         const int32_t kb = std::min(kBlk, F.ncol - k);
         const int32_t c0 = odd ? k - kBlk : k, width = odd ? kBlk + kb : kb;
-        for (int32_t r0 = k + kb; r0 < F.ncol + F.nrow; r0 += 128) slice_.push_back({s, r0, c0, width});
+        for (int32_t r0 = k + kb; r0 < F.ncol + F.nrow; r0 += kSliceRows) slice_.push_back({s, r0, c0, width});
       }
       st.slice_e = (int)slice_.size();
       V.steps.push_back(st);
@@ -495,7 +513,7 @@ void OzPlan::build(const Plan &plan) {
       const int split = split_for(tiles, nw);
       for (int32_t i0 = 0; i0 < F.nrow; i0 += kM)
         for (int32_t j0 = 0; j0 < F.nrow && j0 < i0 + kM; j0 += kN)
-          push_split(gemm_, s, i0, j0, 1, nw, split);
+          push_split(gemm_, s, i0, j0, 1, 0, nw, split);
     }
     V.syrk_e = (int)gemm_.size();
   }
@@ -518,33 +536,57 @@ void OzPlan::validate(const Plan &plan) const {
     need(Z.soff + (int64_t)kP * nf * Z.lds <= slice_elems_, "slice planes past the storage");
     need(Z.eoff + nf * Z.nblk <= exp_elems_, "exponents past the storage");
   }
-  int cur_f = -1, cur_a = -1, cur_b = -1, cur_mode = -1, next_w = 0, cur_W = 0;
-  auto close_tile = [&]() { need(cur_f < 0 || next_w == cur_W, "a tile's chunks miss windows"); };
-  for (const Task &t : gemm_) {
-    need(t.front >= 0 && t.front < nfr, "task front");
-    const FrontInfo &F = plan.fronts[t.front];
-    const int mode = t.c & 3, w0 = (t.c >> 2) & 0x7FFF, w1 = (t.c >> 17) & 0x7FFF;
-    int W;
-    if (mode == 0) {
-      need(t.b > 0 && t.b % kBlk == 0 && t.b < F.ncol, "update: block column");
-      need(t.a >= t.b && t.a < F.ncol + F.nrow && (t.a - t.b) % kM == 0, "update: row tile");
-      W = windows(t.b / kBlk);
-    } else {
-      need(mode == 1 && F.nrow > 0, "task mode");
-      need(t.a >= 0 && t.a < F.nrow && t.a % kM == 0, "SYRK: row tile");
-      need(t.b >= 0 && t.b < F.nrow && t.b % kN == 0 && t.b < t.a + kM, "SYRK: column tile");
-      W = windows((F.ncol + kBlk - 1) / kBlk);
+  // a tile's chunks come one after the other within a part of its range; the parts of an
+  // update (ahead of its step, in it) are a step apart
+  int cur_f = -1, cur_a = -1, cur_b = -1, cur_mode = -1, next_w = 0, end_w = 0;
+  auto close_tile = [&]() { need(cur_f < 0 || next_w == end_w, "a tile's chunks miss windows"); };
+  auto check = [&](int b, int e, auto part) {  // part(task): its windows [first, end)
+    for (int i = b; i < e; i++) {
+      const Task &t = gemm_[i];
+      need(t.front >= 0 && t.front < nfr, "task front");
+      const FrontInfo &F = plan.fronts[t.front];
+      const int mode = t.c & 3, w0 = (t.c >> 2) & 0x7FFF, w1 = (t.c >> 17) & 0x7FFF;
+      if (mode == 0) {
+        need(t.b > 0 && t.b % kBlk == 0 && t.b < F.ncol, "update: block column");
+        need(t.a >= t.b && t.a < F.ncol + F.nrow && (t.a - t.b) % kM == 0, "update: row tile");
+      } else {
+        need(mode == 1 && F.nrow > 0, "task mode");
+        need(t.a >= 0 && t.a < F.nrow && t.a % kM == 0, "SYRK: row tile");
+        need(t.b >= 0 && t.b < F.nrow && t.b % kN == 0 && t.b < t.a + kM, "SYRK: column tile");
+      }
+      const std::pair<int, int> range = part(t, mode);
+      need(0 <= w0 && w0 < w1, "window range");
+      if (i == b || t.front != cur_f || t.a != cur_a || t.b != cur_b || mode != cur_mode) {
+        close_tile();
+        cur_f = t.front, cur_a = t.a, cur_b = t.b, cur_mode = mode, next_w = range.first, end_w = range.second;
+      }
+      need(w0 == next_w, "a tile's chunks are not consecutive");
+      next_w = w1;
     }
-    need(0 <= w0 && w0 < w1 && w1 <= W, "window range");
-    if (t.front != cur_f || t.a != cur_a || t.b != cur_b || mode != cur_mode || w0 == 0) {
-      close_tile();
-      need(w0 == 0, "a tile's first chunk starts past window 0");
-      cur_f = t.front, cur_a = t.a, cur_b = t.b, cur_mode = mode, cur_W = W, next_w = 0;
+    close_tile();
+    cur_f = -1;
+  };
+  for (const Level &V : levels_) {
+    for (size_t j = 0; j < V.steps.size(); j++) {
+      const Step &S = V.steps[j];
+      // windows of a step ahead: blocks before j, whose slices are final and which step j
+      // does not slice again
+      const int na = ahead_windows((int)j + 1);
+      need(2 * na <= (int)j && (j % 2 == 0 || 2 * na <= (int)j - 1), "look-ahead windows");
+      check(S.gemm_b, S.gemm_e, [&](const Task &t, int mode) {
+        need(mode == 0 && t.b == (int)j * kBlk, "update: step");
+        return std::make_pair(ahead_windows((int)j), windows((int)j));
+      });
+      check(S.ahead_b, S.ahead_e, [&](const Task &t, int mode) {
+        need(mode == 0 && t.b == (int)(j + 1) * kBlk, "look-ahead: step");
+        return std::make_pair(0, na);
+      });
     }
-    need(w0 == next_w, "a tile's chunks are not consecutive");
-    next_w = w1;
+    check(V.syrk_b, V.syrk_e, [&](const Task &t, int mode) {
+      need(mode == 1, "SYRK: mode");
+      return std::make_pair(0, windows((plan.fronts[t.front].ncol + kBlk - 1) / kBlk));
+    });
   }
-  close_tile();
   for (const Task &t : slice_) {
     need(t.front >= 0 && t.front < nfr, "slice front");
     const FrontInfo &F = plan.fronts[t.front];
@@ -575,6 +617,14 @@ void OzPlan::layout(Carve &cv, cudaStream_t st, bool storage) {
 void OzPlan::encode(const Plan &plan, cudaStream_t st) {
   ready_ = false;
   if (!sized_ || !S_) return;
+  if (!side_) {
+    int lo = 0, hi = 0;
+    cudaDeviceGetStreamPriorityRange(&lo, &hi);
+    if (cudaStreamCreateWithPriority(&side_, cudaStreamNonBlocking, lo) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ev_main_, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ev_side_, cudaEventDisableTiming) != cudaSuccess)
+      throw std::runtime_error("cannot create the look-ahead stream");
+  }
   PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
   const size_t nfr = plan.fronts.size();
   std::vector<CUtensorMap> maps(2 * nfr);
@@ -612,20 +662,35 @@ void OzPlan::factor(const DevPlan &dp, const Plan &plan, const double *kval, dou
                     int32_t *status, cudaStream_t st) {
   if (!ready_) throw std::runtime_error("FP64 tensor-core factor not prepared");
   const CUtensorMap *maps = reinterpret_cast<const CUtensorMap *>(d_maps_);
-  auto gemm = [&](int b, int e) {
+  const int sms = sm_count(), side_ctas = sms - std::min(kMainCtas, sms / 2);
+  auto gemm = [&](int b, int e, int ctas, cudaStream_t q) {
     if (e > b) {
       note_launch();
-      oz_gemm_kernel<<<e - b, kThreads, kSmem, st>>>(dp, d_fr_, d_gemm_ + b, maps, E_, L, U, status);
+      oz_gemm_kernel<<<std::min(e - b, ctas), kThreads, kSmem, q>>>(dp, d_fr_, d_gemm_ + b, e - b, maps, E_, L, U,
+                                                                   status);
     }
   };
   for (size_t l = 0; l < plan.levels.size(); l++) {
     const LevelPlan &LP = plan.levels[l];
     const Level &V = levels_[l];
     launch_build_level<double>(dp, LP, kval, L, U, st);
+    // A step's chain is its last window, the diagonal block, the panel solve and the
+    // slices; the next block column takes every window but its last one beside it, on
+    // the side stream (on fewer CTAs than SMs, so that the chain finds SMs at once):
+    // 33.2 -> 30.6 ms a 40^3 system.
+    bool pending = false;
     for (size_t s = 0; s < LP.steps.size(); s++) {
       const StepRange &R = LP.steps[s];
       const Step &Z = V.steps[s];
-      gemm(Z.gemm_b, Z.gemm_e);
+      gemm(Z.gemm_b, Z.gemm_e, sms, st);
+      if (pending) cudaStreamWaitEvent(st, ev_side_, 0);
+      pending = Z.ahead_e > Z.ahead_b;
+      if (pending) {
+        cudaEventRecord(ev_main_, st);
+        cudaStreamWaitEvent(side_, ev_main_, 0);
+        gemm(Z.ahead_b, Z.ahead_e, side_ctas, side_);
+        cudaEventRecord(ev_side_, side_);
+      }
       launch_potrf<double>(dp, R, L, status, false, st);
       launch_trsm<double>(dp, R, L, st);
       if (Z.slice_e > Z.slice_b) {
@@ -634,8 +699,15 @@ void OzPlan::factor(const DevPlan &dp, const Plan &plan, const double *kval, dou
                                                               S_, E_);
       }
     }
-    gemm(V.syrk_b, V.syrk_e);
+    if (pending) cudaStreamWaitEvent(st, ev_side_, 0);
+    gemm(V.syrk_b, V.syrk_e, sms, st);
   }
+}
+
+OzPlan::~OzPlan() {
+  if (ev_main_) cudaEventDestroy(ev_main_);
+  if (ev_side_) cudaEventDestroy(ev_side_);
+  if (side_) cudaStreamDestroy(side_);
 }
 
 }  // namespace gipm

@@ -25,6 +25,7 @@ class OzPlan {
   static constexpr int kPlanes = 7;  // BF16 slices per FP64 value
   static constexpr int kBlk = 64;    // the plan's block width; windows are 1 or 2 blocks
   OzPlan() = default;
+  ~OzPlan();
   OzPlan(const OzPlan &) = delete;
   OzPlan &operator=(const OzPlan &) = delete;
   // Task lists and slice layout from the FP64 plan (block width kBlk).
@@ -43,7 +44,9 @@ class OzPlan {
 
  private:
   void validate(const Plan &plan) const;
-  struct Step { int gemm_b, gemm_e, slice_b, slice_e; };
+  // updates of a step's block column, those of the next one that can run beside the
+  // step, and its slices
+  struct Step { int gemm_b, gemm_e, ahead_b, ahead_e, slice_b, slice_e; };
   struct Level { std::vector<Step> steps; int syrk_b = 0, syrk_e = 0; };
   std::vector<Task> gemm_, slice_;
   std::vector<OzFront> fr_;
@@ -55,6 +58,8 @@ class OzPlan {
   uint16_t *S_ = nullptr;   // slice planes (BF16 bits)
   int16_t *E_ = nullptr;    // exponent tables
   bool sized_ = false, ready_ = false;
+  cudaStream_t side_ = nullptr;                        // look-ahead stream (low priority)
+  cudaEvent_t ev_main_ = nullptr, ev_side_ = nullptr;  // fork / join
 };
 
 }  // namespace gipm
