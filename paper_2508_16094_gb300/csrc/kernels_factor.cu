@@ -350,12 +350,15 @@ __device__ __forceinline__ bool pivot_ok(float d) { return d > 0.f && d < INFINI
 // 64 cycles whatever its active lanes (measured; results after 66; a conversion or
 // comparison more), so the count of FP64 warp instructions on each of the four
 // warps is the time, and the chain of 64 pivots is on it too. So the elimination
-// runs on unscaled columns (a_ic -= (a_ij / d_j) a_cj: no square root on the chain),
-// all columns are scaled by 1 / L_jj at the end of their panel, and the block goes in
-// four panels of 16 columns, two threads per row, each column published through
-// shared memory (one barrier per column); past the panel a rank-16 update over 8 x 8
-// blocks of the lower triangle.
-constexpr int kPotrfThreads = 128;
+// runs on unscaled columns (a_ic -= (a_ij / d_j) a_cj: no square root on the chain; all
+// columns are scaled by 1 / L_jj on their way out), and the block goes in four panels of
+// 16 columns, two threads per row, each column published through shared memory (one
+// barrier per column); past the panel a rank-16 update over the entries of the lower
+// triangle, one a thread, on two warps per quarter (one leaves it idle between
+// multiply-adds: 15.4k against 11.3k cycles past the first panel). 64 columns: 95k
+// cycles when each panel was scaled by itself and updated in 8 x 8 blocks on one warp
+// per quarter, 78k now, 49k of them in the panels.
+constexpr int kPotrfThreads = 256;  // the first 128 for the panels
 
 // Barrier 1 over the first `threads` threads of the block (whole warps).
 __device__ __forceinline__ void bar1(int threads) {
@@ -363,10 +366,11 @@ __device__ __forceinline__ void bar1(int threads) {
 }
 
 // Panel at column c0 of the block in S (rows c0 .. 63) on 2 (64 - c0) threads: two
-// per row, thread h of a row holds the columns c0 + h + 2 q.
+// per row, thread h of a row holds the columns c0 + h + 2 q. This form takes every
+// pivot; potrf_panel_fast the usual ones.
 template <typename T>
 __device__ __forceinline__ void potrf_panel(T *S, int ls, int c0, T (*col)[64], const int8_t *neg, T *piv,
-                                            int32_t *status, int perturb, int first) {
+                                            T (*W)[64], int32_t *status, int perturb, int first) {
   const int t = threadIdx.x, i = t / 2, h = t % 2, act = 2 * (64 - c0);  // row c0 + i
   T x[8];
 #pragma unroll
@@ -389,8 +393,9 @@ __device__ __forceinline__ void potrf_panel(T *S, int ls, int c0, T (*col)[64], 
       d = perturb ? big_pivot<T>() : T(1);
     }
     if (t == 0) piv[c0 + j] = d;
-    if (j == 15) break;
     const T w = flip(quotient(aij, d), ng);  // a_ij / d_j
+    if (h == j % 2) W[j][c0 + i] = w;
+    if (j == 15) break;
     // column j + 1 first: published before the barrier, the other columns after it,
     // beside the next pivot's chain (three buffers: the next column but one is
     // written while slower warps still read column j); column j itself is final
@@ -406,16 +411,84 @@ __device__ __forceinline__ void potrf_panel(T *S, int ls, int c0, T (*col)[64], 
     if (h + 2 * q <= i) S[(c0 + i) * ls + c0 + h + 2 * q] = x[q];
 }
 
-// s0, s1 = sum_j x0_j (s_j) y_j, sum_j x1_j (s_j) y_j over a panel's 16 columns
-template <typename T, bool SIGNED>
-__device__ __forceinline__ void panel_dots(const T *x0, const T *x1, const T *y, const int8_t *neg, T &s0, T &s1) {
-  s0 = s1 = T(0);
+// The same without a branch, for pivots of the right sign within FP32's normal range;
+// false (in every thread of the panel, S as it was) if one is not. In one basic block
+// the multiply-adds of column j fill the time in which the loads and the estimate of
+// column j + 1 are under way: 820 cycles a column with the branches, 760 without.
+__device__ __forceinline__ bool potrf_panel_fast(double *S, int ls, int c0, double (*col)[64], const int8_t *neg,
+                                                 double *piv, double (*W)[64]) {
+  const int t = threadIdx.x, i = t / 2, h = t % 2, act = 2 * (64 - c0);  // row c0 + i
+  double x[8];
+#pragma unroll
+  for (int q = 0; q < 8; q++) x[q] = S[(c0 + i) * ls + c0 + h + 2 * q];
+  unsigned sign = 0;  // bit j: column j's pivot sign is negative
+#pragma unroll
+  for (int j = 0; j < 16; j++) sign |= (neg[c0 + j] != 0 ? 1u : 0u) << j;
+  if (h == 0) col[0][i] = x[0];
+  bar1(act);
+  bool good = true;
+  double d = flip(col[0][0], sign & 1u), a = col[0][i], r0 = recip_start(d), v[8], w = 0.0;
+#pragma unroll
+  for (int q = 0; q < 8; q++) v[q] = col[0][h + 2 * q];
 #pragma unroll
   for (int j = 0; j < 16; j++) {
-    const T v = SIGNED ? flip(y[j], neg[j] != 0) : y[j];
-    s0 = fma(x0[j], v, s0);
-    s1 = fma(x1[j], v, s1);
+    good = good && in_fp32(d);
+    if (t == 0) piv[c0 + j] = d;
+    const double w0 = a * r0;
+    w = flip(fma(w0, recip_err(d, r0), w0), sign >> j & 1u);  // a_ij / d_j
+    if (h == j % 2) W[j][c0 + i] = w;
+    if (j == 15) break;
+    const int qn = (j + 1) / 2;
+    if (j % 2 == 1 || h == 1) x[qn] = fma(-w, v[qn], x[qn]);
+    double *cn = col[(j + 1) % 3];
+    if (h == (j + 1) % 2) cn[i] = x[qn];
+    bar1(act);
+    d = flip(cn[j + 1], sign >> (j + 1) & 1u);
+    a = cn[i];
+    double u[8];
+#pragma unroll
+    for (int q = (j + 2) / 2; q < 8; q++) u[q] = cn[h + 2 * q];
+    r0 = recip_start(d);
+#pragma unroll
+    for (int q = qn + 1; q < 8; q++) x[q] = fma(-w, v[q], x[q]);
+#pragma unroll
+    for (int q = (j + 2) / 2; q < 8; q++) v[q] = u[q];
   }
+  if (!good) return false;
+#pragma unroll
+  for (int q = 0; q < 8; q++)
+    if (h + 2 * q <= i) S[(c0 + i) * ls + c0 + h + 2 * q] = x[q];
+  return true;
+}
+__device__ __forceinline__ bool potrf_panel_fast(float *, int, int, float (*)[64], const int8_t *, float *,
+                                                 float (*)[64]) {
+  return false;  // (FP32 arithmetic is not what bounds the FP32 panel)
+}
+
+// Entries e0, e0 + 256, .. (Q of them) of the lower triangle of the m rows and columns past
+// a panel, numbered row by row: a_ic -= sum_j a_ij w_cj. (All sums before the first store:
+// a store to S would hold back the loads of the next sum.)
+template <int Q, typename T>
+__device__ __forceinline__ void panel_trail(T *S, int ls, int c0, int e0, int nout, const T (*W)[64]) {
+  T s[Q];
+  int at[Q], col[Q];
+#pragma unroll
+  for (int q = 0; q < Q; q++) {
+    const int e = min(e0 + kPotrfThreads * q, nout - 1);
+    int bi = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+    if (bi * (bi + 1) / 2 > e) bi--;
+    if ((bi + 1) * (bi + 2) / 2 <= e) bi++;
+    col[q] = c0 + 16 + e - bi * (bi + 1) / 2;
+    at[q] = (c0 + 16 + bi) * ls;
+    s[q] = S[at[q] + col[q]];
+  }
+#pragma unroll
+  for (int j = 0; j < 16; j++)
+#pragma unroll
+    for (int q = 0; q < Q; q++) s[q] = fma(-S[at[q] + c0 + j], W[j][col[q]], s[q]);
+#pragma unroll
+  for (int q = 0; q < Q; q++)
+    if (e0 + kPotrfThreads * q < nout) S[at[q] + col[q]] = s[q];
 }
 
 template <typename T>
@@ -429,15 +502,20 @@ __global__ void __launch_bounds__(kPotrfThreads) potrf_kernel(DevPlan dp, const 
   T *A = L + F.loff + (int64_t)k * F.ld + k;
   const int8_t *sg = dp.sgn ? dp.sgn + F.first + k : nullptr;
   __shared__ T S[NB * LS];  // the block; past kb: zero, with a unit diagonal
-  __shared__ T col[3][NB], piv[NB], rs[NB];
+  __shared__ T col[3][NB], piv[NB], W[16][NB];  // W: a panel's a_ij / d_j
   __shared__ int8_t neg[NB];
   const int tid = threadIdx.x;
-#pragma unroll 16
-  for (int q = 0; q < NB * NB / NT; q++) {
-    const int e = tid + NT * q, r = e / NB, c = e % NB;
-    T v = r == c ? T(1) : T(0);
-    if (r < kb && c <= r) v = A[(int64_t)r * F.ld + c];
-    S[r * LS + c] = v;
+  // 16 bytes at a time (rows are padded to 16 bytes, and zero past their last column)
+  constexpr int VW = 16 / (int)sizeof(T), NV = NB / VW;
+#pragma unroll
+  for (int q = 0; q < NB * NV / NT; q++) {
+    const int e = tid + NT * q, r = e / NV, c = VW * (e % NV);
+    Vec16<T> v;
+#pragma unroll
+    for (int h = 0; h < VW; h++) v.v[h] = T(0);
+    if (r < kb && c <= r) v = ld16(A + (int64_t)r * F.ld + c);
+#pragma unroll
+    for (int h = 0; h < VW; h++) S[r * LS + c + h] = (r < kb && c + h <= r) ? v.v[h] : (r == c + h ? T(1) : T(0));
   }
   if (tid < NB) neg[tid] = sg && tid < kb && sg[tid] < 0;
   __syncthreads();
@@ -445,46 +523,36 @@ __global__ void __launch_bounds__(kPotrfThreads) potrf_kernel(DevPlan dp, const 
   for (int p = 0; p < 4; p++) {
     const int c0 = 16 * p;
     if (c0 >= kb) break;
-    if (tid < 2 * (NB - c0)) potrf_panel<T>(S, LS, c0, col, neg, piv, status, perturb, F.first + k);
-    __syncthreads();
-    if (tid < 16) rs[c0 + tid] = inv_sqrt(piv[c0 + tid]);
-    __syncthreads();
-    {  // the panel's columns: s_j a_ij / L_jj, and L_jj = sqrt(d) from d and 1 / sqrt(d)
-      const int c = c0 + tid % 16;
-      const T r = rs[c];
-      const bool ng = neg[c] != 0;
-#pragma unroll
-      for (int q = 0; q < 8; q++) {
-        const int i = c0 + tid / 16 + 8 * q;
-        if (i < NB && i > c) S[i * LS + c] = flip(S[i * LS + c] * r, ng);
-      }
-      if (tid < 16) {
-        const T d = piv[c], l0 = d * r;
-        S[c * LS + c] = fma(fma(-l0, l0, d), T(0.5) * r, l0);
-      }
+    if (tid < 2 * (NB - c0) && !potrf_panel_fast(S, LS, c0, col, neg, piv, W)) {
+      bar1(2 * (NB - c0));
+      potrf_panel<T>(S, LS, c0, col, neg, piv, W, status, perturb, F.first + k);
     }
     __syncthreads();
     if (p == 3 || c0 + 16 >= kb) break;
-    // rows and columns past the panel: 8 x 8 blocks (bi >= bc) of the lower
-    // triangle, a block per warp, two outputs per lane
-    const int nb8 = (48 - c0) / 8, nblk = nb8 * (nb8 + 1) / 2, l = tid % 32;
-    for (int b = tid / 32; b < nblk; b += NT / 32) {
-      int bi = 0, rest = b;
-      while (rest > bi) rest -= ++bi;  // block row bi holds bi + 1 blocks
-      const int i = c0 + 16 + 8 * bi + l / 8, c = c0 + 16 + 8 * rest + l % 8;
-      const T *x = S + i * LS + c0, *y = S + c * LS + c0;
-      T *o = S + i * LS + c, s0, s1;
-      if (sg) panel_dots<T, true>(x, x + 4 * LS, y, neg + c0, s0, s1);
-      else panel_dots<T, false>(x, x + 4 * LS, y, neg + c0, s0, s1);
-      if (c <= i) o[0] -= s0;
-      if (c <= i + 4) o[4 * LS] -= s1;
-    }
+    const int m = 48 - c0, nout = m * (m + 1) / 2;
+    if (m > 32) panel_trail<5>(S, LS, c0, tid, nout, W);
+    else if (m > 16) panel_trail<3>(S, LS, c0, tid, nout, W);
+    else if (tid < nout) panel_trail<1>(S, LS, c0, tid, nout, W);
     __syncthreads();
   }
-#pragma unroll 16
-  for (int q = 0; q < NB * NB / NT; q++) {
-    const int e = tid + NT * q, r = e / NB, c = e % NB;
-    if (r < kb && c <= r) A[(int64_t)r * F.ld + c] = S[r * LS + c];
+  // L_ij = s_j a_ij / L_jj, L_jj = sqrt(d) from d and 1 / sqrt(d)
+  if (tid < kb) {
+    const T d = piv[tid], r = inv_sqrt(d), l0 = d * r;
+    col[0][tid] = r;
+    col[1][tid] = fma(fma(-l0, l0, d), T(0.5) * r, l0);
+  }
+  __syncthreads();
+#pragma unroll 2
+  for (int q = 0; q < NB * NV / NT; q++) {
+    const int e = tid + NT * q, r = e / NV, c = VW * (e % NV);
+    if (r >= kb || c > r) continue;
+    Vec16<T> v;
+#pragma unroll
+    for (int h = 0; h < VW; h++) {
+      const T x = flip(S[r * LS + c + h] * col[0][c + h], neg[c + h] != 0);
+      v.v[h] = c + h < r ? x : c + h == r ? col[1][r] : T(0);
+    }
+    st16(A + (int64_t)r * F.ld + c, v);
   }
 }
 
