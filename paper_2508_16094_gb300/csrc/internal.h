@@ -76,11 +76,13 @@ enum SolveTaskKind : int32_t {
                      // published, y_i = L_ii^{-1} (.) (explicit inverse), publish y_i
   WS_FWD_BELOW = 1,  // (front, a = first row below the front of a 128-row chunk): gather,
                      // add L_rj y_j for every block j, store the front's update vector
-  WS_BWD_PART = 2,   // (front, b = first row below of a 128-row chunk): partial sums
+  WS_FWD_NARROW = 2, // (front): both of the above for a narrow front (narrow_front) in one task
+  WS_BWD_PART = 3,   // (front, b = first row below of a 128-row chunk): partial sums
                      // L_{r,cb}^T x_r of every column block cb, last first, once the
                      // parent front is done
-  WS_BWD_DIAG = 3    // (front, a = column block cb): the partial sums, L_{i,cb}^T x_i for
+  WS_BWD_DIAG = 4,   // (front, a = column block cb): the partial sums, L_{i,cb}^T x_i for
                      // i > cb as each x_i is published, x_cb = L_cc^{-T} (.), publish x_cb
+  WS_BWD_NARROW = 5  // (front): both of the above for a narrow front in one task
 };
 
 // Work of one level of the supernodal tree, as ranges into the task arrays.
@@ -174,6 +176,10 @@ struct LevelPlan {
 // per slot "partial sums done", per front "update-vector chunks of its children
 // done", "column blocks done".
 constexpr int kSolveB32 = 128, kSolveB64 = 64;  // block widths, FP32 and FP64
+// A front that one task solves in each sweep: its chunks of rows below hold less work
+// than a task costs.
+constexpr int kNarrowCols = 32, kNarrowRows = 512;
+inline bool narrow_front(const FrontInfo &F) { return F.ncol <= kNarrowCols && F.nrow <= kNarrowRows; }
 struct SolvePlan {
   int B = 0;
   std::vector<Task> inv;                  // (front, first column, slot)

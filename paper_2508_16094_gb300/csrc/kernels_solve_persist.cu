@@ -495,9 +495,11 @@ template <> struct FwdTile<double> {
 };
 
 // y = b[first + j + r] = sum_c Dinv[r][c] v[c]  (Dinv staged in S.di, v = S.sv
-// zero past jb), published in the slot's words; a warp's rows stop at their diagonal.
+// zero past jb), published in the slot's words and kept at `keep` if given; a warp's rows
+// stop at their diagonal.
 // FP32: warp w takes rows 16w .. 16w + 15
-__device__ void diag_fwd(const PsArgs<float> &A, PsShared<float> &S, const FrontInfo &F, int j, int slot) {
+__device__ void diag_fwd(const PsArgs<float> &A, PsShared<float> &S, const FrontInfo &F, int j, int slot,
+                         float *keep = nullptr) {
   constexpr int B = Ps<float>::B, RW = Ps<float>::RW;
   const int jb = min(B, F.ncol - j), ldi = (jb + 3) & ~3;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, c = 4 * lane, rw = RW * warp;
@@ -517,10 +519,12 @@ __device__ void diag_fwd(const PsArgs<float> &A, PsShared<float> &S, const Front
   if (lane % 2 == 0 && r < jb) {
     publish(slot_words<float>(A.ly, slot), r, s, A.epoch);
     A.b[F.first + j + r] = s;
+    if (keep) keep[r] = s;
   }
 }
 // FP64: four threads per row
-__device__ void diag_fwd(const PsArgs<double> &A, PsShared<double> &S, const FrontInfo &F, int j, int slot) {
+__device__ void diag_fwd(const PsArgs<double> &A, PsShared<double> &S, const FrontInfo &F, int j, int slot,
+                         double *keep = nullptr) {
   constexpr int B = Ps<double>::B;
   const int jb = min(B, F.ncol - j), ldi = (jb + 1) & ~1, r = threadIdx.x / 4, c = 2 * (threadIdx.x % 4);
   double s = 0.0;
@@ -531,6 +535,7 @@ __device__ void diag_fwd(const PsArgs<double> &A, PsShared<double> &S, const Fro
   if (threadIdx.x % 4 == 0 && r < jb) {
     publish(slot_words<double>(A.ly, slot), r, s, A.epoch);
     A.b[F.first + j + r] = s;
+    if (keep) keep[r] = s;
   }
 }
 
@@ -921,11 +926,134 @@ __device__ void bwd_diag(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R, 
   }
 }
 
+// A narrow front in one task (narrow_front: at most 32 columns and 512 rows below). The
+// lower half of a nested-dissection tree is thousands of such fronts, and a task costs 3
+// to 4 us whatever its size (ticket, record, the children's flag, two dependent gathers,
+// its own flag): one task a front and sweep instead of one per block and chunk of rows,
+// which also hands y to the rows below through shared memory. One solve, TF32x3: 666 ->
+// 574 us at 48^3, 1548 -> 1320 at 64^3, FP64 1302 -> 1180 at 40^3; eight right-hand
+// sides at 56^3 with PCG 15.2 -> 12.6 ms. (64 columns in FP32: 12.0 ms, nothing for one
+// right-hand side.)
+// Forward: a thread per row below (its L row in registers before the wait), the
+// diagonal block as in fwd_diag.
+template <typename T>
+__device__ void fwd_narrow(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R, Next &N) {
+  constexpr int B = Ps<T>::B, VW = Ps<T>::VW, NV = kNarrowCols / VW;
+  const FrontInfo &F = R.front;
+  const int nc = F.ncol, nr = F.nrow, tid = threadIdx.x;
+  if (tid == 0) stage_dinv(A, S, R.slot0, nc);
+  const T *rows = A.L + F.loff + (int64_t)nc * F.ld;
+  Vec<T> l[NV];
+  auto load = [&](int r) {
+#pragma unroll
+    for (int m = 0; m < NV; m++)
+      l[m] = (r < nr && VW * m < nc) ? ldg16(rows + (int64_t)r * F.ld + VW * m) : vzero<T>();
+  };
+  load(tid);
+  const bool ok = wait_children(A, S, F, R);
+  T g = T(0);
+  if (ok) {
+    if (tid < B) S.sv[tid] = tid < nc ? ldcg(A.a + F.first + tid) - gather_children(A, S, F, tid) : T(0);
+    if (tid < nr) g = gather_children(A, S, F, nc + tid);
+  }
+  if (tid >= nc && tid < kNarrowCols) S.xs[tid] = T(0);
+  take_next(A, N);
+  if (!wait_dinv(A, S, ok)) return;  // (a barrier: S.sv is written)
+  diag_fwd(A, S, F, 0, R.slot0, S.xs);
+  __syncthreads();
+  for (int r0 = 0; r0 < nr; r0 += kT) {
+    const int r = r0 + tid;
+    if (r0 > 0) {
+      load(r);
+      g = r < nr ? gather_children(A, S, F, nc + r) : T(0);
+    }
+    T s = T(0);
+#pragma unroll
+    for (int m = 0; m < NV; m++)
+      if (VW * m < nc) {
+        Vec<T> v = l[m];
+#pragma unroll
+        for (int h = 1; h < VW; h++)
+          if (VW * m + h >= nc) v.v[h] = T(0);  // (padding of the row)
+        s = vdot(v, ld16(S.xs + VW * m), s);
+      }
+    if (r < nr) A.t[R.toff + r] = g + s;
+  }
+  if (nr > 0) signal(f_tvec(A, F.parent));
+}
+
+// Backward: 2^lg threads per row, each the VW columns of a 16-byte load, down the rows
+// below; sums across a warp's rows by shuffles and across the warps through shared
+// memory, then the diagonal block as in bwd_diag. The solution at the rows below sits in
+// the part of S.di past the staged inverse.
+template <typename T>
+__device__ void bwd_narrow(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R, Next &N) {
+  constexpr int VW = Ps<T>::VW, NL = 8;
+  static_assert(kNarrowCols * kNarrowCols + kNarrowRows <= Ps<T>::B * Ps<T>::B, "room past the staged inverse");
+  static_assert(kNarrowRows <= 2 * kT && kNarrowCols / VW <= 16 && kNarrowCols <= 32, "rows and columns per thread");
+  const FrontInfo &F = R.front;
+  const int nc = F.ncol, nr = F.nrow, tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+  if (tid == 0) stage_dinv(A, S, R.slot0, nc);
+  int lg = 0;
+  while ((VW << lg) < nc) lg++;
+  const int cg = 1 << lg, c = VW * (tid & (cg - 1)), rr = tid >> lg, rp = kT >> lg;
+  const T *P = A.L + F.loff + (int64_t)nc * F.ld + c;
+  T *xs = S.di + kNarrowCols * kNarrowCols;
+  Vec<T> l[NL];
+  auto load = [&](int r0) {
+#pragma unroll
+    for (int k = 0; k < NL; k++) {
+      const int r = r0 + rr + k * rp;
+      l[k] = (c < nc && r < nr) ? ldg16(P + (int64_t)r * F.ld) : vzero<T>();
+    }
+  };
+  load(0);
+  const int32_t *ri = A.dp.sri + F.rows_off;
+  const int32_t i0 = tid < nr ? ri[tid] : 0, i1 = tid + kT < nr ? ri[tid + kT] : 0;
+  bool ok = F.parent < 0 || wait_flag(A, S, f_front(A, F.parent), (unsigned)R.parent_blocks);
+  take_next(A, N);
+  T bv = T(0);
+  if (ok) {
+    if (tid < nr) xs[tid] = ldcg(A.x + i0);
+    if (tid + kT < nr) xs[tid + kT] = ldcg(A.x + i1);
+    const uint2 *words = slot_words<T>(A.ly, R.slot0);
+    if (A.fwd_here) ok = wait_words(A, words, false, [&]() { return tid >= nc || read_word(words, tid, A.epoch, bv); });
+    else if (tid < nc) bv = ldcg(A.b + F.first + tid);
+  }
+  __syncthreads();
+  Vec<T> acc = vzero<T>();
+  for (int r0 = 0; r0 < nr && ok; r0 += NL * rp) {
+    if (r0 > 0) load(r0);
+#pragma unroll
+    for (int k = 0; k < NL; k++) {
+      const int r = r0 + rr + k * rp;
+      if (r < nr) acc = vfma(l[k], xs[r], acc);
+    }
+  }
+  for (int o = cg; o < 32; o <<= 1)
+#pragma unroll
+    for (int h = 0; h < VW; h++) acc.v[h] += __shfl_xor_sync(0xffffffffu, acc.v[h], o);
+  if (lane < cg) st16(S.red4[warp] + c, acc);
+  __syncthreads();
+  if (tid < nc) {
+    T s = S.red4[0][tid];
+#pragma unroll
+    for (int w = 1; w < kT / 32; w++) s += S.red4[w][tid];
+    S.sv[tid] = bv - s;
+  }
+  if (wait_dinv(A, S, ok)) {  // (ends with a barrier)
+    diag_bwd(A, S, F, 0, R.slot0);
+    signal(f_front(A, R.task.front));
+  }
+}
+
 template <typename T> __device__ __forceinline__ void run_task(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R, Next &N) {
   switch (R.task.c) {
     case WS_FWD_DIAG: fwd_diag(A, S, R, N); break;
     case WS_FWD_BELOW: fwd_below(A, S, R, N); break;
+    case WS_FWD_NARROW: fwd_narrow(A, S, R, N); break;
     case WS_BWD_PART: bwd_part(A, S, R, N); break;
+    case WS_BWD_NARROW: bwd_narrow(A, S, R, N); break;
     default: bwd_diag(A, S, R, N); break;
   }
 }

@@ -843,15 +843,22 @@ void build_fused_solve(const Plan &pl, int B, SolvePlan &sp) {
   }
   sp.dinv_entries = std::max<int64_t>(sp.dinv_entries, 4);
   auto nblk = [&](int32_t s) { return (pl.fronts[s].ncol + B - 1) / B; };
+  auto nbelow = [&](int32_t s) {  // tasks that finish a front's update vector
+    const FrontInfo &F = pl.fronts[s];
+    return narrow_front(F) ? (F.nrow > 0 ? 1 : 0) : (F.nrow + RC - 1) / RC;
+  };
   // forward, leaves to root, level by level: the diagonal chunks of every front
   // of the level (ascending), then the chunks of rows below the fronts
   for (const LevelPlan &LP : pl.levels) {
     for (int32_t t = LP.front_b; t < LP.front_e; t++) {
       const int32_t s = pl.level_fronts[t];
-      for (int32_t i = 0; i < nblk(s); i++) sp.tasks.push_back({s, i, 0, WS_FWD_DIAG});
+      if (narrow_front(pl.fronts[s])) sp.tasks.push_back({s, 0, 0, WS_FWD_NARROW});
+      else
+        for (int32_t i = 0; i < nblk(s); i++) sp.tasks.push_back({s, i, 0, WS_FWD_DIAG});
     }
     for (int32_t t = LP.front_b; t < LP.front_e; t++) {
       const int32_t s = pl.level_fronts[t];
+      if (narrow_front(pl.fronts[s])) continue;
       for (int32_t r0 = 0; r0 < pl.fronts[s].nrow; r0 += RC) sp.tasks.push_back({s, r0, 0, WS_FWD_BELOW});
     }
   }
@@ -870,11 +877,14 @@ void build_fused_solve(const Plan &pl, int B, SolvePlan &sp) {
     const LevelPlan &LP = pl.levels[li];
     for (int32_t t = LP.front_b; t < LP.front_e; t++) {
       const int32_t s = pl.level_fronts[t];
+      if (narrow_front(pl.fronts[s])) continue;
       for (int32_t r0 = 0; r0 < pl.fronts[s].nrow; r0 += RC) sp.tasks.push_back({s, 0, r0, WS_BWD_PART});
     }
     for (int32_t t = LP.front_b; t < LP.front_e; t++) {
       const int32_t s = pl.level_fronts[t];
-      for (int32_t cb = nblk(s) - 1; cb >= 0; cb--) sp.tasks.push_back({s, cb, 0, WS_BWD_DIAG});
+      if (narrow_front(pl.fronts[s])) sp.tasks.push_back({s, 0, 0, WS_BWD_NARROW});
+      else
+        for (int32_t cb = nblk(s) - 1; cb >= 0; cb--) sp.tasks.push_back({s, cb, 0, WS_BWD_DIAG});
     }
   }
   sp.kid_chunks.assign(nfr, 0);
@@ -882,7 +892,7 @@ void build_fused_solve(const Plan &pl, int B, SolvePlan &sp) {
   for (int32_t s = 0; s < nfr; s++) {
     const int32_t par = pl.fronts[s].parent;
     if (par >= 0) {
-      sp.kid_chunks[par] += (pl.fronts[s].nrow + RC - 1) / RC;
+      sp.kid_chunks[par] += nbelow(s);
       sp.parent_blocks[s] = nblk(par);
     }
   }
@@ -901,16 +911,27 @@ void build_fused_solve(const Plan &pl, int B, SolvePlan &sp) {
   std::vector<int32_t> bwd_part_seen(nfr, 0), level_of(nfr, -1);
   for (size_t li = 0; li < pl.levels.size(); li++)
     for (int32_t t = pl.levels[li].front_b; t < pl.levels[li].front_e; t++) level_of[pl.level_fronts[t]] = (int32_t)li;
-  auto nbelow = [&](int32_t s) { return (pl.fronts[s].nrow + RC - 1) / RC; };
   for (size_t q = 0; q < sp.tasks.size(); q++) {
     const Task &t = sp.tasks[q];
     need(t.front >= 0 && t.front < nfr, "task front");
     const FrontInfo &F = pl.fronts[t.front];
     need(F.ld % vw == 0 && F.loff % vw == 0, "panel alignment");
-    need((q < (size_t)sp.fwd_tasks) == (t.c <= WS_FWD_BELOW) && t.c >= 0 && t.c <= WS_BWD_DIAG,
+    need((q < (size_t)sp.fwd_tasks) == (t.c <= WS_FWD_NARROW) && t.c >= 0 && t.c <= WS_BWD_NARROW,
          "task order");
     const int32_t s = t.front;
+    need((t.c == WS_FWD_NARROW || t.c == WS_BWD_NARROW) == narrow_front(F), "narrow front");
     switch (t.c) {
+      case WS_FWD_NARROW:
+        need(nblk(s) == 1 && t.a == 0 && fwd_diag_seen[s]++ == 0, "forward narrow task");
+        for (int32_t ci = F.child_begin; ci < F.child_end; ci++)
+          need(fwd_below_seen[pl.children[ci]] == nbelow(pl.children[ci]), "forward child order");
+        fwd_below_seen[s] = nbelow(s);
+        break;
+      case WS_BWD_NARROW:
+        need(nblk(s) == 1 && t.a == 0 && bwd_diag_seen[s]++ == 0 &&
+                 (F.parent < 0 || bwd_diag_seen[F.parent] == nblk(F.parent)) && (F.parent >= 0 || F.nrow == 0),
+             "backward narrow task");
+        break;
       case WS_FWD_DIAG:
         need(t.a == fwd_diag_seen[s]++ && t.a < nblk(s), "forward diagonal task");
         for (int32_t ci = F.child_begin; ci < F.child_end; ci++)  // children complete before
