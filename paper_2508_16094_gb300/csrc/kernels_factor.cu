@@ -13,6 +13,7 @@
 #include <stdexcept>
 
 #include "launch.h"
+#include "ptx.cuh"
 
 namespace gipm {
 
@@ -317,7 +318,7 @@ __device__ __forceinline__ float inv_sqrt(float d) {
 }
 // 1 / d is r0 (1 + e + e^2), r0 the estimate and e = 1 - d r0 (|e| < 2^-20), and a / d
 // is a r0 plus (e + e^2) of it: a chain of three FP64 operations.
-__device__ __forceinline__ double recip_start(double d) { return widen(__fdividef(1.f, low_float(d))); }
+__device__ __forceinline__ double recip_start(double d) { return widen(ptx::rcp_estimate(low_float(d))); }
 __device__ __forceinline__ double recip_err(double d, double r0) {
   const double e = fma(-d, r0, 1.0);
   return fma(e, e, e);
@@ -418,18 +419,29 @@ __device__ __forceinline__ void potrf_panel(T *S, int ls, int c0, T (*col)[64], 
 __device__ __forceinline__ bool potrf_panel_fast(double *S, int ls, int c0, double (*col)[64], const int8_t *neg,
                                                  double *piv, double (*W)[64]) {
   const int t = threadIdx.x, i = t / 2, h = t % 2, act = 2 * (64 - c0);  // row c0 + i
+  // place of row r in col: the panel's 16 rows by parity, so that a thread's columns come
+  // in 16-byte reads
+  auto place = [](int r) { return r < 16 ? 8 * (r % 2) + r / 2 : r; };
+  const int mine = place(i);
   double x[8];
 #pragma unroll
   for (int q = 0; q < 8; q++) x[q] = S[(c0 + i) * ls + c0 + h + 2 * q];
   unsigned sign = 0;  // bit j: column j's pivot sign is negative
 #pragma unroll
   for (int j = 0; j < 16; j++) sign |= (neg[c0 + j] != 0 ? 1u : 0u) << j;
-  if (h == 0) col[0][i] = x[0];
+  if (h == 0) col[0][mine] = x[0];
   bar1(act);
   bool good = true;
-  double d = flip(col[0][0], sign & 1u), a = col[0][i], r0 = recip_start(d), v[8], w = 0.0;
+  double d = flip(col[0][0], sign & 1u), a = col[0][mine], r0 = recip_start(d), v[8], w = 0.0;
+  auto columns = [&](const double *c, int q0, double (&o)[8]) {  // q0 .. 7 (and one before)
 #pragma unroll
-  for (int q = 0; q < 8; q++) v[q] = col[0][h + 2 * q];
+    for (int q = 0; q < 8; q += 2)
+      if (q + 1 >= q0) {
+        const double2 f = *reinterpret_cast<const double2 *>(c + 8 * h + q);
+        o[q] = f.x, o[q + 1] = f.y;
+      }
+  };
+  columns(col[0], 0, v);
 #pragma unroll
   for (int j = 0; j < 16; j++) {
     good = good && in_fp32(d);
@@ -441,13 +453,12 @@ __device__ __forceinline__ bool potrf_panel_fast(double *S, int ls, int c0, doub
     const int qn = (j + 1) / 2;
     if (j % 2 == 1 || h == 1) x[qn] = fma(-w, v[qn], x[qn]);
     double *cn = col[(j + 1) % 3];
-    if (h == (j + 1) % 2) cn[i] = x[qn];
+    if (h == (j + 1) % 2) cn[mine] = x[qn];
     bar1(act);
-    d = flip(cn[j + 1], sign >> (j + 1) & 1u);
-    a = cn[i];
+    d = flip(cn[place(j + 1)], sign >> (j + 1) & 1u);
+    a = cn[mine];
     double u[8];
-#pragma unroll
-    for (int q = (j + 2) / 2; q < 8; q++) u[q] = cn[h + 2 * q];
+    columns(cn, (j + 2) / 2, u);
     r0 = recip_start(d);
 #pragma unroll
     for (int q = qn + 1; q < 8; q++) x[q] = fma(-w, v[q], x[q]);
@@ -502,7 +513,8 @@ __global__ void __launch_bounds__(kPotrfThreads) potrf_kernel(DevPlan dp, const 
   T *A = L + F.loff + (int64_t)k * F.ld + k;
   const int8_t *sg = dp.sgn ? dp.sgn + F.first + k : nullptr;
   __shared__ T S[NB * LS];  // the block; past kb: zero, with a unit diagonal
-  __shared__ T col[3][NB], piv[NB], W[16][NB];  // W: a panel's a_ij / d_j
+  __shared__ __align__(16) T col[3][NB];
+  __shared__ T piv[NB], W[16][NB];  // W: a panel's a_ij / d_j
   __shared__ int8_t neg[NB];
   const int tid = threadIdx.x;
   // 16 bytes at a time (rows are padded to 16 bytes, and zero past their last column)

@@ -64,6 +64,14 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
 }
 
+// The hardware's estimate of 1 / d for a normal d (no scaling of the extremes, as a
+// division has).
+__device__ __forceinline__ float rcp_estimate(float d) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+  return r;
+}
+
 // Completion of this CTA's issued products, signalled to an mbarrier of this CTA.
 __device__ __forceinline__ void mma_commit(uint64_t *bar) {
   asm volatile(
