@@ -117,51 +117,77 @@ __global__ void __launch_bounds__(128) dinv_kernel(DevPlan dp, const float *__re
   }
 }
 
-// FP64: inverse of one diagonal block (jb <= 64), thread c builds column c in
-// registers, right-looking: x_m is finished, then every row below it takes its
-// multiple (independent multiply-adds, where a row's dot product would be one
-// chain). Warp 1's columns start at row 32, so it skips the rows above. Bound
-// by the FP64 pipe (2608 warp multiply-adds, 20 us of one SM per block).
-template <int N>
-__device__ __forceinline__ void inverse_columns(const double *A, const double *rd, int ls, int r0, int c,
-                                                int jb, double (&x)[N]) {
-#pragma unroll
-  for (int i = 0; i < N; i++) x[i] = r0 + i == c ? 1.0 : 0.0;
-#pragma unroll
-  for (int m = 0; m < N; m++) {
-    if (r0 + m >= jb) break;
-    x[m] *= rd[r0 + m];
-#pragma unroll
-    for (int i = m + 1; i < N; i++) x[i] = fma(-x[m], A[(r0 + m) * ls + r0 + i], x[i]);
-  }
-}
-__global__ void __launch_bounds__(64) dinv64_kernel(DevPlan dp, const double *__restrict__ L,
-                                                    double *__restrict__ Dinv) {
-  constexpr int kB = Ps<double>::B, LS = kB + 1;
+// FP64: inverse of one diagonal block (jb <= 64), right-looking in panels of eight rows:
+// a thread per column finishes the panel's rows, then every row below takes their
+// multiples, two warps per quarter SM (an FP64 instruction occupies the quarter's unit
+// for 64 cycles whatever its active lanes). A 64-column block is 288 warp instructions on
+// the panels' warp and 336 on each quarter after them; with a thread per column down all
+// the rows it was 2080 on one, which a 64-column block took 70 us for wherever it stood,
+// and the last one of a factor waits for nothing else (augmented system of 1716 + 1716
+// unknowns: 78 -> 36 us).
+constexpr int kDinvThreads = 256;
+__global__ void __launch_bounds__(kDinvThreads) dinv64_kernel(DevPlan dp, const double *__restrict__ L,
+                                                              double *__restrict__ Dinv) {
+  constexpr int kB = Ps<double>::B, LS = kB + 1, Q = 4;
   const Task tk = dp.s64.inv[blockIdx.x];
   const FrontInfo F = dp.fronts[tk.front];
-  const int j = tk.a, jb = min(kB, F.ncol - j), ldi = (jb + 1) & ~1, c = threadIdx.x;
-  __shared__ double A[kB * LS];  // column m of the block: A[m * LS + i], zero past jb
+  const int j = tk.a, jb = min(kB, F.ncol - j), ldi = (jb + 1) & ~1, rows = (jb + 7) & ~7, tid = threadIdx.x;
+  extern __shared__ __align__(16) double smd64[];
+  double *A = smd64, *X = smd64 + kB * LS;  // L[i][m] at A[m LS + i] (zero past jb), X[i][c] at X[i kB + c]
   __shared__ double rd[kB];
   const double *g = L + F.loff + (int64_t)j * F.ld + j;
-#pragma unroll 16
-  for (int i = 0; i < kB; i++) A[c * LS + i] = (i < jb && c <= i) ? g[(int64_t)i * F.ld + c] : 0.0;
+  for (int e = tid; e < rows * kB; e += kDinvThreads) {
+    const int i = e / kB, c = e % kB;
+    const double v = (i < jb && c <= i) ? g[(int64_t)i * F.ld + c] : 0.0;
+    A[c * LS + i] = v;
+    X[e] = i == c ? 1.0 : 0.0;
+    if (i == c) rd[i] = i < jb ? 1.0 / v : 0.0;
+  }
   __syncthreads();
-  if (c < jb) rd[c] = 1.0 / A[c * LS + c];
-  __syncthreads();
+  for (int r0 = 0; r0 < rows; r0 += 8) {
+    const int nc = r0 + 8;  // columns that are not zero in these rows
+    if (tid < ((nc + 31) & ~31)) {
+      double x[8];
+#pragma unroll
+      for (int i = 0; i < 8; i++) x[i] = X[(r0 + i) * kB + tid];
+#pragma unroll
+      for (int m = 0; m < 8; m++) {
+        x[m] *= rd[r0 + m];
+#pragma unroll
+        for (int i = m + 1; i < 8; i++) x[i] = fma(-x[m], A[(r0 + m) * LS + r0 + i], x[i]);
+      }
+#pragma unroll
+      for (int i = 0; i < 8; i++) X[(r0 + i) * kB + tid] = x[i];
+    }
+    __syncthreads();
+    const int nout = (rows - nc) * nc;
+    if (tid < nout) {  // (at most 32 x 32 outputs: Q per thread)
+      double s[Q];
+      int at[Q], row[Q], col[Q];
+#pragma unroll
+      for (int q = 0; q < Q; q++) {
+        const int e = min(tid + kDinvThreads * q, nout - 1), i = e / nc;
+        row[q] = nc + i;
+        col[q] = e - nc * i;
+        at[q] = row[q] * kB + col[q];
+        s[q] = X[at[q]];
+      }
+      const int n = (nout - (tid & ~31) + kDinvThreads - 1) / kDinvThreads;  // of this warp
+#pragma unroll
+      for (int m = 0; m < 8; m++)
+#pragma unroll
+        for (int q = 0; q < Q; q++)
+          if (q < n) s[q] = fma(-X[(r0 + m) * kB + col[q]], A[(r0 + m) * LS + row[q]], s[q]);
+#pragma unroll
+      for (int q = 0; q < Q; q++)
+        if (tid + kDinvThreads * q < nout) X[at[q]] = s[q];
+    }
+    __syncthreads();
+  }
   double *out = Dinv + dp.s64.dinv_off[tk.b];
-  if (c < 32) {
-    double x[kB];
-    inverse_columns<kB>(A, rd, LS, 0, c, jb, x);
-#pragma unroll
-    for (int i = 0; i < kB; i++)
-      if (i < jb && c < ldi) out[i * ldi + c] = c < jb ? x[i] : 0.0;
-  } else {
-    double x[kB / 2];
-    inverse_columns<kB / 2>(A, rd, LS, kB / 2, c, jb, x);
-#pragma unroll
-    for (int i = 0; i < kB; i++)
-      if (i < jb && c < ldi) out[i * ldi + c] = (i >= 32 && c < jb) ? x[i >= 32 ? i - 32 : 0] : 0.0;
+  for (int e = tid; e < jb * (ldi / 2); e += kDinvThreads) {
+    const int i = e / (ldi / 2), c = 2 * (e % (ldi / 2));
+    st16(out + i * ldi + c, Vec<double>{{c <= i ? X[i * kB + c] : 0.0, c + 1 <= i ? X[i * kB + c + 1] : 0.0}});
   }
 }
 
@@ -1145,8 +1171,16 @@ void launch_dinv(const DevPlan &dp, const Plan &plan, const double *L, double *D
                  cudaStream_t st) {
   const int n = (int)plan.s64.inv.size();
   if (n == 0) return;
+  constexpr int smem = kSolveB64 * (2 * kSolveB64 + 1) * (int)sizeof(double);
+  static bool attr[64] = {false};  // per device
+  int dev = 0;
+  ck(cudaGetDevice(&dev), "cudaGetDevice");
+  if (!attr[dev & 63]) {
+    ck(cudaFuncSetAttribute(dinv64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem), "dinv attribute");
+    attr[dev & 63] = true;
+  }
   note_launch();
-  dinv64_kernel<<<n, 64, 0, st>>>(dp, L, Dinv);
+  dinv64_kernel<<<n, kDinvThreads, smem, st>>>(dp, L, Dinv);
 }
 
 int64_t solve_words(const SolvePlan &sp) {  // one per FP32 value, two per FP64 value
