@@ -93,10 +93,12 @@ enum SolveTaskKind : int32_t {
 // and a block finds its front by bisection, so a front's O((nf / tile)^2)
 // update tiles need no list.
 constexpr int64_t kSms = 152;  // SMs the schedules are made for
-constexpr int kTrsmRows = 16;  // rows per batch of a panel solve's blocks
-// Batches per block, for `rows` rows in the launch: one while every block has an
-// SM of its own (a launch then lasts one batch), up to four beyond that, which
-// read the diagonal block once per 64 rows.
+// Rows per batch of a panel solve's blocks, for `rows` rows in the launch: as few as give
+// every block an SM of its own (a batch of 16, 8 or 4 rows takes 10, 6 or 4 us of an
+// SM's FP64 units and latencies). Batches per block: one while every block has an SM of
+// its own, up to four beyond that, which read the diagonal block once per 64 rows.
+constexpr int kTrsmRows = 16;
+inline int trsm_rows(int64_t rows) { return rows <= 4 * kSms ? 4 : rows <= 8 * kSms ? 8 : kTrsmRows; }
 inline int trsm_batches(int64_t rows) {
   const int64_t b = (rows + kTrsmRows * kSms - 1) / (kTrsmRows * kSms);
   return (int)(b < 1 ? 1 : b > 4 ? 4 : b);
@@ -110,7 +112,7 @@ struct UpdRange {
   int32_t k0 = 0, k1 = 0, c0 = 0, clim = 0, with_u = 0;
 };
 struct StepRange {
-  int32_t potrf_b = 0, potrf_e = 0, trsm_b = 0, trsm_e = 0, trsm_n = 0, trsm_bat = 1;
+  int32_t potrf_b = 0, potrf_e = 0, trsm_b = 0, trsm_e = 0, trsm_n = 0, trsm_bat = 1, trsm_rows = kTrsmRows;
   UpdRange next64, rest64;  // FP64: the next step's columns (with look-ahead), everything past them
   UpdRange upd32, sup32;  // FP32: the rest of the super-step; at its end everything past it
 };

@@ -569,24 +569,26 @@ __global__ void __launch_bounds__(kPotrfThreads) potrf_kernel(DevPlan dp, const 
 }
 
 // Rows below the diagonal block: X <- X L_kk^{-T} (X L_kk^{-T} S_k with pivot
-// signs) by substitution, kb <= 64, 16 rows at a time on four warps. P = 8 lanes
-// share a row (lane h keeps the columns of residue h mod 8 in registers); with unit
+// signs) by substitution, kb <= 64, R = 128 / P rows at a time on four warps. P lanes
+// share a row (lane h keeps the columns of residue h mod P in registers); with unit
 // columns u_c = L_:c / L_cc and z_c = x_c L_cc the substitution is z_c2 -= z_c
 // u_c2,c, and x = z / diag is formed once at the end, so a column costs its
 // multiply-adds and nothing else. Bound by the FP64 unit (64 cycles per warp
-// instruction on each quarter SM: 10 us per 16 rows and SM). A block takes `batches`
-// times 16 rows: more than one only when the rows exceed 16 per SM (trsm_batches),
+// instruction on each quarter SM: 10 us per 16 rows and SM, P = 8), and where there are
+// SMs to spare by fewer rows on each with more lanes a row (trsm_rows: P = 16 and 32,
+// half and a quarter of the instructions, then the chain of 64 exchanges and
+// multiply-adds; 31 launches of at most 1216 rows: 16.5 us each with P = 8, 12.0 with
+// P = 16 and 8.6 with P = 32). A block takes `batches`
+// times R rows: more than one only when the rows exceed 16 per SM (trsm_batches),
 // so that a 3008-row front reaches every SM (128 rows a block, as before: 24
 // blocks, 169 us a launch on the 32^3 grid); the code of a batch is unrolled over
 // the columns and fits the instruction cache, which wider per-warp tiles (16
 // rows a warp, 56 KB of code run once) did not: 98 us against 55 us a launch on the
 // 40^3 grid.
-constexpr int kTrsmP = 8;
-template <typename T>
+template <typename T, int P>
 __global__ void __launch_bounds__(128) trsm_kernel(DevPlan dp, const Task *__restrict__ ents, int nent,
                                                    int batches, T *__restrict__ L) {
-  constexpr int NB = 64, LS = NB + 1, P = kTrsmP, NQ = NB / P;
-  static_assert(kTrsmRows == 4 * 32 / P, "rows per batch");
+  constexpr int NB = 64, LS = NB + 1, NQ = NB / P, R = 128 / P;
   int lo = 0, hi = nent - 1;  // the front this block's rows belong to
   while (lo < hi) {
     const int mid = (lo + hi + 1) / 2;
@@ -597,7 +599,7 @@ __global__ void __launch_bounds__(128) trsm_kernel(DevPlan dp, const Task *__res
   const FrontInfo F = dp.fronts[tk.front];
   const int nf = F.ncol + F.nrow, k = tk.b, kb = min(NB, F.ncol - k);
   const int tid = threadIdx.x, lane = tid % 32, h = lane % P;
-  int row = k + kb + batches * kTrsmRows * ((int)blockIdx.x - tk.a) + tid / P;
+  int row = k + kb + batches * R * ((int)blockIdx.x - tk.a) + tid / P;
   __shared__ T U[NB * LS];  // column c: u_c2,c at U[c * LS + c2]
   __shared__ T rd[NB];      // s_c / L_cc
   T *Xr = L + F.loff + (int64_t)row * F.ld + k;
@@ -641,8 +643,8 @@ __global__ void __launch_bounds__(128) trsm_kernel(DevPlan dp, const Task *__res
 #pragma unroll
     for (int q = 0; q < NQ; q++)
       if (row < nf && h + P * q < kb) Xr[h + P * q] = z[q] * rd[h + P * q];
-    row += kTrsmRows;
-    Xr += (int64_t)kTrsmRows * F.ld;
+    row += R;
+    Xr += (int64_t)R * F.ld;
     if (b + 1 < batches)
 #pragma unroll
       for (int q = 0; q < NQ; q++) z[q] = (row < nf && h + P * q < kb) ? Xr[h + P * q] : T(0);
@@ -712,7 +714,8 @@ template <typename T>
 void launch_trsm(const DevPlan &dp, const StepRange &S, T *L, cudaStream_t st) {
   if (S.trsm_n <= 0) return;
   note_launch();
-  trsm_kernel<T><<<S.trsm_n, 128, 0, st>>>(dp, dp.trsm + S.trsm_b, S.trsm_e - S.trsm_b, S.trsm_bat, L);
+  auto kernel = S.trsm_rows == 4 ? trsm_kernel<T, 32> : S.trsm_rows == 8 ? trsm_kernel<T, 16> : trsm_kernel<T, 8>;
+  kernel<<<S.trsm_n, 128, 0, st>>>(dp, dp.trsm + S.trsm_b, S.trsm_e - S.trsm_b, S.trsm_bat, L);
 }
 
 static void launch_upd(const DevPlan &dp, const UpdRange &u, double *L, double *U, cudaStream_t st) {

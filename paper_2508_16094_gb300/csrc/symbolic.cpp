@@ -580,11 +580,12 @@ void build_plan(const Problem &P, const Symbolic &S, Plan &plan, int nb, int nbs
       int64_t rows = 0;
       for (int32_t t = LP.front_b; t < LP.front_e; t++) rows += below(plan.fronts[plan.level_fronts[t]]);
       st.trsm_bat = trsm_batches(rows);
+      st.trsm_rows = trsm_rows(rows);
       for (int32_t t = LP.front_b; t < LP.front_e; t++) {
         const int32_t s = plan.level_fronts[t], r = below(plan.fronts[s]);
         if (r <= 0) continue;
         plan.trsm_ents.push_back({s, st.trsm_n, k, 0});
-        st.trsm_n += (r + kTrsmRows * st.trsm_bat - 1) / (kTrsmRows * st.trsm_bat);
+        st.trsm_n += (r + st.trsm_rows * st.trsm_bat - 1) / (st.trsm_rows * st.trsm_bat);
       }
       st.trsm_e = (int32_t)plan.trsm_ents.size();
       if (LP.ahead64 && k + nb < LP.max_ncol) st.next64 = upd_range(k + nb, k, k + nb, k + nb, k + 2 * nb, 0, kUpdTile64);
@@ -762,6 +763,7 @@ void validate_plan(const Problem &P, const Symbolic &S, const Plan &pl) {
   for (const LevelPlan &LP : pl.levels)
     for (const StepRange &S2 : LP.steps) {
       need(S2.trsm_bat >= 1 && S2.trsm_bat <= 4, "panel solve batches");
+      need(S2.trsm_rows == 4 || S2.trsm_rows == 8 || S2.trsm_rows == 16, "panel solve rows per batch");
       need(0 <= S2.trsm_b && S2.trsm_b <= S2.trsm_e && S2.trsm_e <= (int32_t)pl.trsm_ents.size(), "panel solve range");
       int64_t next = 0;
       for (int32_t i = S2.trsm_b; i < S2.trsm_e; i++) {
@@ -769,7 +771,7 @@ void validate_plan(const Problem &P, const Symbolic &S, const Plan &pl) {
         need(in_front(t) && t.a == next && t.b >= 0 && t.b < pl.fronts[t.front].ncol, "panel solve entry");
         const int64_t below = nf(t.front) - (t.b + std::min(pl.nb, pl.fronts[t.front].ncol - t.b));
         need(below > 0, "panel solve rows");
-        next += (below + kTrsmRows * S2.trsm_bat - 1) / (kTrsmRows * S2.trsm_bat);
+        next += (below + S2.trsm_rows * S2.trsm_bat - 1) / (S2.trsm_rows * S2.trsm_bat);
       }
       need(next == S2.trsm_n, "panel solve block count");
       check_upd(S2.next64, kUpdTile64);
