@@ -103,13 +103,16 @@ inline int trsm_batches(int64_t rows) {
   const int64_t b = (rows + kTrsmRows * kSms - 1) / (kTrsmRows * kSms);
   return (int)(b < 1 ? 1 : b > 4 ? 4 : b);
 }
-constexpr int kUpdTile64 = 32;  // update tile, FP64
+// Update tile, FP64: 32, and 16 where the launch has at most half a block of 32 per SM: a
+// 32 x 32 tile of 64 columns is 16 us of an SM's FP64 units, a 16 x 16 tile 4 us, and
+// there are SMs for four times as many.
+constexpr int kUpdTile64 = 32, kUpdTileSmall64 = 16;
 constexpr int kUpdTile32 = 64;  // update tile, FP32
 // One trailing-update launch: columns from min(c0, ncol) to min(clim, ncol) of
 // the panels, and with_u the update matrices, by the columns [k0, min(k1, ncol)).
 struct UpdRange {
   int32_t b = 0, e = 0, n = 0;  // entries, blocks
-  int32_t k0 = 0, k1 = 0, c0 = 0, clim = 0, with_u = 0;
+  int32_t k0 = 0, k1 = 0, c0 = 0, clim = 0, with_u = 0, ts = 0;
 };
 struct StepRange {
   int32_t potrf_b = 0, potrf_e = 0, trsm_b = 0, trsm_e = 0, trsm_n = 0, trsm_bat = 1, trsm_rows = kTrsmRows;

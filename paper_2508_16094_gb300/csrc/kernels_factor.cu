@@ -721,8 +721,8 @@ void launch_trsm(const DevPlan &dp, const StepRange &S, T *L, cudaStream_t st) {
 static void launch_upd(const DevPlan &dp, const UpdRange &u, double *L, double *U, cudaStream_t st) {
   if (u.n <= 0) return;
   note_launch();
-  upd_kernel<double, kUpdTile64, 128, 64><<<u.n, 128, 0, st>>>(dp, dp.upd + u.b, u.e - u.b, u.k0, u.k1, u.c0,
-                                                               u.clim, u.with_u, L, U);
+  auto kernel = u.ts == kUpdTile64 ? upd_kernel<double, kUpdTile64, 128, 64> : upd_kernel<double, kUpdTileSmall64, 128, 64>;
+  kernel<<<u.n, 128, 0, st>>>(dp, dp.upd + u.b, u.e - u.b, u.k0, u.k1, u.c0, u.clim, u.with_u, L, U);
 }
 static void launch_upd(const DevPlan &dp, const UpdRange &u, float *L, float *U, cudaStream_t st) {
   if (u.n <= 0) return;

@@ -532,7 +532,16 @@ void build_plan(const Problem &P, const Symbolic &S, Plan &plan, int nb, int nbs
     LP.steps.clear();
     // the level's fronts with more than `past` columns, numbered for one update launch
     auto upd_range = [&](int32_t past, int32_t k0, int32_t k1, int32_t c0, int32_t clim, int with_u, int TS) {
+      if (TS == kUpdTile64) {
+        int64_t n = 0;
+        for (int32_t t = LP.front_b; t < LP.front_e; t++) {
+          const FrontInfo &F = plan.fronts[plan.level_fronts[t]];
+          if (F.ncol > past) n += upd_tiles(F.ncol, F.nrow, c0, clim, with_u, TS);
+        }
+        if (2 * n <= kSms) TS = kUpdTileSmall64;
+      }
       UpdRange u;
+      u.ts = TS;
       u.b = (int32_t)plan.upd_ents.size();
       u.k0 = k0;
       u.k1 = k1;
@@ -740,7 +749,9 @@ void validate_plan(const Problem &P, const Symbolic &S, const Plan &pl) {
     need(in_front(t) && t.a >= 0 && t.a < pl.fronts[t.front].ncol, "potrf task");
   // block numbering of the panel solves and updates: ranges, consecutive
   // numbers, and the first and last tile of every front inside the front
-  auto check_upd = [&](const UpdRange &u, int TS) {
+  auto check_upd = [&](const UpdRange &u, bool fp64) {
+    const int TS = u.ts;
+    need(u.n == 0 || (fp64 ? TS == kUpdTile64 || TS == kUpdTileSmall64 : TS == kUpdTile32), "update tile size");
     need(0 <= u.b && u.b <= u.e && u.e <= (int32_t)pl.upd_ents.size(), "update range");
     int64_t next = 0;
     for (int32_t i = u.b; i < u.e; i++) {
@@ -774,8 +785,8 @@ void validate_plan(const Problem &P, const Symbolic &S, const Plan &pl) {
         next += (below + S2.trsm_rows * S2.trsm_bat - 1) / (S2.trsm_rows * S2.trsm_bat);
       }
       need(next == S2.trsm_n, "panel solve block count");
-      check_upd(S2.next64, kUpdTile64);
-      check_upd(S2.rest64, kUpdTile64);
+      check_upd(S2.next64, true);
+      check_upd(S2.rest64, true);
       const int32_t c0 = S2.rest64.k1;  // columns past the step's, each in one of the two
       if (S2.next64.n > 0)
         need(S2.next64.c0 == c0 && S2.next64.clim == S2.rest64.c0 && S2.next64.k0 == S2.rest64.k0 &&
@@ -783,8 +794,8 @@ void validate_plan(const Problem &P, const Symbolic &S, const Plan &pl) {
              "update halves");
       else
         need(S2.rest64.c0 == c0 || c0 >= LP.max_ncol, "update columns left out");
-      check_upd(S2.upd32, kUpdTile32);
-      check_upd(S2.sup32, kUpdTile32);
+      check_upd(S2.upd32, false);
+      check_upd(S2.sup32, false);
     }
   for (const Task &t : pl.gath_tasks)
     need(in_front(t) && t.a >= 0 && t.a < nf(t.front), "gather task");
