@@ -103,9 +103,10 @@ inline int trsm_batches(int64_t rows) {
   const int64_t b = (rows + kTrsmRows * kSms - 1) / (kTrsmRows * kSms);
   return (int)(b < 1 ? 1 : b > 4 ? 4 : b);
 }
-// Update tile, FP64: 32, and 16 where the launch has at most half a block of 32 per SM: a
-// 32 x 32 tile of 64 columns is 16 us of an SM's FP64 units, a 16 x 16 tile 4 us, and
-// there are SMs for four times as many.
+// Update tile, FP64: 32, and 16 where the launch has at most two blocks of 32 per SM: a
+// 32 x 32 tile of 64 columns is 16 us of an SM's FP64 units, a 16 x 16 tile 4 us, so the
+// last wave is shorter (31 launches of 3 to 438 tiles: 20.2 us each with 32 throughout;
+// with 16 up to half a block per SM a direction takes 2.48 ms, up to two 2.39).
 constexpr int kUpdTile64 = 32, kUpdTileSmall64 = 16;
 constexpr int kUpdTile32 = 64;  // update tile, FP32
 // One trailing-update launch: columns from min(c0, ncol) to min(clim, ncol) of

@@ -538,7 +538,7 @@ void build_plan(const Problem &P, const Symbolic &S, Plan &plan, int nb, int nbs
           const FrontInfo &F = plan.fronts[plan.level_fronts[t]];
           if (F.ncol > past) n += upd_tiles(F.ncol, F.nrow, c0, clim, with_u, TS);
         }
-        if (2 * n <= kSms) TS = kUpdTileSmall64;
+        if (n <= 2 * kSms) TS = kUpdTileSmall64;
       }
       UpdRange u;
       u.ts = TS;
