@@ -52,10 +52,10 @@ struct ipm_ctx {
   double *jv_copy = nullptr, *D_copy = nullptr, *wv_copy = nullptr;  // inputs kept for refinement
   float *Llo = nullptr;  // low parts of the split-TF32 factor
   float *dinv = nullptr, *fsa = nullptr, *fsb = nullptr, *fsx = nullptr;  // persistent FP32 solve
-  double *dinv64 = nullptr, *dsb = nullptr, *dsx = nullptr, *pspart64 = nullptr;  // FP64 (a: yv)
+  double *dinv64 = nullptr, *dsb = nullptr, *dsx = nullptr;  // FP64 (a: yv)
   unsigned *psflags = nullptr;  // its tickets, flags and counters
-  float *pspart = nullptr;    // its partial sums
-  SolveWords psw32, psw64;    // its published entries
+  void *pspart = nullptr;     // its partial sums, of either type
+  SolveWords psw;             // its published entries, of either type
   // do_solves: r, z, p, q of right-hand sides 1 .. (four n each), and the scalars of all (kRhsScal each)
   double *vrk = nullptr, *rscal = nullptr;
   // learned correction of a stale factor
@@ -292,17 +292,14 @@ void layout(ipm_ctx *c, char *base) {
   c->fsb = cv.take<float>(R * n);
   c->fsx = cv.take<float>(R * n);
   c->psflags = cv.take<unsigned>(R * std::max<int64_t>(std::max(pl.s32.flag_words, pl.s64.flag_words), 32));
-  c->pspart = cv.take<float>(R * std::max<int64_t>(pl.s32.part_entries, 1));
-  const int64_t nw32 = R * solve_words(pl.s32), nw64 = R * solve_words(pl.s64);
-  c->psw32.y = cv.take<uint2>(nw32);
-  c->psw32.x = cv.take<uint2>(nw32);
+  c->pspart = cv.take<double>(R * (std::max(pl.s32.part_entries / 2, pl.s64.part_entries) + 1));
+  c->psw.count = R * std::max(solve_words(pl.s32), solve_words(pl.s64));
+  c->psw.y = cv.take<uint2>(c->psw.count);
+  c->psw.x = cv.take<uint2>(c->psw.count);
   if (!pl.s64.tasks.empty()) {
     c->dinv64 = cv.take<double>(pl.s64.dinv_entries);
     c->dsb = cv.take<double>(R * n);
     c->dsx = cv.take<double>(R * n);
-    c->pspart64 = cv.take<double>(R * pl.s64.part_entries);
-    c->psw64.y = cv.take<uint2>(nw64);
-    c->psw64.x = cv.take<uint2>(nw64);
   }
   {  // learned-correction buffers (only when enabled)
     LearnedBufs &B = c->lb;
@@ -426,20 +423,20 @@ ipm_status do_factor(ipm_ctx *c, int prec, int32_t *bad_col) {
 template <typename T> void launch_held_solve(ipm_ctx *c, int which, int nrhs) {
   constexpr bool f64 = sizeof(T) == 8;
   const SolvePlan &sp = f64 ? c->plan.s64 : c->plan.s32;
-  SolveWords &words = f64 ? c->psw64 : c->psw32;
   SolveBufs<T> v;
   if constexpr (f64) {
-    v.a = c->yv, v.b = c->dsb, v.x = c->dsx, v.t = c->tv, v.part = c->pspart64;
+    v.a = c->yv, v.b = c->dsb, v.x = c->dsx, v.t = c->tv;
   } else {
-    v.a = c->fsa, v.b = c->fsb, v.x = c->fsx, v.t = reinterpret_cast<float *>(c->tv), v.part = c->pspart;
+    v.a = c->fsa, v.b = c->fsb, v.x = c->fsx, v.t = reinterpret_cast<float *>(c->tv);
   }
+  v.part = static_cast<T *>(c->pspart);
   v.flags = c->psflags;
   v.sd = SolveStride{std::max<int64_t>(c->P.n, 1), c->plan.t_entries, sp.part_entries, sp.flag_words,
                      solve_words(sp)};
   const T *Dinv;
   if constexpr (f64) Dinv = c->dinv64;
   else Dinv = c->dinv;
-  launch_psolve<T>(c->dp, c->plan, (const T *)c->L, Dinv, v, nrhs, words, c->status, which != 2, which != 1,
+  launch_psolve<T>(c->dp, c->plan, (const T *)c->L, Dinv, v, nrhs, c->psw, c->status, which != 2, which != 1,
                    c->st, c->test_spins, c->test_withhold);
   c->test_spins = 0;
   c->test_withhold = -1;
@@ -1212,13 +1209,9 @@ ipm_status ipm_set_workspace(ipm_ctx *c, void *buf, size_t bytes) {
     const size_t total = c->ws_need;
     layout(c, base);
     CK(cudaMemsetAsync(c->ticket, 0, sizeof(unsigned), c->st));
-    for (auto [w, sp] : {std::pair<SolveWords *, const SolvePlan *>{&c->psw32, &c->plan.s32},
-                         {&c->psw64, &c->plan.s64}}) {
-      w->epoch = 0;  // no word carries a tag yet
-      if (sp->tasks.empty()) continue;
-      CK(cudaMemsetAsync(w->y, 0, kSolveRhs * solve_words(*sp) * sizeof(uint2), c->st));
-      CK(cudaMemsetAsync(w->x, 0, kSolveRhs * solve_words(*sp) * sizeof(uint2), c->st));
-    }
+    c->psw.epoch = 0;  // no word carries a tag yet
+    CK(cudaMemsetAsync(c->psw.y, 0, c->psw.count * sizeof(uint2), c->st));
+    CK(cudaMemsetAsync(c->psw.x, 0, c->psw.count * sizeof(uint2), c->st));
     CK(cudaStreamSynchronize(c->st));
     if (c->sys) {  // the formulation's system takes the rest of the buffer
       c->ws_need = total;

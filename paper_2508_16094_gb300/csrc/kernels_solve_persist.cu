@@ -1197,7 +1197,7 @@ void launch_psolve(const DevPlan &dp, const Plan &plan, const T *L, const T *Din
   if (q1 <= q0) return;
   ck(cudaMemsetAsync(v.flags, 0, (size_t)(nrhs * v.sd.flags) * sizeof(unsigned), st), "solve flags");
   if (++words.epoch == 0) {  // the tags start over
-    const size_t bytes = (size_t)(kSolveRhs * v.sd.words) * sizeof(uint2);
+    const size_t bytes = (size_t)words.count * sizeof(uint2);
     ck(cudaMemsetAsync(words.y, 0, bytes, st), "solve words");
     ck(cudaMemsetAsync(words.x, 0, bytes, st), "solve words");
     words.epoch = 1;

@@ -54,9 +54,11 @@ void launch_sign(const DevPlan &dp, V *y, cudaStream_t st);
 cudaError_t preload_level_solve();
 
 // Tagged entries the persistent solve hands from block to block (zeroed once, before
-// the first launch; each launch takes the next tag): solve_words(plan) each.
+// the first launch; each launch, of either type, takes the next tag): `count` words
+// each, solve_words(plan) of them per right-hand side.
 struct SolveWords {
   uint2 *y = nullptr, *x = nullptr;
+  int64_t count = 0;
   unsigned epoch = 0;
 };
 int64_t solve_words(const SolvePlan &sp);
