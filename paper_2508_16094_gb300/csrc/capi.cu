@@ -343,6 +343,7 @@ void layout(ipm_ctx *c, char *base) {
   c->Llo = c->storage_bytes == 8 ? (c->L ? reinterpret_cast<float *>(c->L) + pl.l_entries : nullptr)
                                  : cv.take<float>((size_t)pl.l_entries);
   c->U = cv.take<char>((size_t)pl.u_entries * c->storage_bytes);
+  c->dp.build_k = upload(cv, pl.build_k, st);
   c->ws_need = cv.off + 256;
 }
 

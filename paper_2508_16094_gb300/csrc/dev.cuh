@@ -24,6 +24,7 @@ struct DevPlan {
   const Task *build, *potrf, *trsm, *upd, *gath, *sdiag, *sgemv, *rgemv;
   const int64_t *toff;
   DevSolve s32, s64;  // persistent solves (s64: null unless the storage is sized for FP64)
+  const int64_t *build_k;  // K entries of the rows of each assembly tile, levels with LevelPlan::build_k
   const int64_t *k_slot, *k_poff, *k_w, *k_orig;
   const int32_t *k_pa, *k_pb, *k_diag;
   const int32_t *perm;  // final new -> old

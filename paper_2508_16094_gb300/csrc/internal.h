@@ -164,6 +164,7 @@ GIPM_HD inline UpdTile upd_decode(int ncol, int nrow, int k1, int clim, int with
 struct LevelPlan {
   int32_t front_b = 0, front_e = 0;  // into the level-ordered front list
   int32_t build_b = 0, build_e = 0;  // front-assembly tiles
+  int64_t build_k = -1;              // where the level's ranges start in Plan::build_k (-1: K by its own launch)
   int64_t k_b = 0, k_e = 0;          // K entries of this level's fronts
   int32_t gath_b = 0, gath_e = 0;    // solve gather tasks
   int32_t rg_b = 0, rg_e = 0;        // backward-solve tasks on the rows below the block
@@ -221,6 +222,7 @@ struct Plan {
   SolvePlan s32, s64;  // persistent solves (s64: when the storage is sized for FP64)
   // K entries in level-major order
   std::vector<int64_t> k_slot;   // element offset of L(i, j) in the factor storage
+  std::vector<int64_t> build_k;  // per assembly tile of a level with fuse_k: K entries of its rows, [first, end)
   std::vector<int64_t> k_poff;   // products [k_poff[q], k_poff[q+1])
   std::vector<int32_t> k_pa, k_pb;  // CSR positions of the two J factors of each product
   std::vector<int64_t> k_w;      // W value index or -1

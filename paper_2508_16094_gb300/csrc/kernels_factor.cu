@@ -3,7 +3,7 @@
 // elimination-tree parallelism), SIMT FMA path for FP64 and FP32.
 //
 // Per level of the supernodal tree: build every frontal matrix of the level
-// (gather of the children's update matrices, each entry written once), add the
+// (gather of the children's update matrices, each entry written once) and add the
 // K entries owned by the level, then factor the fronts block column by block
 // column: Cholesky of the diagonal block, triangular solve of the rows below,
 // right-looking update of the rest of the panel and of the update matrix
@@ -56,7 +56,9 @@ __device__ __forceinline__ void store4(double *p, double a, double b, double c, 
 // lower triangle per block of 128 threads; thread (row group g, column group
 // q) owns rows r0 + g + 8i (i < 8) and columns c0 + 4q .. c0 + 4q + 3. Each
 // entry is the sum, over the children in ascending order, of the matching
-// entry of the child's update matrix (through the child->front inverse map).
+// entry of the child's update matrix (through the child->front inverse map);
+// then, in levels of few tiles (FUSED), the K entries of the tile's rows that
+// fall in its columns are added to what the block has stored.
 // The maps of up to four children are staged together (one memory round
 // trip), and a child none of whose rows or none of whose columns fall in the
 // tile is skipped by the whole block. Panel tiles start at multiples of 64
@@ -66,12 +68,15 @@ __device__ __forceinline__ void store4(double *p, double a, double b, double c, 
 // enough bytes in flight per block for the chain of dependent loads
 // (task, front, children, maps) a tile starts with.
 constexpr int kBuildThreads = 128, kBuildGroup = 4;
-template <typename T>
-__global__ void __launch_bounds__(kBuildThreads) build_front_kernel(DevPlan dp, int32_t task0,
+template <typename T, bool FUSED>
+__global__ void __launch_bounds__(kBuildThreads) build_front_kernel(DevPlan dp, int32_t task0, int64_t build_k,
+                                                                    const double *__restrict__ kval,
                                                                     T *__restrict__ L,
                                                                     T *__restrict__ U) {
   constexpr int BT = kBuildTile, RS = kBuildThreads / (BT / 4), NR = BT / RS;  // 8 row groups, 8 rows each
   const Task tk = dp.build[task0 + blockIdx.x];
+  longlong2 kr = make_longlong2(0, 0);  // K entries of the tile's rows
+  if (FUSED) kr = *reinterpret_cast<const longlong2 *>(dp.build_k + build_k + 2 * (int64_t)blockIdx.x);
   const FrontInfo F = dp.fronts[tk.front];
   const int nf = F.ncol + F.nrow;
   const int r0 = tk.a, c0 = tk.b, w = tk.c;
@@ -124,20 +129,27 @@ __global__ void __launch_bounds__(kBuildThreads) build_front_kernel(DevPlan dp, 
       }
     }
   }
-  if (q4 >= w) return;
+  if (!FUSED && q4 >= w) return;
   const int c = c0 + q4;
   const bool panel = c0 < F.ncol;
   const int lim = panel ? F.ncol : nf;  // columns past lim are padding
 #pragma unroll
   for (int i = 0; i < NR; i++) {
     const int r = r0 + g + RS * i;
-    if (r >= nf) continue;
+    if (r >= nf || (FUSED && q4 >= w)) continue;
     T o[4];
 #pragma unroll
     for (int j = 0; j < 4; j++) o[j] = (c + j <= r && c + j < lim) ? acc[i][j] : T(0);
     T *dst = panel ? L + F.loff + (int64_t)r * F.ld + c
                    : U + F.uoff + (int64_t)(r - F.ncol) * F.uld + (c - F.ncol);
     if (panel || r >= F.ncol) store4(dst, o[0], o[1], o[2], o[3]);
+  }
+  if (!FUSED || kr.x == kr.y) return;
+  __syncthreads();  // the tile is stored
+  for (int64_t q = kr.x + tid; q < kr.y; q += kBuildThreads) {
+    const int64_t s = dp.k_slot[q], at = s - F.loff;
+    const int col = F.ncol > BT ? (int)(at % F.ld) : c0;
+    if (col >= c0 && col < c0 + w) L[s] = T((double)L[s] + kval[q]);
   }
 }
 
@@ -695,9 +707,14 @@ void launch_assemble(const DevPlan &dp, const double *jv, const double *D, const
 template <typename T>
 void launch_build_level(const DevPlan &dp, const LevelPlan &LP, const double *kval, T *L, T *U,
                         cudaStream_t st) {
+  const bool fused = LP.build_k >= 0;
   if (LP.build_e > LP.build_b)
-    { note_launch(); build_front_kernel<T><<<LP.build_e - LP.build_b, kBuildThreads, 0, st>>>(dp, LP.build_b, L, U); }
-  if (LP.k_e > LP.k_b)
+    {
+      auto kernel = fused ? build_front_kernel<T, true> : build_front_kernel<T, false>;
+      note_launch();
+      kernel<<<LP.build_e - LP.build_b, kBuildThreads, 0, st>>>(dp, LP.build_b, LP.build_k, kval, L, U);
+    }
+  if (!fused && LP.k_e > LP.k_b)
     { note_launch(); kadd_kernel<T><<<grid_for(LP.k_e - LP.k_b, 256), 256, 0, st>>>(dp, LP.k_b, LP.k_e, kval, L); }
 }
 

@@ -498,7 +498,7 @@ void build_plan(const Problem &P, const Symbolic &S, Plan &plan, int nb, int nbs
   const int GR = 256;       // solve gather positions per task
   const int SR = 128;       // solve forward-update rows per task
   const int SC = 256;       // solve backward-update columns per task
-  plan.build_tasks.clear(); plan.potrf_tasks.clear(); plan.trsm_ents.clear();
+  plan.build_tasks.clear(); plan.build_k.clear(); plan.potrf_tasks.clear(); plan.trsm_ents.clear();
   plan.upd_ents.clear(); plan.gath_tasks.clear();
   plan.sdiag_tasks.clear(); plan.sgemv_tasks.clear(); plan.rgemv_tasks.clear();
   plan.toff.assign(ns, 0);
@@ -529,6 +529,24 @@ void build_plan(const Problem &P, const Symbolic &S, Plan &plan, int nb, int nbs
       }
     }
     LP.build_e = (int32_t)plan.build_tasks.size();
+    // K's own launch is 2 to 3 us a level (2 % of a 10^3 system); in levels of many tiles it
+    // costs less than the trip through memory at the end of each of them (1 % of a 64^3
+    // system)
+    LP.build_k = -1;
+    if (LP.build_e - LP.build_b <= 8 * kSms) {
+      LP.build_k = (int64_t)plan.build_k.size();
+      for (int32_t t = LP.build_b; t < LP.build_e; t++) {
+        const Task &tk = plan.build_tasks[t];
+        const FrontInfo &F = plan.fronts[tk.front];
+        auto k_from = [&](int32_t row) {  // the level's entries are in slot order
+          return std::lower_bound(plan.k_slot.begin() + LP.k_b, plan.k_slot.begin() + LP.k_e,
+                                  F.loff + (int64_t)row * F.ld) - plan.k_slot.begin();
+        };
+        const bool panel = tk.b < F.ncol;
+        plan.build_k.push_back(panel ? k_from(tk.a) : 0);
+        plan.build_k.push_back(panel ? k_from(std::min(tk.a + BT, F.ncol + F.nrow)) : 0);
+      }
+    }
     LP.steps.clear();
     // the level's fronts with more than `past` columns, numbered for one update launch
     auto upd_range = [&](int32_t past, int32_t k0, int32_t k1, int32_t c0, int32_t clim, int with_u, int TS) {
@@ -819,6 +837,25 @@ void validate_plan(const Problem &P, const Symbolic &S, const Plan &pl) {
   for (size_t p = 0; p < pl.k_pa.size(); p++)
     need(pl.k_pa[p] >= 0 && pl.k_pa[p] < nnzj && pl.k_pb[p] >= 0 && pl.k_pb[p] < nnzj,
          "K product operands");
+  // every K entry of a level with fused assembly belongs to the rows of one band of tiles
+  for (const LevelPlan &LP : pl.levels) {
+    if (LP.build_k < 0) continue;
+    need(LP.build_k % 2 == 0 && LP.build_k + 2 * (int64_t)(LP.build_e - LP.build_b) <= (int64_t)pl.build_k.size(),
+         "build K ranges");
+    int64_t banded = 0;
+    for (int32_t t = LP.build_b; t < LP.build_e; t++) {
+      const Task &tk = pl.build_tasks[t];
+      const FrontInfo &F = pl.fronts[tk.front];
+      const int64_t kb = pl.build_k[LP.build_k + 2 * (t - LP.build_b)], ke = pl.build_k[LP.build_k + 2 * (t - LP.build_b) + 1];
+      need(0 <= kb && kb <= ke && ke <= (int64_t)pl.k_slot.size(), "build K range");
+      if (ke > kb)
+        need(tk.b < F.ncol && pl.k_slot[kb] >= F.loff + (int64_t)tk.a * F.ld &&
+                 pl.k_slot[ke - 1] < F.loff + (int64_t)std::min(tk.a + kBuildTile, F.ncol + F.nrow) * F.ld,
+             "build K rows");
+      if (tk.b == 0) banded += ke - kb;
+    }
+    need(banded == LP.k_e - LP.k_b, "K entries outside the build tiles");
+  }
   for (const LevelPlan &LP : pl.levels) {
     need(LP.build_b <= LP.build_e && LP.build_e <= (int32_t)pl.build_tasks.size(), "build range");
     need(LP.k_b <= LP.k_e && LP.k_e <= (int64_t)pl.k_slot.size(), "K range");
