@@ -2,10 +2,11 @@
 // factors, 128-wide blocks; FP64 storage: 64-wide blocks, so a lane reads 16
 // bytes of a row either way and a tile holds as many loads in flight).
 //
-// After each factorisation one launch inverts every diagonal block of L
-// (explicit inverse, rows padded to 16 bytes). A solve is then ONE launch of a persistent kernel whose CTAs take the tasks of the plan in
-// order from a global ticket counter (forward sweep leaves -> root, backward
-// sweep root -> leaves). Instead of grid barriers between phases, each task
+// After each factorisation one launch inverts every diagonal block of L (explicit
+// inverse, rows padded to 16 bytes). A solve is then ONE launch of a persistent kernel
+// whose CTAs take the tasks of the plan in order from a global ticket counter (forward
+// sweep leaves -> root, backward sweep root -> leaves), for one right-hand side or for
+// up to kSolveRhs side by side. Instead of grid barriers between phases, each task
 // waits only for the results it reads. Along the diagonal blocks of a front, whose
 // chain is the time of a solve, the entries of y and x carry their own flag: each
 // 32-bit half is stored with the launch's tag in one 8-byte word, and a
@@ -199,7 +200,7 @@ template <typename T> struct PsArgs {
   int32_t q0, q1;    // tasks [q0, q1) of the plan
   unsigned *ticket;  // ticket counter, and the solve plan's flag words, zeroed before the launch
   unsigned *flags;
-  uint2 *ly, *lx;    // published entries of y and x (see LL words), B per slot (FP64: 2 B)
+  uint2 *ly, *lx;    // published entries of y and x, B words per slot (FP64: 2 B)
   unsigned epoch;    // tag of this launch's entries
   int32_t *status;   // ST_SOLVE_TIMEOUT
   unsigned spins;    // polls before a wait gives up
@@ -595,9 +596,10 @@ __device__ __forceinline__ void put_sum(float *row, int c, const Vec<float> &s) 
 }
 __device__ __forceinline__ void put_sum(double *row, int c, double s) { row[c] = s; }
 
-// x[first + j + c] = sum_{r >= c} Dinv[r][c] v[r]  (Dinv staged in S.di, zero
-// above the diagonal; v = S.sv), published in the slot's words. FP32: thread (g, q) takes columns 4q .. and rows
-// 16g ..; FP64: four threads per column, and a warp's eight columns start at their diagonal.
+// x[first + j + c] = sum_{r >= c} Dinv[r][c] v[r]  (Dinv staged in S.di, zero above the
+// diagonal; v = S.sv), published in the slot's words. FP32: thread (g, q) takes columns
+// 4q .. and rows 16g ..; FP64: four threads per column, and a warp's eight columns start
+// at their diagonal.
 __device__ void diag_bwd(const PsArgs<float> &A, PsShared<float> &S, const FrontInfo &F, int j, int slot) {
   constexpr int B = Ps<float>::B, RW = Ps<float>::RW;
   const int jb = min(B, F.ncol - j), ldi = (jb + 3) & ~3;
@@ -1073,7 +1075,8 @@ __device__ void bwd_narrow(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R
   }
 }
 
-template <typename T> __device__ __forceinline__ void run_task(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R, Next &N) {
+template <typename T>
+__device__ __forceinline__ void run_task(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R, Next &N) {
   switch (R.task.c) {
     case WS_FWD_DIAG: fwd_diag(A, S, R, N); break;
     case WS_FWD_BELOW: fwd_below(A, S, R, N); break;

@@ -9,7 +9,8 @@
 // delta_p I is block tridiagonal with 16 x 16 blocks; it is factored by a
 // sequential block Cholesky over the stages.
 //
-// Execution: 16 lanes (half a warp) per instance; lane i holds row i of every
+// Execution (the FP32 variant; FP64 runs in mpc_cta.cu): 16 lanes (half a warp) per
+// instance; lane i holds row i of every
 // 16 x 16 block and the rows of g tied to variable i of the stage (dynamics row
 // i for i < 12, lower and upper bound of variable i). Rows of L blocks move
 // between lanes with width-16 shuffles. Instances come from an atomic queue
