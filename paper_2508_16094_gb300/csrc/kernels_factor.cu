@@ -749,7 +749,11 @@ static void launch_upd(const DevPlan &dp, const UpdRange &u, float *L, float *U,
 }
 
 void ChainStream::create() {
-  if (s) return;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) throw std::runtime_error("no current device");
+  if (s && dev == device) return;
+  destroy();
+  device = dev;
   int lo = 0, hi = 0;
   if (cudaDeviceGetStreamPriorityRange(&lo, &hi) != cudaSuccess ||
       cudaStreamCreateWithPriority(&s, cudaStreamNonBlocking, hi) != cudaSuccess ||
@@ -757,10 +761,12 @@ void ChainStream::create() {
       cudaEventCreateWithFlags(&updated, cudaEventDisableTiming) != cudaSuccess)
     throw std::runtime_error("cannot create the factorisation's chain stream");
 }
-ChainStream::~ChainStream() {
+void ChainStream::destroy() {
   if (solved) cudaEventDestroy(solved);
   if (updated) cudaEventDestroy(updated);
   if (s) cudaStreamDestroy(s);
+  solved = updated = nullptr;
+  s = nullptr;
 }
 
 // FP64 with look-ahead: the chain (diagonal block, panel solve, update of the

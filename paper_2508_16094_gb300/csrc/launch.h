@@ -17,11 +17,13 @@ void launch_assemble(const DevPlan &dp, const double *jv, const double *D, const
 struct ChainStream {
   cudaStream_t s = nullptr;                         // highest priority
   cudaEvent_t solved = nullptr, updated = nullptr;  // fork / join
+  int device = -1;
   ChainStream() = default;
   ChainStream(const ChainStream &) = delete;
   ChainStream &operator=(const ChainStream &) = delete;
-  ~ChainStream();
-  void create();
+  ~ChainStream() { destroy(); }
+  void create();  // on the current device
+  void destroy();
 };
 template <typename T>
 void launch_factor_simt(const DevPlan &dp, const Plan &plan, const double *kval, T *L, T *U,

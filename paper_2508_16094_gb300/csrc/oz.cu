@@ -617,7 +617,11 @@ void OzPlan::layout(Carve &cv, cudaStream_t st, bool storage) {
 void OzPlan::encode(const Plan &plan, cudaStream_t st) {
   ready_ = false;
   if (!sized_ || !S_) return;
-  if (!side_) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) throw std::runtime_error("no current device");
+  if (!side_ || dev != side_device_) {
+    destroy_streams();
+    side_device_ = dev;
     int lo = 0, hi = 0;
     cudaDeviceGetStreamPriorityRange(&lo, &hi);
     if (cudaStreamCreateWithPriority(&side_, cudaStreamNonBlocking, lo) != cudaSuccess ||
@@ -704,10 +708,12 @@ void OzPlan::factor(const DevPlan &dp, const Plan &plan, const double *kval, dou
   }
 }
 
-OzPlan::~OzPlan() {
+void OzPlan::destroy_streams() {
   if (ev_main_) cudaEventDestroy(ev_main_);
   if (ev_side_) cudaEventDestroy(ev_side_);
   if (side_) cudaStreamDestroy(side_);
+  ev_main_ = ev_side_ = nullptr;
+  side_ = nullptr;
 }
 
 }  // namespace gipm
