@@ -347,6 +347,13 @@ void layout(ipm_ctx *c, char *base) {
   c->ws_need = cv.off + 256;
 }
 
+// The larger one, NaN if either is (std::max drops its second argument's).
+double max_or_nan(double a, double b) { return std::isnan(b) || b > a ? b : a; }
+
+// 1 for a direction that is not a number: its iteration counts among the iterations done, as
+// the one after a step along it would find.
+int nan_step(const ipm_solve_info &si) { return std::isnan(si.rel_residual) ? 1 : 0; }
+
 double d2h_scalar(ipm_ctx *c, const double *p) {
   double v = 0;
   CK(cudaMemcpyAsync(&v, p, sizeof(double), cudaMemcpyDeviceToHost, c->st));
@@ -1290,7 +1297,7 @@ ipm_status kkt_solve(ipm_ctx *c, const double *b, double *x, int32_t nrhs, int32
         if (st[q] != IPM_OK && t != c) c->err = t->err;
         all.iterations += one[q].iterations;
         all.used_pcg = std::max(all.used_pcg, one[q].used_pcg);
-        all.rel_residual = std::max(all.rel_residual, one[q].rel_residual);
+        all.rel_residual = max_or_nan(all.rel_residual, one[q].rel_residual);
         if (st[q] != IPM_OK && worst == IPM_OK) worst = st[q];
       }
       k += K;
@@ -1400,13 +1407,12 @@ ipm_status ipm_solve(ipm_ctx *c, const double *jv, const double *b, const double
       res.primal_res = h.primal_inf / bscale;
       res.dual_res = h.dual_inf / cscale;
       res.compl_res = h.compl_inf / fs;
-      res.kkt = std::max(res.primal_res, std::max(res.dual_res, res.compl_res));
+      res.kkt = max_or_nan(res.primal_res, max_or_nan(res.dual_res, res.compl_res));
       res.objective = h.fx;
       res.mu = h.mu;
       if (o.verbose)
         std::fprintf(stderr, "ipm it %3d f % .10e kkt %.3e (p %.2e d %.2e c %.2e) mu %.2e\n", it,
                      h.fx, res.kkt, res.primal_res, res.dual_res, res.compl_res, h.mu);
-      // the maxima skip NaN, the sums (mu, f) do not
       if (!std::isfinite(res.kkt) || !std::isfinite(h.mu) || !std::isfinite(h.fx)) {
         res.status = IPM_ERR_NUMERIC;
         break;
@@ -1498,7 +1504,7 @@ ipm_status ipm_solve(ipm_ctx *c, const double *jv, const double *b, const double
         if (stt == IPM_OK)
           stt = direction(c, jv, b, cc, wv, x, s, lam, nullptr, c->vdx, c->vds, c->vdl, &si);
       }
-      if (stt != IPM_OK) { res.status = stt; c->learned_active = false; break; }
+      if (stt != IPM_OK) { res.status = stt; it += nan_step(si); c->learned_active = false; break; }
       V.ftb(s, c->vds, lam, c->vdl, c->sc, true);
       V.muaff(s, c->vds, lam, c->vdl, c->sc);
       // corrector: w = sigma mu - ds_aff .* dl_aff
@@ -1535,7 +1541,7 @@ ipm_status ipm_solve(ipm_ctx *c, const double *jv, const double *b, const double
       c->refine_override = c->pcg_override = -1;
       if (try_skip && !factored) res.learned_skips++;
       res.worst_rel_residual = std::max(res.worst_rel_residual, si.rel_residual);
-      if (stt != IPM_OK) { res.status = stt; break; }
+      if (stt != IPM_OK) { res.status = stt; it += nan_step(si); break; }
       CK(cudaEventRecord(ev[3], c->st));
       if (keep) {
         CK(cudaMemcpyAsync(keep, x, P.n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
@@ -1942,13 +1948,13 @@ ipm_status nlp_solve(ipm_ctx *c, const NlpFns &F, double *x, double *s, double *
       res.primal_res = h.primal_inf / bscale;
       res.dual_res = h.dual_inf / cscale;
       res.compl_res = h.compl_inf / fs;
-      res.kkt = std::max(res.primal_res, std::max(res.dual_res, res.compl_res));
+      res.kkt = max_or_nan(res.primal_res, max_or_nan(res.dual_res, res.compl_res));
       res.objective = f;
       res.mu = mu;
       if (o.verbose)
         std::fprintf(stderr, "nlp it %3d f % .10e kkt %.3e (p %.2e d %.2e c %.2e) mu %.2e\n", it, f,
                      res.kkt, res.primal_res, res.dual_res, res.compl_res, mu);
-      if (low_step && res.kkt > 10.0 * prev_kkt && o.fallback_fp64 && c->storage_bytes == 8) {
+      if (low_step && !(res.kkt <= 10.0 * prev_kkt) && o.fallback_fp64 && c->storage_bytes == 8) {
         CK(cudaMemcpyAsync(x, keep, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
         CK(cudaMemcpyAsync(s, keep + n, mt * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
         CK(cudaMemcpyAsync(lam, keep + n + mt, mt * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
@@ -2023,7 +2029,7 @@ ipm_status nlp_solve(ipm_ctx *c, const NlpFns &F, double *x, double *s, double *
         c->refine_override = -1;
       }
       res.worst_rel_residual = std::max(res.worst_rel_residual, si.rel_residual);
-      if (stt != IPM_OK) { res.status = stt; break; }
+      if (stt != IPM_OK) { res.status = stt; it += nan_step(si); break; }
       // common step from the fraction to the boundary, then backtracking on the merit
       set_sc(offsetof(IpmScalars, mu), mu);
       V.ftb(s, c->vds, lam, c->vdl, c->sc, false);

@@ -27,7 +27,8 @@ struct VecOps {
   double *partial;   // kRedBlocks * 8 doubles
   unsigned *ticket;  // one word, zero between launches (a reduction counts its finished blocks)
 
-  // out[0] = max |v|; with_scale: out[1] = 1 / out[0] (1 if that is 0 or not finite)
+  // out[0] = max |v| (NaN if one of them is); with_scale: out[1] = 1 / out[0] (1 if that is 0 or
+  // not finite)
   void absmax(int64_t n, const double *v, double *out, bool with_scale = false) const;
   void dot(int64_t n, const double *a, const double *b, double *out) const;
   void jv(const double *jvals, const double *x, double *out) const;

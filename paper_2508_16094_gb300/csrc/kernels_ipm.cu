@@ -14,16 +14,16 @@ namespace {
 
 constexpr int kRedBlock = 256;
 
-// |v| on the integer pipe, NaN as zero (the maxima skip NaN): an FP64 comparison
-// occupies GB300's FP64 unit as long as a multiply-add.
-__device__ __forceinline__ double abs_or_zero(double v) {
-  const long long b = __double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFll;
-  return b > 0x7FF0000000000000ll ? 0.0 : __longlong_as_double(b);
+// |v| and the larger of two of them on the integer pipe: an FP64 comparison
+// occupies GB300's FP64 unit as long as a multiply-add. The bits of a NaN compare above
+// those of infinity, so a maximum over values with a NaN among them is NaN.
+__device__ __forceinline__ double abs_bits(double v) {
+  return __longlong_as_double(__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFll);
 }
 __device__ __forceinline__ double max_nonneg(double a, double b) {
   return __double_as_longlong(a) > __double_as_longlong(b) ? a : b;
 }
-// RED_MAX combines values >= 0 (identity 0)
+// RED_MAX combines values >= 0 or NaN (identity 0)
 template <int OP> __device__ __forceinline__ double red_combine(double a, double b) {
   return OP == RED_SUM ? a + b : (OP == RED_MAX ? max_nonneg(a, b) : fmin(a, b));
 }
@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(kRedBlock) resid_cols_kernel(
   GRID_STRIDE(j, dp.n) {
     const double v = b[j] - kx_col(dp, jv, D, wv, delta_p, tA, x, j);
     r[j] = v;
-    m[0] = max_nonneg(m[0], abs_or_zero(v));
+    m[0] = max_nonneg(m[0], abs_bits(v));
   }
   grid_reduce<RED_MAX>(m, partial, ticket, [&](double (&v)[1]) {
     out[0] = v[0];
@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(kRedBlock) permute_out_dot_kernel(
 __global__ void __launch_bounds__(kRedBlock) absmax_kernel(int64_t n, const double *__restrict__ v, double *out,
                                                            int with_scale, double *partial, unsigned *ticket) {
   double a[1] = {0.0};
-  GRID_STRIDE(i, n) a[0] = max_nonneg(a[0], abs_or_zero(v[i]));
+  GRID_STRIDE(i, n) a[0] = max_nonneg(a[0], abs_bits(v[i]));
   grid_reduce<RED_MAX>(a, partial, ticket, [&](double (&m)[1]) {
     out[0] = m[0];
     if (with_scale) out[1] = scale_of(m[0]);
@@ -311,11 +311,11 @@ __global__ void __launch_bounds__(kRedBlock) kkt_reduce_kernel(
     if (i < dp.mt) {
       const double sl = s[i] * lam[i];
       v[0] += sl;
-      v[1] = max_nonneg(v[1], abs_or_zero(g[i] - s[i]));
-      v[2] = max_nonneg(v[2], abs_or_zero(sl));
+      v[1] = max_nonneg(v[1], abs_bits(g[i] - s[i]));
+      v[2] = max_nonneg(v[2], abs_bits(sl));
     } else {
       const int64_t j = i - dp.mt;
-      v[3] = max_nonneg(v[3], abs_or_zero(rd[j]));
+      v[3] = max_nonneg(v[3], abs_bits(rd[j]));
       v[4] = fma(c[j] + (wx ? 0.5 * wx[j] : 0.0), x[j], v[4]);
     }
   }
@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(kRedBlock) cg_step_kernel(
     x[i] = fma(a, p[i], x[i]);
     const double v = fma(-a, q[i], r[i]);
     r[i] = v;
-    m[0] = max_nonneg(m[0], abs_or_zero(v));
+    m[0] = max_nonneg(m[0], abs_bits(v));
   }
   grid_reduce<RED_MAX>(m, partial, ticket, [&](double (&v)[1]) {
     out[0] = v[0];
