@@ -20,7 +20,6 @@
 // FP64 unit meanwhile (five a SM: 46.1 ms for 4096 instances of 10 to 100 stages; four,
 // without register spills, 49.7; three 58.5). 16 lanes per instance took 180 ms with
 // the default shape (120 with the autotuned one), and 68 ms against 10.4 for 96 instances.
-#include <cfloat>
 #include <cmath>
 #include <stdexcept>
 #include <type_traits>
@@ -122,10 +121,21 @@ __device__ __forceinline__ double recip(double d) {
   const double r0 = recip_estimate(d), e = fma(-d, r0, 1.0);
   return fma(r0, fma(e, e, e), r0);
 }
+__device__ __noinline__ double slow_div(double a, double d) { return a / d; }
 __device__ __forceinline__ double quotient(double a, double d) {
-  if (!in_fp32(d)) return a * slow_recip(d);
+  if (!in_fp32(d) || !in_fp32(a)) return slow_div(a, d);  // (an infinite a stays infinite)
   const double r0 = recip_estimate(d), w0 = a * r0, e = fma(-d, r0, 1.0);
   return fma(w0, fma(e, e, e), w0);
+}
+
+// a / b < c / d of values >= 0 by cross products, by division where one of them may have left
+// FP64's range
+__device__ __noinline__ bool slow_less(double a, double b, double c, double d) { return a / b < c / d; }
+__device__ __forceinline__ bool ratio_less(double a, double b, double c, double d) {
+  const double p = a * d, q = c * b;
+  auto ordinary = [](double v) { return ((unsigned)__double2hiint(v) >> 20) - 100u < 1800u; };
+  if (!ordinary(p) || !ordinary(q)) return slow_less(a, b, c, d);
+  return bits(p) < bits(q);
 }
 
 constexpr int R_SUM = 0, R_MAX = 1, R_MIN = 2;  // max and min of non-negative values
@@ -484,7 +494,7 @@ __device__ __forceinline__ void make_rhs(const Inst &I, int i, int k0) {
 // smallest ratio v / (-dv) of a thread is kept as a fraction, compared by cross products.
 __device__ __forceinline__ void recover(Shared &S, const Inst &I, int i, int k0, double umax, double xmax,
                                         bool corrector, double sig_mu, double &mp, double &md) {
-  double pn = 1.0, pd = 0.0, dn = 1.0, dd = 0.0;  // (1, 0): no bound yet
+  double pn = 1e30, pd = 1.0, dn = 1e30, dd = 1.0;  // (a ratio above 1 bounds no step)
   const double lim = i < NU ? umax : xmax;
   for (int k = k0; k < I.T; k += kThreads / NS) {
     const double zi = I.z[k * NS + i], dzi = I.dz[k * NS + i];
@@ -505,12 +515,12 @@ __device__ __forceinline__ void recover(Shared &S, const Inst &I, int i, int k0,
       const double e = fma(-(s * il), d, wl - s);
       I.dl[q] = d;
       I.ds[q] = e;
-      // e < 0 and s / -e below the smallest so far (all factors positive: compared as integers)
-      if (bits(e) < 0 && bits(s * pd) < bits(pn * neg(e))) { pn = s; pd = neg(e); }
-      if (bits(d) < 0 && bits(lam * dd) < bits(dn * neg(d))) { dn = lam; dd = neg(d); }
+      // e < 0 and s / -e below the smallest so far
+      if (bits(e) < 0 && ratio_less(s, neg(e), pn, pd)) { pn = s; pd = neg(e); }
+      if (bits(d) < 0 && ratio_less(lam, neg(d), dn, dd)) { dn = lam; dd = neg(d); }
     }
   }
-  double v[2] = {bits(pd) != 0 ? quotient(pn, pd) : DBL_MAX, bits(dd) != 0 ? quotient(dn, dd) : DBL_MAX};
+  double v[2] = {quotient(pn, pd), quotient(dn, dd)};
   cta_reduce<R_MIN, R_MIN>(S, v);
   mp = v[0];
   md = v[1];
