@@ -249,10 +249,13 @@ __device__ __forceinline__ unsigned *f_front(const PsArgs<T> &A, int front) {
   return A.flags + 32 + A.nslot + A.nfr + front;
 }
 
+constexpr int kLbStride = 72;  // FP64, row stride of PsShared::lb: two rows of a quarter warp's reads side by side
+
 // Shared scratch of one CTA (dynamic shared memory).
 template <typename T> struct PsShared {
   static constexpr int B = Ps<T>::B;
   T di[B * B];                  // staged inverse of a diagonal block (TMA bulk copy)
+  alignas(16) T lb[sizeof(T) == 8 ? B * kLbStride : 2];  // FP64: its block of L, lower triangle
   alignas(16) T sv[B];          // values handed to the diagonal-block solve
   T xs[B];                      // solution entries of the rows below a front
   alignas(16) T ys[sizeof(T) == 8 ? kT / 32 : 1][B];  // FP64: a warp's copy of the running y block
@@ -268,10 +271,25 @@ template <typename T> struct PsShared {
   alignas(16) SolveRec rec[2];  // the running task's record and the next one's
 };
 
-// Thread 0: start the bulk copy of a diagonal-block inverse into S.di.
+// Start the copies of a diagonal block's inverse into S.di (thread 0: a bulk copy) and, FP64, of
+// its block of L (column j on, zero above the diagonal) into S.lb; wait_dinv ends both.
 template <typename T>
-__device__ __forceinline__ void stage_dinv(const PsArgs<T> &A, PsShared<T> &S, int slot, int jb) {
-  constexpr int VW = Ps<T>::VW;
+__device__ __forceinline__ void stage_dinv(const PsArgs<T> &A, PsShared<T> &S, const FrontInfo &F, int j, int slot) {
+  constexpr int VW = Ps<T>::VW, B = Ps<T>::B;
+  const int jb = min(B, F.ncol - j);
+  if constexpr (sizeof(T) == 8) {
+    const T *g = A.L + F.loff + (int64_t)j * F.ld + j;
+    for (int e = threadIdx.x; e < jb * (B / 2); e += kT) {
+      const int r = e / (B / 2), c = 2 * (e % (B / 2));
+      T *dst = S.lb + r * kLbStride + c;
+      if (c <= r)  // (the factor holds a zero beside an even row's diagonal entry)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(g + (int64_t)r * F.ld + c)
+                     : "memory");
+      else if (c < (r | 7))  // up to the end of the diagonal's group of eight
+        st16(dst, vzero<T>());
+    }
+  }
+  if (threadIdx.x != 0) return;
   const uint32_t bytes = (uint32_t)(jb * ((jb + VW - 1) & ~(VW - 1)) * (int)sizeof(T));
   const T *src = A.Dinv + A.sv.dinv_off[slot];
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -291,6 +309,7 @@ __device__ __forceinline__ void stage_dinv(const PsArgs<T> &A, PsShared<T> &S, i
 template <typename T>
 __device__ bool wait_dinv(const PsArgs<T> &A, PsShared<T> &S, bool ok_in) {
   const uint32_t par = S.parity;
+  if constexpr (sizeof(T) == 8) asm volatile("cp.async.wait_all;" ::: "memory");  // (the barrier below shares it)
   auto try_wait = [&]() {
     uint32_t done;
     asm volatile(
@@ -549,17 +568,45 @@ __device__ void diag_fwd(const PsArgs<float> &A, PsShared<float> &S, const Front
     if (keep) keep[r] = s;
   }
 }
-// FP64: four threads per row
+// Row (forward) or column (backward) of a diagonal block for this quad of lanes, eight a warp.
+// Warps w and w + 4 share a quarter SM's FP64 unit: theirs are paired so that the triangle gives
+// each quarter the same work.
+__device__ __forceinline__ int quad_row() {
+  const int w = threadIdx.x / 32;
+  return 8 * (w < 4 ? w : 11 - w) + threadIdx.x % 32 / 4;
+}
+// FP64: four threads per row. A product with the inverse alone leaves a residual of |L| |L^-1|
+// |v| u where substitution leaves |L| |y| u (a thousand times as much for a block with entries of
+// either sign and condition 1e6), so its result is corrected once: y += Dinv (v - L y). That
+// is three triangular products a block on the FP64 unit instead of one (a solve at 40^3 takes
+// 1675 us, 1195 with the product alone; 2632 and 1915 at 48^3); a chain of 64 exchanges and
+// multiply-adds, as substitution has, would be longer still.
 __device__ void diag_fwd(const PsArgs<double> &A, PsShared<double> &S, const FrontInfo &F, int j, int slot,
                          double *keep = nullptr) {
   constexpr int B = Ps<double>::B;
-  const int jb = min(B, F.ncol - j), ldi = (jb + 1) & ~1, r = threadIdx.x / 4, c = 2 * (threadIdx.x % 4);
-  double s = 0.0;
-  for (int m = 0; m <= (int)threadIdx.x / 32; m++)
-    if (r < jb && 8 * m + c < ldi)
-      s = vdot(ld16(S.di + r * ldi + 8 * m + c), ld16(S.sv + 8 * m + c), s);
-  s = quad_sum(s);
-  if (threadIdx.x % 4 == 0 && r < jb) {
+  const int jb = min(B, F.ncol - j), ldi = (jb + 1) & ~1, r = quad_row(), h = threadIdx.x % 4, c = 2 * h;
+  const int last = 8 * (r / 8) < jb ? r / 8 : -1;  // column groups of this warp's rows (uniform per warp)
+  double *y0 = S.red4[0], *rs = S.red4[1], s = 0.0;
+  auto product = [&](const double *row, int end, const double *v) {  // both triangles are zero past r
+    double a = 0.0;
+#pragma unroll 4
+    for (int m = 0; m <= last; m++)
+      if (r < jb && 8 * m + c < end) a = vdot(ld16(row + 8 * m + c), ld16(v + 8 * m + c), a);
+    return quad_sum(a);
+  };
+  if (last >= 0) {
+    s = product(S.di + r * ldi, ldi, S.sv);
+    if (h == 0) y0[r] = s;
+  }
+  __syncthreads();
+  if (last >= 0) {
+    const double t = product(S.lb + r * kLbStride, B, y0);
+    if (h == 0) rs[r] = S.sv[r] - t;
+  }
+  __syncthreads();
+  if (last < 0) return;
+  s += product(S.di + r * ldi, ldi, rs);
+  if (h == 0 && r < jb) {
     publish(slot_words<double>(A.ly, slot), r, s, A.epoch);
     A.b[F.first + j + r] = s;
     if (keep) keep[r] = s;
@@ -598,8 +645,8 @@ __device__ __forceinline__ void put_sum(double *row, int c, double s) { row[c] =
 
 // x[first + j + c] = sum_{r >= c} Dinv[r][c] v[r]  (Dinv staged in S.di, zero above the
 // diagonal; v = S.sv), published in the slot's words. FP32: thread (g, q) takes columns
-// 4q .. and rows 16g ..; FP64: four threads per column, and a warp's eight columns start
-// at their diagonal.
+// 4q .. and rows 16g ..; FP64: four threads per column, a warp's eight columns start
+// at their diagonal, and the result is corrected as in diag_fwd.
 __device__ void diag_bwd(const PsArgs<float> &A, PsShared<float> &S, const FrontInfo &F, int j, int slot) {
   constexpr int B = Ps<float>::B, RW = Ps<float>::RW;
   const int jb = min(B, F.ncol - j), ldi = (jb + 3) & ~3;
@@ -625,13 +672,30 @@ __device__ void diag_bwd(const PsArgs<float> &A, PsShared<float> &S, const Front
 }
 __device__ void diag_bwd(const PsArgs<double> &A, PsShared<double> &S, const FrontInfo &F, int j, int slot) {
   constexpr int B = Ps<double>::B;
-  const int jb = min(B, F.ncol - j), ldi = (jb + 1) & ~1, c = threadIdx.x / 4, h = threadIdx.x % 4;
-  double s = 0.0;
-  for (int m = 2 * (threadIdx.x / 32); m < B / 4; m++) {
-    const int r = 4 * m + h;
-    if (r < jb && c < jb) s = fma(S.di[r * ldi + c], S.sv[r], s);
+  const int jb = min(B, F.ncol - j), ldi = (jb + 1) & ~1, c = quad_row(), h = threadIdx.x % 4;
+  const int m0 = 2 * (c / 8), m1 = (jb + 3) / 4;  // row groups of this warp's columns (uniform per warp)
+  double *x0 = S.red4[0], *rs = S.red4[1], s = 0.0;
+  auto product = [&](const double *M, int ld, const double *v) {
+    double a = 0.0;
+#pragma unroll 4
+    for (int m = m0; m < m1; m++) {
+      const int r = 4 * m + h;
+      if (r < jb && c < jb) a = fma(M[r * ld + c], v[r], a);
+    }
+    return quad_sum(a);
+  };
+  if (m0 < m1) {
+    s = product(S.di, ldi, S.sv);
+    if (h == 0) x0[c] = s;
   }
-  s = quad_sum(s);
+  __syncthreads();
+  if (m0 < m1) {
+    const double t = product(S.lb, kLbStride, x0);
+    if (h == 0) rs[c] = S.sv[c] - t;
+  }
+  __syncthreads();
+  if (m0 >= m1) return;
+  s += product(S.di, ldi, rs);
   if (h == 0 && c < jb) {
     publish(slot_words<double>(A.lx, slot), c, s, A.epoch);
     A.x[F.first + j + c] = s;
@@ -775,7 +839,7 @@ __device__ void fwd_diag(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R, 
   const Task &tk = R.task;
   const FrontInfo &F = R.front;
   const int i = tk.a, j0 = B * i, jb = min(B, F.ncol - j0), slot0 = R.slot0;
-  if (threadIdx.x == 0) stage_dinv(A, S, slot0 + i, jb);
+  stage_dinv(A, S, F, j0, slot0 + i);
   bool ok = wait_children(A, S, F, R);
   if (ok && threadIdx.x < B)
     S.sv[threadIdx.x] = threadIdx.x < jb
@@ -894,7 +958,7 @@ __device__ void bwd_diag(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R, 
   const FrontInfo &F = R.front;
   const int cb = tk.a, c0 = B * cb, jb = min(B, F.ncol - c0), nb = (F.ncol + B - 1) / B;
   const int nbl = (F.nrow + B - 1) / B, slot0 = R.slot0;
-  if (threadIdx.x == 0) stage_dinv(A, S, slot0 + cb, jb);
+  stage_dinv(A, S, F, c0, slot0 + cb);
   bool ok = true;
   if (nbl > 0) ok = wait_flag(A, S, f_part(A, slot0 + cb), nbl);  // implies the parent is done
   else if (ok && F.parent >= 0)
@@ -969,7 +1033,7 @@ __device__ void fwd_narrow(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R
   constexpr int B = Ps<T>::B, VW = Ps<T>::VW, NV = kNarrowCols / VW;
   const FrontInfo &F = R.front;
   const int nc = F.ncol, nr = F.nrow, tid = threadIdx.x;
-  if (tid == 0) stage_dinv(A, S, R.slot0, nc);
+  stage_dinv(A, S, F, 0, R.slot0);
   const T *rows = A.L + F.loff + (int64_t)nc * F.ld;
   Vec<T> l[NV];
   auto load = [&](int r) {
@@ -1021,7 +1085,7 @@ __device__ void bwd_narrow(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R
   static_assert(kNarrowRows <= 2 * kT && kNarrowCols / VW <= 16 && kNarrowCols <= 32, "rows and columns per thread");
   const FrontInfo &F = R.front;
   const int nc = F.ncol, nr = F.nrow, tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
-  if (tid == 0) stage_dinv(A, S, R.slot0, nc);
+  stage_dinv(A, S, F, 0, R.slot0);
   int lg = 0;
   while ((VW << lg) < nc) lg++;
   const int cg = 1 << lg, c = VW * (tid & (cg - 1)), rr = tid >> lg, rp = kT >> lg;
