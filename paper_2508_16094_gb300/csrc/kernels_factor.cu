@@ -341,6 +341,13 @@ __device__ __forceinline__ double quotient(double a, double d) {
   return fma(w0, recip_err(d, r0), w0);
 }
 __device__ __forceinline__ float quotient(float a, float d) { return a * (1.f / d); }
+// a / l from r = 1 / l, for an entry of the factor: correctly rounded in FP32 and, EXACT, in FP64
+// (one correction of the product, r being correctly rounded); else the product.
+template <bool EXACT> __device__ __forceinline__ double entry(double a, double l, double r) {
+  const double q = a * r;
+  return EXACT ? fma(fma(-q, l, a), r, q) : q;
+}
+template <bool EXACT> __device__ __forceinline__ float entry(float a, float l, float) { return a / l; }
 // s v for s = +-1 and 0 < d < big_pivot^2 (false for NaN) on the integer pipe:
 // an FP64 multiplication or comparison costs as much as a multiply-add.
 __device__ __forceinline__ double flip(double v, bool neg) {
@@ -514,7 +521,7 @@ __device__ __forceinline__ void panel_trail(T *S, int ls, int c0, int e0, int no
     if (e0 + kPotrfThreads * q < nout) S[at[q] + col[q]] = s[q];
 }
 
-template <typename T>
+template <typename T, bool SGN>
 __global__ void __launch_bounds__(kPotrfThreads) potrf_kernel(DevPlan dp, const Task *__restrict__ tasks,
                                                               T *__restrict__ L, int32_t *status,
                                                               int perturb) {
@@ -523,7 +530,7 @@ __global__ void __launch_bounds__(kPotrfThreads) potrf_kernel(DevPlan dp, const 
   const FrontInfo F = dp.fronts[tk.front];
   const int k = tk.a, kb = min(NB, F.ncol - k);
   T *A = L + F.loff + (int64_t)k * F.ld + k;
-  const int8_t *sg = dp.sgn ? dp.sgn + F.first + k : nullptr;
+  const int8_t *sg = SGN ? dp.sgn + F.first + k : nullptr;
   __shared__ T S[NB * LS];  // the block; past kb: zero, with a unit diagonal
   __shared__ __align__(16) T col[3][NB];
   __shared__ T piv[NB], W[16][NB];  // W: a panel's a_ij / d_j
@@ -561,9 +568,9 @@ __global__ void __launch_bounds__(kPotrfThreads) potrf_kernel(DevPlan dp, const 
   }
   // L_ij = s_j a_ij / L_jj, L_jj = sqrt(d) from d and 1 / sqrt(d)
   if (tid < kb) {
-    const T d = piv[tid], r = inv_sqrt(d), l0 = d * r;
-    col[0][tid] = r;
-    col[1][tid] = fma(fma(-l0, l0, d), T(0.5) * r, l0);
+    const T d = piv[tid], r = inv_sqrt(d), l0 = d * r, l = fma(fma(-l0, l0, d), T(0.5) * r, l0);
+    col[0][tid] = quotient(T(1), l);
+    col[1][tid] = l;
   }
   __syncthreads();
 #pragma unroll 2
@@ -573,7 +580,7 @@ __global__ void __launch_bounds__(kPotrfThreads) potrf_kernel(DevPlan dp, const 
     Vec16<T> v;
 #pragma unroll
     for (int h = 0; h < VW; h++) {
-      const T x = flip(S[r * LS + c + h] * col[0][c + h], neg[c + h] != 0);
+      const T x = flip(entry<SGN>(S[r * LS + c + h], col[1][c + h], col[0][c + h]), neg[c + h] != 0);
       v.v[h] = c + h < r ? x : c + h == r ? col[1][r] : T(0);
     }
     st16(A + (int64_t)r * F.ld + c, v);
@@ -597,7 +604,7 @@ __global__ void __launch_bounds__(kPotrfThreads) potrf_kernel(DevPlan dp, const 
 // the columns and fits the instruction cache, which wider per-warp tiles (16
 // rows a warp, 56 KB of code run once) did not: 98 us against 55 us a launch on the
 // 40^3 grid.
-template <typename T, int P>
+template <typename T, int P, bool SGN>
 __global__ void __launch_bounds__(128) trsm_kernel(DevPlan dp, const Task *__restrict__ ents, int nent,
                                                    int batches, T *__restrict__ L) {
   constexpr int NB = 64, LS = NB + 1, NQ = NB / P, R = 128 / P;
@@ -612,17 +619,18 @@ __global__ void __launch_bounds__(128) trsm_kernel(DevPlan dp, const Task *__res
   const int nf = F.ncol + F.nrow, k = tk.b, kb = min(NB, F.ncol - k);
   const int tid = threadIdx.x, lane = tid % 32, h = lane % P;
   int row = k + kb + batches * R * ((int)blockIdx.x - tk.a) + tid / P;
-  __shared__ T U[NB * LS];  // column c: u_c2,c at U[c * LS + c2]
-  __shared__ T rd[NB];      // s_c / L_cc
+  __shared__ T U[NB * LS];      // column c: u_c2,c at U[c * LS + c2]
+  __shared__ T rd[NB], dg[NB];  // s_c / L_cc, s_c L_cc
   T *Xr = L + F.loff + (int64_t)row * F.ld + k;
   T z[NQ];
 #pragma unroll
   for (int q = 0; q < NQ; q++) z[q] = (row < nf && h + P * q < kb) ? Xr[h + P * q] : T(0);
-  const int8_t *sg = dp.sgn ? dp.sgn + F.first + k : nullptr;
+  const int8_t *sg = SGN ? dp.sgn + F.first + k : nullptr;
   const T *A = L + F.loff + (int64_t)k * F.ld + k;
   if (tid < kb) {
     const T d = A[(int64_t)tid * F.ld + tid];
     rd[tid] = flip(quotient(T(1), d), sg && sg[tid] < 0);
+    dg[tid] = flip(d, sg && sg[tid] < 0);
   }
   T u[NB * NB / 128];
 #pragma unroll
@@ -634,11 +642,12 @@ __global__ void __launch_bounds__(128) trsm_kernel(DevPlan dp, const Task *__res
   {
     // column c of this thread: u = L_c2,c / L_cc (the signs of L and of the scale cancel)
     const int c = tid % NB;
-    const T s = c < kb ? flip(rd[c], sg && sg[c] < 0) : T(0);
+    const bool ng = sg && c < kb && sg[c] < 0;
+    const T s = c < kb ? flip(rd[c], ng) : T(0), d = c < kb ? flip(dg[c], ng) : T(1);
 #pragma unroll
     for (int q = 0; q < NB * NB / 128; q++) {
       const int c2 = 2 * q + tid / NB;
-      U[c * LS + c2] = 2 * q + 1 > (c & 32) ? u[q] * s : T(0);  // (uniform per warp)
+      U[c * LS + c2] = 2 * q + 1 > (c & 32) ? entry<SGN>(u[q], d, s) : T(0);  // (uniform per warp)
     }
   }
   __syncthreads();
@@ -654,7 +663,7 @@ __global__ void __launch_bounds__(128) trsm_kernel(DevPlan dp, const Task *__res
     }
 #pragma unroll
     for (int q = 0; q < NQ; q++)
-      if (row < nf && h + P * q < kb) Xr[h + P * q] = z[q] * rd[h + P * q];
+      if (row < nf && h + P * q < kb) Xr[h + P * q] = entry<SGN>(z[q], dg[h + P * q], rd[h + P * q]);
     row += R;
     Xr += (int64_t)R * F.ld;
     if (b + 1 < batches)
@@ -723,15 +732,18 @@ void launch_potrf(const DevPlan &dp, const StepRange &S, T *L, int32_t *status, 
                   cudaStream_t st) {
   if (S.potrf_e <= S.potrf_b) return;
   note_launch();
-  potrf_kernel<T><<<S.potrf_e - S.potrf_b, kPotrfThreads, 0, st>>>(dp, dp.potrf + S.potrf_b, L, status,
-                                                                   perturb ? 1 : 0);
+  auto kernel = dp.sgn ? potrf_kernel<T, true> : potrf_kernel<T, false>;
+  kernel<<<S.potrf_e - S.potrf_b, kPotrfThreads, 0, st>>>(dp, dp.potrf + S.potrf_b, L, status, perturb ? 1 : 0);
 }
 
+template <typename T, bool SGN> auto trsm_for(int rows) {
+  return rows == 4 ? trsm_kernel<T, 32, SGN> : rows == 8 ? trsm_kernel<T, 16, SGN> : trsm_kernel<T, 8, SGN>;
+}
 template <typename T>
 void launch_trsm(const DevPlan &dp, const StepRange &S, T *L, cudaStream_t st) {
   if (S.trsm_n <= 0) return;
   note_launch();
-  auto kernel = S.trsm_rows == 4 ? trsm_kernel<T, 32> : S.trsm_rows == 8 ? trsm_kernel<T, 16> : trsm_kernel<T, 8>;
+  auto kernel = dp.sgn ? trsm_for<T, true>(S.trsm_rows) : trsm_for<T, false>(S.trsm_rows);
   kernel<<<S.trsm_n, 128, 0, st>>>(dp, dp.trsm + S.trsm_b, S.trsm_e - S.trsm_b, S.trsm_bat, L);
 }
 
