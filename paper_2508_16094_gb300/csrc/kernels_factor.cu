@@ -340,7 +340,7 @@ __device__ __forceinline__ double quotient(double a, double d) {
   const double r0 = recip_start(d), w0 = a * r0;
   return fma(w0, recip_err(d, r0), w0);
 }
-__device__ __forceinline__ float quotient(float a, float d) { return a * (1.f / d); }
+__device__ __forceinline__ float quotient(float a, float d) { return a / d; }  // (1 / d overflows below 2^-128)
 // a / l from r = 1 / l, for an entry of the factor: correctly rounded in FP32 and, EXACT, in FP64
 // (one correction of the product, r being correctly rounded); else the product.
 template <bool EXACT> __device__ __forceinline__ double entry(double a, double l, double r) {

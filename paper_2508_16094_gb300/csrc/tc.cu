@@ -753,18 +753,11 @@ __device__ __forceinline__ void blk_nt(const float *A, int lda, const float *B, 
   }
 }
 
-// 1 / d of a pivot (reciprocal estimate and one Newton step); one that is not
-// positive is replaced and counted (by thread 0: the branch is uniform).
-__device__ __forceinline__ float pivot_inverse(float &d, int32_t *status) {
-  if (d >= 1e-37f && d <= 8e37f) {
-    const float i = __fdividef(1.f, d);
-    return fmaf(i, fmaf(-d, i, 1.f), i);
-  }
-  if (!(d > 0.f) || !(d < 3.0e38f)) {
-    d = 1e30f;
-    if (threadIdx.x == 0) atomicAdd(&status[ST_PERTURBED], 1);
-  }
-  return 1.f / d;
+// A pivot that is not positive is replaced and counted (by thread 0: the branch is uniform).
+__device__ __forceinline__ void check_pivot(float &d, int32_t *status) {
+  if (d > 0.f && d < 3.0e38f) return;
+  d = 1e30f;
+  if (threadIdx.x == 0) atomicAdd(&status[ST_PERTURBED], 1);
 }
 
 // Barrier over `threads` threads (whole warps) of the block; id 0 is __syncthreads.
@@ -908,15 +901,20 @@ __device__ __forceinline__ bool inv_panel(float *S, int c0, int act, float (*cp)
       v1[r] = f1.x, v1[r + 1] = f1.y, v1[r + 2] = f1.z, v1[r + 3] = f1.w;
       v2[r] = f2.x, v2[r + 1] = f2.y, v2[r + 2] = f2.z, v2[r + 3] = f2.w;
     }
-    const float i1 = FAST ? usual_inverse(d1, good) : pivot_inverse(d1, status);
-    const float t = a21 * i1;
+    // a / d (not FAST: by division, since 1 / d overflows for a d below 2^-128)
+    auto over = [](float a, float d, float inv) { return FAST ? a * inv : a / d; };
+    float i1 = 0.f, i2 = 0.f;
+    if (FAST) i1 = usual_inverse(d1, good);
+    else check_pivot(d1, status);
+    const float t = over(a21, d1, i1);
     d2 = fmaf(-t, a21, d2);
-    const float i2 = FAST ? usual_inverse(d2, good) : pivot_inverse(d2, status);
+    if (FAST) i2 = usual_inverse(d2, good);
+    else check_pivot(d2, status);
     if (tid == 0) {
       piv[c0 + 2 * q] = d1;
       piv[c0 + 2 * q + 1] = d2;
     }
-    const float w1 = a1 * i1, a2p = fmaf(-w1, a21, a2), w2 = a2p * i2;
+    const float w1 = over(a1, d1, i1), a2p = fmaf(-w1, a21, a2), w2 = over(a2p, d2, i2);
     if (h == 1) x[q] = a2p;
     if (q == 7) break;
     // the next pair first
