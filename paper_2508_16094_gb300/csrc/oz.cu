@@ -686,8 +686,9 @@ void OzPlan::factor(const DevPlan &dp, const Plan &plan, const double *kval, dou
     for (size_t s = 0; s < LP.steps.size(); s++) {
       const StepRange &R = LP.steps[s];
       const Step &Z = V.steps[s];
-      gemm(Z.gemm_b, Z.gemm_e, sms, st);
+      // both parts of a column's sum are added to the same entries: in this order, always
       if (pending) cudaStreamWaitEvent(st, ev_side_, 0);
+      gemm(Z.gemm_b, Z.gemm_e, sms, st);
       pending = Z.ahead_e > Z.ahead_b;
       if (pending) {
         cudaEventRecord(ev_main_, st);
