@@ -43,8 +43,8 @@ struct ipm_ctx {
   DevPlan dp{};
   double *kval = nullptr;
   void *L = nullptr, *U = nullptr;
-  double *yv = nullptr, *tv = nullptr;  // solve scratch (doubles; float views), kSolveRhs of each
-  double *vx = nullptr, *vr = nullptr, *vc = nullptr, *vz = nullptr, *vp = nullptr,
+  double *yv = nullptr, *tv = nullptr;  // solve scratch (doubles; float views)
+  double *vr = nullptr, *vc = nullptr, *vz = nullptr, *vp = nullptr,
          *vq = nullptr, *vb = nullptr, *vdx = nullptr, *vrd = nullptr, *vwx = nullptr;
   double *vg = nullptr, *vD = nullptr, *vw = nullptr, *vds = nullptr, *vdl = nullptr,
          *vt = nullptr, *vjd = nullptr, *vjx = nullptr, *vtA = nullptr;
@@ -52,12 +52,18 @@ struct ipm_ctx {
   double *jv_copy = nullptr, *D_copy = nullptr, *wv_copy = nullptr;  // inputs kept for refinement
   float *Llo = nullptr;  // low parts of the split-TF32 factor
   float *dinv = nullptr, *fsa = nullptr, *fsb = nullptr, *fsx = nullptr;  // persistent FP32 solve
-  double *dinv64 = nullptr, *dsb = nullptr, *dsx = nullptr;  // FP64 (a: yv)
-  unsigned *psflags = nullptr;  // its tickets, flags and counters
-  void *pspart = nullptr;     // its partial sums, of either type
-  SolveWords psw;             // its published entries, of either type
-  // do_solves: r, z, p, q of right-hand sides 1 .. (four n each), and the scalars of all (kRhsScal each)
-  double *vrk = nullptr, *rscal = nullptr;
+  unsigned *psflags = nullptr;  // the persistent solves' tickets, flags and counters
+  float *pspart = nullptr;      // FP32 partial sums
+  uint2 *wy = nullptr, *wx = nullptr;  // published entries, of either type
+  unsigned epoch = 0;                  // tag of the last launch
+  // In the place of the update matrices, which are dead outside a factorisation: inverses and vectors of
+  // the FP64 solve (a: yv), and the vectors of up to rhs_max right-hand sides that go side by side
+  // (GroupBufs), whose published entries are to be zeroed again after each factorisation
+  double *dinv64 = nullptr, *dsb = nullptr, *dsx = nullptr, *part64 = nullptr;
+  char *group = nullptr;
+  int rhs_max = 1;
+  bool group_clean = false;
+  double *rscal = nullptr;  // do_solves: device scalars (kRhsScal per right-hand side)
   // learned correction of a stale factor
   LearnedBufs lb;
   bool learned_active = false;  // PCG preconditioner = corrected stale factor
@@ -175,6 +181,46 @@ void w_full(const Problem &P, std::vector<int64_t> &fp, std::vector<int32_t> &fi
     }
 }
 
+// Words of published entries (y or x) of one right-hand side, of either type.
+int64_t own_words(const ipm_ctx *c) { return std::max(c->plan.s32.words, c->plan.s64.words); }
+
+// What the FP64 solve keeps between a factorisation and the next.
+void layout_fp64_solve(ipm_ctx *c, Carve &cv) {
+  const SolvePlan &sp = c->plan.s64;
+  if (sp.tasks.empty()) return;
+  const size_t n = std::max<int64_t>(c->P.n, 1);
+  c->dinv64 = cv.take<double>(sp.dinv_entries);
+  c->dsb = cv.take<double>(n);
+  c->dsx = cv.take<double>(n);
+  c->part64 = cv.take<double>(std::max<int64_t>(sp.part_entries, 1));
+}
+
+// Vectors of R right-hand sides that are solved side by side, at `base` (null: the size only), and
+// r, z, p, q of the right-hand sides 1 .. R - 1 (four n each).
+template <typename T> struct GroupBufs {
+  SolveBufs<T> v;
+  double *vrk;
+  size_t bytes;
+};
+template <typename T> GroupBufs<T> group_layout(const ipm_ctx *c, char *base, int R) {
+  const SolvePlan &sp = sizeof(T) == 8 ? c->plan.s64 : c->plan.s32;
+  GroupBufs<T> g{};
+  const size_t n = std::max<int64_t>(c->P.n, 1);
+  Carve cv{base};
+  g.v.sd = SolveStride{(int64_t)n, c->plan.t_entries, sp.part_entries, sp.flag_words, sp.words};
+  g.v.wy = cv.take<uint2>(R * sp.words);
+  g.v.wx = cv.take<uint2>(R * sp.words);
+  g.v.flags = cv.take<unsigned>(R * sp.flag_words);
+  g.v.a = cv.take<T>(R * n);
+  g.v.b = cv.take<T>(R * n);
+  g.v.x = cv.take<T>(R * n);
+  g.v.t = cv.take<T>(R * c->plan.t_entries);
+  g.v.part = cv.take<T>(R * sp.part_entries);
+  g.vrk = cv.take<double>(4 * (R - 1) * n);
+  g.bytes = cv.off;
+  return g;
+}
+
 // Assign every device pointer of the context inside the workspace.
 void layout(ipm_ctx *c, char *base) {
   Carve cv{base};
@@ -272,12 +318,10 @@ void layout(ipm_ctx *c, char *base) {
   const size_t n = std::max<int64_t>(P.n, 1), mt = std::max<int64_t>(P.mt, 1),
                m = std::max<int32_t>(P.m, 1);
   c->kval = cv.take<double>(std::max<int64_t>(d.nk, 1));
-  constexpr size_t R = kSolveRhs;  // right-hand sides of one persistent solve
-  c->yv = cv.take<double>(R * n);
-  c->tv = cv.take<double>(R * pl.t_entries);
-  c->vrk = cv.take<double>(4 * (R - 1) * n);
-  c->rscal = cv.take<double>(kRhsScal * R);
-  for (double **v : {&c->vx, &c->vr, &c->vc, &c->vz, &c->vp, &c->vq, &c->vb, &c->vdx, &c->vrd,
+  c->yv = cv.take<double>(n);
+  c->tv = cv.take<double>(pl.t_entries);
+  c->rscal = cv.take<double>(kRhsScal * kSolveRhs);
+  for (double **v : {&c->vr, &c->vc, &c->vz, &c->vp, &c->vq, &c->vb, &c->vdx, &c->vrd,
                      &c->vwx})
     *v = cv.take<double>(n);
   for (double **v : {&c->vg, &c->vD, &c->vw, &c->vds, &c->vdl, &c->vt, &c->vjd})
@@ -288,19 +332,13 @@ void layout(ipm_ctx *c, char *base) {
   c->vjx = cv.take<double>(m);
   c->vtA = cv.take<double>(m);
   c->dinv = cv.take<float>(std::max<int64_t>(pl.s32.dinv_entries, 4));
-  c->fsa = cv.take<float>(R * n);
-  c->fsb = cv.take<float>(R * n);
-  c->fsx = cv.take<float>(R * n);
-  c->psflags = cv.take<unsigned>(R * std::max<int64_t>(std::max(pl.s32.flag_words, pl.s64.flag_words), 32));
-  c->pspart = cv.take<double>(R * (std::max(pl.s32.part_entries / 2, pl.s64.part_entries) + 1));
-  c->psw.count = R * std::max(solve_words(pl.s32), solve_words(pl.s64));
-  c->psw.y = cv.take<uint2>(c->psw.count);
-  c->psw.x = cv.take<uint2>(c->psw.count);
-  if (!pl.s64.tasks.empty()) {
-    c->dinv64 = cv.take<double>(pl.s64.dinv_entries);
-    c->dsb = cv.take<double>(R * n);
-    c->dsx = cv.take<double>(R * n);
-  }
+  c->fsa = cv.take<float>(n);
+  c->fsb = cv.take<float>(n);
+  c->fsx = cv.take<float>(n);
+  c->psflags = cv.take<unsigned>(std::max<int64_t>(std::max(pl.s32.flag_words, pl.s64.flag_words), 32));
+  c->pspart = cv.take<float>(std::max<int64_t>(pl.s32.part_entries, 1));
+  c->wy = cv.take<uint2>(own_words(c));
+  c->wx = cv.take<uint2>(own_words(c));
   {  // learned-correction buffers (only when enabled)
     LearnedBufs &B = c->lb;
     const bool on = c->opts.learned != 0 || c->opts.learned_probes > 0;
@@ -342,7 +380,24 @@ void layout(ipm_ctx *c, char *base) {
   // buffer, else their own array
   c->Llo = c->storage_bytes == 8 ? (c->L ? reinterpret_cast<float *>(c->L) + pl.l_entries : nullptr)
                                  : cv.take<float>((size_t)pl.l_entries);
-  c->U = cv.take<char>((size_t)pl.u_entries * c->storage_bytes);
+  {
+    // The update matrices, and in their place what only solves use. As many right-hand sides side by
+    // side as find room there (a factor without update matrices: in 256 KB).
+    const size_t ub = (size_t)pl.u_entries * c->storage_bytes;
+    Carve sz{nullptr};
+    layout_fp64_solve(c, sz);
+    const size_t room = std::max(ub, sz.off + (256u << 10));
+    auto need = [&](int R) {
+      const size_t g32 = group_layout<float>(c, nullptr, R).bytes;
+      return sz.off + 256 + (pl.s64.tasks.empty() ? g32 : std::max(g32, group_layout<double>(c, nullptr, R).bytes));
+    };
+    c->rhs_max = kSolveRhs;
+    while (c->rhs_max > 1 && need(c->rhs_max) > room) c->rhs_max--;
+    c->U = cv.take<char>(std::max(ub, c->rhs_max > 1 ? need(c->rhs_max) : sz.off));
+    Carve uv{static_cast<char *>(c->U)};
+    layout_fp64_solve(c, uv);
+    c->group = uv.take<char>(0);
+  }
   c->dp.build_k = upload(cv, pl.build_k, st);
   c->ws_need = cv.off + 256;
 }
@@ -370,6 +425,7 @@ ipm_status do_factor(ipm_ctx *c, int prec, int32_t *bad_col) {
   if (c->dp.sgn && prec != IPM_FP64 && prec != IPM_FP32)
     throw Fail{IPM_ERR_UNSUPPORTED, "the signed factorisation of a quasi-definite system runs in FP64 or FP32"};
   int32_t init[ST_COUNT] = {INT32_MAX, 0, 0, 0, 0, 0, 0, 0};
+  c->group_clean = false;  // (the update matrices are about to be written)
   CK(cudaMemcpyAsync(c->status, init, sizeof(init), cudaMemcpyHostToDevice, c->st));
   if (prec == IPM_FP64 && c->opts.fp64_tc && !c->dp.sgn) {
     if (!c->ozp.ready())
@@ -425,72 +481,106 @@ ipm_status do_factor(ipm_ctx *c, int prec, int32_t *bad_col) {
   return IPM_OK;
 }
 
-// One persistent solve launch over the workspace vectors: which = 0 both sweeps
-// (fsa -> fsx; FP64: yv -> dsx), 1 forward only (fsa -> fsb; yv -> dsb), 2 backward
-// only (fsb -> fsx; dsb -> dsx), of the first nrhs right-hand sides there
-template <typename T> void launch_held_solve(ipm_ctx *c, int which, int nrhs) {
-  constexpr bool f64 = sizeof(T) == 8;
-  const SolvePlan &sp = f64 ? c->plan.s64 : c->plan.s32;
+// The vectors of one right-hand side, or (K > 1) of a group.
+template <typename T> SolveBufs<T> solve_bufs(const ipm_ctx *c, int K) {
+  if (K > 1) return group_layout<T>(c, c->group, c->rhs_max).v;
   SolveBufs<T> v;
-  if constexpr (f64) {
-    v.a = c->yv, v.b = c->dsb, v.x = c->dsx, v.t = c->tv;
+  if constexpr (sizeof(T) == 8) {
+    v.a = c->yv, v.b = c->dsb, v.x = c->dsx, v.t = c->tv, v.part = c->part64;
+    v.sd.flags = c->plan.s64.flag_words;
   } else {
-    v.a = c->fsa, v.b = c->fsb, v.x = c->fsx, v.t = reinterpret_cast<float *>(c->tv);
+    v.a = c->fsa, v.b = c->fsb, v.x = c->fsx, v.t = reinterpret_cast<float *>(c->tv), v.part = c->pspart;
+    v.sd.flags = c->plan.s32.flag_words;
   }
-  v.part = static_cast<T *>(c->pspart);
   v.flags = c->psflags;
-  v.sd = SolveStride{std::max<int64_t>(c->P.n, 1), c->plan.t_entries, sp.part_entries, sp.flag_words,
-                     solve_words(sp)};
+  v.wy = c->wy, v.wx = c->wx;
+  return v;
+}
+template <typename T> void zero_group_words(ipm_ctx *c) {
+  const SolveBufs<T> v = solve_bufs<T>(c, 2);
+  const size_t bytes = (size_t)(c->rhs_max * v.sd.words) * sizeof(uint2);
+  CK(cudaMemsetAsync(v.wy, 0, bytes, c->st));
+  CK(cudaMemsetAsync(v.wx, 0, bytes, c->st));
+}
+void zero_own_words(ipm_ctx *c) {
+  CK(cudaMemsetAsync(c->wy, 0, own_words(c) * sizeof(uint2), c->st));
+  CK(cudaMemsetAsync(c->wx, 0, own_words(c) * sizeof(uint2), c->st));
+}
+
+// One persistent solve launch over v: which = 0 both sweeps (a -> x), 1 forward only
+// (a -> b), 2 backward only (b -> x), of the first nrhs right-hand sides there
+template <typename T> void launch_held_solve(ipm_ctx *c, SolveBufs<T> v, int which, int nrhs) {
+  if (++c->epoch == 0) {  // the tags start over
+    zero_own_words(c);
+    if (c->group_clean) zero_group_words<T>(c);
+    c->epoch = 1;
+  }
+  v.epoch = c->epoch;
   const T *Dinv;
-  if constexpr (f64) Dinv = c->dinv64;
+  if constexpr (sizeof(T) == 8) Dinv = c->dinv64;
   else Dinv = c->dinv;
-  launch_psolve<T>(c->dp, c->plan, (const T *)c->L, Dinv, v, nrhs, c->psw, c->status, which != 2, which != 1,
-                   c->st, c->test_spins, c->test_withhold);
+  launch_psolve<T>(c->dp, c->plan, (const T *)c->L, Dinv, v, nrhs, c->status, which != 2, which != 1, c->st,
+                   c->test_spins, c->test_withhold);
   c->test_spins = 0;
   c->test_withhold = -1;
 }
-void launch_fp32_solve(ipm_ctx *c, int which) { launch_held_solve<float>(c, which, 1); }
+void launch_fp32_solve(ipm_ctx *c, int which) { launch_held_solve<float>(c, solve_bufs<float>(c, 1), which, 1); }
 // Both sweeps, with K = L S L^T's signs between them for a quasi-definite system.
-template <typename T> void launch_both_sweeps(ipm_ctx *c, T *mid, int nrhs) {
-  if (!c->dp.sgn) return launch_held_solve<T>(c, 0, nrhs);
-  launch_held_solve<T>(c, 1, nrhs);
-  for (int k = 0; k < nrhs; k++) launch_sign<T>(c->dp, mid + (int64_t)k * c->P.n, c->st);
-  launch_held_solve<T>(c, 2, nrhs);
+template <typename T> void launch_both_sweeps(ipm_ctx *c, const SolveBufs<T> &v, int nrhs) {
+  if (!c->dp.sgn) return launch_held_solve<T>(c, v, 0, nrhs);
+  launch_held_solve<T>(c, v, 1, nrhs);
+  for (int k = 0; k < nrhs; k++) launch_sign<T>(c->dp, v.b + (int64_t)k * c->P.n, c->st);
+  launch_held_solve<T>(c, v, 2, nrhs);
 }
 
-// The preconditioner up to the final numbering's result: P b (times scale[0] for an
-// FP32-storage factor) into right-hand side k of the sweeps' vectors, the sweeps.
 bool factor_is_fp64(const ipm_ctx *c) { return c->storage_bytes == 8 && c->factor_prec == IPM_FP64; }
-void sweeps_in(ipm_ctx *c, const double *b, const double *scale, int k) {
-  VecOps V = c->vec();
-  const int64_t off = (int64_t)k * c->P.n;
-  if (factor_is_fp64(c)) V.permute_in<double>(b, nullptr, c->yv + off);
-  else V.permute_in<float>(b, scale, c->fsa + off);
-}
-void sweeps_run(ipm_ctx *c, int nrhs) {
-  if (factor_is_fp64(c)) return launch_both_sweeps<double>(c, c->dsb, nrhs);
-  if (c->learned_active) {  // P^T L_s^{-T} (Delta + U U^T)^{-1} L_s^{-1} P b (one right-hand side)
-    launch_fp32_solve(c, 1);
-    learned_apply(c->lb, c->fsb, c->st);
-    launch_fp32_solve(c, 2);
-  } else {
-    launch_both_sweeps<float>(c, c->fsb, nrhs);
+// The held factor's solve for K right-hand sides: the preconditioner up to the final numbering's
+// result, P b (times scale[0] for an FP32-storage factor) into right-hand side k of the sweeps' vectors,
+// the sweeps, and the way back.
+struct Sweeps {
+  ipm_ctx *c;
+  SolveBufs<double> v64;
+  SolveBufs<float> v32;
+  double *vrk = nullptr;
+  const bool f64;
+  Sweeps(ipm_ctx *ctx, int K) : c(ctx), f64(factor_is_fp64(ctx)) {
+    if (f64) v64 = solve_bufs<double>(c, K);
+    else v32 = solve_bufs<float>(c, K);
+    if (K == 1) return;
+    vrk = f64 ? group_layout<double>(c, c->group, c->rhs_max).vrk : group_layout<float>(c, c->group, c->rhs_max).vrk;
+    if (c->group_clean) return;
+    if (f64) zero_group_words<double>(c);
+    else zero_group_words<float>(c);
+    c->group_clean = true;
   }
-}
-void sweeps_out(ipm_ctx *c, const double *scale, int k, double *out, bool accumulate) {
-  VecOps V = c->vec();
-  const int64_t off = (int64_t)k * c->P.n;
-  if (factor_is_fp64(c)) V.permute_out<double>(c->dsx + off, nullptr, out, accumulate);
-  else V.permute_out<float>(c->fsx + off, scale, out, accumulate);
-}
-// As sweeps_out, with rz = r . out and beta = rz / rz_old (when given).
-void sweeps_out_dot(ipm_ctx *c, const double *scale, int k, const double *r, double *out, const double *rz_old,
-                    double *rz, double *beta) {
-  VecOps V = c->vec();
-  const int64_t off = (int64_t)k * c->P.n;
-  if (factor_is_fp64(c)) V.permute_out_dot<double>(c->dsx + off, nullptr, r, out, rz_old, rz, beta);
-  else V.permute_out_dot<float>(c->fsx + off, scale, r, out, rz_old, rz, beta);
-}
+  void in(const double *b, const double *scale, int k) const {
+    const int64_t off = (int64_t)k * c->P.n;
+    if (f64) c->vec().permute_in<double>(b, nullptr, v64.a + off);
+    else c->vec().permute_in<float>(b, scale, v32.a + off);
+  }
+  void run(int nrhs) const {
+    if (f64) return launch_both_sweeps<double>(c, v64, nrhs);
+    if (c->learned_active) {  // P^T L_s^{-T} (Delta + U U^T)^{-1} L_s^{-1} P b (one right-hand side)
+      launch_fp32_solve(c, 1);
+      learned_apply(c->lb, c->fsb, c->st);
+      launch_fp32_solve(c, 2);
+    } else {
+      launch_both_sweeps<float>(c, v32, nrhs);
+    }
+  }
+  void out(const double *scale, int k, double *x, bool accumulate) const {
+    const int64_t off = (int64_t)k * c->P.n;
+    if (f64) c->vec().permute_out<double>(v64.x + off, nullptr, x, accumulate);
+    else c->vec().permute_out<float>(v32.x + off, scale, x, accumulate);
+  }
+  // As out, with rz = r . x and beta = rz / rz_old (when given).
+  void out_dot(const double *scale, int k, const double *r, double *x, const double *rz_old, double *rz,
+               double *beta) const {
+    const int64_t off = (int64_t)k * c->P.n;
+    if (f64) c->vec().permute_out_dot<double>(v64.x + off, nullptr, r, x, rz_old, rz, beta);
+    else c->vec().permute_out_dot<float>(v32.x + off, scale, r, x, rz_old, rz, beta);
+  }
+};
 
 // A wait of the persistent solve that ran out of time: the launch drained and
 // its result is invalid; clear the word (each launch zeroes its own flags) and
@@ -518,7 +608,7 @@ struct RhsRun {
   bool going = false;  // in the loop that runs
 };
 
-// Solves with K <= kSolveRhs right-hand sides, b[k n ..] -> x[k n ..] (K > 1: b and x
+// Solves with K <= c->rhs_max right-hand sides, b[k n ..] -> x[k n ..] (K > 1: b and x
 // apart, no learned correction or warm start). They go through refinement and PCG side
 // by side: the triangular solves of a step are one launch, its residuals one
 // synchronisation, and who has converged drops out. info, status: K entries each.
@@ -528,12 +618,13 @@ void do_solves(ipm_ctx *c, int K, const double *b, double *x, int refine, ipm_so
   VecOps V = c->vec();
   const int64_t n = c->P.n;
   const ipm_options &o = c->opts;
+  const Sweeps sweeps(c, K);
   RhsRun run[kSolveRhs];
   for (int k = 0; k < K; k++) {
     RhsRun &u = run[k];
     u.b = b + k * n;
     u.x = x + k * n;
-    double *v = c->vrk + 4 * (k - 1) * n;
+    double *v = sweeps.vrk + 4 * (k - 1) * n;
     u.r = k == 0 ? c->vr : v;
     u.z = k == 0 ? c->vz : v + n;
     u.p = k == 0 ? c->vp : v + 2 * n;
@@ -588,18 +679,18 @@ void do_solves(ipm_ctx *c, int K, const double *b, double *x, int refine, ipm_so
   // x (+)= M^{-1} (b, or its residual) with the current factor
   auto apply = [&](bool from_b, bool accumulate) {
     const int sc = from_b ? 1 : 3;
-    for (int k = 0; k < na; k++) sweeps_in(c, from_b ? act[k]->b : act[k]->r, act[k]->s + sc, k);
-    sweeps_run(c, na);
-    for (int k = 0; k < na; k++) sweeps_out(c, act[k]->s + sc, k, act[k]->x, accumulate);
+    for (int k = 0; k < na; k++) sweeps.in(from_b ? act[k]->b : act[k]->r, act[k]->s + sc, k);
+    sweeps.run(na);
+    for (int k = 0; k < na; k++) sweeps.out(act[k]->s + sc, k, act[k]->x, accumulate);
   };
   // PCG: z (first: p) = M^{-1} r, r . z and beta
   auto precondition = [&](bool first) {
-    for (int k = 0; k < na; k++) sweeps_in(c, act[k]->r, act[k]->s + 3, k);
-    sweeps_run(c, na);
+    for (int k = 0; k < na; k++) sweeps.in(act[k]->r, act[k]->s + 3, k);
+    sweeps.run(na);
     for (int k = 0; k < na; k++) {
       RhsRun &u = *act[k];
       double *now = u.s + 8 + u.it % 2, *old = u.s + 8 + (u.it + 1) % 2;
-      sweeps_out_dot(c, u.s + 3, k, u.r, first ? u.p : u.z, first ? nullptr : old, now, first ? nullptr : u.s + 11);
+      sweeps.out_dot(u.s + 3, k, u.r, first ? u.p : u.z, first ? nullptr : old, now, first ? nullptr : u.s + 11);
     }
   };
   collect([](const RhsRun &) { return true; });
@@ -1217,9 +1308,9 @@ ipm_status ipm_set_workspace(ipm_ctx *c, void *buf, size_t bytes) {
     const size_t total = c->ws_need;
     layout(c, base);
     CK(cudaMemsetAsync(c->ticket, 0, sizeof(unsigned), c->st));
-    c->psw.epoch = 0;  // no word carries a tag yet
-    CK(cudaMemsetAsync(c->psw.y, 0, c->psw.count * sizeof(uint2), c->st));
-    CK(cudaMemsetAsync(c->psw.x, 0, c->psw.count * sizeof(uint2), c->st));
+    c->epoch = 0;  // no word carries a tag yet
+    c->group_clean = false;
+    zero_own_words(c);
     CK(cudaStreamSynchronize(c->st));
     if (c->sys) {  // the formulation's system takes the rest of the buffer
       c->ws_need = total;
@@ -1289,7 +1380,7 @@ ipm_status kkt_solve(ipm_ctx *c, const double *b, double *x, int32_t nrhs, int32
     // then overwrite the next right-hand side)
     const bool apart = !(b < x + nrhs * n && x < b + nrhs * n) && !t->learned_active && !t->warm_x;
     for (int32_t k = 0; k < nrhs;) {
-      const int K = apart ? std::min(nrhs - k, kSolveRhs) : 1;
+      const int K = apart ? std::min(nrhs - k, t->rhs_max) : 1;
       ipm_solve_info one[kSolveRhs];
       ipm_status st[kSolveRhs];
       do_solves(t, K, b + k * n, x + k * n, refine, one, st);
@@ -1697,7 +1788,7 @@ ipm_status kkt_time_kernel(ipm_ctx *c, int32_t kernel, int32_t reps, double *ms)
       else if (kernel == 3 || kernel == 4)
         launch_fp32_solve(c, kernel == 3 ? 1 : 2);
       else
-        launch_held_solve<double>(c, 0, 1);
+        launch_held_solve<double>(c, solve_bufs<double>(c, 1), 0, 1);
     }
     CK(cudaEventRecord(e1, c->st));
     CK(cudaEventSynchronize(e1));

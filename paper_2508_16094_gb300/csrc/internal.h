@@ -62,7 +62,7 @@ struct SolveRec {
   int32_t slot0;  // slot of its first diagonal block
   int32_t kid_chunks;     // below-front chunks of all its children
   int32_t parent_blocks;  // diagonal blocks of its parent (0 at a root)
-  int32_t pad;
+  int32_t word0;          // its first column among the published entries
 };
 static_assert(sizeof(SolveRec) == 112 && sizeof(SolveRec) % 16 == 0, "SolveRec layout");
 
@@ -201,6 +201,7 @@ struct SolvePlan {
   std::vector<int32_t> parent_blocks;     // per front: diagonal blocks of its parent (0 at roots)
   int64_t part_entries = 0;               // values of partial sums
   int64_t flag_words = 0;
+  int64_t words = 0;                      // 8-byte words of published entries, y or x (FP64: two per value)
 };
 
 // Numeric plan: everything the kernels need, built on the host by analysis.

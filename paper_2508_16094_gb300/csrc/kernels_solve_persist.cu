@@ -200,7 +200,7 @@ template <typename T> struct PsArgs {
   int32_t q0, q1;    // tasks [q0, q1) of the plan
   unsigned *ticket;  // ticket counter, and the solve plan's flag words, zeroed before the launch
   unsigned *flags;
-  uint2 *ly, *lx;    // published entries of y and x, B words per slot (FP64: 2 B)
+  uint2 *ly, *lx;    // published entries of y and x, one word each (FP64: two)
   unsigned epoch;    // tag of this launch's entries
   int32_t *status;   // ST_SOLVE_TIMEOUT
   unsigned spins;    // polls before a wait gives up
@@ -364,8 +364,9 @@ __device__ __forceinline__ void publish(uint2 *slot, int r, double v, unsigned t
                : "memory");
 }
 __device__ __forceinline__ double word_double(unsigned lo, unsigned hi) { return __hiloint2double((int)hi, (int)lo); }
-template <typename T> __device__ __forceinline__ uint2 *slot_words(uint2 *base, int slot) {
-  return base + (int64_t)slot * (Ps<T>::B * (int)(sizeof(T) / 4));
+// The words of block j of a record's front.
+template <typename T> __device__ __forceinline__ uint2 *block_words(uint2 *base, const SolveRec &R, int j) {
+  return base + ((int64_t)R.word0 + Ps<T>::B * j) * (int)(sizeof(T) / 4);
 }
 
 // One warp: until load() holds in every lane (it reads the lane's words and tells
@@ -544,7 +545,7 @@ template <> struct FwdTile<double> {
 // zero past jb), published in the slot's words and kept at `keep` if given; a warp's rows
 // stop at their diagonal.
 // FP32: warp w takes rows 16w .. 16w + 15
-__device__ void diag_fwd(const PsArgs<float> &A, PsShared<float> &S, const FrontInfo &F, int j, int slot,
+__device__ void diag_fwd(const PsArgs<float> &A, PsShared<float> &S, const FrontInfo &F, int j, uint2 *words,
                          float *keep = nullptr) {
   constexpr int B = Ps<float>::B, RW = Ps<float>::RW;
   const int jb = min(B, F.ncol - j), ldi = (jb + 3) & ~3;
@@ -563,7 +564,7 @@ __device__ void diag_fwd(const PsArgs<float> &A, PsShared<float> &S, const Front
   const float s = rows_reduce(p);
   const int r = rw + lane / 2;
   if (lane % 2 == 0 && r < jb) {
-    publish(slot_words<float>(A.ly, slot), r, s, A.epoch);
+    publish(words, r, s, A.epoch);
     A.b[F.first + j + r] = s;
     if (keep) keep[r] = s;
   }
@@ -581,7 +582,7 @@ __device__ __forceinline__ int quad_row() {
 // is three triangular products a block on the FP64 unit instead of one (a solve at 40^3 takes
 // 1675 us, 1195 with the product alone; 2632 and 1915 at 48^3); a chain of 64 exchanges and
 // multiply-adds, as substitution has, would be longer still.
-__device__ void diag_fwd(const PsArgs<double> &A, PsShared<double> &S, const FrontInfo &F, int j, int slot,
+__device__ void diag_fwd(const PsArgs<double> &A, PsShared<double> &S, const FrontInfo &F, int j, uint2 *words,
                          double *keep = nullptr) {
   constexpr int B = Ps<double>::B;
   const int jb = min(B, F.ncol - j), ldi = (jb + 1) & ~1, r = quad_row(), h = threadIdx.x % 4, c = 2 * h;
@@ -607,7 +608,7 @@ __device__ void diag_fwd(const PsArgs<double> &A, PsShared<double> &S, const Fro
   if (last < 0) return;
   s += product(S.di + r * ldi, ldi, rs);
   if (h == 0 && r < jb) {
-    publish(slot_words<double>(A.ly, slot), r, s, A.epoch);
+    publish(words, r, s, A.epoch);
     A.b[F.first + j + r] = s;
     if (keep) keep[r] = s;
   }
@@ -647,7 +648,7 @@ __device__ __forceinline__ void put_sum(double *row, int c, double s) { row[c] =
 // diagonal; v = S.sv), published in the slot's words. FP32: thread (g, q) takes columns
 // 4q .. and rows 16g ..; FP64: four threads per column, a warp's eight columns start
 // at their diagonal, and the result is corrected as in diag_fwd.
-__device__ void diag_bwd(const PsArgs<float> &A, PsShared<float> &S, const FrontInfo &F, int j, int slot) {
+__device__ void diag_bwd(const PsArgs<float> &A, PsShared<float> &S, const FrontInfo &F, int j, uint2 *words) {
   constexpr int B = Ps<float>::B, RW = Ps<float>::RW;
   const int jb = min(B, F.ncol - j), ldi = (jb + 3) & ~3;
   const int q = threadIdx.x % 32, g = threadIdx.x / 32, c = 4 * q;
@@ -665,12 +666,12 @@ __device__ void diag_bwd(const PsArgs<float> &A, PsShared<float> &S, const Front
   groups_sum(S, [&](int c0, auto s) {
     each_sum(c0, s, [&](int cc, float v) {
       if (cc >= jb) return;
-      publish(slot_words<float>(A.lx, slot), cc, v, A.epoch);
+      publish(words, cc, v, A.epoch);
       xo[cc] = v;
     });
   });
 }
-__device__ void diag_bwd(const PsArgs<double> &A, PsShared<double> &S, const FrontInfo &F, int j, int slot) {
+__device__ void diag_bwd(const PsArgs<double> &A, PsShared<double> &S, const FrontInfo &F, int j, uint2 *words) {
   constexpr int B = Ps<double>::B;
   const int jb = min(B, F.ncol - j), ldi = (jb + 1) & ~1, c = quad_row(), h = threadIdx.x % 4;
   const int m0 = 2 * (c / 8), m1 = (jb + 3) / 4;  // row groups of this warp's columns (uniform per warp)
@@ -697,7 +698,7 @@ __device__ void diag_bwd(const PsArgs<double> &A, PsShared<double> &S, const Fro
   if (m0 >= m1) return;
   s += product(S.di, ldi, rs);
   if (h == 0 && c < jb) {
-    publish(slot_words<double>(A.lx, slot), c, s, A.epoch);
+    publish(words, c, s, A.epoch);
     A.x[F.first + j + c] = s;
   }
 }
@@ -851,14 +852,14 @@ __device__ void fwd_diag(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R, 
   const T *row = A.L + F.loff + (int64_t)j0 * F.ld;
   for (int j = 0; j < i && ok; j++) {  // block j < i is a full block
     tile.template load<true>(row + B * j, F.ld, jb, B);
-    ok = tile.wait_y(A, slot_words<T>(A.ly, slot0 + j), B, j == i - 1);
+    ok = tile.wait_y(A, block_words<T>(A.ly, R, j), B, j == i - 1);
     if (ok) tile.template mul<true>(S, B);
   }
   take_next(A, N);
   tile.finish(ok ? jb : 0, [&](int r, T v) { S.sv[r] -= v; });
   // the staged copy always lands before S.di is reused; the wait ends with a
   // barrier, after which every row of S.sv is final
-  if (wait_dinv(A, S, ok)) diag_fwd(A, S, F, j0, slot0 + i);
+  if (wait_dinv(A, S, ok)) diag_fwd(A, S, F, j0, block_words<T>(A.ly, R, i));
 }
 
 // Forward, rows r0 .. r0 + nr below front s: the children's entries plus
@@ -881,7 +882,7 @@ __device__ void fwd_below(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R,
     const T *P = row + B * j;
     if (jbj == B) tile.template load<true>(P, F.ld, nr, B);
     else tile.template load<false>(P, F.ld, nr, jbj);
-    ok = tile.wait_y(A, slot_words<T>(A.ly, slot0 + j), jbj, false);
+    ok = tile.wait_y(A, block_words<T>(A.ly, R, j), jbj, false);
     if (!ok) break;
     if (jbj == B) tile.template mul<true>(S, B);
     else tile.template mul<false>(S, jbj);
@@ -971,7 +972,7 @@ __device__ void bwd_diag(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R, 
     const int cc = threadIdx.x / TPC;
     const bool mine = threadIdx.x % TPC == 0 && cc < jb;
     T bv = T(0);
-    const uint2 *words = slot_words<T>(A.ly, slot0 + cb);
+    const uint2 *words = block_words<T>(A.ly, R, cb);
     if (A.fwd_here)
       ok = wait_words(A, words, false, [&]() { return !mine || read_word(words, cc, A.epoch, bv); });
     else if (mine)
@@ -997,7 +998,7 @@ __device__ void bwd_diag(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R, 
     // lane k < RW reads x of row RW g + k of block i; the warp shares them
     T xv = T(0);
     const bool mine = q < RW && RW * g + q < jbi;
-    const uint2 *words = slot_words<T>(A.lx, slot0 + i);
+    const uint2 *words = block_words<T>(A.lx, R, i);
     ok = wait_words(A, words, i == cb + 1, [&]() { return !mine || read_word(words, RW * g + q, A.epoch, xv); });
     if (!ok) break;
 #pragma unroll
@@ -1013,7 +1014,7 @@ __device__ void bwd_diag(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R, 
       });
     });
   if (wait_dinv(A, S, ok)) {  // (ends with a barrier)
-    diag_bwd(A, S, F, c0, slot0 + cb);
+    diag_bwd(A, S, F, c0, block_words<T>(A.lx, R, cb));
     signal(f_front(A, tk.front));
   }
 }
@@ -1051,7 +1052,7 @@ __device__ void fwd_narrow(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R
   if (tid >= nc && tid < kNarrowCols) S.xs[tid] = T(0);
   take_next(A, N);
   if (!wait_dinv(A, S, ok)) return;  // (a barrier: S.sv is written)
-  diag_fwd(A, S, F, 0, R.slot0, S.xs);
+  diag_fwd(A, S, F, 0, block_words<T>(A.ly, R, 0), S.xs);
   __syncthreads();
   for (int r0 = 0; r0 < nr; r0 += kT) {
     const int r = r0 + tid;
@@ -1108,7 +1109,7 @@ __device__ void bwd_narrow(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R
   if (ok) {
     if (tid < nr) xs[tid] = ldcg(A.x + i0);
     if (tid + kT < nr) xs[tid + kT] = ldcg(A.x + i1);
-    const uint2 *words = slot_words<T>(A.ly, R.slot0);
+    const uint2 *words = block_words<T>(A.ly, R, 0);
     if (A.fwd_here) ok = wait_words(A, words, false, [&]() { return tid >= nc || read_word(words, tid, A.epoch, bv); });
     else if (tid < nc) bv = ldcg(A.b + F.first + tid);
   }
@@ -1134,7 +1135,7 @@ __device__ void bwd_narrow(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R
     S.sv[tid] = bv - s;
   }
   if (wait_dinv(A, S, ok)) {  // (ends with a barrier)
-    diag_bwd(A, S, F, 0, R.slot0);
+    diag_bwd(A, S, F, 0, block_words<T>(A.lx, R, 0));
     signal(f_front(A, R.task.front));
   }
 }
@@ -1250,27 +1251,17 @@ void launch_dinv(const DevPlan &dp, const Plan &plan, const double *L, double *D
   dinv64_kernel<<<n, kDinvThreads, smem, st>>>(dp, L, Dinv);
 }
 
-int64_t solve_words(const SolvePlan &sp) {  // one per FP32 value, two per FP64 value
-  return std::max<int64_t>((int64_t)sp.dinv_off.size() * sp.B * (sp.B == kSolveB64 ? 2 : 1), 2);
-}
-
 template <typename T>
 void launch_psolve(const DevPlan &dp, const Plan &plan, const T *L, const T *Dinv, const SolveBufs<T> &v,
-                   int nrhs, SolveWords &words, int32_t *status, bool fwd, bool bwd, cudaStream_t st,
+                   int nrhs, int32_t *status, bool fwd, bool bwd, cudaStream_t st,
                    unsigned test_spins, int test_withhold) {
   const SolvePlan &sp = sizeof(T) == 8 ? plan.s64 : plan.s32;
   const int32_t q0 = fwd ? 0 : sp.fwd_tasks;
   const int32_t q1 = bwd ? (int32_t)sp.tasks.size() : sp.fwd_tasks;
   if (q1 <= q0) return;
   ck(cudaMemsetAsync(v.flags, 0, (size_t)(nrhs * v.sd.flags) * sizeof(unsigned), st), "solve flags");
-  if (++words.epoch == 0) {  // the tags start over
-    const size_t bytes = (size_t)words.count * sizeof(uint2);
-    ck(cudaMemsetAsync(words.y, 0, bytes, st), "solve words");
-    ck(cudaMemsetAsync(words.x, 0, bytes, st), "solve words");
-    words.epoch = 1;
-  }
   PsArgs<T> A{dp, sizeof(T) == 8 ? dp.s64 : dp.s32, L, Dinv, v.a, v.b, v.x, v.t, v.part, q0, q1, v.flags, v.flags,
-              words.y, words.x, words.epoch, status, test_spins ? test_spins : kBarrierSpins, test_withhold,
+              v.wy, v.wx, v.epoch, status, test_spins ? test_spins : kBarrierSpins, test_withhold,
               (int32_t)sp.dinv_off.size(), (int32_t)plan.fronts.size(), fwd && bwd ? 1 : 0, nrhs, v.sd};
   const int64_t tickets = (int64_t)(q1 - q0) * nrhs;
   note_launch();
@@ -1279,10 +1270,10 @@ void launch_psolve(const DevPlan &dp, const Plan &plan, const T *L, const T *Din
   ck(cudaGetLastError(), "solve launch");
 }
 template void launch_psolve<float>(const DevPlan &, const Plan &, const float *, const float *,
-                                   const SolveBufs<float> &, int, SolveWords &, int32_t *, bool, bool,
-                                   cudaStream_t, unsigned, int);
+                                   const SolveBufs<float> &, int, int32_t *, bool, bool, cudaStream_t, unsigned,
+                                   int);
 template void launch_psolve<double>(const DevPlan &, const Plan &, const double *, const double *,
-                                    const SolveBufs<double> &, int, SolveWords &, int32_t *, bool, bool,
-                                    cudaStream_t, unsigned, int);
+                                    const SolveBufs<double> &, int, int32_t *, bool, bool, cudaStream_t, unsigned,
+                                    int);
 
 }  // namespace gipm

@@ -55,19 +55,11 @@ void launch_sign(const DevPlan &dp, V *y, cudaStream_t st);
 // commits no device memory (lazy module loading); used by the allocation-free solve.
 cudaError_t preload_level_solve();
 
-// Tagged entries the persistent solve hands from block to block (zeroed once, before
-// the first launch; each launch, of either type, takes the next tag): `count` words
-// each, solve_words(plan) of them per right-hand side.
-struct SolveWords {
-  uint2 *y = nullptr, *x = nullptr;
-  int64_t count = 0;
-  unsigned epoch = 0;
-};
-int64_t solve_words(const SolvePlan &sp);
-
 // The vectors of a persistent solve: right-hand sides, forward results, solutions,
-// update vectors, partial sums and flags of up to kSolveRhs right-hand sides, each
-// kind `sd` apart from one to the next (t in values of T). A solve is bound by its
+// update vectors, partial sums, flags and published entries of up to kSolveRhs right-hand sides,
+// each kind `sd` apart from one to the next (t in values of T). The entries wy, wx handed from
+// block to block carry the tag of their launch: zeroed before the first one, and no two launches
+// between have the same tag `epoch` (not 0). A solve is bound by its
 // chain of diagonal blocks, so right-hand sides side by side cost little until they
 // fill the chip: 56^3 TF32x3, eight right-hand sides with PCG: 27.4 ms one by one,
 // 16.6 in fours, 15.2 as eight.
@@ -78,6 +70,8 @@ struct SolveStride {
 template <typename T> struct SolveBufs {
   T *a = nullptr, *b = nullptr, *x = nullptr, *t = nullptr, *part = nullptr;
   unsigned *flags = nullptr;
+  uint2 *wy = nullptr, *wx = nullptr;
+  unsigned epoch = 0;
   SolveStride sd;
 };
 
@@ -94,8 +88,8 @@ void launch_dinv(const DevPlan &dp, const Plan &plan, const float *L, float *Din
 void launch_dinv(const DevPlan &dp, const Plan &plan, const double *L, double *Dinv, cudaStream_t st);
 template <typename T>
 void launch_psolve(const DevPlan &dp, const Plan &plan, const T *L, const T *Dinv, const SolveBufs<T> &v,
-                   int nrhs, SolveWords &words, int32_t *status, bool fwd, bool bwd, cudaStream_t st,
-                   unsigned test_spins = 0, int test_withhold = -1);
+                   int nrhs, int32_t *status, bool fwd, bool bwd, cudaStream_t st, unsigned test_spins = 0,
+                   int test_withhold = -1);
 
 // Sampled entries of L (final numbering).
 template <typename T>
