@@ -81,7 +81,7 @@ struct ipm_ctx {
   unsigned *ticket = nullptr;  // of the reductions (VecOps), zeroed when the workspace is set
   IpmScalars *sc = nullptr;
   int32_t *status = nullptr, *col2s = nullptr;
-  ChainStream chain;   // of the FMA-pipe FP64 factor
+  SideStream chain;    // of the FMA-pipe FP64 factor
   TcPlan tcp;
   OzPlan ozp;          // FP64 factor on tensor cores (Ozaki slices), with options.fp64_tc
   bool oz_on = false;  // its task lists and slice storage were sized by kkt_analyze
@@ -1326,7 +1326,7 @@ ipm_status ipm_set_workspace(ipm_ctx *c, void *buf, size_t bytes) {
     CK(preload_vec_kernels());
     c->have_stale = false;
     if (c->lb_on) learned_init_weights(c);
-    if (!c->sys) c->chain.create();
+    if (!c->sys && !c->chain.create(true)) throw Fail{IPM_ERR_CUDA, "cannot create the factorisation's chain stream"};
     try {  // tensor maps of the FP32 panels for the tensor-core path
       if (!c->sys) c->tcp.encode(c->plan, (float *)c->L, c->Llo, (float *)c->U, c->st);
     } catch (const std::exception &e) {

@@ -760,27 +760,6 @@ static void launch_upd(const DevPlan &dp, const UpdRange &u, float *L, float *U,
                                                               u.clim, u.with_u, L, U);
 }
 
-void ChainStream::create() {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) throw std::runtime_error("no current device");
-  if (s && dev == device) return;
-  destroy();
-  device = dev;
-  int lo = 0, hi = 0;
-  if (cudaDeviceGetStreamPriorityRange(&lo, &hi) != cudaSuccess ||
-      cudaStreamCreateWithPriority(&s, cudaStreamNonBlocking, hi) != cudaSuccess ||
-      cudaEventCreateWithFlags(&solved, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&updated, cudaEventDisableTiming) != cudaSuccess)
-    throw std::runtime_error("cannot create the factorisation's chain stream");
-}
-void ChainStream::destroy() {
-  if (solved) cudaEventDestroy(solved);
-  if (updated) cudaEventDestroy(updated);
-  if (s) cudaStreamDestroy(s);
-  solved = updated = nullptr;
-  s = nullptr;
-}
-
 // FP64 with look-ahead: the chain (diagonal block, panel solve, update of the
 // next step's columns) goes on its own stream ahead of the update of everything past
 // them, whose blocks it would otherwise wait for; it has the higher priority, so its
@@ -788,30 +767,30 @@ void ChainStream::destroy() {
 // steps 0 .. s in order: rest(s - 1) is complete before next(s) starts. 32^3 grid LP
 // (FP64): 47.2 -> 43.7 ms a system.
 static void factor_steps64(const DevPlan &dp, const LevelPlan &LP, double *L, double *U, int32_t *status, bool perturb,
-                           const ChainStream &ch, cudaStream_t st) {
-  cudaEventRecord(ch.updated, st);  // the level's fronts are built
-  cudaStreamWaitEvent(ch.s, ch.updated, 0);
+                           const SideStream &chain, cudaStream_t st) {
+  cudaEventRecord(chain.fork, st);  // the level's fronts are built
+  cudaStreamWaitEvent(chain.s, chain.fork, 0);
   for (size_t k = 0; k < LP.steps.size(); k++) {
     const StepRange &S = LP.steps[k];
-    launch_potrf<double>(dp, S, L, status, perturb, ch.s);
-    launch_trsm<double>(dp, S, L, ch.s);
-    cudaEventRecord(ch.solved, ch.s);
-    if (k > 0) cudaStreamWaitEvent(ch.s, ch.updated, 0);
-    launch_upd(dp, S.next64, L, U, ch.s);
-    cudaStreamWaitEvent(st, ch.solved, 0);
+    launch_potrf<double>(dp, S, L, status, perturb, chain.s);
+    launch_trsm<double>(dp, S, L, chain.s);
+    cudaEventRecord(chain.join, chain.s);
+    if (k > 0) cudaStreamWaitEvent(chain.s, chain.fork, 0);
+    launch_upd(dp, S.next64, L, U, chain.s);
+    cudaStreamWaitEvent(st, chain.join, 0);
     launch_upd(dp, S.rest64, L, U, st);
-    if (k + 1 < LP.steps.size()) cudaEventRecord(ch.updated, st);
+    if (k + 1 < LP.steps.size()) cudaEventRecord(chain.fork, st);
   }
 }
 
 template <typename T>
 void launch_factor_simt(const DevPlan &dp, const Plan &plan, const double *kval, T *L, T *U,
-                        int32_t *status, bool perturb, const ChainStream &ch, cudaStream_t st) {
+                        int32_t *status, bool perturb, const SideStream &chain, cudaStream_t st) {
   for (const LevelPlan &LP : plan.levels) {
     launch_build_level<T>(dp, LP, kval, L, U, st);
     if constexpr (sizeof(T) == 8) {
       if (LP.ahead64) {
-        factor_steps64(dp, LP, L, U, status, perturb, ch, st);
+        factor_steps64(dp, LP, L, U, status, perturb, chain, st);
         continue;
       }
     }
@@ -844,9 +823,9 @@ template void launch_potrf<double>(const DevPlan &, const StepRange &, double *,
                                    cudaStream_t);
 template void launch_trsm<double>(const DevPlan &, const StepRange &, double *, cudaStream_t);
 template void launch_factor_simt<double>(const DevPlan &, const Plan &, const double *, double *,
-                                         double *, int32_t *, bool, const ChainStream &, cudaStream_t);
+                                         double *, int32_t *, bool, const SideStream &, cudaStream_t);
 template void launch_factor_simt<float>(const DevPlan &, const Plan &, const double *, float *,
-                                        float *, int32_t *, bool, const ChainStream &, cudaStream_t);
+                                        float *, int32_t *, bool, const SideStream &, cudaStream_t);
 template void launch_factor_entries<double>(const DevPlan &, const double *, const int32_t *,
                                             int64_t, const int32_t *, const int32_t *, double *,
                                             cudaStream_t);

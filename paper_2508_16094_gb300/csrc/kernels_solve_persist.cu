@@ -1221,16 +1221,22 @@ template <typename T, bool MANY> int psolve_grid(int64_t ntask) {
 
 }  // namespace
 
+// Allow a kernel this much shared memory on the current device (`once`: the kernel's).
+template <typename K> static void allow_smem(K kernel, int smem, DeviceOnce &once) {
+  int dev = 0;
+  ck(cudaGetDevice(&dev), "cudaGetDevice");
+  if (!once.needed(dev)) return;
+  ck(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem), "dinv attribute");
+  once.done(dev);
+}
+
 void launch_dinv(const DevPlan &dp, const Plan &plan, const float *L, float *Dinv,
                  cudaStream_t st) {
   const int n = (int)plan.s32.inv.size();
   if (n == 0) return;
   const int smem = 2 * 128 * 129 * (int)sizeof(float);
-  static bool attr = false;
-  if (!attr) {
-    ck(cudaFuncSetAttribute(dinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem), "dinv attribute");
-    attr = true;
-  }
+  static DeviceOnce once;
+  allow_smem(dinv_kernel, smem, once);
   note_launch();
   dinv_kernel<<<n, 128, smem, st>>>(dp, L, Dinv);
 }
@@ -1240,13 +1246,8 @@ void launch_dinv(const DevPlan &dp, const Plan &plan, const double *L, double *D
   const int n = (int)plan.s64.inv.size();
   if (n == 0) return;
   constexpr int smem = kSolveB64 * (2 * kSolveB64 + 1) * (int)sizeof(double);
-  static bool attr[64] = {false};  // per device
-  int dev = 0;
-  ck(cudaGetDevice(&dev), "cudaGetDevice");
-  if (!attr[dev & 63]) {
-    ck(cudaFuncSetAttribute(dinv64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem), "dinv attribute");
-    attr[dev & 63] = true;
-  }
+  static DeviceOnce once;
+  allow_smem(dinv64_kernel, smem, once);
   note_launch();
   dinv64_kernel<<<n, kDinvThreads, smem, st>>>(dp, L, Dinv);
 }

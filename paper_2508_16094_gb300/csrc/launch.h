@@ -2,6 +2,7 @@
 #pragma once
 
 #include "dev.cuh"
+#include "side_stream.h"
 
 namespace gipm {
 
@@ -10,24 +11,27 @@ namespace gipm {
 void launch_assemble(const DevPlan &dp, const double *jv, const double *D, const double *wv,
                      double delta_p, double *kval, cudaStream_t st);
 
-// Multifrontal factorisation of all levels with SIMT FMA kernels. status must
-// be initialised by the caller (ST_FAIL_COL = INT32_MAX, ST_PERTURBED = 0).
-// Stream and events of the FP64 factor's look-ahead (one per context; see
-// factor_steps64).
-struct ChainStream {
-  cudaStream_t s = nullptr;                         // highest priority
-  cudaEvent_t solved = nullptr, updated = nullptr;  // fork / join
-  int device = -1;
-  ChainStream() = default;
-  ChainStream(const ChainStream &) = delete;
-  ChainStream &operator=(const ChainStream &) = delete;
-  ~ChainStream() { destroy(); }
-  void create();  // on the current device
-  void destroy();
+struct CudaApi {
+  using Stream = cudaStream_t;
+  using Event = cudaEvent_t;
+  static bool current_device(int &dev) { return cudaGetDevice(&dev) == cudaSuccess; }
+  static bool create(bool high, Stream &s) {
+    int lo = 0, hi = 0;
+    return cudaDeviceGetStreamPriorityRange(&lo, &hi) == cudaSuccess &&
+           cudaStreamCreateWithPriority(&s, cudaStreamNonBlocking, high ? hi : lo) == cudaSuccess;
+  }
+  static bool create(Event &e) { return cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess; }
+  static void destroy(Stream s) { cudaStreamDestroy(s); }
+  static void destroy(Event e) { cudaEventDestroy(e); }
 };
+using SideStream = SideStreamOf<CudaApi>;
+
+// Multifrontal factorisation of all levels with SIMT FMA kernels. status must
+// be initialised by the caller (ST_FAIL_COL = INT32_MAX, ST_PERTURBED = 0). chain: the
+// highest-priority stream of the FP64 factor's look-ahead (one per context; see factor_steps64).
 template <typename T>
 void launch_factor_simt(const DevPlan &dp, const Plan &plan, const double *kval, T *L, T *U,
-                        int32_t *status, bool perturb, const ChainStream &ch, cudaStream_t st);
+                        int32_t *status, bool perturb, const SideStream &chain, cudaStream_t st);
 
 // Pieces of a level of the factorisation, shared with the tensor-core path:
 // front assembly (+ K entries), diagonal-block Cholesky (64 wide) and the

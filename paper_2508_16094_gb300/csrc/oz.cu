@@ -617,18 +617,7 @@ void OzPlan::layout(Carve &cv, cudaStream_t st, bool storage) {
 void OzPlan::encode(const Plan &plan, cudaStream_t st) {
   ready_ = false;
   if (!sized_ || !S_) return;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) throw std::runtime_error("no current device");
-  if (!side_ || dev != side_device_) {
-    destroy_streams();
-    side_device_ = dev;
-    int lo = 0, hi = 0;
-    cudaDeviceGetStreamPriorityRange(&lo, &hi);
-    if (cudaStreamCreateWithPriority(&side_, cudaStreamNonBlocking, lo) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ev_main_, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ev_side_, cudaEventDisableTiming) != cudaSuccess)
-      throw std::runtime_error("cannot create the look-ahead stream");
-  }
+  if (!side_.create(false)) throw std::runtime_error("cannot create the look-ahead stream");
   PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
   const size_t nfr = plan.fronts.size();
   std::vector<CUtensorMap> maps(2 * nfr);
@@ -687,14 +676,14 @@ void OzPlan::factor(const DevPlan &dp, const Plan &plan, const double *kval, dou
       const StepRange &R = LP.steps[s];
       const Step &Z = V.steps[s];
       // both parts of a column's sum are added to the same entries: in this order, always
-      if (pending) cudaStreamWaitEvent(st, ev_side_, 0);
+      if (pending) cudaStreamWaitEvent(st, side_.join, 0);
       gemm(Z.gemm_b, Z.gemm_e, sms, st);
       pending = Z.ahead_e > Z.ahead_b;
       if (pending) {
-        cudaEventRecord(ev_main_, st);
-        cudaStreamWaitEvent(side_, ev_main_, 0);
-        gemm(Z.ahead_b, Z.ahead_e, side_ctas, side_);
-        cudaEventRecord(ev_side_, side_);
+        cudaEventRecord(side_.fork, st);
+        cudaStreamWaitEvent(side_.s, side_.fork, 0);
+        gemm(Z.ahead_b, Z.ahead_e, side_ctas, side_.s);
+        cudaEventRecord(side_.join, side_.s);
       }
       launch_potrf<double>(dp, R, L, status, false, st);
       launch_trsm<double>(dp, R, L, st);
@@ -704,17 +693,9 @@ void OzPlan::factor(const DevPlan &dp, const Plan &plan, const double *kval, dou
                                                               S_, E_);
       }
     }
-    if (pending) cudaStreamWaitEvent(st, ev_side_, 0);
+    if (pending) cudaStreamWaitEvent(st, side_.join, 0);
     gemm(V.syrk_b, V.syrk_e, sms, st);
   }
-}
-
-void OzPlan::destroy_streams() {
-  if (ev_main_) cudaEventDestroy(ev_main_);
-  if (ev_side_) cudaEventDestroy(ev_side_);
-  if (side_) cudaStreamDestroy(side_);
-  ev_main_ = ev_side_ = nullptr;
-  side_ = nullptr;
 }
 
 }  // namespace gipm

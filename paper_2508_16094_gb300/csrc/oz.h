@@ -6,7 +6,7 @@
 
 #include <vector>
 
-#include "dev.cuh"
+#include "launch.h"
 
 namespace gipm {
 
@@ -25,7 +25,6 @@ class OzPlan {
   static constexpr int kPlanes = 7;  // BF16 slices per FP64 value
   static constexpr int kBlk = 64;    // the plan's block width; windows are 1 or 2 blocks
   OzPlan() = default;
-  ~OzPlan() { destroy_streams(); }
   OzPlan(const OzPlan &) = delete;
   OzPlan &operator=(const OzPlan &) = delete;
   // Task lists and slice layout from the FP64 plan (block width kBlk).
@@ -44,7 +43,6 @@ class OzPlan {
 
  private:
   void validate(const Plan &plan) const;
-  void destroy_streams();
   // updates of a step's block column, those of the next one that can run beside the
   // step, and its slices
   struct Step { int gemm_b, gemm_e, ahead_b, ahead_e, slice_b, slice_e; };
@@ -59,9 +57,7 @@ class OzPlan {
   uint16_t *S_ = nullptr;   // slice planes (BF16 bits)
   int16_t *E_ = nullptr;    // exponent tables
   bool sized_ = false, ready_ = false;
-  cudaStream_t side_ = nullptr;                        // look-ahead stream (low priority)
-  int side_device_ = -1;
-  cudaEvent_t ev_main_ = nullptr, ev_side_ = nullptr;  // fork / join
+  SideStream side_;  // look-ahead (default priority: the launches leave SMs to the chain)
 };
 
 }  // namespace gipm

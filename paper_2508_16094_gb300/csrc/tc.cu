@@ -1225,14 +1225,7 @@ void TcPlan::layout(Carve &cv, cudaStream_t st) {
 
 void TcPlan::encode(const Plan &plan, float *L, float *Llo, float *U, cudaStream_t st) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
-  if (!side_) {
-    int lo = 0, hi = 0;
-    cudaDeviceGetStreamPriorityRange(&lo, &hi);
-    if (cudaStreamCreateWithPriority(&side_, cudaStreamNonBlocking, lo) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ev_main_, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&ev_side_, cudaEventDisableTiming) != cudaSuccess)
-      throw std::runtime_error("cannot create the look-ahead stream");
-  }
+  if (!side_.create(false)) throw std::runtime_error("cannot create the look-ahead stream");
   L_ = L;
   Llo_ = Llo;
   U_ = U;
@@ -1333,15 +1326,11 @@ void TcPlan::encode(const Plan &plan, float *L, float *Llo, float *U, cudaStream
   ready_ = true;
 }
 
-static int sm_count() {
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (sms <= 0) sms = 1;
-  }
-  return sms;
+static int sm_count() {  // of the current device
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return std::max(sms, 1);
 }
 
 // Persistent launch: at most ctas CTAs (one per SM), each taking tiles ctas apart.
@@ -1369,12 +1358,6 @@ static void pair_launch(int npair, int ctas, const DevPlan &dp, const Task *pair
       dp, pairs, npair, maps, maps_lo, umaps, lmaps, maps_bf, status);
 }
 
-TcPlan::~TcPlan() {
-  if (ev_main_) cudaEventDestroy(ev_main_);
-  if (ev_side_) cudaEventDestroy(ev_side_);
-  if (side_) cudaStreamDestroy(side_);
-}
-
 void TcPlan::factor(const DevPlan &dp, const Plan &plan, const double *kval, float *L, float *U,
                     float *Dinv, int32_t *status, int split, cudaStream_t st) {
   auto gemm3 = split == 3 ? gemm_launch<3, 128>
@@ -1382,7 +1365,7 @@ void TcPlan::factor(const DevPlan &dp, const Plan &plan, const double *kval, flo
   auto pair3 = split == 3 ? pair_launch<3> : (split == kBf16 ? pair_launch<kBf16> : pair_launch<1>);
   const CUtensorMap *maps = static_cast<const CUtensorMap *>(d_maps_);
   if (L != L_ || U != U_) throw std::runtime_error("tensor maps were encoded for other factor buffers");
-  if (!side_) throw std::runtime_error("tensor-core factor streams not created");
+  if (!side_.s) throw std::runtime_error("tensor-core factor streams not created");
   const int sms = sm_count();
   const int main_ctas = std::min(kMainCtas, sms / 2), side_ctas = sms - main_ctas;
   auto gemm = [&](const Task *t, int n, int ctas, cudaStream_t s) {
@@ -1397,19 +1380,19 @@ void TcPlan::factor(const DevPlan &dp, const Plan &plan, const double *kval, flo
     launch_build_level<float>(dp, plan.levels[li], kval, L, U, st);
     for (const Super &sp : lv.supers) {
       if (pending) {  // this super-step's columns took the look-ahead update
-        cudaStreamWaitEvent(st, ev_side_, 0);
+        cudaStreamWaitEvent(st, side_.join, 0);
         pending = false;
       }
       const bool ahead = sp.ahead_e > sp.ahead_b;
       if (ahead) {  // the columns before this super-step are final: fork
-        cudaEventRecord(ev_main_, st);
-        cudaStreamWaitEvent(side_, ev_main_, 0);
+        cudaEventRecord(side_.fork, st);
+        cudaStreamWaitEvent(side_.s, side_.fork, 0);
       }
       pair(sp.now_b, sp.now_e, sms, st);
       const int ctas = ahead ? main_ctas : sms;
       if (ahead) {
-        pair(sp.ahead_b, sp.ahead_e, side_ctas, side_);
-        cudaEventRecord(ev_side_, side_);
+        pair(sp.ahead_b, sp.ahead_e, side_ctas, side_.s);
+        cudaEventRecord(side_.join, side_.s);
         pending = true;
       }
       for (int i = sp.step_b; i < sp.step_e; i++) {
@@ -1421,7 +1404,7 @@ void TcPlan::factor(const DevPlan &dp, const Plan &plan, const double *kval, flo
       }
     }
     if (pending) {
-      cudaStreamWaitEvent(st, ev_side_, 0);
+      cudaStreamWaitEvent(st, side_.join, 0);
       pending = false;
     }
     pair(lv.pair_b, lv.pair_e, sms, st);  // the level's update matrices

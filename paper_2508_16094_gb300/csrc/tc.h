@@ -8,7 +8,7 @@
 
 #include <vector>
 
-#include "dev.cuh"
+#include "launch.h"
 
 namespace gipm {
 
@@ -21,15 +21,14 @@ class TcPlan {
   TcPlan() = default;
   TcPlan(const TcPlan &) = delete;
   TcPlan &operator=(const TcPlan &) = delete;
-  ~TcPlan();
   // Host task lists (after the symbolic analysis and plan).
   void build(const Plan &plan);
   // Carve device memory for tasks and tensor maps (cv.base == nullptr: size only).
   void layout(Carve &cv, cudaStream_t st);
   // Encode one TMA tensor map per front panel of the FP32 factor storage L and
   // of Llo (low parts x - tf32(x) of the finished entries, same layout), and
-  // one per update matrix in U; also creates the side stream and events of
-  // the look-ahead (once).
+  // one per update matrix in U; also creates the look-ahead's side stream, on the
+  // current device.
   void encode(const Plan &plan, float *L, float *Llo, float *U, cudaStream_t st);
   bool ready() const { return ready_; }
   // split = 1: plain TF32 products; split = 3: A_lo B + A B_lo + A B
@@ -60,8 +59,7 @@ class TcPlan {
   Task *d_gemm_ = nullptr, *d_potrf_ = nullptr, *d_trsm_ = nullptr, *d_pairs_ = nullptr;
   void *d_maps_ = nullptr;  // 7 nfronts_ + 1 CUtensorMap (128 bytes each)
   float *L_ = nullptr, *Llo_ = nullptr, *U_ = nullptr;
-  cudaStream_t side_ = nullptr;                              // look-ahead stream (low priority)
-  cudaEvent_t ev_main_ = nullptr, ev_side_ = nullptr;        // fork / join
+  SideStream side_;  // look-ahead (default priority: the launches leave SMs to the panel steps)
   bool ready_ = false;
 };
 
