@@ -14,7 +14,7 @@
 // trip through L2 and no fence (a counter behind a release, polled and
 // acquired before the values are read, takes three: 2.6 us a block of the root
 // against 1.8; a whole solve, TF32x3: 834 -> 666 us at 48^3, 1845 -> 1548 at
-// 64^3, FP64 1484 -> 1302 at 40^3). A
+// 64^3). The words lie in the order of the columns, each front on lines of its own. A
 // diagonal block of the forward sweep subtracts L_ij y_j as each y_j of its front
 // appears (a wavefront down the front's blocks), rows below a front take every
 // y_j and then count towards the front's update vector, which the parent's gathers
@@ -1024,7 +1024,7 @@ __device__ void bwd_diag(const PsArgs<T> &A, PsShared<T> &S, const SolveRec &R, 
 // to 4 us whatever its size (ticket, record, the children's flag, two dependent gathers,
 // its own flag): one task a front and sweep instead of one per block and chunk of rows,
 // which also hands y to the rows below through shared memory. One solve, TF32x3: 666 ->
-// 574 us at 48^3, 1548 -> 1320 at 64^3, FP64 1302 -> 1180 at 40^3; eight right-hand
+// 574 us at 48^3, 1548 -> 1320 at 64^3; eight right-hand
 // sides at 56^3 with PCG 15.2 -> 12.6 ms. (64 columns in FP32: 12.0 ms, nothing for one
 // right-hand side.)
 // Forward: a thread per row below (its L row in registers before the wait), the

@@ -1017,21 +1017,21 @@ void build_fused_solve(const Plan &pl, int B, SolvePlan &sp) {
     }
     need(kids == sp.kid_chunks[s], "children's chunk count");
   }
-  // published entries in the order of the columns, every front at an even place (16-byte reads of
-  // FP32 words) and room for a last read past the end
-  auto word0 = [&](int32_t s) { return ((int64_t)pl.fronts[s].first + s + 1) & ~int64_t(1); };
+  // published entries in the order of the columns, every front from a 128-byte line of its own on
+  // (lines that two fronts share: the forward sweep 3 % slower)
+  std::vector<int32_t> word0(nfr);
   int64_t end = 0;
   for (int32_t s = 0; s < nfr; s++) {
-    need(word0(s) >= end, "published entries overlap");
-    end = word0(s) + pl.fronts[s].ncol;
+    word0[s] = (int32_t)end;
+    end += round_up(pl.fronts[s].ncol, 16);
+    need(end < INT32_MAX, "published entries");
   }
-  need(end + 4 < INT32_MAX, "published entries");
-  sp.words = ((end + 5) & ~int64_t(1)) * (B == kSolveB64 ? 2 : 1);
+  sp.words = std::max<int64_t>(end, 16) * (B == kSolveB64 ? 2 : 1);
   sp.recs.resize(sp.tasks.size());
   for (size_t q = 0; q < sp.tasks.size(); q++) {
     const int32_t s = sp.tasks[q].front;
     sp.recs[q] = SolveRec{sp.tasks[q], pl.fronts[s], pl.toff[s], sp.pbase[s],
-                             sp.first_slot[s], sp.kid_chunks[s], sp.parent_blocks[s], (int32_t)word0(s)};
+                             sp.first_slot[s], sp.kid_chunks[s], sp.parent_blocks[s], word0[s]};
   }
 }
 
