@@ -236,7 +236,8 @@ IPM_API ipm_status ipm_set_options(ipm_ctx *ctx, const ipm_options *opts);
  * with relaxed amalgamation, supernode row structures, level sets and every
  * index map the numeric phase uses. Host only; no GPU work.
  * h_perm: length n, new->old, or NULL for the identity.
- * info (may be NULL) receives sizes and the workspace the numeric phase needs.
+ * info (may be NULL) receives sizes and the workspace the numeric phase needs (the
+ * scratch of solves shares the place of the factorisation's update matrices).
  * Errors: IPM_ERR_ARG if h_perm is not a permutation. */
 IPM_API ipm_status kkt_analyze(ipm_ctx *ctx, const int32_t *h_perm, ipm_symbolic_info *info);
 
@@ -279,10 +280,12 @@ IPM_API ipm_status kkt_factor(ipm_ctx *ctx, int32_t precision, int32_t *bad_col)
  * solutions of length n each, stored one after the other (column k at offset
  * k n), original numbering (may alias). Each right-hand side is solved and
  * refined on its own; info (may be NULL) receives the summed iterations and
- * the largest final relative residual.
+ * the largest final relative residual. d_x is also the running iterate, so after
+ * an error it holds an unspecified one.
  * Errors: IPM_ERR_ARG for nrhs < 1; IPM_ERR_STATE before kkt_factor;
- * IPM_ERR_NUMERIC if a residual misses accept_tol (the other right-hand sides
- * are still solved). */
+ * IPM_ERR_NUMERIC if a residual misses accept_tol or is not a number (the other
+ * right-hand sides are still solved); IPM_ERR_TIMEOUT if a bounded wait of the
+ * triangular solve, FP32 or FP64, ran out. */
 IPM_API ipm_status kkt_solve(ipm_ctx *ctx, const double *d_b, double *d_x, int32_t nrhs,
                      int32_t refine, ipm_solve_info *info);
 
@@ -332,7 +335,9 @@ typedef struct {
 
 typedef struct {
   int32_t precision;          /* IPM_FP64, or IPM_FP32: FP32 block factor and solves with
-                                 two FP64 refinement steps per solve */
+                                 two FP64 refinement steps per solve (on a GB300 about
+                                 three times slower than IPM_FP64: its kernel keeps 16
+                                 lanes per instance) */
   int32_t instances_per_cta;  /* 2, 4, 8 or 16. IPM_FP32: instances of one CTA (16 lanes
                                  each). IPM_FP64: one CTA per instance, and
                                  instances_per_cta * ctas instances in flight */
@@ -360,7 +365,9 @@ IPM_API ipm_status ipm_solve_batched(const ipm_mpc_batch *b, const ipm_mpc_confi
  * uneven horizons) for the precision in best->precision on this batch (one
  * warm-up solve, then the mean of two timed solves per shape) and writes the
  * fastest shape to best; h_ms (may be NULL) receives the 16 timings in that
- * order (float[16]). */
+ * order (float[16]). IPM_FP64 knows its own grid (ctas = 0): only instances_per_cta
+ * * ctas counts there, every shape tried is past what the GPU holds at once, and the
+ * timings differ by their scatter. */
 IPM_API ipm_status ipm_mpc_autotune(const ipm_mpc_batch *b, void *d_work, size_t bytes, double tol,
                                     int32_t max_iter, void *stream, double *d_z, double *d_obj,
                                     double *d_kkt, int32_t *d_iters, int32_t *d_status,

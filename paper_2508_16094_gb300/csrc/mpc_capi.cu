@@ -122,9 +122,10 @@ ipm_status ipm_mpc_autotune(const ipm_mpc_batch *b, void *d_work, size_t bytes, 
                             ipm_mpc_config *best, float *h_ms) {
   if (!best) return IPM_ERR_ARG;
   const int ipcs[4] = {2, 4, 8, 16};
-  // persistent CTAs per SM relative to the lane budget, in quarters: 1 and 2
+  // IPM_FP32: persistent CTAs per SM relative to the lane budget, in quarters: 1 and 2
   // leave fewer slots than a large batch has instances, so the queue balances
-  // the uneven horizons; 4 and 8 start every instance at once
+  // the uneven horizons; 4 and 8 start every instance at once. (IPM_FP64 runs a CTA per
+  // instance on a grid of its own: every shape here is past what the GPU holds.)
   const int occ[4] = {1, 2, 4, 8};
   cudaStream_t st = (cudaStream_t)stream;
   cudaEvent_t e0, e1;
