@@ -16,12 +16,13 @@ constexpr int kRedBlock = 256;
 
 // |v| and the larger of two of them on the integer pipe: an FP64 comparison
 // occupies GB300's FP64 unit as long as a multiply-add. The bits of a NaN compare above
-// those of infinity, so a maximum over values with a NaN among them is NaN.
+// those of infinity, so a maximum over values with a NaN among them is NaN; the comparison
+// leaves the sign bit out, which the compiler's |v| may leave set on a NaN.
 __device__ __forceinline__ double abs_bits(double v) {
   return __longlong_as_double(__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFll);
 }
 __device__ __forceinline__ double max_nonneg(double a, double b) {
-  return __double_as_longlong(a) > __double_as_longlong(b) ? a : b;
+  return (unsigned long long)__double_as_longlong(a) << 1 > (unsigned long long)__double_as_longlong(b) << 1 ? a : b;
 }
 // RED_MAX combines values >= 0 or NaN (identity 0)
 template <int OP> __device__ __forceinline__ double red_combine(double a, double b) {

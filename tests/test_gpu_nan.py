@@ -71,6 +71,25 @@ def test_nan_in_the_matrix(prec, refine):
     assert solve_status(ctx, b, torch.empty_like(b), refine) != OK
 
 
+@pytest.mark.parametrize("n,at", [(4, 0), (4, 3), (700, 300)])
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+@pytest.mark.parametrize("refine", [gb.IPM_REFINE_NONE, gb.IPM_REFINE_IR, gb.IPM_REFINE_PCG])
+def test_a_solution_past_the_largest_number(n, at, sign, refine):
+    # bounds only: K is diagonal, and one entry of the solution, 5 / 1e-308, overflows
+    ctx = gb.IpmContext(n, 0, np.zeros(1, np.int64), np.zeros(0, np.int32), np.zeros(n), np.ones(n),
+                        options=gb.default_options(storage_fp64=1))
+    ctx.kkt_analyze(None)
+    ctx.ipm_set_workspace()
+    D, b = np.ones(2 * n), np.ones((2, n))
+    D[at], D[n + at], b[1, at] = 1e-308, 0.0, 5.0 * sign
+    ctx.kkt_assemble(dev(np.zeros(1)), dev(D), 0.0)
+    ctx.kkt_factor(gb.IPM_FP64)
+    x, X = torch.empty(n, dtype=torch.float64, device="cuda"), torch.empty((2, n), dtype=torch.float64, device="cuda")
+    assert solve_status(ctx, dev(b[0]), x, refine) == OK
+    assert solve_status(ctx, dev(b[1]), x, refine) != OK
+    assert solve_status(ctx, dev(b), X, refine) != OK
+
+
 @pytest.mark.parametrize("prec", [gb.IPM_FP64, gb.IPM_TF32X3])
 @pytest.mark.parametrize("what", ["val", "b", "c"])
 def test_nan_in_a_problem(prec, what):
