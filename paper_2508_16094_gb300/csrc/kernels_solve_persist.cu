@@ -239,7 +239,7 @@ __device__ __forceinline__ unsigned *f_part(const PsArgs<T> &A, int slot) {
   return A.flags + 32 + slot;
 }
 // per front: chunks of rows below its children that are done (the children's
-// update vectors are complete once it reaches ps_kid_chunks[front])
+// update vectors are complete once it reaches the record's kid_chunks)
 template <typename T>
 __device__ __forceinline__ unsigned *f_tvec(const PsArgs<T> &A, int front) {
   return A.flags + 32 + A.nslot + front;
